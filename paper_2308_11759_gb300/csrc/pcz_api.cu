@@ -426,17 +426,30 @@ BoxJob make_job(const pc_streams* s, int k0, int k, const int64_t lo[3], const i
   J.nbox = J.bn[0] * J.bn[1] * J.bn[2];
   J.k0 = k0;
   J.k = k;
-  J.umult = retrieve_unit_mult(k - k0);
   if (J.nbox < (1ll << 32)) {
     J.dv_bn0 = div_magic((uint64_t)J.bn[0]);
     J.dv_bn1 = div_magic((uint64_t)J.bn[1]);
   }
-  J.dv_ub = div_magic(16ull * (uint64_t)J.umult);
   J.out = d_out;
   return J;
 }
 
-int64_t job_units(const BoxJob& J) { return (J.nbox + 16 * J.umult - 1) / (16 * J.umult); }
+// Cuts the jobs of one launch into units (retrieve_unit_mult on the launch's
+// brick total) and places them one after the other; returns the units.  Units
+// of 1D/2D jobs are bricks.
+int64_t place_job_list(BoxJob* jobs, int nj, int dtype, int ndims) {
+  int64_t bricks = 0, units = 0;
+  for (int j = 0; j < nj; ++j) bricks += jobs[j].nbox;
+  for (int j = 0; j < nj; ++j) {
+    BoxJob& J = jobs[j];
+    J.unit_begin = units;
+    J.umult = retrieve_unit_mult(dtype, J.k - J.k0, J.nbox, bricks);
+    const int64_t ub = 16 * (int64_t)J.umult;
+    J.dv_ub = div_magic((uint64_t)ub);
+    units += ndims == 3 ? (J.nbox + ub - 1) / ub : J.nbox;
+  }
+  return units;
+}
 
 // Runs Algorithm 2 on the box: components k0+1..k added into d_out (device).
 pc_status run_retrieve(const pc_streams* s, int k0, int k, const int64_t lo[3], const int64_t hi[3], void* d_out,
@@ -453,7 +466,7 @@ pc_status run_retrieve(const pc_streams* s, int k0, int k, const int64_t lo[3], 
   R.job0 = make_job(s, k0, k, lo, hi, d_out);
   R.jobs = nullptr;
   R.njobs = 1;
-  R.nunits = job_units(R.job0);
+  R.nunits = place_job_list(&R.job0, 1, s->dtype, s->ndims);
   R.write = write;
   R.err = s->d_err;
   R.grid = retrieve_grid(s->dtype, s->ndims, R.nunits);
@@ -478,7 +491,7 @@ pc_status pcz::check_box(const pc_streams* s, const pc_box* box, int64_t lo[3], 
 BoxJob pcz::make_box_job(const pc_streams* s, int k0, int k, const int64_t lo[3], const int64_t hi[3], void* out) {
   return make_job(s, k0, k, lo, hi, out);
 }
-int64_t pcz::box_job_units(const BoxJob& J) { return job_units(J); }
+int64_t pcz::place_jobs(BoxJob* jobs, int nj, int dtype, int ndims) { return place_job_list(jobs, nj, dtype, ndims); }
 double pcz::value_of_bits(uint64_t b, pc_dtype dt) { return bits_to_double(b, dt); }
 int pcz::floor_log2_of(double tau) { return floor_log2_bits(tau); }
 uint64_t pcz::tau_bits_of(double tau, pc_dtype dt) { return tau_threshold_bits(tau, dt); }

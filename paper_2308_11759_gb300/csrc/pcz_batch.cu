@@ -975,8 +975,6 @@ pc_status pc_retrieve_batch(int nq, const pc_streams* const* s, const int* k, co
     }
     Group& G = groups[s[q]->dtype == PC_F64][s[q]->ndims];
     BoxJob J = make_box_job(s[q], 0, k[q], lo, hi, d_out[q]);
-    J.unit_begin = G.units;
-    G.units += s[q]->ndims == 3 ? box_job_units(J) : J.nbox;  // 1D/2D units are bricks
     G.jobs.push_back(J);
     err = s[q]->d_err;
   }
@@ -985,6 +983,7 @@ pc_status pc_retrieve_batch(int nq, const pc_streams* const* s, const int* k, co
       Group& G = groups[t][d];
       if (G.jobs.empty()) continue;
       const int dt = t ? PC_F64 : PC_F32;
+      G.units = place_jobs(G.jobs.data(), (int)G.jobs.size(), dt, d);
       void* mem = nullptr;
       const size_t jb = align256(sizeof(BoxJob) * G.jobs.size());
       const size_t spill = d == 3 ? 8 * retrieve_spill_words(dt, 3, retrieve_grid(dt, 3, G.units)) : 0;

@@ -68,9 +68,10 @@ size_t dtype_size(pc_dtype t);
 // Box of a query in element units (whole field when box is null); PC_ERR_ARG
 // when it is empty or leaves the field.
 pc_status check_box(const pc_streams* s, const pc_box* box, int64_t lo[3], int64_t hi[3]);
-// Retrieval job over a box (components k0+1..k into out); unit_begin = 0.
+// Retrieval job over a box (components k0+1..k into out), not yet cut into
+// units; place_jobs does that for the jobs of one launch and returns its units.
 BoxJob make_box_job(const pc_streams* s, int k0, int k, const int64_t lo[3], const int64_t hi[3], void* out);
-int64_t box_job_units(const BoxJob& J);
+int64_t place_jobs(BoxJob* jobs, int nj, int dtype, int ndims);
 // Exact double of a T bit pattern.
 double value_of_bits(uint64_t b, pc_dtype dt);
 // floor(log2 tau) and the bit pattern of the largest T not above tau.

@@ -169,10 +169,10 @@ uint32_t check_word_batch(int reset);
 void set_last_error(const char* msg);
 
 // CTAs of a persistent retrieval launch over nunits units, brick pairs per
-// warp of a unit for ncomp components, and the spill words a launch of grid
-// CTAs needs.
+// warp of a unit for a job of nbox bricks and ncomp components in a launch of
+// `bricks` bricks, and the spill words a launch of grid CTAs needs.
 int retrieve_grid(int dtype, int ndims, int64_t nunits);
-int retrieve_unit_mult(int ncomp);
+int retrieve_unit_mult(int dtype, int ncomp, int64_t nbox, int64_t bricks);
 size_t retrieve_spill_words(int dtype, int ndims, int grid);
 
 // Finite-difference derivatives (pcz_fd.cu): omega_z = v_x - u_y and the

@@ -34,6 +34,7 @@
 // plane and converted to double without the FP64 pipe, which the partial-sum
 // adds keep busy; this form is a second instantiation of the kernel, used
 // when a brick decodes at least 3 components.
+#include <algorithm>
 #include <type_traits>
 
 #include "pcz_device.cuh"
@@ -702,7 +703,7 @@ __global__ void __launch_bounds__(kRThreads, 3) k_retrieve3(const RetrieveParams
       parse_round<T>(J, R.err, unit0, ub, J.k0, nc, &s_next, slots, meta, spill, lut, order, hist);
       __syncthreads();
       for (int q = 0; q < umult; ++q) {
-        const int uA = 2 * (umult * warp + q);  // unit-local index of the pair's first brick
+        const int uA = 2 * (kRWarps * q + warp);  // unit-local index of the pair's first brick
         const BrickLane BL = brick_lane<sizeof(T) == 8>(J, unit0 + uA + h, t);
         T xt[4];
         start_sum<T>(J, R.write, BL, xt);
@@ -759,15 +760,6 @@ __global__ void __launch_bounds__(kRThreads, 3) k_retrieve3(const RetrieveParams
   }
 }
 
-// Brick pairs per warp in a unit (a unit is 16 * umult bricks): as many as
-// keep one round's parse tasks (bricks x components) within kTasks, two per
-// thread, so that warps can steal work; several rounds use 2 pairs per warp.
-int retrieve_unit_mult(int ncomp) {
-  if (ncomp <= 0 || ncomp > kRound) return 2;
-  const int m = (kTasks / 16) / ncomp;
-  return m < 1 ? 1 : m;
-}
-
 template <typename T>
 static int retrieve_grid_t(int64_t nunits) {
   // CTAs that fit on the GPU at once, queried once per type (a function-local
@@ -785,6 +777,22 @@ static int retrieve_grid_t(int64_t nunits) {
     return (int64_t)(ps < 1 ? 1 : ps) * (sms < 1 ? 1 : sms);
   }();
   return (int)(nunits < g ? (nunits > 0 ? nunits : 1) : g);
+}
+
+// Brick pairs per warp in a unit (a unit is 16 * umult bricks): as many as
+// keep one round's parse tasks (bricks x components) within kTasks, two per
+// thread, so that warps can steal work -- but no more than leave every CTA
+// that fits on the GPU two units of the launch's bricks, and no more than the
+// job fills.  A 64^3 box at k = 4 (4096 bricks) in units of 128 ran on 32 of
+// 456 CTAs: 43.6 us, in units of 16 26 us; four reconstructions of a 64^3
+// field took 240 us, now 90 us.  (One, two and four units per CTA measured
+// alike.)  Several rounds use 2 pairs per warp.
+int retrieve_unit_mult(int dtype, int ncomp, int64_t nbox, int64_t bricks) {
+  if (ncomp <= 0 || ncomp > kRound) return 2;
+  const int64_t fit = dtype == 1 ? retrieve_grid_t<float>(INT64_MAX) : retrieve_grid_t<double>(INT64_MAX);
+  const int64_t most = std::max((kTasks / 16) / ncomp, 1);
+  const int64_t share = bricks / (16 * fit * 2);
+  return (int)std::max<int64_t>(1, std::min(std::min(most, share), (nbox + 15) / 16));
 }
 
 int retrieve_grid(int dtype, int ndims, int64_t nunits) {

@@ -347,17 +347,15 @@ cudaError_t issue_batch(pc_server* S, Slot& sl, const std::vector<int>& others) 
         e = cudaStreamWaitEvent(sl.st, S->slots[o].done, 0);
         if (e != cudaSuccess) return e;
       }
-  int64_t nunits = 0, nitems = 0;
+  int64_t nitems = 0;
   for (int j = 0; j < nj; ++j) {
     const Query& q = sl.qs[j];
     const ServeField& F = S->fields[q.field];
     BoxJob J = make_box_job(F.s, 0, q.k, q.lo, q.hi, S->arena_mem + sl.offs[j]);
-    J.unit_begin = nunits;
     if (cache) {
       J.cache = F.cache;
       J.level = F.level;
     }
-    nunits += box_job_units(J);
     sl.h_jobs[j] = J;
     CacheAux A;
     A.cache = F.cache;
@@ -369,6 +367,7 @@ cudaError_t issue_batch(pc_server* S, Slot& sl, const std::vector<int>& others) 
     sl.h_aux[j] = A;
     nitems += J.nbox;
   }
+  const int64_t nunits = place_jobs(sl.h_jobs, nj, dt, 3);
   e = cudaMemcpyAsync(sl.d_jobs, sl.h_jobs, sizeof(BoxJob) * nj, cudaMemcpyHostToDevice, sl.st);
   if (e == cudaSuccess && cache)
     e = cudaMemcpyAsync(sl.d_aux, sl.h_aux, sizeof(CacheAux) * nj, cudaMemcpyHostToDevice, sl.st);

@@ -1,0 +1,94 @@
+"""Kernel variants and dispatch rules at the sizes where they change: against
+the oracle, numpy or the general path, bit for bit."""
+import numpy as np
+import pytest
+
+import synth_fields as S
+from oracle import derivatives as D
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+
+@pytest.fixture(scope="module")
+def P():
+    import paper_2308_11759_gb300 as pcz
+
+    pcz.lib()
+    return pcz
+
+
+def _bits(a):
+    a = np.ascontiguousarray(a)
+    return a.view(np.uint32 if a.dtype == np.float32 else np.uint64)
+
+
+@pytest.mark.parametrize("dtype", [np.float32, np.float64])
+@pytest.mark.parametrize("n", [1, 2, 3, 5, 17, 1023, 4097, 100003])
+@pytest.mark.parametrize("off", [0, 1, 3])
+def test_range_of_any_length_and_alignment(P, dtype, n, off):
+    rng = np.random.default_rng(1000 * n + off)
+    x = (rng.standard_normal(n) * 2.0 ** rng.integers(-60, 60, n)).astype(dtype)
+    buf = torch.empty(n + off, dtype=torch.float32 if dtype == np.float32 else torch.float64, device="cuda")
+    view = buf[off:]
+    for at in (0, n // 2, n - 1):  # an extreme at the head, in the middle and at the tail
+        for sign in (1, -1):
+            y = x.copy()
+            y[at] = sign * dtype(3e30)
+            view.copy_(torch.from_numpy(y))
+            assert P.field_range(view) == (float(y.min()), float(y.max()))
+        for bad in (np.inf, -np.inf, np.nan, -np.nan):
+            y = x.copy()
+            y[at] = bad
+            view.copy_(torch.from_numpy(y))
+            with pytest.raises(P.PczError) as e:
+                P.field_range(view)
+            assert e.value.name == "PC_ERR_NONFINITE"
+
+
+@pytest.mark.parametrize("n", [1, 3, 8])
+def test_units_of_every_size_give_the_same(P, n):
+    # 128 x 130 x 127: enough bricks for units of several pairs per warp; the
+    # sub-boxes below it take smaller ones
+    x = torch.from_numpy(S.powerlaw((127, 130, 128), seed=77, dtype=np.float32)).cuda()
+    st = P.compress(x, P.field_tau_schedule(x, "decade", n))
+    for k in {1, n}:
+        full = st.retrieve(k=k)
+        for lo, hi in (([0, 0, 0], [64, 130, 128]), ([64, 0, 0], [127, 130, 128]), ([3, 5, 7], [4, 6, 8]),
+                       ([1, 2, 3], [40, 39, 41])):
+            part = st.retrieve(k=k, box=(lo, hi))
+            sl = tuple(slice(a, b) for a, b in zip(lo, hi))
+            assert torch.equal(part, full[sl])
+        boxes = [([0, 0, 0], [127, 130, 128]), ([100, 100, 100], [101, 102, 103]), ([8, 8, 8], [72, 72, 72])]
+        outs = P.retrieve_batch([st] * 3, [k] * 3, boxes)
+        for (lo, hi), o in zip(boxes, outs):
+            assert torch.equal(o, full[tuple(slice(a, b) for a, b in zip(lo, hi))])
+
+
+@pytest.mark.parametrize("h", [0.5, 1.0, 2.0 ** -500, 2.0 ** 400, 0.3])
+def test_derivatives_outside_the_normal_range(P, h):
+    # zeros, subnormals, values near the largest and infinities beside ordinary
+    # ones: the float64 kernels scale exponent fields and redo such values
+    shape = (9, 11, 70)
+    rng = np.random.default_rng(5)
+    def field():
+        f = rng.standard_normal(shape)
+        pick = rng.integers(0, 12, shape)
+        f[pick == 0] = 0.0
+        f[pick == 1] = -0.0
+        f[pick == 2] *= 2.0 ** -1060
+        f[pick == 3] *= 2.0 ** 1020
+        f[(pick == 4) & (rng.random(shape) < 0.1)] = np.inf
+        f[:, 4:6] = 1.25  # equal neighbours: exact zeros
+        return f
+    u, v = field(), field()
+    with np.errstate(all="ignore"):
+        want = [D.vorticity_z(u, v, h)] + [D.second(u, a, h) for a in range(3)]
+    ud, vd = torch.from_numpy(u).cuda(), torch.from_numpy(v).cuda()
+    got = [P.fd_vorticity_z(ud, vd, h)] + [P.fd_second(ud, a, h) for a in range(3)]
+    for w, g in zip(want, got):
+        g = g.cpu().numpy()
+        nan = np.isnan(w)
+        assert np.array_equal(nan, np.isnan(g))
+        assert np.array_equal(_bits(w)[~nan], _bits(g)[~nan])
