@@ -45,6 +45,7 @@ struct Ar<float> {
   static __device__ __forceinline__ float div(float a, float b) { return __fdiv_rn(a, b); }
   // x * 2^k, with p = 2^k
   static __device__ __forceinline__ float mul2k(float x, int, float p) { return __fmul_rn(x, p); }
+  static __device__ __forceinline__ float shift2k(float x, int, float p, bool&) { return __fmul_rn(x, p); }
 };
 template <>
 struct Ar<double> {
@@ -62,6 +63,21 @@ struct Ar<double> {
     if (e != 0 && e != 0x7ff && e + k >= 1 && e + k <= 2046) return __longlong_as_double(b + ((long long)k << 52));
     return __dmul_rn(x, p);
   }
+  // mul2k without the multiplication: sets `rare` where the exponent field
+  // alone does not give the product (the caller then redoes its values with
+  // mul2k).  A multiplication predicated off still passes through the FP64
+  // pipe, so a fallback beside the fast path costs as much as using it: the
+  // interior loops of the vorticity kernel issued 6.35 FP64 instructions per
+  // value for 3 subtractions.
+  static __device__ __forceinline__ double shift2k(double x, int k, double, bool& rare) {
+    const int hi = __double2hiint(x), lo = __double2loint(x);
+    const int e = hi & 0x7ff00000;  // 0 for zeros and subnormals
+    const int least = max(1, 1 - k) << 20, most = min(2046, 2046 - k) << 20;
+    const bool zero = ((hi & 0x7fffffff) | lo) == 0;
+    const bool in = e >= least && e <= most;
+    rare = rare || !(zero || in);
+    return __hiloint2double(zero ? hi : hi + k * (1 << 20), lo);
+  }
 };
 
 // Division by the denominator d (2h or h^2 in T): when d = 2^-k is a power of
@@ -72,6 +88,14 @@ struct Den {
   T d, inv;
   int pow2, k;
   __device__ __forceinline__ T apply(T x) const { return pow2 ? Ar<T>::mul2k(x, k, inv) : Ar<T>::div(x, d); }
+  // apply in the interior loops of a kernel built for POW2 or for the division
+  template <bool POW2>
+  __device__ __forceinline__ T fast(T x, bool& rare) const {
+    if constexpr (POW2)
+      return Ar<T>::shift2k(x, k, inv, rare);
+    else
+      return Ar<T>::div(x, d);
+  }
 };
 
 // First derivative at coordinate c of n along a line of stride s from p
@@ -89,6 +113,12 @@ template <typename T>
 __device__ __forceinline__ T second_inner(T fp, T f0, T fm, const Den<T>& hh) {
   using A = Ar<T>;
   return hh.apply(A::add(A::sub(fp, A::mul2k(f0, 1, T(2))), fm));
+}
+
+template <typename T, bool POW2>
+__device__ __forceinline__ T second_fast(T fp, T f0, T fm, const Den<T>& hh, bool& rare) {
+  using A = Ar<T>;
+  return hh.template fast<POW2>(A::add(A::sub(fp, A::shift2k(f0, 1, T(2), rare)), fm), rare);
 }
 
 template <typename T>
@@ -118,17 +148,43 @@ __device__ __forceinline__ Column column(int nx, int ny, int nz, int zchunk) {
   return c;
 }
 
-// omega_z = v_x - u_y.
+// The columns at the two ends of x of one tile row, by a CTA of their own
+// (the last along x): 8 rows, 2 ends, 16 planes at a time.  Beside interior
+// columns an end column would make its whole warp run both code paths.
+// body(x, y, z) computes one value.
+template <typename F>
+__device__ __forceinline__ void x_ends(int nx, int ny, int nz, int zchunk, F body) {
+  const int y = blockIdx.y * kTileY + (threadIdx.x & 7), x = threadIdx.x & 8 ? nx - 1 : 0;
+  const int z0 = blockIdx.z * zchunk, z1 = min(nz, z0 + zchunk);
+  if (y >= ny) return;
+  for (int z = z0 + 2 * threadIdx.y + (threadIdx.x >> 4); z < z1; z += 2 * kTileY) body(x, y, z);
+}
+
+// omega_z = v_x - u_y at one value, by the general formulas.
 template <typename T>
+__device__ __noinline__ void vorticity_value(const T* __restrict__ u, const T* __restrict__ v, T* __restrict__ out,
+                                             int x, int y, int z, int nx, int ny, const Den<T>& h2) {
+  const int64_t i = ((int64_t)z * ny + y) * nx + x;
+  out[i] = Ar<T>::sub(first_at<T>(v + i, x, nx, 1, h2), first_at<T>(u + i, y, ny, nx, h2));
+}
+
+// omega_z = v_x - u_y.  float64 is bound by the FP64 pipe (3 subtractions per
+// value at 2 lanes per SM and clock) next to HBM: 384 x 384 x 256 527 us ->
+// 267 us.
+template <typename T, bool POW2>
 __global__ void __launch_bounds__(kTileX * kTileY) k_vorticity_z(const T* __restrict__ u, const T* __restrict__ v,
                                                                  T* __restrict__ out, int nx, int ny, int nz,
                                                                  int zchunk, Den<T> h2) {
+  if (blockIdx.x == gridDim.x - 1) {
+    x_ends(nx, ny, nz, zchunk, [&](int x, int y, int z) { vorticity_value<T>(u, v, out, x, y, z, nx, ny, h2); });
+    return;
+  }
   const Column c = column(nx, ny, nz, zchunk);
-  if (!c.ok) return;
+  if (!c.ok || c.x == 0 || c.x == nx - 1) return;
   const int64_t plane = (int64_t)nx * ny;
   const int64_t i0 = ((int64_t)c.z0 * ny + c.y) * nx + c.x;
   int z = c.z0;
-  if (c.x > 0 && c.x < nx - 1 && c.y > 0 && c.y < ny - 1) {
+  if (c.y > 0 && c.y < ny - 1) {
     // interior column: the loads of 4 planes are issued before any is used
     using A = Ar<T>;
     for (; z + 4 <= c.z1; z += 4) {
@@ -141,15 +197,16 @@ __global__ void __launch_bounds__(kTileX * kTileY) k_vorticity_z(const T* __rest
         up[j] = __ldg(u + i + j * plane + nx);
         um[j] = __ldg(u + i + j * plane - nx);
       }
+      bool rare = false;
 #pragma unroll
       for (int j = 0; j < 4; ++j)
-        out[i + j * plane] = A::sub(h2.apply(A::sub(vp[j], vm[j])), h2.apply(A::sub(up[j], um[j])));
+        out[i + j * plane] = A::sub(h2.template fast<POW2>(A::sub(vp[j], vm[j]), rare),
+                                    h2.template fast<POW2>(A::sub(up[j], um[j]), rare));
+      if (rare)
+        for (int j = 0; j < 4; ++j) vorticity_value<T>(u, v, out, c.x, c.y, z + j, nx, ny, h2);
     }
   }
-  for (; z < c.z1; ++z) {
-    const int64_t i = i0 + (int64_t)(z - c.z0) * plane;
-    out[i] = Ar<T>::sub(first_at<T>(v + i, c.x, nx, 1, h2), first_at<T>(u + i, c.y, ny, nx, h2));
-  }
+  for (; z < c.z1; ++z) vorticity_value<T>(u, v, out, c.x, c.y, z, nx, ny, h2);
 }
 
 // omega_z = v_x - u_y for float32 rows whose length is a multiple of 4 (and
@@ -213,12 +270,25 @@ __global__ void __launch_bounds__(kTileX * kTileY) k_vorticity_z4(const float* _
   }
 }
 
-// d2w/da2 along x (axis 0) or y (axis 1).
+// d2w/da2 at one value c of n along a line of stride s, by the general formulas.
 template <typename T>
+__device__ __noinline__ void second_value(const T* __restrict__ w, T* __restrict__ out, int64_t i, int c, int n,
+                                          int64_t s, const Den<T>& hh) {
+  out[i] = second_at<T>(w + i, c, n, s, hh);
+}
+
+// d2w/da2 along x (axis 0) or y (axis 1).
+template <typename T, bool POW2>
 __global__ void __launch_bounds__(kTileX * kTileY) k_second_xy(const T* __restrict__ w, T* __restrict__ out, int nx,
                                                                int ny, int nz, int zchunk, int axis, Den<T> hh) {
+  if (axis == 0 && blockIdx.x == gridDim.x - 1) {
+    x_ends(nx, ny, nz, zchunk, [&](int x, int y, int z) {
+      second_value<T>(w, out, ((int64_t)z * ny + y) * nx + x, x, nx, 1, hh);
+    });
+    return;
+  }
   const Column c = column(nx, ny, nz, zchunk);
-  if (!c.ok) return;
+  if (!c.ok || (axis == 0 && (c.x == 0 || c.x == nx - 1))) return;
   const int64_t plane = (int64_t)nx * ny;
   const int cc = axis == 0 ? c.x : c.y, n = axis == 0 ? nx : ny;
   const int64_t s = axis == 0 ? 1 : nx;
@@ -234,18 +304,19 @@ __global__ void __launch_bounds__(kTileX * kTileY) k_second_xy(const T* __restri
         f0[j] = __ldg(w + i + j * plane);
         fm[j] = __ldg(w + i + j * plane - s);
       }
+      bool rare = false;
 #pragma unroll
-      for (int j = 0; j < 4; ++j) out[i + j * plane] = second_inner<T>(fp[j], f0[j], fm[j], hh);
+      for (int j = 0; j < 4; ++j) out[i + j * plane] = second_fast<T, POW2>(fp[j], f0[j], fm[j], hh, rare);
+      if (rare)
+        for (int j = 0; j < 4; ++j) second_value<T>(w, out, i + j * plane, cc, n, s, hh);
     }
   }
-  for (; z < c.z1; ++z) {
-    const int64_t i = i0 + (int64_t)(z - c.z0) * plane;
-    out[i] = second_at<T>(w + i, cc, n, s, hh);
-  }
+  for (; z < c.z1; ++z) second_value<T>(w, out, i0 + (int64_t)(z - c.z0) * plane, cc, n, s, hh);
 }
 
 // d2w/dz2: the column's window w[z-1], w[z], w[z+1] stays in registers.
-template <typename T>
+// float64 384 x 384 x 256: 288 us -> 160 us.
+template <typename T, bool POW2>
 __global__ void __launch_bounds__(kTileX * kTileY) k_second_z(const T* __restrict__ w, T* __restrict__ out, int nx,
                                                               int ny, int nz, int zchunk, Den<T> hh) {
   const Column c = column(nx, ny, nz, zchunk);
@@ -254,11 +325,11 @@ __global__ void __launch_bounds__(kTileX * kTileY) k_second_z(const T* __restric
   const int64_t col = (int64_t)c.y * nx + c.x;
   int za = c.z0, zb = c.z1;  // the slice's interior planes [za, zb)
   if (za == 0) {             // the four-point ends
-    out[col] = second_at<T>(w + col, 0, nz, plane, hh);
+    second_value<T>(w, out, col, 0, nz, plane, hh);
     za = 1;
   }
   if (zb == nz) {
-    out[col + (int64_t)(nz - 1) * plane] = second_at<T>(w + col + (int64_t)(nz - 1) * plane, nz - 1, nz, plane, hh);
+    second_value<T>(w, out, col + (int64_t)(nz - 1) * plane, nz - 1, nz, plane, hh);
     zb = nz - 1;
   }
   if (za >= zb) return;
@@ -271,20 +342,17 @@ __global__ void __launch_bounds__(kTileX * kTileY) k_second_z(const T* __restric
     T wp[4];
 #pragma unroll
     for (int j = 0; j < 4; ++j) wp[j] = __ldg(p + o + (j + 1) * plane);
+    bool rare = false;
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-      q[o + j * plane] = second_inner<T>(wp[j], w0, wm, hh);
+      q[o + j * plane] = second_fast<T, POW2>(wp[j], w0, wm, hh, rare);
       wm = w0;
       w0 = wp[j];
     }
+    if (rare)
+      for (int j = 0; j < 4; ++j) second_value<T>(w, out, col + (int64_t)(z + j) * plane, z + j, nz, plane, hh);
   }
-  for (; z < zb; ++z) {
-    const int64_t o = (int64_t)(z - za) * plane;
-    const T wp = __ldg(p + o + plane);
-    q[o] = second_inner<T>(wp, w0, wm, hh);
-    wm = w0;
-    w0 = wp;
-  }
+  for (; z < zb; ++z) second_value<T>(w, out, col + (int64_t)z * plane, z, nz, plane, hh);
 }
 
 template <typename T>
@@ -302,7 +370,8 @@ Den<T> make_den(double h, int twice) {
 }
 
 // Grid of tiles, with z split so that about 16 CTAs per SM are launched.
-dim3 fd_grid(int nx, int ny, int nz, int* zchunk) {
+// ends: one more CTA along x, for the columns at the ends of x.
+dim3 fd_grid(int nx, int ny, int nz, bool ends, int* zchunk) {
   static const int sms = [] {  // once, thread-safe
     int dev = 0, n = 0;
     cudaGetDevice(&dev);
@@ -314,7 +383,7 @@ dim3 fd_grid(int nx, int ny, int nz, int* zchunk) {
   split = std::max<int64_t>(1, std::min<int64_t>(split, nz));
   *zchunk = (int)((nz + split - 1) / split);
   const int gz = (nz + *zchunk - 1) / *zchunk;
-  return dim3((unsigned)((nx + kTileX - 1) / kTileX), (unsigned)((ny + kTileY - 1) / kTileY), (unsigned)gz);
+  return dim3((unsigned)((nx + kTileX - 1) / kTileX + (ends ? 1 : 0)), (unsigned)((ny + kTileY - 1) / kTileY), (unsigned)gz);
 }
 
 }  // namespace
@@ -325,41 +394,45 @@ cudaError_t launch_fd_vorticity_z(int dtype, const void* u, const void* v, void*
   const dim3 block(kTileX, kTileY);
   const bool vec4 = dtype == 1 && nx % 4 == 0 && ((uintptr_t)u | (uintptr_t)v | (uintptr_t)out) % 16 == 0;
   if (vec4) {  // the tiles are 128 values wide
-    dim3 grid = fd_grid((int)(nx / 4), (int)ny, (int)nz, &zc);
+    dim3 grid = fd_grid((int)(nx / 4), (int)ny, (int)nz, false, &zc);
     k_vorticity_z4<<<grid, block, 0, st>>>((const float*)u, (const float*)v, (float*)out, (int)nx, (int)ny, (int)nz,
                                            zc, make_den<float>(h, 1));
     return cudaGetLastError();
   }
-  const dim3 grid = fd_grid((int)nx, (int)ny, (int)nz, &zc);
+  const dim3 grid = fd_grid((int)nx, (int)ny, (int)nz, true, &zc);
+  auto run = [&](auto one) {
+    using T = decltype(one);
+    const Den<T> D = make_den<T>(h, 1);
+    auto* kernel = D.pow2 ? &k_vorticity_z<T, true> : &k_vorticity_z<T, false>;
+    kernel<<<grid, block, 0, st>>>((const T*)u, (const T*)v, (T*)out, (int)nx, (int)ny, (int)nz, zc, D);
+  };
   if (dtype == 1)
-    k_vorticity_z<float><<<grid, block, 0, st>>>((const float*)u, (const float*)v, (float*)out, (int)nx, (int)ny,
-                                                 (int)nz, zc, make_den<float>(h, 1));
+    run(float());
   else
-    k_vorticity_z<double><<<grid, block, 0, st>>>((const double*)u, (const double*)v, (double*)out, (int)nx, (int)ny,
-                                                  (int)nz, zc, make_den<double>(h, 1));
+    run(double());
   return cudaGetLastError();
 }
 
 cudaError_t launch_fd_second(int dtype, const void* w, void* out, int64_t nx, int64_t ny, int64_t nz, int axis,
                              double h, cudaStream_t st) {
   int zc = 1;
-  const dim3 grid = fd_grid((int)nx, (int)ny, (int)nz, &zc);
+  const dim3 grid = fd_grid((int)nx, (int)ny, (int)nz, axis == 0, &zc);
   const dim3 block(kTileX, kTileY);
-  if (dtype == 1) {
-    if (axis == 2)
-      k_second_z<float><<<grid, block, 0, st>>>((const float*)w, (float*)out, (int)nx, (int)ny, (int)nz, zc,
-                                                make_den<float>(h, 0));
-    else
-      k_second_xy<float><<<grid, block, 0, st>>>((const float*)w, (float*)out, (int)nx, (int)ny, (int)nz, zc, axis,
-                                                 make_den<float>(h, 0));
-  } else {
-    if (axis == 2)
-      k_second_z<double><<<grid, block, 0, st>>>((const double*)w, (double*)out, (int)nx, (int)ny, (int)nz, zc,
-                                                 make_den<double>(h, 0));
-    else
-      k_second_xy<double><<<grid, block, 0, st>>>((const double*)w, (double*)out, (int)nx, (int)ny, (int)nz, zc, axis,
-                                                  make_den<double>(h, 0));
-  }
+  auto run = [&](auto one) {
+    using T = decltype(one);
+    const Den<T> D = make_den<T>(h, 0);
+    if (axis == 2) {
+      auto* kernel = D.pow2 ? &k_second_z<T, true> : &k_second_z<T, false>;
+      kernel<<<grid, block, 0, st>>>((const T*)w, (T*)out, (int)nx, (int)ny, (int)nz, zc, D);
+    } else {
+      auto* kernel = D.pow2 ? &k_second_xy<T, true> : &k_second_xy<T, false>;
+      kernel<<<grid, block, 0, st>>>((const T*)w, (T*)out, (int)nx, (int)ny, (int)nz, zc, axis, D);
+    }
+  };
+  if (dtype == 1)
+    run(float());
+  else
+    run(double());
   return cudaGetLastError();
 }
 
