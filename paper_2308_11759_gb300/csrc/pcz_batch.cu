@@ -58,10 +58,16 @@ __device__ __forceinline__ void find_item(const BatchParams* __restrict__ bp, in
   *nd_out = bp->slot_ndims[lo];
 }
 
-// 3D part of a batch: CTAs of 16 warps claim chunks of the 3D
+// CTAs per SM of the 3D kernel's two variants: the stand-alone kernel's, and
+// one fewer with more registers a thread.
+template <typename T>
+constexpr int batch3_ctas(int variant) {
+  return (sizeof(T) == 4 ? 4 : 3) - (variant == 2 ? 0 : 1);
+}
+
+// 3D part of a batch: CTAs of 4 warps claim chunks of the 3D
 // fields (one chunk of 32 bricks per item) and code each as pc_compress does.
-// MINB = CTAs per SM the variant is compiled for: 1 (up to 128 registers per
-// thread) or 2 (at most 64, two CTAs sharing an SM).
+// MINB = CTAs per SM the variant is compiled for.
 template <typename T, int MINB>
 __global__ void __launch_bounds__(kCompressThreads3, MINB) k_batch3(const BatchParams* __restrict__ bp) {
   extern __shared__ __align__(16) unsigned char smem[];
@@ -159,16 +165,24 @@ __global__ void __launch_bounds__(32 * W, sizeof(T) == 4 ? 16 / W : 1) k_batch_s
 
 // Both parts in one kernel: CTAs of 16 warps (up to 128 registers per thread)
 // claim items of one work list holding the 3D and the 1D/2D fields; a 3D item
-// takes the whole CTA, a 1D/2D item one chunk per warp at a time.  With one
-// queue the two kinds of work share the SMs to the end.
+// is 4 chunks, one for every 4 warps, a 1D/2D item one chunk per warp at a
+// time.  With one queue the two kinds of work share the SMs to the end.
+constexpr int kMixedThreads = 512;
+constexpr int kMixedGroups = kMixedThreads / kCompressThreads3;
+
 template <typename T>
-__global__ void __launch_bounds__(kCompressThreads3, 1) k_batch_mixed(const BatchParams* __restrict__ bp) {
+__host__ __device__ constexpr size_t mixed_group_smem() {
+  return (compress_smem3<T>() + 127) / 128 * 128;
+}
+
+template <typename T>
+__global__ void __launch_bounds__(kMixedThreads, 1) k_batch_mixed(const BatchParams* __restrict__ bp) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ CompressParams sP;
   __shared__ long long s_first, s_chunk0;
   __shared__ int s_field, s_nchunks, s_ndims;
   constexpr int PW = (int)(sizeof(CompressParams) / 8);
-  constexpr int WARPS = kCompressThreads3 / 32;
+  constexpr int WARPS = kMixedThreads / 32;
   const int tid = threadIdx.x, warp = tid >> 5;
   const int64_t nitems = bp->nitems;
   const int per = bp->per_fetch;
@@ -194,13 +208,14 @@ __global__ void __launch_bounds__(kCompressThreads3, 1) k_batch_mixed(const Batc
       {
         const uint64_t* src = reinterpret_cast<const uint64_t*>(bp->fields + s_field);
         uint64_t* dst = reinterpret_cast<uint64_t*>(&sP);
-        for (int w = tid; w < PW; w += kCompressThreads3) dst[w] = src[w];
+        for (int w = tid; w < PW; w += kMixedThreads) dst[w] = src[w];
       }
       __syncthreads();
       const int64_t c0 = s_chunk0;
       const int nch = s_nchunks;
       if (s_ndims == 3) {
-        compress3_chunk<T>(sP, c0, smem);
+        const int g = warp / kWarps3;
+        if (g < nch) compress3_chunk<T>(sP, c0 + g, smem + g * mixed_group_smem<T>(), 1 + g);
       } else if (s_ndims == 2) {
         uint32_t* cbuf = reinterpret_cast<uint32_t*>(smem) + (size_t)warp * chunk_words_small<T, 2>();
         for (int c = warp; c < nch; c += WARPS) compress_small_chunk<T, 2>(sP, c0 + c, cbuf);
@@ -214,8 +229,8 @@ __global__ void __launch_bounds__(kCompressThreads3, 1) k_batch_mixed(const Batc
 
 template <typename T>
 __host__ __device__ constexpr size_t batch_mixed_smem() {
-  const size_t a = compress_smem3<T>();
-  const size_t b = (size_t)(kCompressThreads3 / 32) * chunk_words_small<T, 2>() * 4;
+  const size_t a = kMixedGroups * mixed_group_smem<T>();
+  const size_t b = (size_t)(kMixedThreads / 32) * chunk_words_small<T, 2>() * 4;
   return a > b ? a : b;
 }
 
@@ -229,7 +244,7 @@ static int batch_mixed_grid_t() {
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     cudaFuncSetAttribute(k_batch_mixed<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)batch_mixed_smem<T>());
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_batch_mixed<T>, kCompressThreads3, batch_mixed_smem<T>()) !=
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_batch_mixed<T>, kMixedThreads, batch_mixed_smem<T>()) !=
         cudaSuccess) {
       cudaGetLastError();
       per = 1;
@@ -246,7 +261,7 @@ int compress_batch_mixed_grid(int dtype) { return dtype == 1 ? batch_mixed_grid_
 
 cudaError_t launch_compress_batch_mixed(int dtype, const BatchParams* d_bp, int grid, cudaStream_t s) {
   if (dtype != 1) return cudaErrorNotSupported;
-  k_batch_mixed<float><<<grid, kCompressThreads3, batch_mixed_smem<float>(), s>>>(d_bp);
+  k_batch_mixed<float><<<grid, kMixedThreads, batch_mixed_smem<float>(), s>>>(d_bp);
   return cudaGetLastError();
 }
 
@@ -294,8 +309,8 @@ static int batch_small_grid_t() {
 uint32_t check_word_batch(int reset) { return read_check_word(reset); }
 
 int compress_batch_grid(int dtype, int minb) {
-  if (dtype == 1) return minb == 2 ? batch3_grid_t<float, 2>() : batch3_grid_t<float, 1>();
-  return minb == 2 ? batch3_grid_t<double, 2>() : batch3_grid_t<double, 1>();
+  if (dtype == 1) return minb == 2 ? batch3_grid_t<float, batch3_ctas<float>(2)>() : batch3_grid_t<float, batch3_ctas<float>(1)>();
+  return minb == 2 ? batch3_grid_t<double, batch3_ctas<double>(2)>() : batch3_grid_t<double, batch3_ctas<double>(1)>();
 }
 
 int compress_batch_small_grid(int dtype, int warps) {
@@ -313,14 +328,14 @@ int compress_batch_small_grid(int dtype, int warps) {
 cudaError_t launch_compress_batch(int dtype, int minb, const BatchParams* d_bp, int grid, cudaStream_t s) {
   if (dtype == 1) {
     if (minb == 2)
-      k_batch3<float, 2><<<grid, kCompressThreads3, compress_smem3<float>(), s>>>(d_bp);
+      k_batch3<float, batch3_ctas<float>(2)><<<grid, kCompressThreads3, compress_smem3<float>(), s>>>(d_bp);
     else
-      k_batch3<float, 1><<<grid, kCompressThreads3, compress_smem3<float>(), s>>>(d_bp);
+      k_batch3<float, batch3_ctas<float>(1)><<<grid, kCompressThreads3, compress_smem3<float>(), s>>>(d_bp);
   } else {
     if (minb == 2)
-      k_batch3<double, 2><<<grid, kCompressThreads3, compress_smem3<double>(), s>>>(d_bp);
+      k_batch3<double, batch3_ctas<double>(2)><<<grid, kCompressThreads3, compress_smem3<double>(), s>>>(d_bp);
     else
-      k_batch3<double, 1><<<grid, kCompressThreads3, compress_smem3<double>(), s>>>(d_bp);
+      k_batch3<double, batch3_ctas<double>(1)><<<grid, kCompressThreads3, compress_smem3<double>(), s>>>(d_bp);
   }
   return cudaGetLastError();
 }
@@ -511,7 +526,7 @@ void set_schedule(pc_batch* B, const Schedule& sc) {
     const int base = list * F;
     for (int f : ord) {
       if (sc.ctas3 == 0 ? list == 1 : (B->ndims[f] == 3) != (list == 0)) continue;
-      const int w = B->ndims[f] == 3 ? 1 : sc.warps_small * sc.chunks_per_warp;
+      const int w = B->ndims[f] != 3 ? sc.warps_small * sc.chunks_per_warp : sc.ctas3 == 0 ? kMixedGroups : 1;
       B->h_slot_field[base + ns] = f;
       B->h_slot_width[base + ns] = w;
       B->h_slot_ndims[base + ns] = B->ndims[f];

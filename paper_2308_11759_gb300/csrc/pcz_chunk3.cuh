@@ -15,31 +15,70 @@
 
 namespace pcz {
 
-static __constant__ PermTable kPerm3 = make_perm(64);
+// Rank of each brick position in coded order (R8).
+constexpr PermTable make_rank() {
+  const PermTable perm = make_perm(64);
+  PermTable t{};
+  for (int r = 0; r < 64; ++r) t.pos[perm.pos[r]] = (int8_t)r;
+  return t;
+}
+static __constant__ PermTable kRank3 = make_rank();
 
-// Largest bit string of one brick and component: CODED with every plane
-// non-empty (each plane at most 2N + 1 bits) plus the header.
+// Largest bit string of one brick and component: the header, at most one
+// verbatim or run bit per coefficient and plane, and at most one test bit per
+// coefficient plus one closing test bit per plane (R11); RAW is shorter still.
 template <typename T>
 __host__ __device__ constexpr int max_brick_bits3() {
-  return 2 + 3 + Fmt<T>::EBITS + Fmt<T>::P * (2 * 64 + 1);
+  return 2 + 3 + Fmt<T>::EBITS + 64 * Fmt<T>::P + 64 + Fmt<T>::P;
 }
 
 template <typename T>
-__host__ __device__ constexpr int chunk_buf_words3() {  // u32 words, rounded to whole u64 words
-  return ((kChunk * max_brick_bits3<T>() + 63) / 64) * 2;
+__host__ __device__ constexpr int chunk_buf_words3() {  // u32 words, whole 16-byte vectors
+  return ((kChunk * max_brick_bits3<T>() + 127) / 128) * 4;
 }
 
-constexpr int kCompressThreads3 = 512;
+constexpr int kCompressThreads3 = 128;  // threads that code a chunk: 4 warps of 8 bricks
+constexpr int kWarps3 = kCompressThreads3 / 32;
 
-// The per-plane tables of a warp's two bricks share the warp's brick buffer,
-// which is free from the end of the decode-back until the next component's
-// forward transform: the plane words (8 bytes per plane) for 64-bit
-// coefficients, the plane offsets and counts (4 bytes) for 32-bit ones --
-// whichever has the buffer's element size.
+// A warp's work area in shared memory, in u32 words.  Three uses follow one
+// another within a component:
+//  (a) exchanges between the z-planes and the y-planes of the lifting passes:
+//      16-byte vectors of 4 values along x (float64: two such sets, 2 values
+//      each), vector (y, z) of brick b at (b >> 1) * 38 + (b & 1) + 10 z + 2 y.
+//      Both directions are free of bank conflicts.
+//  (b) the digits in coded order, brick b from word 72 b (or 36 b as halves);
+//  (c) the plane words, brick b from word b * kPlaneStride: word j of the
+//      lane's 16 coefficients q at 4 j + q; a RAW brick's residual in their place.
 template <typename T>
-__host__ __device__ constexpr bool planes_in_brick_buffer() {
-  return sizeof(typename Fmt<T>::S) == 8;
+struct Area3 {
+  static constexpr int kSet = 38 * 4;                                     // vectors of one set of (a)
+  static constexpr int kWords = kSet * 4 * (int)(sizeof(T) / 4);
+  static constexpr int kPlaneStride = 16 * (int)sizeof(T) + 4;
+  static constexpr int kInfoStride = Fmt<T>::P + 4;                       // plane table, words per brick
+};
+
+// Group-test code of 8 coefficient bits (R11): each bit in turn, and after
+// each 1 the 1 of the next token's test bit.  Its length is 8 + popc(bits).
+struct SpreadTable {
+  uint16_t code[256];
+};
+constexpr SpreadTable make_spread() {
+  SpreadTable t{};
+  for (int v = 0; v < 256; ++v) {
+    unsigned code = 0, len = 0;
+    for (int j = 0; j < 8; ++j)
+      if ((v >> j) & 1) {
+        code |= 3u << len;
+        len += 2;
+      } else {
+        ++len;
+      }
+    t.code[v] = (uint16_t)code;
+  }
+  return t;
 }
+static __device__ const SpreadTable kSpread3 = make_spread();
+constexpr int kSpreadBytes = (int)sizeof(SpreadTable);
 
 // Bytes of the staging area in front of the rest (TMA-staged form only).
 template <typename T>
@@ -48,85 +87,191 @@ __host__ __device__ constexpr size_t staging_bytes3(bool staged) {
 }
 
 template <typename T>
-constexpr size_t compress_smem3(bool staged = false) {
-  using S = typename Fmt<T>::S;
+__host__ __device__ constexpr size_t compress_smem3(bool staged = false) {
   return staging_bytes3<T>(staged)
-         + (size_t)chunk_buf_words3<T>() * 4 * 2  // chunk bit buffers (two components in flight)
-         + (size_t)kChunk * 64 * sizeof(S)     // brick buffers, 128 elements per warp
-         + (planes_in_brick_buffer<T>() ? 0 : (size_t)kChunk * 64 * 8)  // plane words of every brick
-         + (planes_in_brick_buffer<T>() ? (size_t)kChunk * 64 * 4 : 0)  // plane offsets and counts
-         + 2 * 32 * 4 * 4                      // per component parity: lengths, modes, escalations, violations
-         + 16                                  // pool base of the two components in flight
-         + 2 * 32 * 8                          // per component parity and brick: bits of max |x - x~_i|
-         + 16;                                 // chunk bits of the two components in flight
+         + (size_t)chunk_buf_words3<T>() * 4                        // chunk bit buffer
+         + (size_t)kWarps3 * Area3<T>::kWords * 4                   // work areas
+         + (size_t)kChunk * Area3<T>::kInfoStride * 4               // plane offsets and counts
+         + (sizeof(T) == 8 ? (size_t)kChunk * 64 * sizeof(T) : 0)   // the chunk's values (float32: in registers)
+         + kSpreadBytes                                             // group-test code table
+         + 4 * 32 * 4                                               // lengths, modes, escalations, violations
+         + 32 * 8                                                   // per brick: bits of max |x - x~_i|
+         + 16;                                                      // pool base and chunk bits
 }
 
-// R11 group-test bits of one coefficient c that turns significant in plane
-// pc (its highest set bit, at or above the lowest coded plane): when n
-// coefficients are significant before pc and c >= n, c is a token of that
-// plane.  With k its rank among the plane's tokens (1-based), the group part
-// of the plane (which follows the n verbatim bits) holds c's 1 at c - n + k,
-// the next token's test bit right after it unless c is the plane's last
-// token (c + 1 == hi, hi one past the plane word's highest 1), and the
-// plane's first test bit at 0 (set by the token with k = 1).  Zeros (runs and
-// the closing test bit) need no write.  The two bits span at most two words.
-__device__ __forceinline__ void write_token(uint32_t* buf, uint32_t cap_bits, uint32_t group_base, uint64_t W,
-                                            int n, int c, int hi) {
-  const uint64_t before = W & low_mask64(c) & ~low_mask64(n);
-  const int k = 1 + __popcll((long long)before);
-  const uint32_t pos = group_base + (uint32_t)(c - n + k);
-  const bool two = c + 1 != hi;
-  if (PCZ_CHECK(pos + (two ? 2u : 1u) <= cap_bits, 0)) {
-    atomicOr(buf + (pos >> 5), (two ? 3u : 1u) << (pos & 31));
-    if (two && (pos & 31) == 31) atomicOr(buf + (pos >> 5) + 1, 1u);
-  }
-  if (k == 1 && PCZ_CHECK(group_base < cap_bits, 0)) atomicOr(buf + (group_base >> 5), 1u << (group_base & 31));
+// The barrier of the 4 warps that code a chunk (id 0 in CTAs of 4 warps).
+__device__ __forceinline__ void group_sync(int id) {
+  asm volatile("bar.sync %0, 128;" ::"r"(id) : "memory");
 }
 
-// Suffix scans of one round of 32 planes of a warp's two bricks (lane l =
-// plane base + l, coded in descending order): per brick, n before each plane
-// (max of the one-past-highest set position over the planes above), the
-// plane's own one-past-highest position and its bit offset.  The two bricks'
-// offsets share one scan in 16-bit halves (a brick's code is below 2^14 bits).
-template <int N>
-__device__ __forceinline__ void plane_scan2(uint64_t WA, bool actA, uint64_t WB, bool actB, int lane, int& cmaxA,
-                                            int& cmaxB, uint32_t& csum, int& nA, int& nB, int& hiA, int& hiB,
-                                            int& offA, int& offB) {
-  constexpr unsigned FULL = 0xffffffffu;
-  hiA = (actA && WA) ? 64 - __clzll((long long)WA) : 0;
-  hiB = (actB && WB) ? 64 - __clzll((long long)WB) : 0;
-  int vA = hiA, vB = hiB;
+// Bit transposes within a lane.  transpose16: word i holds 16 bits (planes) of
+// coefficient i in its low half and of coefficient i + 8 in its high half;
+// afterwards word j holds plane j of the 16 coefficients in its low half and
+// plane j + 8 in its high half.  transpose32: word i holds 32 bits of
+// coefficient i; afterwards word j holds planes j and j + 16.  Stages of 4, 2
+// and 1 exchange bit groups between two words with a shift and a logic op per
+// result; the stage of 8 is one byte permute per result.
+template <int N, int K>
+__device__ __forceinline__ void exchange_stage(uint32_t (&a)[N], uint32_t m) {
 #pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const int yA = __shfl_down_sync(FULL, vA, o);
-    const int yB = __shfl_down_sync(FULL, vB, o);
-    if (lane + o < 32) {
-      vA = max(vA, yA);
-      vB = max(vB, yB);
+  for (int i = 0; i < N; ++i)
+    if (!(i & K)) {
+      const uint32_t x = a[i], y = a[i + K];
+      a[i] = (x & m) | ((y << K) & ~m);
+      a[i + K] = ((x >> K) & m) | (y & ~m);
     }
-  }
-  int exA = __shfl_down_sync(FULL, vA, 1);
-  int exB = __shfl_down_sync(FULL, vB, 1);
-  if (lane == 31) exA = exB = 0;
-  nA = max(exA, cmaxA);
-  nB = max(exB, cmaxB);
-  const uint32_t len = (uint32_t)(actA ? plane_len<N>(WA, nA) : 0) | ((uint32_t)(actB ? plane_len<N>(WB, nB) : 0) << 16);
-  uint32_t sum = len;
+}
+__device__ __forceinline__ void transpose16(uint32_t (&a)[8]) {
 #pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const uint32_t y = __shfl_down_sync(FULL, sum, o);
-    if (lane + o < 32) sum += y;
+  for (int i = 0; i < 8; ++i) a[i] = __byte_perm(a[i], 0u, 0x3120);
+  exchange_stage<8, 4>(a, 0x0F0F0F0Fu);
+  exchange_stage<8, 2>(a, 0x33333333u);
+  exchange_stage<8, 1>(a, 0x55555555u);
+}
+__device__ __forceinline__ void transpose32_lane(uint32_t (&a)[16]) {
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const uint32_t x = a[i], y = a[i + 8];
+    a[i] = __byte_perm(x, y, 0x6240);
+    a[i + 8] = __byte_perm(x, y, 0x7351);
   }
-  const uint32_t off = sum - len + csum;
-  offA = (int)(off & 0xffffu);
-  offB = (int)(off >> 16);
-  cmaxA = max(cmaxA, __shfl_sync(FULL, vA, 0));
-  cmaxB = max(cmaxB, __shfl_sync(FULL, vB, 0));
-  csum += __shfl_sync(FULL, sum, 0);
+  exchange_stage<16, 4>(a, 0x0F0F0F0Fu);
+  exchange_stage<16, 2>(a, 0x33333333u);
+  exchange_stage<16, 1>(a, 0x55555555u);
 }
 
-// Byte m of a register of four packed shared-memory slots.
-__device__ __forceinline__ int slot_of(uint32_t packed, int m) { return (int)((packed >> (8 * m)) & 0xffu); }
+// |v| as an integer that orders like it (NaN above +inf above every finite
+// value): the bit pattern without its sign.  float64 masks the high word only:
+// masking the whole pattern is recognised as fabs and emitted on the FP64 pipe.
+__device__ __forceinline__ uint32_t magnitude(float v) { return __float_as_uint(v) & 0x7FFFFFFFu; }
+__device__ __forceinline__ uint64_t magnitude(double v) {
+  return ((uint64_t)((uint32_t)__double2hiint(v) & 0x7FFFFFFFu) << 32) | (uint32_t)__double2loint(v);
+}
+
+// The largest magnitude of a brick: over a lane's 16 values, then its 4 lanes.
+template <typename T>
+__device__ __forceinline__ typename Fmt<T>::U brick_max(const T* e) {
+  using U = typename Fmt<T>::U;
+  constexpr unsigned FULL = 0xffffffffu;
+  U m = magnitude(e[0]);
+#pragma unroll
+  for (int v = 1; v < 16; ++v) {
+    const U a = magnitude(e[v]);
+    m = a > m ? a : m;
+  }
+#pragma unroll
+  for (int o = 1; o <= 2; o <<= 1) {
+    const U a = __shfl_xor_sync(FULL, m, o);
+    m = a > m ? a : m;
+  }
+  return m;
+}
+
+// R4 padding of a brick in a lane's layout (value x + 4 y, plane z = q):
+// values past the field repeat the nearest in-field value along x, then y,
+// then z.  Every lane of the warp calls it.
+template <typename T>
+__device__ __forceinline__ void pad_brick(T* e, int nvx, int nvy, int nvz, int lane) {
+#pragma unroll
+  for (int y = 0; y < 4; ++y)
+#pragma unroll
+    for (int x = 1; x < 4; ++x)
+      if (x >= nvx) e[x + 4 * y] = e[x - 1 + 4 * y];
+#pragma unroll
+  for (int y = 1; y < 4; ++y)
+#pragma unroll
+    for (int x = 0; x < 4; ++x)
+      if (y >= nvy) e[x + 4 * y] = e[x + 4 * (y - 1)];
+  const int src = (lane & ~3) | min(lane & 3, nvz - 1);
+#pragma unroll
+  for (int v = 0; v < 16; ++v) e[v] = __shfl_sync(0xffffffffu, e[v], src);
+}
+
+// 4 values along x to and from the work area, in 16-byte vectors (`set`
+// vectors between a 64-bit line's two halves).
+__device__ __forceinline__ void put_line(uint4* a, int, const int32_t* v) {
+  *a = make_uint4((uint32_t)v[0], (uint32_t)v[1], (uint32_t)v[2], (uint32_t)v[3]);
+}
+__device__ __forceinline__ void get_line(const uint4* a, int, int32_t* v) {
+  const uint4 r = *a;
+  v[0] = (int32_t)r.x;
+  v[1] = (int32_t)r.y;
+  v[2] = (int32_t)r.z;
+  v[3] = (int32_t)r.w;
+}
+__device__ __forceinline__ void put_line(uint4* a, int set, const int64_t* v) {
+  longlong2* d = reinterpret_cast<longlong2*>(a);
+  d[0] = make_longlong2(v[0], v[1]);
+  d[set] = make_longlong2(v[2], v[3]);
+}
+__device__ __forceinline__ void get_line(const uint4* a, int set, int64_t* v) {
+  const longlong2* d = reinterpret_cast<const longlong2*>(a);
+  const longlong2 p = d[0], r = d[set];
+  v[0] = p.x;
+  v[1] = p.y;
+  v[2] = r.x;
+  v[3] = r.y;
+}
+
+// R7 on a warp's 8 bricks.  v: the lane's z-plane q (value x + 4 y) on entry;
+// on return its y-plane q of coefficients (coefficient x + 4 z).  One exchange
+// through the work area: a lane lifts along x and y in registers, then along z.
+template <typename S>
+__device__ __forceinline__ void lift_fwd_bricks(S* v, uint4* zw, uint4* yw, int set) {
+#pragma unroll
+  for (int y = 0; y < 4; ++y) lift_fwd(v[4 * y], v[4 * y + 1], v[4 * y + 2], v[4 * y + 3]);
+#pragma unroll
+  for (int x = 0; x < 4; ++x) lift_fwd(v[x], v[x + 4], v[x + 8], v[x + 12]);
+#pragma unroll
+  for (int y = 0; y < 4; ++y) put_line(zw + 2 * y, set, v + 4 * y);
+  __syncwarp();
+#pragma unroll
+  for (int z = 0; z < 4; ++z) get_line(yw + 10 * z, set, v + 4 * z);
+  __syncwarp();
+#pragma unroll
+  for (int x = 0; x < 4; ++x) lift_fwd(v[x], v[x + 4], v[x + 8], v[x + 12]);
+}
+
+// The inverse: coefficients of the lane's y-plane in, values of its z-plane out.
+template <typename S>
+__device__ __forceinline__ void lift_inv_bricks(S* v, uint4* zw, uint4* yw, int set) {
+#pragma unroll
+  for (int x = 0; x < 4; ++x) lift_inv(v[x], v[x + 4], v[x + 8], v[x + 12]);
+#pragma unroll
+  for (int z = 0; z < 4; ++z) put_line(yw + 10 * z, set, v + 4 * z);
+  __syncwarp();
+#pragma unroll
+  for (int y = 0; y < 4; ++y) get_line(zw + 2 * y, set, v + 4 * y);
+  __syncwarp();
+#pragma unroll
+  for (int x = 0; x < 4; ++x) lift_inv(v[x], v[x + 4], v[x + 8], v[x + 12]);
+#pragma unroll
+  for (int y = 0; y < 4; ++y) lift_inv(v[4 * y], v[4 * y + 1], v[4 * y + 2], v[4 * y + 3]);
+}
+
+// R6 and R13 for blocks whose scale is outside the common range, out of line.
+template <typename T>
+__device__ __noinline__ typename Fmt<T>::S quantize_any(typename Fmt<T>::U b, int s) {
+  return quantize<T>(b, s);
+}
+template <typename T>
+__device__ __noinline__ typename Fmt<T>::U dequantize_any(typename Fmt<T>::S q, int s) {
+  return dequantize_bits<T>(q, s);
+}
+
+// R6 for float64 in a block whose scale s lies in [-960, 1000] (c = 1078 - s):
+// q = sign(e) * ((the 53-bit significand << 3) >> r) with r = c - biased
+// exponent, which is at least 0 because |q| < 2^56.  A subnormal e, taken with
+// a hidden bit it does not have, is shifted out entirely (r >= 78).  c = 4096
+// gives 0 for every e.
+__device__ __forceinline__ int64_t quantize_f64_normal(double e, int c) {
+  const uint32_t hi = (uint32_t)__double2hiint(e), lo = (uint32_t)__double2loint(e);
+  const uint64_t m = ((uint64_t)((hi & 0xFFFFFu) | 0x100000u) << 32) | lo;
+  const int r = min(c - (int)((hi >> 20) & 0x7FFu), 63);
+  const int64_t a = (int64_t)((m << 3) >> r);
+  const int64_t sg = (int64_t)((int32_t)hi >> 31);
+  return (a ^ sg) - sg;
+}
 
 // Staging of a chunk's field values in shared memory with TMA (the
 // persistent construction kernel, pcz_compress.cu): when the field's rows of
@@ -213,16 +358,7 @@ __device__ __forceinline__ void staged_line(const T* xs, bool row_box, int slot,
   for (int m = 0; m < 4; ++m) v[m] = src[min(m, nvx - 1)];
 }
 
-// Algorithm 1 on every brick of index chunk `chunk` of a 3D field, all
-// components, by the whole CTA (kCompressThreads3 threads); smem holds
-// compress_smem3<T>(map != nullptr) bytes, 128-byte aligned.  With a tensor
-// map, xs (= smem) holds the chunk's field values staged by TMA (row layout when
-// row_box, brick layout otherwise): each lane reads its line from there, and
-// after a CTA barrier thread 0 starts the copy of chunk `next` (if below
-// nchunks) into xs on barrier `bar`, so that it lands while this chunk is
-// coded.  Without a tensor map each lane loads its line from the field with
-// vector loads.  Every thread of the CTA must call it.
-// Copies one component's finished chunk from its shared buffer to the pool
+// Copies a component's finished chunk from its shared buffer to the pool
 // (base ~0: the pool was too small) and clears the buffer for reuse.
 __device__ __forceinline__ void append_chunk(const CompressParams& P, uint32_t* buf, unsigned long long base,
                                              int chunk_bits, int tid) {
@@ -234,52 +370,64 @@ __device__ __forceinline__ void append_chunk(const CompressParams& P, uint32_t* 
   }
 }
 
+// Algorithm 1 on every brick of index chunk `chunk` of a 3D field, all
+// components, by 4 warps (barrier `bar_id`); smem holds compress_smem3<T>(map
+// != nullptr) bytes, 128-byte aligned.  With a tensor map, xs (= smem) holds
+// the chunk's field values staged by TMA (row layout when row_box, brick layout
+// otherwise): each lane reads its lines from there, and after a barrier thread
+// 0 starts the copy of chunk `next` (if below nchunks) into xs on barrier
+// `bar`, so that it lands while this chunk is coded.  Without a tensor map each
+// lane loads its lines from the field with vector loads.  Every thread of the
+// 4 warps must call it.
+//
+// A warp codes 8 bricks, 4 lanes each; lane q of a brick holds the z-plane q
+// (16 values), and after the forward transform the coefficients of the y-plane
+// q.  The kernel is bound by instruction issue, and this split spends the
+// fewest: both in-plane lifting passes run in registers, the bits are
+// transposed in registers, reductions over a brick take two shuffles, and what
+// a component costs per warp (votes, scans, the barrier) is shared by 512
+// values.  With 16 lanes per brick and 4 values per lane, as before, it took
+// 582 (float32) and 997 (float64) warp instructions per brick and component.
 template <typename T>
 __device__ __forceinline__ void compress3_chunk(const CompressParams& P, int64_t chunk, unsigned char* smem,
-                                                const CUtensorMap* map = nullptr, bool row_box = false,
-                                                uint64_t* bar = nullptr, int64_t next = -1) {
+                                                int bar_id = 0, const CUtensorMap* map = nullptr,
+                                                bool row_box = false, uint64_t* bar = nullptr, int64_t next = -1) {
   using F = Fmt<T>;
   using U = typename F::U;
   using S = typename F::S;
-  constexpr int N = 64;
+  using A3 = Area3<T>;
+  constexpr bool WIDE = F::P == 64;
   constexpr int Q = F::P - 2 - Geo<3>::G;  // quantisation bits (R6)
   constexpr int C = Geo<3>::C;             // guard planes (R10)
   constexpr int HDR = 2 + 3 + F::EBITS;    // mode, escalation, block exponent
-  constexpr int LEN_RAW = 2 + N * F::P;
+  constexpr int LEN_RAW = 2 + 64 * F::P;
   constexpr int BUFW = chunk_buf_words3<T>();
-  constexpr uint32_t CAP = (uint32_t)BUFW * 32;  // bits of one chunk buffer
-  constexpr bool WIDE = F::P == 64;
+  constexpr uint32_t CAP = (uint32_t)BUFW * 32;  // bits of the chunk buffer
   constexpr unsigned FULL = 0xffffffffu;
+  constexpr int SET = A3::kSet;
 
-  // component i's bits go to buffer i & 1; it is appended to the pool while
-  // component i + 1 is written, which saves a barrier per component
-  uint32_t* cbufs = reinterpret_cast<uint32_t*>(smem + staging_bytes3<T>(map != nullptr));
-  S* bbuf = reinterpret_cast<S*>(cbufs + (size_t)BUFW * 2);
-  // [warp][brick][plane] plane words, and offsets | n << 14 | hi << 21; one of
-  // the two lives in the brick buffer
-  uint64_t* s_pw = planes_in_brick_buffer<T>() ? reinterpret_cast<uint64_t*>(bbuf)
-                                               : reinterpret_cast<uint64_t*>(bbuf + kChunk * 64);
-  uint32_t* s_pi = planes_in_brick_buffer<T>() ? reinterpret_cast<uint32_t*>(bbuf + kChunk * 64)
-                                               : reinterpret_cast<uint32_t*>(bbuf);
-  // per-brick tables, one set per component parity: a warp that runs ahead
-  // into component i + 1 never overwrites what slower warps still read of i
-  int* s_len = reinterpret_cast<int*>(planes_in_brick_buffer<T>() ? (void*)(s_pi + kChunk * 64)
-                                                                  : (void*)(s_pw + kChunk * 64));  // [2][32]
-  int* s_mode = s_len + 64;
-  int* s_esc = s_mode + 64;
-  int* s_viol = s_esc + 64;
-  unsigned long long* s_base = reinterpret_cast<unsigned long long*>(s_viol + 64);
-  uint64_t* s_merr = reinterpret_cast<uint64_t*>(s_base + 2);  // [2][32]
-  int* s_cbits = reinterpret_cast<int*>(s_merr + 64);
+  uint32_t* cbuf = reinterpret_cast<uint32_t*>(smem + staging_bytes3<T>(map != nullptr));
+  uint32_t* areas = cbuf + BUFW;
+  uint32_t* infos = areas + kWarps3 * A3::kWords;  // [brick][k]: plane offset << 8 | n
+  double2* s_x = reinterpret_cast<double2*>(infos + kChunk * A3::kInfoStride);  // float64: [16-byte part][thread]
+  uint16_t* s_spread = reinterpret_cast<uint16_t*>(s_x + (WIDE ? kChunk * 64 * sizeof(T) / 16 : 0));
+  int* s_len = reinterpret_cast<int*>(s_spread + 256);
+  int* s_mode = s_len + 32;
+  int* s_esc = s_mode + 32;
+  int* s_viol = s_esc + 32;
+  uint64_t* s_merr = reinterpret_cast<uint64_t*>(s_viol + 32);
+  unsigned long long* s_base = reinterpret_cast<unsigned long long*>(s_merr + 32);
+  int* s_cbits = reinterpret_cast<int*>(s_base + 1);
 
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int h = lane >> 4, t = lane & 15;
-  const unsigned HALF = h ? 0xffff0000u : 0x0000ffffu;
-  const int slot = warp * 2 + h;
+  const int tid = threadIdx.x & (kCompressThreads3 - 1), warp = tid >> 5, lane = tid & 31;
+  const int bq = lane >> 2, q = lane & 3;  // brick of the warp, z- or y-plane of the brick
+  const int slot = warp * 8 + bq;
   const int64_t b = chunk * kChunk + slot;
   const bool have = b < P.nbricks;
 
-  for (int w = tid; w < 2 * BUFW; w += kCompressThreads3) cbufs[w] = 0u;
+  for (int w = tid; w < BUFW / 4; w += kCompressThreads3) reinterpret_cast<uint4*>(cbuf)[w] = make_uint4(0, 0, 0, 0);
+  reinterpret_cast<uint32_t*>(s_spread)[tid] = reinterpret_cast<const uint32_t*>(kSpread3.code)[tid];
+  static_assert(kSpreadBytes == 4 * kCompressThreads3, "one word per thread");
 
   int64_t bx = 0, by = 0, bz = 0;
   if (have) {
@@ -288,477 +436,526 @@ __device__ __forceinline__ void compress3_chunk(const CompressParams& P, int64_t
     by = r % P.nb[1];
     bz = r / P.nb[1];
   }
-  const int ly = t & 3, lz = t >> 2;
   int nvx = 4, nvy = 4, nvz = 4;  // in-field extent of the brick per axis
   if (have) {
     nvx = (int)(P.dims[0] - 4 * bx < 4 ? P.dims[0] - 4 * bx : 4);
     nvy = (int)(P.dims[1] - 4 * by < 4 ? P.dims[1] - 4 * by : 4);
     nvz = (int)(P.dims[2] - 4 * bz < 4 ? P.dims[2] - 4 * bz : 4);
   }
-  const bool line_in = have && ly < nvy && lz < nvz;
-  // R4: a lane outside the field takes the nearest in-field line's values
-  const int srcl = 16 * h + min(ly, nvy - 1) + 4 * min(lz, nvz - 1);
-  const bool partial = have && (nvx < 4 || nvy < 4 || nvz < 4);
-  const bool any_partial = __any_sync(FULL, partial);
+  const bool any_partial = __any_sync(FULL, nvx < 4 || nvy < 4 || nvz < 4);
 
-  T x[4], xt[4], e[4];
-  T* xs = reinterpret_cast<T*>(smem);
-  if (map) {
-    if (have) {
-      staged_line<T>(xs, row_box, slot, ly, lz, nvx, nvy, nvz, x);
-    } else {
+  // The values (float64: kept in shared memory, read back twice a component),
+  // padded (R4).  Algorithm 1 starts from x~ = 0, so the first residual is x
+  // itself (x - 0 in IEEE arithmetic, -0 included).
+  T x[16], xt[16], e[16];
+  if (have) {
+    const T* field = reinterpret_cast<const T*>(P.field);
+    const int64_t gz = 4 * bz + min(q, nvz - 1);
 #pragma unroll
-      for (int m = 0; m < 4; ++m) x[m] = T(0);
+    for (int y = 0; y < 4; ++y) {
+      if (map)
+        staged_line<T>(reinterpret_cast<const T*>(smem), row_box, slot, y, q, nvx, nvy, nvz, e + 4 * y);
+      else
+        load_line<T>(field + (gz * P.dims[1] + 4 * by + min(y, nvy - 1)) * P.dims[0] + 4 * bx, nvx, e + 4 * y);
     }
-    __syncthreads();  // every lane has its values: xs is free for the next chunk
+  } else {
+#pragma unroll
+    for (int v = 0; v < 16; ++v) e[v] = T(0);
+  }
+  if (map) {
+    group_sync(bar_id);  // every lane has its values: xs is free for the next chunk
     if (tid == 0 && next >= 0 && next < P.nchunks) {
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // the reads above before the copy's writes
-      issue_chunk_copy<T>(P, map, row_box, next, xs, bar);
+      issue_chunk_copy<T>(P, map, row_box, next, reinterpret_cast<T*>(smem), bar);
     }
-  } else if (!have) {
-#pragma unroll
-    for (int m = 0; m < 4; ++m) x[m] = T(0);
-  } else {
-    const int64_t gy = 4 * by + min(ly, nvy - 1), gz = 4 * bz + min(lz, nvz - 1);
-    const T* row = reinterpret_cast<const T*>(P.field) + (gz * P.dims[1] + gy) * P.dims[0] + 4 * bx;
-    load_line<T>(row, nvx, x);
   }
-  {
-    bool bad = false;
+  auto load_x = [&](int part, T* two) {  // float64: values 2 part, 2 part + 1
+    const double2 d = s_x[part * kCompressThreads3 + tid];
+    two[0] = (T)d.x;
+    two[1] = (T)d.y;
+  };
 #pragma unroll
-    for (int m = 0; m < 4; ++m)
-      if (line_in && m < nvx && not_finite<T>(x[m])) bad = true;
-    if (__any_sync(FULL, bad) && lane == 0) atomicOr(P.flags, kFlagNonFinite);
+  for (int v = 0; v < 16; ++v) {
+    xt[v] = T(0);
+    if constexpr (!WIDE) x[v] = e[v];
   }
-  // Algorithm 1 starts from x~ = 0; the first residual is x - 0, which is x
-  // itself in IEEE arithmetic (-0 - +0 = -0), so no subtraction is issued
+  if constexpr (WIDE) {
 #pragma unroll
-  for (int m = 0; m < 4; ++m) {
-    xt[m] = T(0);
-    e[m] = x[m];
+    for (int h = 0; h < 8; ++h)
+      s_x[h * kCompressThreads3 + tid] = make_double2(e[2 * h], e[2 * h + 1]);
   }
-  S* buf = bbuf + warp * 128;
-  // buffer slots (each below 128) of this lane's line in each pass and of its
-  // coded coefficients, four to a register: slot m of a pass is byte m
-  const int xx = t & 3, yq = t >> 2;
-  uint32_t pix = 0u, piy = 0u, piz = 0u, pir = 0u;
+  U m = brick_max<T>(e);  // the largest magnitude of the residual, by brick
+  if (__any_sync(FULL, m >= F::INF) && lane == 0) atomicOr(P.flags, kFlagNonFinite);
+
+  uint32_t* area = areas + warp * A3::kWords;
+  uint4* zw = reinterpret_cast<uint4*>(area) + (bq >> 1) * 38 + (bq & 1) + 10 * q;  // + 2 y: line (y, z = q)
+  uint4* yw = reinterpret_cast<uint4*>(area) + (bq >> 1) * 38 + (bq & 1) + 2 * q;   // + 10 z: line (y = q, z)
+  uint32_t* planes = area + bq * A3::kPlaneStride;
+  uint32_t* info = infos + slot * A3::kInfoStride;
+  // places of this lane's coefficients in coded order, four to a register:
+  // byte offset 32 (r / 16) + 4 (r & 7) + 2 ((r >> 3) & 1) of rank r
+  uint32_t place[4];
 #pragma unroll
-  for (int m = 0; m < 4; ++m) {
-    pix |= (uint32_t)sidx<T>(m, ly, lz, h) << (8 * m);   // x-line of (y = ly, z = lz)
-    piy |= (uint32_t)sidx<T>(xx, m, yq, h) << (8 * m);   // y-line of (x = xx, z = yq)
-    piz |= (uint32_t)sidx<T>(xx, yq, m, h) << (8 * m);   // z-line of (x = xx, y = yq)
-    const int pos = kPerm3.pos[t + 16 * m];
-    pir |= (uint32_t)sidx<T>(pos & 3, (pos >> 2) & 3, pos >> 4, h) << (8 * m);
+  for (int z = 0; z < 4; ++z) {
+    place[z] = 0u;
+#pragma unroll
+    for (int xx = 0; xx < 4; ++xx) {
+      const int r = kRank3.pos[xx + 4 * q + 16 * z];
+      place[z] |= (uint32_t)(32 * (r >> 4) + 4 * (r & 7) + 2 * ((r >> 3) & 1)) << (8 * xx);
+    }
   }
-  unsigned long long pool_base = 0;  // thread 0 only
-  unsigned pool_nw = 0;
 
   for (int i = 0; i < P.n; ++i) {  // one component per tau_i
-    uint32_t* cbuf = cbufs + (i & 1) * BUFW;
-    __syncwarp();  // the last component's plane tables (in the brick buffer) are read
     const U tb = (U)P.tau_bits[i];
-    if (any_partial) {  // R4 padding of the residual
-      const T last = nvx == 1 ? e[0] : nvx == 2 ? e[1] : nvx == 3 ? e[2] : e[3];
-#pragma unroll
-      for (int m = 1; m < 4; ++m)
-        if (m >= nvx) e[m] = last;
-#pragma unroll
-      for (int m = 0; m < 4; ++m) e[m] = __shfl_sync(FULL, e[m], srcl);
-    }
-    // R5: a brick whose residual meets tau_i on every in-field value is ZERO.
-    // (Every lane takes part in each vote: a vote behind && or || would be
-    // skipped by one half of the warp and leave the other half waiting.)
-    bool small = true;
-#pragma unroll
-    for (int m = 0; m < 4; ++m)
-      if (line_in && m < nvx && !within<T>(e[m], tb)) small = false;
-    const unsigned big_votes = __ballot_sync(FULL, !small);
-    const bool zero_blk = !have || ((big_votes & HALF) == 0u);
-    // R6: block exponent and exact quantisation.  The largest biased exponent
-    // of the brick is also its finiteness test: an infinite or NaN residual
-    // (all-ones exponent) forces RAW.
-    int be = 0;
-#pragma unroll
-    for (int m = 0; m < 4; ++m) be = max(be, biased_exp<T>(F::bits(e[m])));
-    {  // the maximum over each brick's 16 lanes: two warp reductions (redux)
-      const unsigned lo = __reduce_max_sync(FULL, h ? 0u : (unsigned)be);
-      const unsigned hi = __reduce_max_sync(FULL, h ? (unsigned)be : 0u);
-      be = (int)(h ? hi : lo);
-    }
-    const bool raw_forced = !zero_blk && be == (1 << F::EXPW) - 1;
-    const int emax = block_emax_from_be<T>(be);
-    const int s = Q - emax;
-    S q[4];
-    bool qdone = false;
-    if constexpr (sizeof(T) == 4) {
-      if (s >= -126 && s <= 127) {
-        // 2^s is a normal float: e * 2^s is exact whenever |q| >= 1 (at most
-        // 2^Q, no overflow; a product below the normal range truncates to 0
-        // either way), so truncating the product is the R6 quantisation
-        const float sc = __uint_as_float((uint32_t)(127 + s) << 23);
-#pragma unroll
-        for (int m = 0; m < 4; ++m) q[m] = __float2int_rz(__fmul_rn(e[m], sc));
-        qdone = true;
-      }
-    }
-    if (!qdone) {
-#pragma unroll
-      for (int m = 0; m < 4; ++m) q[m] = quantize<T>(F::bits(e[m]), s);
-    }
-
-    // R7: lifting along x (in the lane), y and z (shared buffer)
-    lift_fwd(q[0], q[1], q[2], q[3]);
-#pragma unroll
-    for (int m = 0; m < 4; ++m) buf[slot_of(pix, m)] = q[m];
-    __syncwarp();
-    {
-      S a = buf[slot_of(piy, 0)], bq = buf[slot_of(piy, 1)], c = buf[slot_of(piy, 2)], d = buf[slot_of(piy, 3)];
-      lift_fwd(a, bq, c, d);
-      buf[slot_of(piy, 0)] = a; buf[slot_of(piy, 1)] = bq; buf[slot_of(piy, 2)] = c; buf[slot_of(piy, 3)] = d;
-    }
-    __syncwarp();
-    {
-      S a = buf[slot_of(piz, 0)], bq = buf[slot_of(piz, 1)], c = buf[slot_of(piz, 2)], d = buf[slot_of(piz, 3)];
-      lift_fwd(a, bq, c, d);
-      buf[slot_of(piz, 0)] = a; buf[slot_of(piz, 1)] = bq; buf[slot_of(piz, 2)] = c; buf[slot_of(piz, 3)] = d;
-    }
-    __syncwarp();
-    // R8, R9: coded order, negabinary.  Lane t holds coefficients t + 16j.
-    U u[4];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) u[j] = nb_fwd<T>(buf[slot_of(pir, j)]);
-    __syncwarp();
-
-    // R10, R13: lowest coded plane; lowered until Eq. 1 holds in T
     const int L = P.L[i];
-    int esc = 0, p = 0;
-    bool done = zero_blk || raw_forced, pass = false;
-    // x~ + x_i of the passing precision; the carried residual e takes its
-    // x - (x~ + x_i) at the same time (a RAW brick recomputes the residual it
-    // stores from x - x~, which is the same value)
-    T xtc[4];
+    // R5: a brick whose residual meets tau_i is ZERO.  R6: the block exponent
+    // comes from the largest magnitude; an infinite or NaN residual forces RAW.
+    const bool zero_blk = !have || m <= tb;
+    const int be = (int)(m >> (F::MANT - 1));
+    const bool coded = !zero_blk && be != (1 << F::EXPW) - 1;
+    const int emax = block_emax_from_be<T>(be);
+    const int s = coded ? Q - emax : 0;
+    int esc = 0;
+    for (;;) {  // again, with more planes in some brick, while Eq. 1 fails (R13): at most 8 times
+      // The blocks' common scales let every value take the short forms of R6
+      // and R13; other scales take the general ones.
+      const bool common = __all_sync(FULL, WIDE ? s >= -960 && s <= 1000 : s >= -126 && s <= 126);
+      S v[16];
+      if constexpr (!WIDE) {
+        if (common) {
+          // e * 2^s is exact whenever |q| >= 1 (at most 2^Q, no overflow; a
+          // product below the normal range truncates to 0 either way), so
+          // truncating the product is the R6 quantisation.  0 where not coded.
+          const float sc = coded ? __uint_as_float((uint32_t)(127 + s) << 23) : 0.0f;
 #pragma unroll
-    for (int m = 0; m < 4; ++m) xtc[m] = xt[m];
-    for (int round = 0; round < 8; ++round) {  // esc runs 0..7: at most 8 rounds
-      const bool active = !done;
-      const int pp = min(max(L + s - C - esc, 0), F::P);
-      const U keep = pp >= F::P ? U(0) : (U)~((U(1) << pp) - 1);
+          for (int k = 0; k < 16; ++k) v[k] = __float2int_rz(__fmul_rn(e[k], sc));
+        } else {
 #pragma unroll
-      for (int j = 0; j < 4; ++j) buf[slot_of(pir, j)] = nb_inv<T>((U)(u[j] & keep));
-      __syncwarp();
-      {
-        S a = buf[slot_of(piz, 0)], bq = buf[slot_of(piz, 1)], c = buf[slot_of(piz, 2)], d = buf[slot_of(piz, 3)];
-        lift_inv(a, bq, c, d);
-        buf[slot_of(piz, 0)] = a; buf[slot_of(piz, 1)] = bq; buf[slot_of(piz, 2)] = c; buf[slot_of(piz, 3)] = d;
-      }
-      __syncwarp();
-      {
-        S a = buf[slot_of(piy, 0)], bq = buf[slot_of(piy, 1)], c = buf[slot_of(piy, 2)], d = buf[slot_of(piy, 3)];
-        lift_inv(a, bq, c, d);
-        buf[slot_of(piy, 0)] = a; buf[slot_of(piy, 1)] = bq; buf[slot_of(piy, 2)] = c; buf[slot_of(piy, 3)] = d;
-      }
-      __syncwarp();
-      S r[4];
-#pragma unroll
-      for (int m = 0; m < 4; ++m) r[m] = buf[slot_of(pix, m)];
-      __syncwarp();
-      lift_inv(r[0], r[1], r[2], r[3]);
-      bool ok = true;
-      T xtn[4], en[4];
-      if constexpr (sizeof(T) == 4) {
-        T xi[4];
-        dequantize_line<T, false>(r, s, xi);  // x_i = D(y_i)
-#pragma unroll
-        for (int m = 0; m < 4; ++m) {
-          xtn[m] = F::add(xt[m], xi[m]);  // x~ + x_i (candidate)
-          en[m] = F::sub(x[m], xtn[m]);   // the next residual
-          if (line_in && m < nvx && !within<T>(en[m], tb)) ok = false;
+          for (int k = 0; k < 16; ++k) v[k] = coded ? quantize_any<T>(F::bits(e[k]), s) : S(0);
         }
       } else {
-        const bool normal = s >= -960 && s <= 1022;  // every result normal and finite
+        if (common) {
+          const int c = coded ? 1078 - s : 4096;
 #pragma unroll
-        for (int m = 0; m < 4; ++m) {
-          const T xi = normal ? Fmt<T>::val(dequantize_f64_normal(r[m], s)) : dequantize_val<T>(r[m], s);  // x_i = D(y_i)
-          // x~ + x_i (candidate); for the first component +0 + x_i, which is
-          // x_i with -0 turned to +0 -- a bit test instead of an FP64 add
-          const U xb = F::bits(xi);
-          xtn[m] = i == 0 ? F::val(xb == F::SIGN ? U(0) : xb) : F::add(xt[m], xi);
-          en[m] = F::sub(x[m], xtn[m]);             // the next residual
-          if (line_in && m < nvx && !within<T>(en[m], tb)) ok = false;
-        }
-      }
-      const bool pass_h = (__ballot_sync(FULL, !ok) & HALF) == 0u;
-      if (active) {
-        if (pass_h) {
-          pass = true;
-          done = true;
-          p = pp;
-#pragma unroll
-          for (int m = 0; m < 4; ++m) {
-            xtc[m] = xtn[m];
-            if constexpr (sizeof(T) == 8) e[m] = en[m];  // float32 recomputes it below
-          }
-        } else if (esc == 7 || pp == 0) {
-          done = true;
+          for (int k = 0; k < 16; ++k) v[k] = quantize_f64_normal(e[k], c);
         } else {
-          ++esc;
+#pragma unroll
+          for (int k = 0; k < 16; ++k) v[k] = coded ? quantize_any<T>(F::bits(e[k]), s) : S(0);
         }
       }
-      if (__all_sync(FULL, done)) break;
-    }
+      lift_fwd_bricks<S>(v, zw, yw, SET);  // R7
+      // R9, and the highest plane that is not empty
+      U any = 0;
+#pragma unroll
+      for (int k = 0; k < 16; ++k) {
+        const U u = nb_fwd<T>(v[k]);
+        any |= u;
+        v[k] = (S)u;
+      }
+      any |= __shfl_xor_sync(FULL, any, 1);
+      any |= __shfl_xor_sync(FULL, any, 2);
+      // R10: the lowest coded plane
+      const int p = coded ? min(max(L + s - C - esc, 0), F::P) : F::P;
+      const int top = any ? F::P - 1 - F::clz(any) : -1;
+      const int nw = top - p + 1;  // planes from the highest that is not empty down to p
+      // the coded digits, from plane p up
+#pragma unroll
+      for (int k = 0; k < 16; ++k) v[k] = (S)(p >= F::P ? U(0) : (U)v[k] >> (p & (F::P - 1)));
+      const int span = (int)__reduce_max_sync(FULL, (unsigned)max(nw, 0));
 
-    // R11: plane words by transposing the coefficient bits across the warp:
-    // lane l then holds plane l (and l + 32) of both bricks.
-    uint64_t WA0, WB0, WA1 = 0, WB1 = 0;
-    {
-      uint32_t tkeep[5];
-      transpose_masks(lane, tkeep);
-      uint32_t tl[4];
+      // the digits in coded order (R8), 16 ranks per lane, and their transpose:
+      // plane words from word 4 j + q of the brick's plane area
+      auto planes16 = [&] {
+        unsigned char* put = reinterpret_cast<unsigned char*>(area + 36 * bq);
 #pragma unroll
-      for (int j = 0; j < 4; ++j) tl[j] = transpose32((uint32_t)u[j], lane, tkeep);
-      WA0 = (uint64_t)__byte_perm(tl[0], tl[1], 0x5410) | ((uint64_t)__byte_perm(tl[2], tl[3], 0x5410) << 32);
-      WB0 = (uint64_t)__byte_perm(tl[0], tl[1], 0x7632) | ((uint64_t)__byte_perm(tl[2], tl[3], 0x7632) << 32);
-      if constexpr (WIDE) {
-        uint32_t th[4];
+        for (int k = 0; k < 16; ++k)
+          *reinterpret_cast<uint16_t*>(put + ((place[k >> 2] >> (8 * (k & 3))) & 0xffu)) = (uint16_t)v[k];
+        __syncwarp();
+        uint32_t a[8];
+        const uint4* get = reinterpret_cast<const uint4*>(area + 36 * bq + 8 * q);
 #pragma unroll
-        for (int j = 0; j < 4; ++j) th[j] = transpose32((uint32_t)((uint64_t)u[j] >> 32), lane, tkeep);
-        WA1 = (uint64_t)__byte_perm(th[0], th[1], 0x5410) | ((uint64_t)__byte_perm(th[2], th[3], 0x5410) << 32);
-        WB1 = (uint64_t)__byte_perm(th[0], th[1], 0x7632) | ((uint64_t)__byte_perm(th[2], th[3], 0x7632) << 32);
-      }
-    }
-    const int pA = __shfl_sync(FULL, p, 0), pB = __shfl_sync(FULL, p, 16);
-    const bool passA = __shfl_sync(FULL, (int)pass, 0) != 0, passB = __shfl_sync(FULL, (int)pass, 16) != 0;
-    // planes P-1 .. p are coded, from the top: the high round (planes 32 + l)
-    // first for 64-bit coefficients, then planes l
-    int nA0 = 0, nA1 = 0, nB0 = 0, nB1 = 0, oA0 = 0, oA1 = 0, oB0 = 0, oB1 = 0;
-    int hA0 = 0, hA1 = 0, hB0 = 0, hB1 = 0;
-    int totA = 0, totB = 0;
-    {
-      int cmaxA = 0, cmaxB = 0;
-      uint32_t csum = 0;
-      if constexpr (WIDE)
-        plane_scan2<N>(WA1, passA && lane + 32 >= pA, WB1, passB && lane + 32 >= pB, lane, cmaxA, cmaxB, csum, nA1, nB1,
-                       hA1, hB1, oA1, oB1);
-      plane_scan2<N>(WA0, passA && lane >= pA, WB0, passB && lane >= pB, lane, cmaxA, cmaxB, csum, nA0, nB0, hA0, hB0,
-                     oA0, oB0);
-      totA = (int)(csum & 0xffffu);
-      totB = (int)(csum >> 16);
-    }
-    const int lenC = HDR + (h ? totB : totA);
-    {  // plane p's word, code offset and significance count, for the coefficient lanes
-      uint64_t* pw = s_pw + warp * 128;
-      uint32_t* pi = s_pi + warp * 128;
-      pw[lane] = WA0;
-      pi[lane] = (uint32_t)oA0 | ((uint32_t)nA0 << 14) | ((uint32_t)hA0 << 21);
-      pw[64 + lane] = WB0;
-      pi[64 + lane] = (uint32_t)oB0 | ((uint32_t)nB0 << 14) | ((uint32_t)hB0 << 21);
-      if constexpr (WIDE) {
-        pw[32 + lane] = WA1;
-        pi[32 + lane] = (uint32_t)oA1 | ((uint32_t)nA1 << 14) | ((uint32_t)hA1 << 21);
-        pw[96 + lane] = WB1;
-        pi[96 + lane] = (uint32_t)oB1 | ((uint32_t)nB1 << 14) | ((uint32_t)hB1 << 21);
-      }
-    }
+        for (int k = 0; k < 2; ++k) {
+          const uint4 r = get[k];
+          a[4 * k] = r.x;
+          a[4 * k + 1] = r.y;
+          a[4 * k + 2] = r.z;
+          a[4 * k + 3] = r.w;
+        }
+        __syncwarp();
+        transpose16(a);
+#pragma unroll
+        for (int j = 0; j < 8; ++j) planes[4 * j + q] = a[j];
+        __syncwarp();
+      };
+      // 32 planes: the digits of 16 ranks, then (half 0: planes p + j) their words
+      auto ranks32 = [&](const uint32_t* w, uint32_t (&a)[16]) {
+        unsigned char* put = reinterpret_cast<unsigned char*>(area + 72 * bq);
+#pragma unroll
+        for (int k = 0; k < 16; ++k)
+          *reinterpret_cast<uint32_t*>(put + 2 * ((place[k >> 2] >> (8 * (k & 3))) & 0xffu)) = w[k];
+        __syncwarp();
+        const uint4* get = reinterpret_cast<const uint4*>(area + 72 * bq + 16 * q);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {  // ranks 2k, 2k + 8, 2k + 1, 2k + 9
+          const uint4 r = get[k];
+          a[2 * k] = r.x;
+          a[2 * k + 8] = r.y;
+          a[2 * k + 1] = r.z;
+          a[2 * k + 9] = r.w;
+        }
+        __syncwarp();
+      };
+      auto words32 = [&](uint32_t (&a)[16], int half) {
+        transpose32_lane(a);
+#pragma unroll
+        for (int j = 0; j < 16; ++j) planes[64 * half + 4 * j + q] = a[j];
+      };
+      auto planes32 = [&](const uint32_t* w) {
+        uint32_t a[16];
+        ranks32(w, a);
+        words32(a, 0);
+        __syncwarp();
+      };
 
-    // the residual x - x~_{i-1} again, padded (R4), where a brick may be RAW:
-    // the value the coder started from, which the loop above has replaced
-    // by the next residual in passing bricks
-    T eo[4];
-    const bool need_eo = __any_sync(FULL, !zero_blk && (!pass || lenC > LEN_RAW));
-    if (need_eo) {
+      // R13: decode-back x_i = D(y_i), the candidate x~ + x_i and the residual
+      // it leaves.  Bricks that are not coded decode to 0, which leaves x~ and
+      // the residual as they are.
+      T xtn[16], en[16];
+      auto residual = [&] {
+        if constexpr (WIDE) {
 #pragma unroll
-      for (int m = 0; m < 4; ++m) eo[m] = F::sub(x[m], xt[m]);
-      if (any_partial) {
-        const T last = nvx == 1 ? eo[0] : nvx == 2 ? eo[1] : nvx == 3 ? eo[2] : eo[3];
+          for (int h = 0; h < 8; ++h) {
+            T two[2];
+            load_x(h, two);
+            en[2 * h] = F::sub(two[0], xtn[2 * h]);
+            en[2 * h + 1] = F::sub(two[1], xtn[2 * h + 1]);
+          }
+        } else {
 #pragma unroll
-        for (int m = 1; m < 4; ++m)
-          if (m >= nvx) eo[m] = last;
+          for (int k = 0; k < 16; ++k) en[k] = F::sub(x[k], xtn[k]);
+        }
+        if (any_partial) pad_brick<T>(en, nvx, nvy, nvz, lane);
+      };
+      int H = 8;  // plane words: plane j in half j / H of word j mod H
+      if constexpr (!WIDE) {
+        {
+          S r[16];
 #pragma unroll
-        for (int m = 0; m < 4; ++m) eo[m] = __shfl_sync(FULL, eo[m], srcl);
+          for (int k = 0; k < 16; ++k) r[k] = nb_inv<T>(p >= 32 ? 0u : (U)v[k] << (p & 31));
+          lift_inv_bricks<S>(r, zw, yw, SET);
+          if (common) {
+            const float sc = __uint_as_float((uint32_t)(127 - s) << 23);
+#pragma unroll
+            for (int k = 0; k < 16; ++k) xtn[k] = F::add(xt[k], __fmul_rn(__int2float_rn(r[k]), sc));
+          } else {
+#pragma unroll
+            for (int k = 0; k < 16; ++k) xtn[k] = F::add(xt[k], F::val(dequantize_any<T>(r[k], s)));
+          }
+        }
+        residual();
+        if (span <= 16) {
+          planes16();
+        } else {
+          uint32_t w[16];
+#pragma unroll
+          for (int k = 0; k < 16; ++k) w[k] = (uint32_t)v[k];
+          planes32(w);
+          H = 16;
+        }
+      } else {
+        // Digits within 20 planes from plane p >= 6 on, none above plane 58:
+        // decoded in 32-bit integers in units of 2^(p - 6).  A coefficient with
+        // negabinary digits d from plane p is ((d ^ M) - M) * 2^p with M =
+        // NBM >> p (M's bits above d's do not matter).  In these units each
+        // inverse lifting pass turns multiples of 2^a into multiples of
+        // 2^(a - 2), so from 2^6 on every shift divides an even number exactly;
+        // |value| < 2^(19 + 6.42) * 2.75^3 < 2^30 (2.75: the largest row sum of
+        // the inverse lifting's coefficients), while the unscaled value stays
+        // below 2^(58 + 4.8) <= 2^63: neither form wraps, so the result is the
+        // 64-bit decoding's exactly, in half the instructions.
+        const bool narrow = common && __all_sync(FULL, nw <= 0 || (nw <= 20 && p >= 6 && top <= 58));
+        auto add = [&](int k, T xi) {  // x~ + x_i; the first component's +0 + x_i is x_i with -0 turned to +0
+          if (i == 0)
+            xtn[k] = F::val(F::bits(xi) == F::SIGN ? U(0) : F::bits(xi));
+          else
+            xtn[k] = F::add(xt[k], xi);
+        };
+        if (narrow) {
+          uint32_t w[16];
+#pragma unroll
+          for (int k = 0; k < 16; ++k) w[k] = (uint32_t)v[k];
+          int32_t r[16];
+          const uint32_t M = (uint32_t)(F::NBM >> min(p, 63));
+#pragma unroll
+          for (int k = 0; k < 16; ++k) r[k] = (int32_t)(((w[k] ^ M) - M) << 6);
+          lift_inv_bricks<int32_t>(r, zw, yw, SET);
+          const uint32_t eb = (uint32_t)(1053 + (p - 6) - s) << 20;
+#pragma unroll
+          for (int k = 0; k < 16; ++k) add(k, scaled_i32_to_f64(r[k], eb));
+          residual();
+          if (span <= 16) {
+            planes16();
+          } else {
+            planes32(w);
+            H = 16;
+          }
+        } else {
+          S r[16];
+#pragma unroll
+          for (int k = 0; k < 16; ++k) r[k] = nb_inv<T>(p >= 64 ? U(0) : (U)v[k] << (p & 63));
+          lift_inv_bricks<S>(r, zw, yw, SET);
+#pragma unroll
+          for (int k = 0; k < 16; ++k)
+            add(k, F::val(common ? dequantize_f64_normal(r[k], s) : dequantize_any<T>(r[k], s)));
+          residual();
+          H = 16;
+          uint32_t w[16];
+#pragma unroll
+          for (int k = 0; k < 16; ++k) w[k] = (uint32_t)v[k];
+          if (span <= 32) {
+            planes32(w);
+          } else {  // both halves' digits are read before the words take their place
+            uint32_t a0[16], a1[16];
+            ranks32(w, a0);
+#pragma unroll
+            for (int k = 0; k < 16; ++k) w[k] = (uint32_t)((U)v[k] >> 32);
+            ranks32(w, a1);
+            words32(a0, 0);
+            words32(a1, 1);
+            __syncwarp();
+          }
+        }
       }
-    }
-    // R14: RAW replaces a longer CODED brick only if it also meets tau_i
-    bool raw_ok = false;
-    if (__any_sync(FULL, pass && lenC > LEN_RAW)) {
-      bool ok = true;
+      const U mn = brick_max<T>(en);
+      const bool pass = !zero_blk && coded && mn <= tb;
+      const bool again = coded && !pass && p > 0 && esc < 7;
+      if (__any_sync(FULL, again)) {  // rare: code the warp's bricks again from the same residual
+        if (again) ++esc;
+        if constexpr (WIDE) {
 #pragma unroll
-      for (int m = 0; m < 4; ++m) {
-        const T a = F::add(xt[m], eo[m]);
-        if (line_in && m < nvx && !within<T>(F::sub(x[m], a), tb)) ok = false;
+          for (int h = 0; h < 8; ++h) {
+            T two[2];
+            load_x(h, two);
+            e[2 * h] = F::sub(two[0], xt[2 * h]);
+            e[2 * h + 1] = F::sub(two[1], xt[2 * h + 1]);
+          }
+        } else {
+#pragma unroll
+          for (int k = 0; k < 16; ++k) e[k] = F::sub(x[k], xt[k]);
+        }
+        if (any_partial) pad_brick<T>(e, nvx, nvy, nvz, lane);
+        continue;
       }
-      raw_ok = (__ballot_sync(FULL, !ok) & HALF) == 0u;
-    }
-    const int mode = zero_blk ? kModeZero : (pass && !(lenC > LEN_RAW && raw_ok)) ? kModeCoded : kModeRaw;
-    const int blen = !have ? 0 : mode == kModeZero ? 2 : mode == kModeRaw ? LEN_RAW : lenC;
 
-    // x~_i and the next residual (a RAW brick stores the residual it started
-    // from); the next residual is in e already for CODED and ZERO bricks
-    int viol = 0;  // Eq. 1 failures left (only a RAW brick can have them)
-    U merr = 0;    // max |x - x~_i| over this lane's in-field values, as bits (Sec. 4.3)
-    if (need_eo) {
+      // R11, lengths: the planes above `top` are one 0 test bit each; then 4
+      // planes at a time, one per lane of the brick: the significance count n
+      // before a plane is the largest one-past-highest position over the planes
+      // above it, and the planes' offsets are a running sum of their lengths.
+      const int nrow = (span + 3) >> 2;
+      int lenC = HDR + F::P - max(top + 1, p);
+      {
+        int carry = 0;
+        for (int k = 0; k < nrow; ++k) {
+          const int j = nw - 1 - 4 * k - q;  // plane p + j
+          uint64_t W = 0;
+          if (j >= 0) {
+            const uint4 r = *reinterpret_cast<const uint4*>(planes + 64 * (j >> 5) + 4 * (j & (H - 1)));
+            const uint32_t sel = j & H ? 0x7632u : 0x5410u;
+            W = (uint64_t)__byte_perm(r.x, r.y, sel) | ((uint64_t)__byte_perm(r.z, r.w, sel) << 32);
+          }
+          const int hi = W ? 64 - __clzll((long long)W) : 0;
+          int n = hi;
+          int t = __shfl_up_sync(FULL, n, 1, 4);
+          if (q >= 1) n = max(n, t);
+          t = __shfl_up_sync(FULL, n, 2, 4);
+          if (q >= 2) n = max(n, t);
+          const int all = max(carry, __shfl_sync(FULL, n, 3, 4));
+          t = __shfl_up_sync(FULL, n, 1, 4);
+          n = q ? max(carry, t) : carry;
+          carry = all;
+          int len = 0;
+          if (j >= 0) {
+            len = n;
+            if (n < 64) len += hi > n ? __popcll((long long)(W >> n)) + hi - n + (hi < 64 ? 1 : 0) : 1;
+          }
+          int sum = len;
+          t = __shfl_up_sync(FULL, sum, 1, 4);
+          if (q >= 1) sum += t;
+          t = __shfl_up_sync(FULL, sum, 2, 4);
+          if (q >= 2) sum += t;
+          if (PCZ_CHECK(4 * k + q < A3::kInfoStride, 1)) info[4 * k + q] = (uint32_t)(lenC + sum - len) << 8 | (uint32_t)n;
+          lenC += __shfl_sync(FULL, sum, 3, 4);
+        }
+      }
+
+      // R14: RAW replaces a longer CODED brick only if it also meets tau_i
+      int mode = zero_blk ? kModeZero : pass ? kModeCoded : kModeRaw;
+      int viol = 0;  // Eq. 1 failures left (only a RAW brick can have them)
+      U mnew = mn;
+      if (__any_sync(FULL, mode == kModeRaw || (pass && lenC > LEN_RAW))) {
+        // the residual the brick started from, and x~ and the residual after it
+        T eo[16], xr[16], er[16];
+        if constexpr (WIDE) {
 #pragma unroll
-      for (int m = 0; m < 4; ++m) {
+          for (int h = 0; h < 8; ++h) {
+            T two[2];
+            load_x(h, two);
+            eo[2 * h] = F::sub(two[0], xt[2 * h]);
+            eo[2 * h + 1] = F::sub(two[1], xt[2 * h + 1]);
+          }
+        } else {
+#pragma unroll
+          for (int k = 0; k < 16; ++k) eo[k] = F::sub(x[k], xt[k]);
+        }
+        if (any_partial) pad_brick<T>(eo, nvx, nvy, nvz, lane);
+#pragma unroll
+        for (int h = 0; h < 8; ++h) {
+          T two[2];
+          if constexpr (WIDE) {
+            load_x(h, two);
+          } else {
+            two[0] = x[2 * h];
+            two[1] = x[2 * h + 1];
+          }
+#pragma unroll
+          for (int o = 0; o < 2; ++o) {
+            xr[2 * h + o] = F::add(xt[2 * h + o], eo[2 * h + o]);
+            er[2 * h + o] = F::sub(two[o], xr[2 * h + o]);
+          }
+        }
+        if (any_partial) pad_brick<T>(er, nvx, nvy, nvz, lane);
+        const U mr = brick_max<T>(er);
+        if (pass && lenC > LEN_RAW && mr <= tb) mode = kModeRaw;
         if (mode == kModeRaw) {
-          xtc[m] = F::add(xt[m], eo[m]);
-          if constexpr (sizeof(T) == 8) e[m] = F::sub(x[m], xtc[m]);
+          S* raw = reinterpret_cast<S*>(planes);  // the residual, for the bit writes
+          mnew = mr;
+#pragma unroll
+          for (int k = 0; k < 16; ++k) {
+            raw[16 * q + k] = (S)F::bits(eo[k]);
+            xtn[k] = xr[k];
+            en[k] = er[k];
+            if ((k & 3) < nvx && (k >> 2) < nvy && q < nvz && magnitude(er[k]) > tb) ++viol;
+          }
+        }
+        viol += __shfl_xor_sync(FULL, viol, 1);
+        viol += __shfl_xor_sync(FULL, viol, 2);
+      }
+#pragma unroll
+      for (int k = 0; k < 16; ++k) {
+        xt[k] = xtn[k];
+        e[k] = en[k];
+      }
+      m = mnew;
+      const int blen = !have ? 0 : mode == kModeZero ? 2 : mode == kModeRaw ? LEN_RAW : lenC;
+      if (q == 0) {
+        s_len[slot] = blen;
+        s_mode[slot] = have ? mode : -1;
+        s_esc[slot] = mode == kModeCoded ? esc : 0;
+        s_viol[slot] = have ? viol : 0;
+        s_merr[slot] = have ? (uint64_t)mnew : 0ull;
+      }
+      group_sync(bar_id);  // (the previous component's chunk is appended)
+
+      // chunk layout: every warp scans the 32 brick lengths
+      const int l0 = s_len[lane];
+      int incl = l0;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int t = __shfl_up_sync(FULL, incl, o);
+        if (lane >= o) incl += t;
+      }
+      const int total = __shfl_sync(FULL, incl, 31);
+      const uint32_t boff = (uint32_t)__shfl_sync(FULL, incl - l0, slot);
+      // bookkeeping, spread over the warps: warp 0 sizes the chunk and
+      // reserves its pool space (the atomic's result is needed after the bit
+      // writes), warp 1 gathers the block counters, warp 2 writes the index
+      unsigned long long pool_base = 0;
+      const unsigned cw = (unsigned)((total + 63) >> 6);
+      if (tid == 0) {
+        *s_cbits = total;
+        pool_base = cw ? atomicAdd(P.pool_used, (unsigned long long)cw) : 0ull;
+        P.chunk_nwords[(int64_t)i * P.nchunks + chunk] = cw;
+      }
+      if (warp == 1) {
+        const int md = s_mode[lane];
+        const unsigned cz = __popc(__ballot_sync(FULL, md == kModeZero));
+        const unsigned cc = __popc(__ballot_sync(FULL, md == kModeCoded));
+        const unsigned cr = __popc(__ballot_sync(FULL, md == kModeRaw));
+        const unsigned se = __reduce_add_sync(FULL, (unsigned)s_esc[lane]);
+        const unsigned sv = __reduce_add_sync(FULL, (unsigned)s_viol[lane]);
+        const unsigned long long me = warp_max_u64(FULL, s_merr[lane]);
+        if (lane == 0) {
+          const int64_t ci = (int64_t)i * P.nchunks + chunk;
+          uint32_t* cnt = P.chunk_counts + ci * 5;
+          cnt[0] = cz;
+          cnt[1] = cc;
+          cnt[2] = cr;
+          cnt[3] = se;
+          cnt[4] = sv;
+          if (P.chunk_maxerr) P.chunk_maxerr[ci] = me;
         }
       }
-    }
-    if constexpr (sizeof(T) == 4) {
-      // float32: the next residual x - x~_i for every mode, recomputed here so
-      // that it is not live across the escalation loop (fewer spills; the
-      // same values: a passing brick's candidate residual was x - x~_i, and
-      // lanes outside the field are padded again at the next component).
-      // Float64 keeps the loop's value: a second FP64 subtraction costs more
-      // than the spills it saves.
-#pragma unroll
-      for (int m = 0; m < 4; ++m) e[m] = F::sub(x[m], xtc[m]);
-    }
-#pragma unroll
-    for (int m = 0; m < 4; ++m) {
-      if (line_in && m < nvx) {
-        U a;  // float64: |e|'s pattern doubled (mag2_bits), halved after the maximum
-        if constexpr (sizeof(U) == 8)
-          a = mag2_bits(e[m]);
-        else
-          a = F::bits(e[m]) & F::ABS;
-        merr = a > merr ? a : merr;
+      if (warp == 2 && chunk * kChunk + lane < P.nbricks) {
+        const int64_t at = (int64_t)i * P.nbricks + chunk * kChunk + lane;
+        P.brick_len[at] = (uint16_t)l0;
+        if (P.brick_off) P.brick_off[at] = (uint32_t)(incl - l0);
       }
-    }
-    if constexpr (sizeof(U) == 4) {  // per brick half: two warp reductions (redux)
-      const unsigned lo = __reduce_max_sync(FULL, h ? 0u : (unsigned)merr);
-      const unsigned hi = __reduce_max_sync(FULL, h ? (unsigned)merr : 0u);
-      merr = (U)(h ? hi : lo);
-    } else {  // per brick half: the two halves' 64-bit maxima, four warp reductions
-      const unsigned long long lo = warp_max_u64(FULL, h ? 0ull : (unsigned long long)merr);
-      const unsigned long long hi = warp_max_u64(FULL, h ? (unsigned long long)merr : 0ull);
-      merr = (U)(h ? hi : lo) >> 1;
-    }
-    // failures are counted only where a brick of the warp is RAW (a CODED or
-    // ZERO brick meets tau_i on every value by construction)
-    if (__any_sync(FULL, have && mode == kModeRaw)) {
-#pragma unroll
-      for (int m = 0; m < 4; ++m)
-        if (line_in && m < nvx && !within<T>(e[m], tb)) ++viol;
-#pragma unroll
-      for (int o = 8; o >= 1; o >>= 1) viol += __shfl_xor_sync(FULL, viol, o);
-    }
 
-    const int par = (i & 1) * 32;
-    if (t == 0) {
-      s_len[par + slot] = blen;
-      s_mode[par + slot] = have ? mode : -1;
-      s_esc[par + slot] = (have && mode == kModeCoded) ? esc : 0;
-      s_viol[par + slot] = have ? viol : 0;
-      s_merr[par + slot] = have ? (uint64_t)merr : 0ull;
-    }
-    __syncthreads();
-    // chunk layout: every warp scans the 32 brick lengths for its own bricks'
-    // offsets (no second barrier); warp 0 also records the chunk
-    // this warp's two bricks start after the lengths of the bricks before them:
-    // one warp sum (redux) over the lanes below 2 * warp
-    const int l0 = s_len[par + lane];
-    const int offA = (int)__reduce_add_sync(FULL, lane < 2 * warp ? (unsigned)l0 : 0u);
-    const int offB = offA + __shfl_sync(FULL, l0, 2 * warp);
-    // chunk bookkeeping, spread so that no warp carries much more than the
-    // others to the next barrier: warp 0 sizes the chunk and reserves its
-    // pool space, warp 1 gathers the block counters, and each warp writes its
-    // own bricks' index entries
-    if (warp == 0) {
-      const int total = (int)__reduce_add_sync(FULL, (unsigned)l0);
-      const unsigned nw = (unsigned)((total + 63) >> 6);
-      if (lane == 0) {
-        s_cbits[i & 1] = total;
-        // pool space for the chunk; the atomic's result is first needed after
-        // this warp's share of the bit writes, which hides its latency
-        pool_base = nw ? atomicAdd(P.pool_used, (unsigned long long)nw) : 0ull;
-        pool_nw = nw;
-        P.chunk_nwords[(int64_t)i * P.nchunks + chunk] = nw;
+      // the bits of the warp's bricks, into the chunk buffer
+      if (have && mode == kModeRaw) {
+        if (q == 0) or_bits_in(cbuf, boff, (uint64_t)kModeRaw, CAP, 0);
+        const U* raw = reinterpret_cast<const U*>(planes) + 16 * q;
+        for (int k = 0; k < 16; ++k)
+          or_bits_in(cbuf, boff + 2 + (uint32_t)(F::P * (16 * q + k)), (uint64_t)raw[k], CAP, 0);
       }
-    } else if (warp == 1) {
-      const int md = s_mode[par + lane];
-      const unsigned cz = __popc(__ballot_sync(FULL, md == kModeZero));
-      const unsigned cc = __popc(__ballot_sync(FULL, md == kModeCoded));
-      const unsigned cr = __popc(__ballot_sync(FULL, md == kModeRaw));
-      int se = s_esc[par + lane], sv = s_viol[par + lane];
-      const unsigned long long me = warp_max_u64(FULL, s_merr[par + lane]);
-      if (__any_sync(FULL, se != 0 || sv != 0)) {  // escalations and failures are rare
-#pragma unroll
-        for (int o = 16; o >= 1; o >>= 1) {
-          se += __shfl_xor_sync(FULL, se, o);
-          sv += __shfl_xor_sync(FULL, sv, o);
+      const bool emit = have && mode == kModeCoded;
+      if (emit && q == 0)
+        or_bits_in(cbuf, boff, (uint64_t)kModeCoded | ((uint64_t)esc << 2) | ((uint64_t)(emax + F::EBIAS) << 5), CAP, 0);
+      // R11: each plane by a lane: its n verbatim bits and, if a coefficient
+      // turns significant, the first test bit; then the group-test code, 16
+      // coefficients at a time through the byte table.  The code of the last 16
+      // drops the test 1 after the plane's last 1; zeros need no write.
+      for (int k = 0; k < nrow; ++k) {
+        const int j = nw - 1 - 4 * k - q;
+        if (!emit || j < 0) continue;
+        const uint4 r = *reinterpret_cast<const uint4*>(planes + 64 * (j >> 5) + 4 * (j & (H - 1)));
+        const uint32_t sel = j & H ? 0x7632u : 0x5410u;
+        const uint64_t W = (uint64_t)__byte_perm(r.x, r.y, sel) | ((uint64_t)__byte_perm(r.z, r.w, sel) << 32);
+        if (!W) continue;
+        const uint32_t nf = info[4 * k + q];
+        const int n = (int)(nf & 0xffu);
+        const uint32_t at = boff + (nf >> 8);
+        uint64_t rest = n < 64 ? W >> n : 0ull;
+        or_bits_in(cbuf, at, (W & low_mask64(n)) | (rest ? 1ull << n : 0ull), CAP, 0);
+        uint32_t pos = at + (uint32_t)n + 1u;
+        while (rest) {
+          const uint32_t b0 = (uint32_t)rest & 0xffu, b1 = ((uint32_t)rest >> 8) & 0xffu;
+          const uint32_t l0c = 8u + (uint32_t)__popc(b0);
+          uint32_t code = s_spread[b0] | ((uint32_t)s_spread[b1] << l0c);
+          rest >>= 16;
+          if (!rest) code ^= 0x80000000u >> __clz((int)code);
+          const uint32_t sh = pos & 31u, w0 = pos >> 5;
+          const uint32_t clo = code << sh, chi = __funnelshift_l(code, 0u, sh);
+          if (PCZ_CHECK(pos + 32u - (uint32_t)__clz((int)(code | 1u)) <= CAP, 0)) {
+            if (clo) atomicOr(cbuf + w0, clo);
+            if (chi) atomicOr(cbuf + w0 + 1, chi);
+          }
+          pos += l0c + 8u + (uint32_t)__popc(b1);
         }
       }
-      if (lane == 0) {
-        const int64_t ci = (int64_t)i * P.nchunks + chunk;
-        uint32_t* cnt = P.chunk_counts + ci * 5;
-        cnt[0] = cz;
-        cnt[1] = cc;
-        cnt[2] = cr;
-        cnt[3] = (uint32_t)se;
-        cnt[4] = (uint32_t)sv;
-        if (P.chunk_maxerr) P.chunk_maxerr[ci] = me;
+      if (tid == 0) {
+        if (pool_base + cw > P.pool_words) {
+          atomicOr(P.flags, kFlagPoolOverflow);
+          pool_base = ~0ull;
+        }
+        *s_base = pool_base;
+        P.chunk_pool[(int64_t)i * P.nchunks + chunk] = pool_base;
       }
+      group_sync(bar_id);  // the chunk is complete, and its pool place known
+      append_chunk(P, cbuf, *s_base, *s_cbits, tid);
+      break;
     }
-    if (t == 0 && have) {
-      P.brick_len[(int64_t)i * P.nbricks + b] = (uint16_t)blen;
-      if (P.brick_off) P.brick_off[(int64_t)i * P.nbricks + b] = (uint32_t)(h ? offB : offA);
-    }
-
-    // this component's bits of the warp's two bricks, into the chunk buffer
-    const uint32_t boff = (uint32_t)(h ? offB : offA);
-    if (have && mode == kModeRaw) {
-      if (t == 0) or_bits_in(cbuf, boff, (uint64_t)kModeRaw, CAP, 0);
-#pragma unroll
-      for (int m = 0; m < 4; ++m) or_bits_in(cbuf, boff + 2 + F::P * (4 * t + m), (uint64_t)F::bits(eo[m]), CAP, 0);
-    } else if (have && mode == kModeCoded && t == 0) {
-      or_bits_in(cbuf, boff, (uint64_t)kModeCoded | ((uint64_t)esc << 2) | ((uint64_t)(emax + F::EBIAS) << 5), CAP,
-                 0);
-    }
-    const int modeA = __shfl_sync(FULL, mode, 0), modeB = __shfl_sync(FULL, mode, 16);
-    const bool haveA = __shfl_sync(FULL, (int)have, 0) != 0, haveB = __shfl_sync(FULL, (int)have, 16) != 0;
-    // R11: each coded plane's verbatim bits, by the plane's owner lane ...
-    if (haveA && modeA == kModeCoded) {
-      const uint32_t base = (uint32_t)offA + HDR;
-      if (lane >= pA && nA0 > 0) or_bits_in(cbuf, base + oA0, WA0 & low_mask64(nA0), CAP, 0);
-      if (WIDE && lane + 32 >= pA && nA1 > 0) or_bits_in(cbuf, base + oA1, WA1 & low_mask64(nA1), CAP, 0);
-    }
-    if (haveB && modeB == kModeCoded) {
-      const uint32_t base = (uint32_t)offB + HDR;
-      if (lane >= pB && nB0 > 0) or_bits_in(cbuf, base + oB0, WB0 & low_mask64(nB0), CAP, 0);
-      if (WIDE && lane + 32 >= pB && nB1 > 0) or_bits_in(cbuf, base + oB1, WB1 & low_mask64(nB1), CAP, 0);
-    }
-    // ... and its group-test bits, one token per newly significant coefficient,
-    // by the lane that holds the coefficient
-    if (have && mode == kModeCoded && p < F::P) {
-      const uint64_t* pw = s_pw + warp * 128 + 64 * h;
-      const uint32_t* pi = s_pi + warp * 128 + 64 * h;
-      const uint32_t base = boff + HDR;
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        if ((u[j] >> p) == 0) continue;  // no bit at or above the lowest coded plane
-        const int pc = F::P - 1 - F::clz(u[j]);
-        if (!PCZ_CHECK(pc >= 0 && pc < 64, 1)) continue;
-        const uint32_t info = pi[pc];
-        const int n = (int)((info >> 14) & 127u), c = t + 16 * j;
-        if (c >= n) write_token(cbuf, CAP, base + (info & 0x3fffu) + (uint32_t)n, pw[pc], n, c, (int)(info >> 21));
-      }
-    }
-#pragma unroll
-    for (int m = 0; m < 4; ++m) xt[m] = xtc[m];
-    if (tid == 0) {
-      unsigned long long base = pool_base;
-      if (base + pool_nw > P.pool_words) {
-        atomicOr(P.flags, kFlagPoolOverflow);
-        base = ~0ull;
-      }
-      s_base[i & 1] = base;
-      P.chunk_pool[(int64_t)i * P.nchunks + chunk] = base;
-    }
-    if (i > 0) append_chunk(P, cbufs + ((i - 1) & 1) * BUFW, s_base[(i - 1) & 1], s_cbits[(i - 1) & 1], tid);
   }
-  __syncthreads();
-  append_chunk(P, cbufs + ((P.n - 1) & 1) * BUFW, s_base[(P.n - 1) & 1], s_cbits[(P.n - 1) & 1], tid);
 }
 
 }  // namespace pcz

@@ -32,9 +32,14 @@
 
 namespace pcz {
 
+// CTAs that share an SM: 4 at 128 registers a thread for float32, 3 at 168 for
+// float64.
+template <typename T>
+constexpr int kCtas3 = sizeof(T) == 4 ? 4 : 3;
+
 // One chunk per CTA, each lane's line loaded straight into registers.
 template <typename T>
-__global__ void __launch_bounds__(kCompressThreads3, 2) k_compress3(const CompressParams P) {
+__global__ void __launch_bounds__(kCompressThreads3, kCtas3<T>) k_compress3(const CompressParams P) {
   extern __shared__ __align__(128) unsigned char smem[];
   compress3_chunk<T>(P, (int64_t)blockIdx.x, smem);
 }
@@ -42,7 +47,7 @@ __global__ void __launch_bounds__(kCompressThreads3, 2) k_compress3(const Compre
 // Persistent CTAs with the chunks staged by TMA: chunk c's values are copied
 // into shared memory while chunk c - grid is coded.
 template <typename T>
-__global__ void __launch_bounds__(kCompressThreads3, 2)
+__global__ void __launch_bounds__(kCompressThreads3, kCtas3<T>)
     k_compress3_tma(const CompressParams P, const __grid_constant__ CUtensorMap tmap, int row_box) {
   extern __shared__ __align__(128) unsigned char smem[];
   T* xs = reinterpret_cast<T*>(smem);
@@ -62,7 +67,7 @@ __global__ void __launch_bounds__(kCompressThreads3, 2)
       return;
     }
     parity ^= 1u;
-    compress3_chunk<T>(P, c, smem, &tmap, row_box != 0, bar, c + gridDim.x);
+    compress3_chunk<T>(P, c, smem, 0, &tmap, row_box != 0, bar, c + gridDim.x);
   }
 }
 
