@@ -3,9 +3,9 @@
 // Algorithm 2 (Sec. 4.2) over a batch of boxes of several fields.
 //
 // Construction: two kernels run side by side (two branches of one CUDA
-// graph), or one kernel does both parts.  In the 3D kernel, CTAs of 512
-// threads claim items from a work counter; an item is one chunk of 32 bricks of a 3D field, which the
-// whole CTA codes as pcz_compress.cu does.  In the 1D/2D kernel, CTAs of a
+// graph), or one kernel does both parts.  In the 3D kernel, CTAs of 4
+// warps claim items from a work counter; an item is one chunk of 32 bricks of a
+// 3D field, which the CTA codes as pcz_compress.cu does.  In the 1D/2D kernel, CTAs of a
 // few warps claim items of several chunks of a 1D or 2D field from a second
 // counter, and each warp codes one chunk at a time, a brick per lane, as
 // pcz_small.cu does (no register cap: a 2D brick of float64 values lives in
@@ -62,7 +62,7 @@ __device__ __forceinline__ void find_item(const BatchParams* __restrict__ bp, in
 // one fewer with more registers a thread.
 template <typename T>
 constexpr int batch3_ctas(int variant) {
-  return (sizeof(T) == 4 ? 4 : 3) - (variant == 2 ? 0 : 1);
+  return (sizeof(T) == 4 ? 6 : 3) - (variant == 2 ? 0 : 1);
 }
 
 // 3D part of a batch: CTAs of 4 warps claim chunks of the 3D
@@ -389,14 +389,14 @@ struct BatchArena {
 
 // A schedule of the batched construction: the order of the fields' work,
 // the block shapes of the two persistent kernels and how much a claim takes.
-// A 3D item is one chunk of 32 bricks for a whole CTA of 16 warps (two bricks
-// per warp); `ctas3` such CTAs share an SM (1 at up to 128 registers per
-// thread, 2 at 64).  A 1D/2D item is warps_small * chunks_per_warp chunks
+// A 3D item is one chunk of 32 bricks for a CTA of 4 warps (8 bricks
+// per warp); `ctas3` chooses the kernel variant by the CTAs that share an SM
+// (batch3_ctas).  A 1D/2D item is warps_small * chunks_per_warp chunks
 // for a CTA of warps_small warps, one chunk (a brick per lane) per warp at a
 // time.
 struct Schedule {
   int order;            // 0: fields in the caller's order; 1: largest first
-  int ctas3;            // CTAs per SM of the 3D kernel: 1 or 2; 0: one kernel for both parts, whose
+  int ctas3;            // variant of the 3D kernel: 1 or 2; 0: one kernel for both parts, whose
                         // CTAs of 16 warps take 3D and 1D/2D items from one queue
   int warps_small;      // warps per CTA of the 1D/2D kernel: 2, 4, 8 or 16
   int chunks_per_warp;  // chunks per warp in a 1D/2D item: 1 or 2
@@ -947,7 +947,7 @@ pc_status pc_batch_info(const pc_batch* B, pc_batch_info_t* info) {
     info->order = sc.order;
     info->chunks_per_item = sc.warps_small * sc.chunks_per_warp;
     info->items_per_claim = sc.per_fetch;
-    info->ctas_per_sm = sc.ctas3 ? sc.ctas3 : 1;
+    info->ctas_per_sm = !sc.ctas3 ? 1 : B->dtype == PC_F32 ? batch3_ctas<float>(sc.ctas3) : batch3_ctas<double>(sc.ctas3);
     info->warps_small = sc.warps_small;
     info->mixed = sc.ctas3 == 0;
   }

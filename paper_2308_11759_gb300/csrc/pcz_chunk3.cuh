@@ -46,7 +46,8 @@ constexpr int kWarps3 = kCompressThreads3 / 32;
 //      16-byte vectors of 4 values along x (float64: two such sets, 2 values
 //      each), vector (y, z) of brick b at (b >> 1) * 38 + (b & 1) + 10 z + 2 y.
 //      Both directions are free of bank conflicts.
-//  (b) the digits in coded order, brick b from word 72 b (or 36 b as halves);
+//  (b) the digits in coded order, brick b from word 72 b (36 b as halves, 20 b
+//      as bytes);
 //  (c) the plane words, brick b from word b * kPlaneStride: word j of the
 //      lane's 16 coefficients q at 4 j + q; a RAW brick's residual in their place.
 template <typename T>
@@ -92,7 +93,7 @@ __host__ __device__ constexpr size_t compress_smem3(bool staged = false) {
          + (size_t)chunk_buf_words3<T>() * 4                        // chunk bit buffer
          + (size_t)kWarps3 * Area3<T>::kWords * 4                   // work areas
          + (size_t)kChunk * Area3<T>::kInfoStride * 4               // plane offsets and counts
-         + (sizeof(T) == 8 ? (size_t)kChunk * 64 * sizeof(T) : 0)   // the chunk's values (float32: in registers)
+         + (size_t)kChunk * 64 * sizeof(T)                          // the chunk's values
          + kSpreadBytes                                             // group-test code table
          + 4 * 32 * 4                                               // lengths, modes, escalations, violations
          + 32 * 8                                                   // per brick: bits of max |x - x~_i|
@@ -104,7 +105,9 @@ __device__ __forceinline__ void group_sync(int id) {
   asm volatile("bar.sync %0, 128;" ::"r"(id) : "memory");
 }
 
-// Bit transposes within a lane.  transpose16: word i holds 16 bits (planes) of
+// Bit transposes within a lane.  transpose8: word i holds 8 bits (planes) each
+// of the coefficients i, i + 8, i + 4 and i + 12 (from its low byte up);
+// afterwards word j holds planes j and j + 4 of the 16 coefficients.  transpose16: word i holds 16 bits (planes) of
 // coefficient i in its low half and of coefficient i + 8 in its high half;
 // afterwards word j holds plane j of the 16 coefficients in its low half and
 // plane j + 8 in its high half.  transpose32: word i holds 32 bits of
@@ -120,6 +123,15 @@ __device__ __forceinline__ void exchange_stage(uint32_t (&a)[N], uint32_t m) {
       a[i] = (x & m) | ((y << K) & ~m);
       a[i + K] = ((x >> K) & m) | (y & ~m);
     }
+}
+__device__ __forceinline__ void transpose8(uint32_t (&a)[4]) {
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const uint32_t t = (a[i] ^ (a[i] >> 12)) & 0x0000F0F0u;
+    a[i] ^= t ^ (t << 12);
+  }
+  exchange_stage<4, 2>(a, 0x33333333u);
+  exchange_stage<4, 1>(a, 0x55555555u);
 }
 __device__ __forceinline__ void transpose16(uint32_t (&a)[8]) {
 #pragma unroll
@@ -149,15 +161,35 @@ __device__ __forceinline__ uint64_t magnitude(double v) {
 }
 
 // The largest magnitude of a brick: over a lane's 16 values, then its 4 lanes.
+// float32 takes the maximum of |v| with NaN propagated, one instruction per
+// value; a NaN's own bits, which that maximum does not keep, are looked up.
+__device__ __forceinline__ float max_abs_nan(float a, float b) {
+  float r;
+  asm("{\n .reg .f32 t;\n abs.f32 t, %2;\n max.NaN.f32 %0, %1, t;\n}\n" : "=f"(r) : "f"(a), "f"(b));
+  return r;
+}
 template <typename T>
 __device__ __forceinline__ typename Fmt<T>::U brick_max(const T* e) {
   using U = typename Fmt<T>::U;
   constexpr unsigned FULL = 0xffffffffu;
-  U m = magnitude(e[0]);
+  U m;
+  if constexpr (sizeof(T) == 4) {
+    float f = 0.0f;
 #pragma unroll
-  for (int v = 1; v < 16; ++v) {
-    const U a = magnitude(e[v]);
-    m = a > m ? a : m;
+    for (int v = 0; v < 16; ++v) f = max_abs_nan(f, e[v]);
+    m = __float_as_uint(f);
+    if (m > Fmt<T>::INF) {
+      m = 0;
+#pragma unroll
+      for (int v = 0; v < 16; ++v) m = max(m, magnitude(e[v]));
+    }
+  } else {
+    m = magnitude(e[0]);
+#pragma unroll
+    for (int v = 1; v < 16; ++v) {
+      const U a = magnitude(e[v]);
+      m = a > m ? a : m;
+    }
   }
 #pragma unroll
   for (int o = 1; o <= 2; o <<= 1) {
@@ -185,6 +217,32 @@ __device__ __forceinline__ void pad_brick(T* e, int nvx, int nvy, int nvz, int l
   const int src = (lane & ~3) | min(lane & 3, nvz - 1);
 #pragma unroll
   for (int v = 0; v < 16; ++v) e[v] = __shfl_sync(0xffffffffu, e[v], src);
+}
+
+// Bits 0 .. n - 1 of a 64-bit mask, n in 0..64.
+__device__ __forceinline__ void low_mask(int n, uint32_t* lo, uint32_t* hi) {
+  asm("bmsk.clamp.b32 %0, 0, %1;" : "=r"(*lo) : "r"(n));
+  asm("bmsk.clamp.b32 %0, 0, %1;" : "=r"(*hi) : "r"(max(n - 32, 0)));
+}
+
+// OR of the three words that 64 bits hi:lo span from bit pos of a bit buffer.
+__device__ __forceinline__ void or_words(uint32_t* buf, uint32_t pos, uint32_t lo, uint32_t hi) {
+  uint32_t* w = buf + (pos >> 5);
+  const uint32_t a = lo << (pos & 31u), b = __funnelshift_l(lo, hi, pos), c = __funnelshift_l(hi, 0u, pos);
+  if (a) atomicOr(w, a);
+  if (b) atomicOr(w + 1, b);
+  if (c) atomicOr(w + 2, c);
+}
+
+// The plane word at plane p + j of a brick (layout of Area3's use (c)): its two
+// halves, from the 4 lanes' 16 coefficients each; 0 for j < 0.
+template <bool WIDE>
+__device__ __forceinline__ void plane_at(const uint32_t* planes, int j, int H, uint32_t* lo, uint32_t* hi) {
+  const int at = 4 * (j & (H - 1)) + (WIDE && j >= 32 ? 64 : 0);
+  const uint4 r = *reinterpret_cast<const uint4*>(planes + at);
+  const uint32_t sel = j & H ? 0x7632u : 0x5410u;
+  *lo = j >= 0 ? __byte_perm(r.x, r.y, sel) : 0u;
+  *hi = j >= 0 ? __byte_perm(r.z, r.w, sel) : 0u;
 }
 
 // 4 values along x to and from the work area, in 16-byte vectors (`set`
@@ -386,8 +444,11 @@ __device__ __forceinline__ void append_chunk(const CompressParams& P, uint32_t* 
 // fewest: both in-plane lifting passes run in registers, the bits are
 // transposed in registers, reductions over a brick take two shuffles, and what
 // a component costs per warp (votes, scans, the barrier) is shared by 512
-// values.  With 16 lanes per brick and 4 values per lane, as before, it took
-// 582 (float32) and 997 (float64) warp instructions per brick and component.
+// values.  With 16 lanes per brick and 4 values per lane it took 582 (float32)
+// and 997 (float64) warp instructions per brick and component, now 187 and 284;
+// 512^3 float32, 8 components: 10.16 -> 3.52 ms, 256 x 384 x 384 float64, 12
+// components: 8.77 -> 3.35 ms.  It runs at 0.71 (float32; ALU pipe 0.67) and
+// 0.47 (float64) of the issue peak.
 template <typename T>
 __device__ __forceinline__ void compress3_chunk(const CompressParams& P, int64_t chunk, unsigned char* smem,
                                                 int bar_id = 0, const CUtensorMap* map = nullptr,
@@ -397,6 +458,7 @@ __device__ __forceinline__ void compress3_chunk(const CompressParams& P, int64_t
   using S = typename F::S;
   using A3 = Area3<T>;
   constexpr bool WIDE = F::P == 64;
+  constexpr int XV = 16 / (int)sizeof(T);  // values of a 16-byte part
   constexpr int Q = F::P - 2 - Geo<3>::G;  // quantisation bits (R6)
   constexpr int C = Geo<3>::C;             // guard planes (R10)
   constexpr int HDR = 2 + 3 + F::EBITS;    // mode, escalation, block exponent
@@ -409,8 +471,8 @@ __device__ __forceinline__ void compress3_chunk(const CompressParams& P, int64_t
   uint32_t* cbuf = reinterpret_cast<uint32_t*>(smem + staging_bytes3<T>(map != nullptr));
   uint32_t* areas = cbuf + BUFW;
   uint32_t* infos = areas + kWarps3 * A3::kWords;  // [brick][k]: plane offset << 8 | n
-  double2* s_x = reinterpret_cast<double2*>(infos + kChunk * A3::kInfoStride);  // float64: [16-byte part][thread]
-  uint16_t* s_spread = reinterpret_cast<uint16_t*>(s_x + (WIDE ? kChunk * 64 * sizeof(T) / 16 : 0));
+  uint4* s_x = reinterpret_cast<uint4*>(infos + kChunk * A3::kInfoStride);  // [16-byte part][thread]
+  uint16_t* s_spread = reinterpret_cast<uint16_t*>(s_x + kChunk * 64 * sizeof(T) / 16);
   int* s_len = reinterpret_cast<int*>(s_spread + 256);
   int* s_mode = s_len + 32;
   int* s_esc = s_mode + 32;
@@ -444,10 +506,12 @@ __device__ __forceinline__ void compress3_chunk(const CompressParams& P, int64_t
   }
   const bool any_partial = __any_sync(FULL, nvx < 4 || nvy < 4 || nvz < 4);
 
-  // The values (float64: kept in shared memory, read back twice a component),
-  // padded (R4).  Algorithm 1 starts from x~ = 0, so the first residual is x
-  // itself (x - 0 in IEEE arithmetic, -0 included).
-  T x[16], xt[16], e[16];
+  // The values, padded (R4), are kept in shared memory, each lane's own, and
+  // read back once per component: that leaves float32 the registers for 6 CTAs
+  // per SM instead of 4 (512^3, 8 components: 3.98 -> 3.55 ms).  Algorithm 1
+  // starts from x~ = 0, so the first residual is x itself (x - 0 in IEEE
+  // arithmetic, -0 included).
+  T xt[16], e[16];
   if (have) {
     const T* field = reinterpret_cast<const T*>(P.field);
     const int64_t gz = 4 * bz + min(q, nvz - 1);
@@ -469,21 +533,31 @@ __device__ __forceinline__ void compress3_chunk(const CompressParams& P, int64_t
       issue_chunk_copy<T>(P, map, row_box, next, reinterpret_cast<T*>(smem), bar);
     }
   }
-  auto load_x = [&](int part, T* two) {  // float64: values 2 part, 2 part + 1
-    const double2 d = s_x[part * kCompressThreads3 + tid];
-    two[0] = (T)d.x;
-    two[1] = (T)d.y;
+#pragma unroll
+  for (int v = 0; v < 16; ++v) xt[v] = T(0);
+  union Part {
+    uint4 w;
+    T v[XV];
+    __device__ Part() {}
   };
 #pragma unroll
-  for (int v = 0; v < 16; ++v) {
-    xt[v] = T(0);
-    if constexpr (!WIDE) x[v] = e[v];
-  }
-  if constexpr (WIDE) {
+  for (int h = 0; h < 16 / XV; ++h) {
+    Part t;
 #pragma unroll
-    for (int h = 0; h < 8; ++h)
-      s_x[h * kCompressThreads3 + tid] = make_double2(e[2 * h], e[2 * h + 1]);
+    for (int o = 0; o < XV; ++o) t.v[o] = e[XV * h + o];
+    s_x[h * kCompressThreads3 + tid] = t.w;
   }
+  // r = x - a, padded
+  auto residual_of = [&](const T* a, T* r) {
+#pragma unroll
+    for (int h = 0; h < 16 / XV; ++h) {
+      Part t;
+      t.w = s_x[h * kCompressThreads3 + tid];
+#pragma unroll
+      for (int o = 0; o < XV; ++o) r[XV * h + o] = F::sub(t.v[o], a[XV * h + o]);
+    }
+    if (any_partial) pad_brick<T>(r, nvx, nvy, nvz, lane);
+  };
   U m = brick_max<T>(e);  // the largest magnitude of the residual, by brick
   if (__any_sync(FULL, m >= F::INF) && lane == 0) atomicOr(P.flags, kFlagNonFinite);
 
@@ -492,8 +566,9 @@ __device__ __forceinline__ void compress3_chunk(const CompressParams& P, int64_t
   uint4* yw = reinterpret_cast<uint4*>(area) + (bq >> 1) * 38 + (bq & 1) + 2 * q;   // + 10 z: line (y = q, z)
   uint32_t* planes = area + bq * A3::kPlaneStride;
   uint32_t* info = infos + slot * A3::kInfoStride;
-  // places of this lane's coefficients in coded order, four to a register:
-  // byte offset 32 (r / 16) + 4 (r & 7) + 2 ((r >> 3) & 1) of rank r
+  // places of this lane's coefficients in coded order, a byte each: rank r at
+  // 16 (r / 16) + 4 (r & 3) + 2 ((r >> 2) & 1) + ((r >> 3) & 1), in elements of
+  // 1, 2 or 4 bytes
   uint32_t place[4];
 #pragma unroll
   for (int z = 0; z < 4; ++z) {
@@ -501,7 +576,7 @@ __device__ __forceinline__ void compress3_chunk(const CompressParams& P, int64_t
 #pragma unroll
     for (int xx = 0; xx < 4; ++xx) {
       const int r = kRank3.pos[xx + 4 * q + 16 * z];
-      place[z] |= (uint32_t)(32 * (r >> 4) + 4 * (r & 7) + 2 * ((r >> 3) & 1)) << (8 * xx);
+      place[z] |= (uint32_t)((r & 48) + 4 * (r & 3) + 2 * ((r >> 2) & 1) + ((r >> 3) & 1)) << (8 * xx);
     }
   }
 
@@ -519,7 +594,7 @@ __device__ __forceinline__ void compress3_chunk(const CompressParams& P, int64_t
     for (;;) {  // again, with more planes in some brick, while Eq. 1 fails (R13): at most 8 times
       // The blocks' common scales let every value take the short forms of R6
       // and R13; other scales take the general ones.
-      const bool common = __all_sync(FULL, WIDE ? s >= -960 && s <= 1000 : s >= -126 && s <= 126);
+      const bool common = __all_sync(FULL, WIDE ? s >= -960 && s <= 1000 : s >= -96 && s <= 126);
       S v[16];
       if constexpr (!WIDE) {
         if (common) {
@@ -544,42 +619,77 @@ __device__ __forceinline__ void compress3_chunk(const CompressParams& P, int64_t
         }
       }
       lift_fwd_bricks<S>(v, zw, yw, SET);  // R7
-      // R9, and the highest plane that is not empty
-      U any = 0;
+      // R9, and the highest plane that is not empty.  Float64 takes it from the
+      // high words; where they are empty in a coded brick, from the low ones.
+      uint32_t any = 0;
+      int top = -1;
 #pragma unroll
       for (int k = 0; k < 16; ++k) {
         const U u = nb_fwd<T>(v[k]);
-        any |= u;
+        any |= (uint32_t)(u >> (F::P - 32));
         v[k] = (S)u;
       }
       any |= __shfl_xor_sync(FULL, any, 1);
       any |= __shfl_xor_sync(FULL, any, 2);
+      if (any) top = F::P - 1 - __clz((int)any);
+      if constexpr (WIDE) {
+        if (__any_sync(FULL, coded && !any)) {
+          uint32_t low = 0;
+#pragma unroll
+          for (int k = 0; k < 16; ++k) low |= (uint32_t)v[k];
+          low |= __shfl_xor_sync(FULL, low, 1);
+          low |= __shfl_xor_sync(FULL, low, 2);
+          if (!any && low) top = 31 - __clz((int)low);
+        }
+      }
       // R10: the lowest coded plane
       const int p = coded ? min(max(L + s - C - esc, 0), F::P) : F::P;
-      const int top = any ? F::P - 1 - F::clz(any) : -1;
       const int nw = top - p + 1;  // planes from the highest that is not empty down to p
-      // the coded digits, from plane p up
-#pragma unroll
-      for (int k = 0; k < 16; ++k) v[k] = (S)(p >= F::P ? U(0) : (U)v[k] >> (p & (F::P - 1)));
       const int span = (int)__reduce_max_sync(FULL, (unsigned)max(nw, 0));
+
+      // the coded digits, from plane p up: 32 of them (float64 where p >= 32 ...)
+      auto digits = [&](int k) {
+        if constexpr (WIDE)
+          return __funnelshift_rc((uint32_t)((U)v[k] >> 32), 0u, p - 32);
+        else
+          return __funnelshift_rc((uint32_t)v[k], 0u, p);
+      };
+      auto digits64 = [&](int k) { return p >= F::P ? U(0) : (U)v[k] >> (p & (F::P - 1)); };  // (... and all)
 
       // the digits in coded order (R8), 16 ranks per lane, and their transpose:
       // plane words from word 4 j + q of the brick's plane area
-      auto planes16 = [&] {
-        unsigned char* put = reinterpret_cast<unsigned char*>(area + 36 * bq);
+      auto planes8 = [&](const uint32_t* w) {
+        const uint32_t put = smem_addr(area + 20 * bq);
+#pragma unroll
+        for (int k = 0; k < 16; ++k)  // the address: put + byte k & 3 of place
+          asm volatile("st.shared.u8 [%0], %1;" ::"r"(__dp4a(place[k >> 2], 1u << (8 * (k & 3)), put)), "r"(w[k])
+                       : "memory");
+        __syncwarp();
+        const uint4 r = *reinterpret_cast<const uint4*>(area + 20 * bq + 4 * q);
+        uint32_t a[4] = {r.x, r.y, r.z, r.w};
+        __syncwarp();
+        transpose8(a);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) planes[4 * j + q] = a[j];
+        __syncwarp();
+      };
+      auto planes16 = [&](const uint32_t* w) {
+        const uint32_t put = smem_addr(area + 36 * bq);
 #pragma unroll
         for (int k = 0; k < 16; ++k)
-          *reinterpret_cast<uint16_t*>(put + ((place[k >> 2] >> (8 * (k & 3))) & 0xffu)) = (uint16_t)v[k];
+          asm volatile("st.shared.u16 [%0], %1;" ::"r"(__dp4a(place[k >> 2], 2u << (8 * (k & 3)), put)),
+                       "h"((uint16_t)w[k])
+                       : "memory");
         __syncwarp();
         uint32_t a[8];
         const uint4* get = reinterpret_cast<const uint4*>(area + 36 * bq + 8 * q);
 #pragma unroll
-        for (int k = 0; k < 2; ++k) {
+        for (int k = 0; k < 2; ++k) {  // ranks 2k, 2k + 4, 2k + 1, 2k + 5, each with the one 8 above it
           const uint4 r = get[k];
-          a[4 * k] = r.x;
-          a[4 * k + 1] = r.y;
-          a[4 * k + 2] = r.z;
-          a[4 * k + 3] = r.w;
+          a[2 * k] = r.x;
+          a[2 * k + 4] = r.y;
+          a[2 * k + 1] = r.z;
+          a[2 * k + 5] = r.w;
         }
         __syncwarp();
         transpose16(a);
@@ -589,19 +699,20 @@ __device__ __forceinline__ void compress3_chunk(const CompressParams& P, int64_t
       };
       // 32 planes: the digits of 16 ranks, then (half 0: planes p + j) their words
       auto ranks32 = [&](const uint32_t* w, uint32_t (&a)[16]) {
-        unsigned char* put = reinterpret_cast<unsigned char*>(area + 72 * bq);
+        const uint32_t put = smem_addr(area + 72 * bq);
 #pragma unroll
         for (int k = 0; k < 16; ++k)
-          *reinterpret_cast<uint32_t*>(put + 2 * ((place[k >> 2] >> (8 * (k & 3))) & 0xffu)) = w[k];
+          asm volatile("st.shared.u32 [%0], %1;" ::"r"(__dp4a(place[k >> 2], 4u << (8 * (k & 3)), put)), "r"(w[k])
+                       : "memory");
         __syncwarp();
         const uint4* get = reinterpret_cast<const uint4*>(area + 72 * bq + 16 * q);
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {  // ranks 2k, 2k + 8, 2k + 1, 2k + 9
+        for (int k = 0; k < 4; ++k) {  // ranks k, k + 8, k + 4, k + 12
           const uint4 r = get[k];
-          a[2 * k] = r.x;
-          a[2 * k + 8] = r.y;
-          a[2 * k + 1] = r.z;
-          a[2 * k + 9] = r.w;
+          a[k] = r.x;
+          a[k + 8] = r.y;
+          a[k + 4] = r.z;
+          a[k + 12] = r.w;
         }
         __syncwarp();
       };
@@ -617,63 +728,61 @@ __device__ __forceinline__ void compress3_chunk(const CompressParams& P, int64_t
         __syncwarp();
       };
 
+      // the plane words of at most 32 planes; returns how many words hold planes
+      auto planes_of = [&](const uint32_t* w) {
+        if (span <= 8) {
+          planes8(w);
+          return 4;
+        }
+        if (span <= 16) {
+          planes16(w);
+          return 8;
+        }
+        planes32(w);
+        return 16;
+      };
+
       // R13: decode-back x_i = D(y_i), the candidate x~ + x_i and the residual
       // it leaves.  Bricks that are not coded decode to 0, which leaves x~ and
       // the residual as they are.
       T xtn[16], en[16];
-      auto residual = [&] {
-        if constexpr (WIDE) {
-#pragma unroll
-          for (int h = 0; h < 8; ++h) {
-            T two[2];
-            load_x(h, two);
-            en[2 * h] = F::sub(two[0], xtn[2 * h]);
-            en[2 * h + 1] = F::sub(two[1], xtn[2 * h + 1]);
-          }
-        } else {
-#pragma unroll
-          for (int k = 0; k < 16; ++k) en[k] = F::sub(x[k], xtn[k]);
-        }
-        if (any_partial) pad_brick<T>(en, nvx, nvy, nvz, lane);
-      };
-      int H = 8;  // plane words: plane j in half j / H of word j mod H
+      int H;  // plane p + j is in half (j / H) & 1 of word j mod H
       if constexpr (!WIDE) {
         {
           S r[16];
+          const U keep = __funnelshift_lc(0u, ~0u, p);  // planes p and up
 #pragma unroll
-          for (int k = 0; k < 16; ++k) r[k] = nb_inv<T>(p >= 32 ? 0u : (U)v[k] << (p & 31));
+          for (int k = 0; k < 16; ++k) r[k] = nb_inv<T>((U)v[k] & keep);
           lift_inv_bricks<S>(r, zw, yw, SET);
           if (common) {
+            // int -> float rounds once; the product by 2^-s is exact (normal, and
+            // below 2^127 for s >= -96), so one fused add is x~ + x_i
             const float sc = __uint_as_float((uint32_t)(127 - s) << 23);
 #pragma unroll
-            for (int k = 0; k < 16; ++k) xtn[k] = F::add(xt[k], __fmul_rn(__int2float_rn(r[k]), sc));
+            for (int k = 0; k < 16; ++k) xtn[k] = __fmaf_rn(__int2float_rn(r[k]), sc, xt[k]);
           } else {
 #pragma unroll
             for (int k = 0; k < 16; ++k) xtn[k] = F::add(xt[k], F::val(dequantize_any<T>(r[k], s)));
           }
         }
-        residual();
-        if (span <= 16) {
-          planes16();
-        } else {
-          uint32_t w[16];
+        residual_of(xtn, en);
+        uint32_t w[16];
 #pragma unroll
-          for (int k = 0; k < 16; ++k) w[k] = (uint32_t)v[k];
-          planes32(w);
-          H = 16;
-        }
+        for (int k = 0; k < 16; ++k) w[k] = digits(k);
+        H = planes_of(w);
       } else {
-        // Digits within 20 planes from plane p >= 6 on, none above plane 58:
-        // decoded in 32-bit integers in units of 2^(p - 6).  A coefficient with
-        // negabinary digits d from plane p is ((d ^ M) - M) * 2^p with M =
-        // NBM >> p (M's bits above d's do not matter).  In these units each
-        // inverse lifting pass turns multiples of 2^a into multiples of
-        // 2^(a - 2), so from 2^6 on every shift divides an even number exactly;
-        // |value| < 2^(19 + 6.42) * 2.75^3 < 2^30 (2.75: the largest row sum of
-        // the inverse lifting's coefficients), while the unscaled value stays
-        // below 2^(58 + 4.8) <= 2^63: neither form wraps, so the result is the
-        // 64-bit decoding's exactly, in half the instructions.
-        const bool narrow = common && __all_sync(FULL, nw <= 0 || (nw <= 20 && p >= 6 && top <= 58));
+        // Digits within 20 planes from plane p in 32..57 on: decoded in 32-bit
+        // integers in units of 2^(p - 6).  A coefficient with negabinary digits d
+        // from plane p is ((d ^ M) - M) * 2^p with M = NBM >> p (M's bits above
+        // d's do not matter).  In these units each inverse lifting pass turns
+        // multiples of 2^a into multiples of 2^(a - 2), so from 2^6 on every
+        // shift divides an even number exactly; |value| < 2^(19 + 6.42) * 2.75^3
+        // < 2^30 (2.75: the largest row sum of the inverse lifting's
+        // coefficients).  The 64-bit form does not wrap either: without the
+        // truncation its values are the forward transform's, below 2^62, and the
+        // truncation moves them by less than 2.75^3 * 2^p < 2^62.  So the result
+        // is the 64-bit decoding's exactly, in half the instructions.
+        const bool narrow = common && __all_sync(FULL, !coded || (nw <= 20 && p >= 32 && p <= 57));
         auto add = [&](int k, T xi) {  // x~ + x_i; the first component's +0 + x_i is x_i with -0 turned to +0
           if (i == 0)
             xtn[k] = F::val(F::bits(xi) == F::SIGN ? U(0) : F::bits(xi));
@@ -683,42 +792,38 @@ __device__ __forceinline__ void compress3_chunk(const CompressParams& P, int64_t
         if (narrow) {
           uint32_t w[16];
 #pragma unroll
-          for (int k = 0; k < 16; ++k) w[k] = (uint32_t)v[k];
+          for (int k = 0; k < 16; ++k) w[k] = digits(k);
           int32_t r[16];
-          const uint32_t M = (uint32_t)(F::NBM >> min(p, 63));
+          const uint32_t M = (uint32_t)(F::NBM >> min(p, 63)), M64 = M << 6;
 #pragma unroll
-          for (int k = 0; k < 16; ++k) r[k] = (int32_t)(((w[k] ^ M) - M) << 6);
+          for (int k = 0; k < 16; ++k) r[k] = (int32_t)(((w[k] ^ M) << 6) - M64);
           lift_inv_bricks<int32_t>(r, zw, yw, SET);
           const uint32_t eb = (uint32_t)(1053 + (p - 6) - s) << 20;
 #pragma unroll
           for (int k = 0; k < 16; ++k) add(k, scaled_i32_to_f64(r[k], eb));
-          residual();
-          if (span <= 16) {
-            planes16();
-          } else {
-            planes32(w);
-            H = 16;
-          }
+          residual_of(xtn, en);
+          H = planes_of(w);
         } else {
           S r[16];
+          const U keep = p >= 64 ? U(0) : ~U(0) << p;  // planes p and up
 #pragma unroll
-          for (int k = 0; k < 16; ++k) r[k] = nb_inv<T>(p >= 64 ? U(0) : (U)v[k] << (p & 63));
+          for (int k = 0; k < 16; ++k) r[k] = nb_inv<T>((U)v[k] & keep);
           lift_inv_bricks<S>(r, zw, yw, SET);
 #pragma unroll
           for (int k = 0; k < 16; ++k)
             add(k, F::val(common ? dequantize_f64_normal(r[k], s) : dequantize_any<T>(r[k], s)));
-          residual();
+          residual_of(xtn, en);
           H = 16;
           uint32_t w[16];
 #pragma unroll
-          for (int k = 0; k < 16; ++k) w[k] = (uint32_t)v[k];
+          for (int k = 0; k < 16; ++k) w[k] = (uint32_t)digits64(k);
           if (span <= 32) {
             planes32(w);
           } else {  // both halves' digits are read before the words take their place
             uint32_t a0[16], a1[16];
             ranks32(w, a0);
 #pragma unroll
-            for (int k = 0; k < 16; ++k) w[k] = (uint32_t)((U)v[k] >> 32);
+            for (int k = 0; k < 16; ++k) w[k] = (uint32_t)(digits64(k) >> 32);
             ranks32(w, a1);
             words32(a0, 0);
             words32(a1, 1);
@@ -731,19 +836,7 @@ __device__ __forceinline__ void compress3_chunk(const CompressParams& P, int64_t
       const bool again = coded && !pass && p > 0 && esc < 7;
       if (__any_sync(FULL, again)) {  // rare: code the warp's bricks again from the same residual
         if (again) ++esc;
-        if constexpr (WIDE) {
-#pragma unroll
-          for (int h = 0; h < 8; ++h) {
-            T two[2];
-            load_x(h, two);
-            e[2 * h] = F::sub(two[0], xt[2 * h]);
-            e[2 * h + 1] = F::sub(two[1], xt[2 * h + 1]);
-          }
-        } else {
-#pragma unroll
-          for (int k = 0; k < 16; ++k) e[k] = F::sub(x[k], xt[k]);
-        }
-        if (any_partial) pad_brick<T>(e, nvx, nvy, nvz, lane);
+        residual_of(xt, e);
         continue;
       }
 
@@ -757,27 +850,22 @@ __device__ __forceinline__ void compress3_chunk(const CompressParams& P, int64_t
         int carry = 0;
         for (int k = 0; k < nrow; ++k) {
           const int j = nw - 1 - 4 * k - q;  // plane p + j
-          uint64_t W = 0;
-          if (j >= 0) {
-            const uint4 r = *reinterpret_cast<const uint4*>(planes + 64 * (j >> 5) + 4 * (j & (H - 1)));
-            const uint32_t sel = j & H ? 0x7632u : 0x5410u;
-            W = (uint64_t)__byte_perm(r.x, r.y, sel) | ((uint64_t)__byte_perm(r.z, r.w, sel) << 32);
-          }
-          const int hi = W ? 64 - __clzll((long long)W) : 0;
-          int n = hi;
+          uint32_t lo, hi;
+          plane_at<WIDE>(planes, j, H, &lo, &hi);
+          int n = (int)(31 - __clz((int)(hi ? hi : lo))) + 1 + (hi ? 32 : 0);  // one past the highest position
           int t = __shfl_up_sync(FULL, n, 1, 4);
           if (q >= 1) n = max(n, t);
           t = __shfl_up_sync(FULL, n, 2, 4);
           if (q >= 2) n = max(n, t);
-          const int all = max(carry, __shfl_sync(FULL, n, 3, 4));
-          t = __shfl_up_sync(FULL, n, 1, 4);
-          n = q ? max(carry, t) : carry;
-          carry = all;
-          int len = 0;
-          if (j >= 0) {
-            len = n;
-            if (n < 64) len += hi > n ? __popcll((long long)(W >> n)) + hi - n + (hi < 64 ? 1 : 0) : 1;
-          }
+          const int after = max(n, carry);  // significant after the plane
+          t = __shfl_up_sync(FULL, after, 1, 4);
+          n = q ? t : carry;  // and before it
+          carry = __shfl_sync(FULL, after, 3, 4);
+          // n verbatim bits, the positions and 1s from n on, the closing 0
+          uint32_t mlo, mhi;
+          low_mask(n, &mlo, &mhi);
+          int len = after + __popc(lo & ~mlo) + __popc(hi & ~mhi) + (after < 64 ? 1 : 0);
+          if (j < 0) len = 0;
           int sum = len;
           t = __shfl_up_sync(FULL, sum, 1, 4);
           if (q >= 1) sum += t;
@@ -795,35 +883,10 @@ __device__ __forceinline__ void compress3_chunk(const CompressParams& P, int64_t
       if (__any_sync(FULL, mode == kModeRaw || (pass && lenC > LEN_RAW))) {
         // the residual the brick started from, and x~ and the residual after it
         T eo[16], xr[16], er[16];
-        if constexpr (WIDE) {
+        residual_of(xt, eo);
 #pragma unroll
-          for (int h = 0; h < 8; ++h) {
-            T two[2];
-            load_x(h, two);
-            eo[2 * h] = F::sub(two[0], xt[2 * h]);
-            eo[2 * h + 1] = F::sub(two[1], xt[2 * h + 1]);
-          }
-        } else {
-#pragma unroll
-          for (int k = 0; k < 16; ++k) eo[k] = F::sub(x[k], xt[k]);
-        }
-        if (any_partial) pad_brick<T>(eo, nvx, nvy, nvz, lane);
-#pragma unroll
-        for (int h = 0; h < 8; ++h) {
-          T two[2];
-          if constexpr (WIDE) {
-            load_x(h, two);
-          } else {
-            two[0] = x[2 * h];
-            two[1] = x[2 * h + 1];
-          }
-#pragma unroll
-          for (int o = 0; o < 2; ++o) {
-            xr[2 * h + o] = F::add(xt[2 * h + o], eo[2 * h + o]);
-            er[2 * h + o] = F::sub(two[o], xr[2 * h + o]);
-          }
-        }
-        if (any_partial) pad_brick<T>(er, nvx, nvy, nvz, lane);
+        for (int k = 0; k < 16; ++k) xr[k] = F::add(xt[k], eo[k]);
+        residual_of(xr, er);
         const U mr = brick_max<T>(er);
         if (pass && lenC > LEN_RAW && mr <= tb) mode = kModeRaw;
         if (mode == kModeRaw) {
@@ -918,15 +981,23 @@ __device__ __forceinline__ void compress3_chunk(const CompressParams& P, int64_t
       for (int k = 0; k < nrow; ++k) {
         const int j = nw - 1 - 4 * k - q;
         if (!emit || j < 0) continue;
-        const uint4 r = *reinterpret_cast<const uint4*>(planes + 64 * (j >> 5) + 4 * (j & (H - 1)));
-        const uint32_t sel = j & H ? 0x7632u : 0x5410u;
-        const uint64_t W = (uint64_t)__byte_perm(r.x, r.y, sel) | ((uint64_t)__byte_perm(r.z, r.w, sel) << 32);
-        if (!W) continue;
+        uint32_t lo, hi, mlo, mhi;
+        plane_at<WIDE>(planes, j, H, &lo, &hi);
+        if (!(lo | hi)) continue;
         const uint32_t nf = info[4 * k + q];
         const int n = (int)(nf & 0xffu);
         const uint32_t at = boff + (nf >> 8);
-        uint64_t rest = n < 64 ? W >> n : 0ull;
-        or_bits_in(cbuf, at, (W & low_mask64(n)) | (rest ? 1ull << n : 0ull), CAP, 0);
+        low_mask(n, &mlo, &mhi);
+        const uint32_t rlo = lo & ~mlo, rhi = hi & ~mhi;  // from position n on
+        lo &= mlo;
+        hi &= mhi;
+        if (rlo | rhi) {  // the first test 1, at position n < 64
+          lo |= mlo + 1u;  // bit n below 32: the mask's end (0 when the mask is full)
+          hi |= mlo == ~0u ? mhi + 1u : 0u;
+        }
+        if (PCZ_CHECK(at + (hi ? 64u - (uint32_t)__clz((int)hi) : 32u - (uint32_t)__clz((int)lo)) <= CAP, 0))
+          or_words(cbuf, at, lo, hi);
+        uint64_t rest = n < 64 ? (((uint64_t)rhi << 32) | rlo) >> n : 0ull;
         uint32_t pos = at + (uint32_t)n + 1u;
         while (rest) {
           const uint32_t b0 = (uint32_t)rest & 0xffu, b1 = ((uint32_t)rest >> 8) & 0xffu;

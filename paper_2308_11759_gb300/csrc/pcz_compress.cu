@@ -6,23 +6,22 @@
 // x_i = D(y_i) from the coded planes and adds it into x~.  x and x~ never
 // leave registers, so the field is read once.
 //
-// Layout: one CTA per index chunk of 32 bricks (R15), 16 warps, two CTAs per
-// SM; each lane loads its line of the field with 16-byte vector loads.  (A
-// second form, k_compress3_tma, stages the chunks in shared memory with TMA
-// tile copies in persistent CTAs; it is selected by PCZ_COMPRESS_TMA=1.)
-// A warp codes two bricks, 16 lanes each; lane t of a brick holds the x-line y = t & 3,
-// z = t >> 2, and after the transform the coded coefficients t + 16j.  The y
-// and z lifting passes and the reorder go through a bank-conflict-free brick
-// buffer in shared memory.  Bit planes come from 32x32 bit transposes across
-// the warp, after which lane p owns plane p (and p + 32): each lane emits its
-// plane's verbatim bits (R11), with the significance count before the plane
-// and the plane's bit offset from suffix scans over lanes (planes are coded
-// from the top down); the lane holding a coefficient writes the bits of the
-// token that makes it significant, at positions that follow from the plane's
-// offset, its significance count and the coefficient's rank among the plane's
-// new coefficients.  The chunk's bits are assembled in shared memory and
-// appended to a scratch pool with one atomic per chunk; pcz_misc.cu then scans
-// the chunk sizes and packs the final streams.
+// Layout: one CTA per index chunk of 32 bricks (R15), 4 warps; each lane loads
+// its lines of the field with 16-byte vector loads.  (A second form,
+// k_compress3_tma, stages the chunks in shared memory with TMA tile copies in
+// persistent CTAs; it is selected by PCZ_COMPRESS_TMA=1.)  A warp codes 8
+// bricks, 4 lanes each: lane q of a brick holds its z-plane q, lifts it along x
+// and y in registers, and after one exchange through shared memory holds the
+// y-plane q of coefficients and lifts it along z.  The coded digits are brought
+// into coded order through shared memory and transposed in registers into plane
+// words of 16 coefficients per lane.  Then 4 planes of a brick at a time, one per
+// lane (planes are coded from the top down): the significance count before a
+// plane and its bit offset come from scans over the 4 lanes, and a second pass,
+// when the bricks' places in the chunk are known, writes each plane's verbatim
+// bits and its group-test code, 16 coefficients at a time through a byte table.
+// The chunk's bits are assembled in shared memory and appended to a scratch pool
+// with one atomic per chunk; pcz_misc.cu then scans the chunk sizes and packs the
+// final streams.
 #include <algorithm>
 #include <cstdlib>
 #include <cstring>
@@ -32,10 +31,11 @@
 
 namespace pcz {
 
-// CTAs that share an SM: 4 at 128 registers a thread for float32, 3 at 168 for
-// float64.
+// CTAs that share an SM: 6 at 80 registers a thread for float32 (5 at 96
+// measured 1.5 % slower, 4 at 128 11 %), 3 at 168 for float64 (2 at 254, which
+// spills nothing, measured 25 % slower).
 template <typename T>
-constexpr int kCtas3 = sizeof(T) == 4 ? 4 : 3;
+constexpr int kCtas3 = sizeof(T) == 4 ? 6 : 3;
 
 // One chunk per CTA, each lane's line loaded straight into registers.
 template <typename T>

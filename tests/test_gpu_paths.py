@@ -3,8 +3,10 @@ the oracle, numpy or the general path, bit for bit."""
 import numpy as np
 import pytest
 
+import oracle as O
 import synth_fields as S
 from oracle import derivatives as D
+from tests.gpu_helpers import parse_serialized
 
 pytestmark = pytest.mark.gpu
 
@@ -92,3 +94,27 @@ def test_derivatives_outside_the_normal_range(P, h):
         nan = np.isnan(w)
         assert np.array_equal(nan, np.isnan(g))
         assert np.array_equal(_bits(w)[~nan], _bits(g)[~nan])
+
+
+# components whose coded planes span at most 8, 16 and 32 planes and more, at
+# block scales on both sides of the common range (float32 s in [-96, 126],
+# float64 [-960, 1000]; s = 24 or 56 minus the block exponent) and of the
+# 32-bit decode-back of float64
+@pytest.mark.parametrize("dtype", [np.float32, np.float64])
+@pytest.mark.parametrize("exp", ["low", "low+", "mid", "high-", "high"])
+@pytest.mark.parametrize("rel", [[0.25, 2.0 ** -4], [2.0 ** -9, 2.0 ** -14], [2.0 ** -20], [2.0 ** -45]])
+def test_construction_by_span_and_scale(P, dtype, exp, rel):
+    e = {np.float32: {"low": -103, "low+": -99, "mid": 3, "high-": 117, "high": 121},
+         np.float64: {"low": -946, "low+": -940, "mid": 3, "high-": 1012, "high": 1017}}[dtype][exp]
+    x = np.ldexp(S.powerlaw((9, 10, 37), seed=61, dtype=np.float64) / 4.0, e).astype(dtype)
+    tau = [float(np.ldexp(r, e)) for r in rel]
+    st, ref = P.compress(torch.from_numpy(x).cuda(), tau), O.Streams(x, tau, nthreads=4)
+    d = parse_serialized(st.serialize())
+    for i in range(len(tau)):
+        c = d["comps"][i]
+        assert np.array_equal(c["brick_len"], ref.brick_len(i))
+        assert np.array_equal(c["payload"], ref.payload(i))
+        assert c["counts"] == [int(v) for v in ref.stats(i)]
+        assert c["measured"] == ref.measured(i)
+    got = st.retrieve(k=len(tau)).cpu().numpy()
+    assert np.array_equal(_bits(got), _bits(ref.retrieve(len(tau))))
