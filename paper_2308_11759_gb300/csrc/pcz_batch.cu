@@ -8,8 +8,7 @@
 // 3D field, which the CTA codes as pcz_compress.cu does.  In the 1D/2D kernel, CTAs of a
 // few warps claim items of several chunks of a 1D or 2D field from a second
 // counter, and each warp codes one chunk at a time, a brick per lane, as
-// pcz_small.cu does (no register cap: a 2D brick of float64 values lives in
-// one thread's registers).  All fields share one scratch pool and one set of
+// pcz_small.cu does.  All fields share one scratch pool and one set of
 // chunk arrays; a segmented scan (one segment per field and component) places
 // every chunk in its component's stream, and a packing kernel copies the
 // chunks there.  The schedule (field order, CTAs per SM of the 3D kernel,
@@ -33,7 +32,7 @@ namespace pcz {
 
 template <typename T, int W>
 __host__ __device__ constexpr size_t batch_small_smem() {  // a chunk buffer per warp, sized for 2D bricks
-  return (size_t)W * chunk_words_small<T, 2>() * 4;
+  return small_smem<T, 2>(W);
 }
 
 // The item of work list `bp` that `it` falls in: its slot's field, first chunk,
@@ -111,11 +110,15 @@ __global__ void __launch_bounds__(kCompressThreads3, MINB) k_batch3(const BatchP
 
 // 1D/2D part of a batch: CTAs of W warps claim items of `width`
 // chunks of the 1D and 2D fields; the CTA's warps take the item's chunks one
-// at a time (a brick per lane, as in pcz_small.cu).  Float32 variants are
-// held to 128 registers so that 16 warps share an SM; float64 ones have no
-// cap, because a 2D brick of float64 values lives in one thread's registers.
+// at a time (a brick per lane, as in pcz_small.cu).  As many CTAs share an SM
+// as make the stand-alone kernel's warps: 20 for float32, 12 for float64.
 template <typename T, int W>
-__global__ void __launch_bounds__(32 * W, sizeof(T) == 4 ? 16 / W : 1) k_batch_small(const BatchParams* __restrict__ bp) {
+constexpr int batch_small_ctas() {
+  constexpr int warps = sizeof(T) == 4 ? 20 : 12;
+  return warps / W > 0 ? warps / W : 1;
+}
+template <typename T, int W>
+__global__ void __launch_bounds__(32 * W, (batch_small_ctas<T, W>())) k_batch_small(const BatchParams* __restrict__ bp) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ CompressParams sP;
   __shared__ long long s_first, s_chunk0;
@@ -123,6 +126,7 @@ __global__ void __launch_bounds__(32 * W, sizeof(T) == 4 ? 16 / W : 1) k_batch_s
   constexpr int PW = (int)(sizeof(CompressParams) / 8);
   constexpr int NT = 32 * W;
   const int tid = threadIdx.x, warp = tid >> 5;
+  const uint16_t* spread = load_spread<NT>(smem + batch_small_smem<T, W>() - kSpreadBytes);  // read after the first barrier
   const int64_t nitems = bp->nitems;
   const int per = bp->per_fetch;
   for (;;) {
@@ -153,11 +157,11 @@ __global__ void __launch_bounds__(32 * W, sizeof(T) == 4 ? 16 / W : 1) k_batch_s
       const int64_t c0 = s_chunk0;
       const int nch = s_nchunks;
       if (s_ndims == 2) {
-        uint32_t* cbuf = reinterpret_cast<uint32_t*>(smem) + (size_t)warp * chunk_words_small<T, 2>();
-        for (int c = warp; c < nch; c += W) compress_small_chunk<T, 2>(sP, c0 + c, cbuf);
+        uint32_t* area = reinterpret_cast<uint32_t*>(smem) + (size_t)warp * SmallArea<T, 2>::kWords;
+        for (int c = warp; c < nch; c += W) compress_small_chunk<T, 2>(sP, c0 + c, area, spread);
       } else {
-        uint32_t* cbuf = reinterpret_cast<uint32_t*>(smem) + (size_t)warp * chunk_words_small<T, 1>();
-        for (int c = warp; c < nch; c += W) compress_small_chunk<T, 1>(sP, c0 + c, cbuf);
+        uint32_t* area = reinterpret_cast<uint32_t*>(smem) + (size_t)warp * SmallArea<T, 1>::kWords;
+        for (int c = warp; c < nch; c += W) compress_small_chunk<T, 1>(sP, c0 + c, area, spread);
       }
     }
   }
@@ -183,7 +187,9 @@ __global__ void __launch_bounds__(kMixedThreads, 1) k_batch_mixed(const BatchPar
   __shared__ int s_field, s_nchunks, s_ndims;
   constexpr int PW = (int)(sizeof(CompressParams) / 8);
   constexpr int WARPS = kMixedThreads / 32;
+  __shared__ uint32_t s_spread[kSpreadBytes / 4];
   const int tid = threadIdx.x, warp = tid >> 5;
+  const uint16_t* spread = load_spread<kMixedThreads>(s_spread);  // read after the first barrier
   const int64_t nitems = bp->nitems;
   const int per = bp->per_fetch;
   for (;;) {
@@ -217,11 +223,11 @@ __global__ void __launch_bounds__(kMixedThreads, 1) k_batch_mixed(const BatchPar
         const int g = warp / kWarps3;
         if (g < nch) compress3_chunk<T>(sP, c0 + g, smem + g * mixed_group_smem<T>(), 1 + g);
       } else if (s_ndims == 2) {
-        uint32_t* cbuf = reinterpret_cast<uint32_t*>(smem) + (size_t)warp * chunk_words_small<T, 2>();
-        for (int c = warp; c < nch; c += WARPS) compress_small_chunk<T, 2>(sP, c0 + c, cbuf);
+        uint32_t* area = reinterpret_cast<uint32_t*>(smem) + (size_t)warp * SmallArea<T, 2>::kWords;
+        for (int c = warp; c < nch; c += WARPS) compress_small_chunk<T, 2>(sP, c0 + c, area, spread);
       } else {
-        uint32_t* cbuf = reinterpret_cast<uint32_t*>(smem) + (size_t)warp * chunk_words_small<T, 1>();
-        for (int c = warp; c < nch; c += WARPS) compress_small_chunk<T, 1>(sP, c0 + c, cbuf);
+        uint32_t* area = reinterpret_cast<uint32_t*>(smem) + (size_t)warp * SmallArea<T, 1>::kWords;
+        for (int c = warp; c < nch; c += WARPS) compress_small_chunk<T, 1>(sP, c0 + c, area, spread);
       }
     }
   }
@@ -230,7 +236,7 @@ __global__ void __launch_bounds__(kMixedThreads, 1) k_batch_mixed(const BatchPar
 template <typename T>
 __host__ __device__ constexpr size_t batch_mixed_smem() {
   const size_t a = kMixedGroups * mixed_group_smem<T>();
-  const size_t b = (size_t)(kMixedThreads / 32) * chunk_words_small<T, 2>() * 4;
+  const size_t b = small_smem<T, 2>(kMixedThreads / 32) - kSpreadBytes;
   return a > b ? a : b;
 }
 

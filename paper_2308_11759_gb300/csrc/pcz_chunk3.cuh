@@ -58,29 +58,6 @@ struct Area3 {
   static constexpr int kInfoStride = Fmt<T>::P + 4;                       // plane table, words per brick
 };
 
-// Group-test code of 8 coefficient bits (R11): each bit in turn, and after
-// each 1 the 1 of the next token's test bit.  Its length is 8 + popc(bits).
-struct SpreadTable {
-  uint16_t code[256];
-};
-constexpr SpreadTable make_spread() {
-  SpreadTable t{};
-  for (int v = 0; v < 256; ++v) {
-    unsigned code = 0, len = 0;
-    for (int j = 0; j < 8; ++j)
-      if ((v >> j) & 1) {
-        code |= 3u << len;
-        len += 2;
-      } else {
-        ++len;
-      }
-    t.code[v] = (uint16_t)code;
-  }
-  return t;
-}
-static __device__ const SpreadTable kSpread3 = make_spread();
-constexpr int kSpreadBytes = (int)sizeof(SpreadTable);
-
 // Bytes of the staging area in front of the rest (TMA-staged form only).
 template <typename T>
 __host__ __device__ constexpr size_t staging_bytes3(bool staged) {
@@ -105,95 +82,14 @@ __device__ __forceinline__ void group_sync(int id) {
   asm volatile("bar.sync %0, 128;" ::"r"(id) : "memory");
 }
 
-// Bit transposes within a lane.  transpose8: word i holds 8 bits (planes) each
-// of the coefficients i, i + 8, i + 4 and i + 12 (from its low byte up);
-// afterwards word j holds planes j and j + 4 of the 16 coefficients.  transpose16: word i holds 16 bits (planes) of
-// coefficient i in its low half and of coefficient i + 8 in its high half;
-// afterwards word j holds plane j of the 16 coefficients in its low half and
-// plane j + 8 in its high half.  transpose32: word i holds 32 bits of
-// coefficient i; afterwards word j holds planes j and j + 16.  Stages of 4, 2
-// and 1 exchange bit groups between two words with a shift and a logic op per
-// result; the stage of 8 is one byte permute per result.
-template <int N, int K>
-__device__ __forceinline__ void exchange_stage(uint32_t (&a)[N], uint32_t m) {
-#pragma unroll
-  for (int i = 0; i < N; ++i)
-    if (!(i & K)) {
-      const uint32_t x = a[i], y = a[i + K];
-      a[i] = (x & m) | ((y << K) & ~m);
-      a[i + K] = ((x >> K) & m) | (y & ~m);
-    }
-}
-__device__ __forceinline__ void transpose8(uint32_t (&a)[4]) {
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const uint32_t t = (a[i] ^ (a[i] >> 12)) & 0x0000F0F0u;
-    a[i] ^= t ^ (t << 12);
-  }
-  exchange_stage<4, 2>(a, 0x33333333u);
-  exchange_stage<4, 1>(a, 0x55555555u);
-}
-__device__ __forceinline__ void transpose16(uint32_t (&a)[8]) {
-#pragma unroll
-  for (int i = 0; i < 8; ++i) a[i] = __byte_perm(a[i], 0u, 0x3120);
-  exchange_stage<8, 4>(a, 0x0F0F0F0Fu);
-  exchange_stage<8, 2>(a, 0x33333333u);
-  exchange_stage<8, 1>(a, 0x55555555u);
-}
-__device__ __forceinline__ void transpose32_lane(uint32_t (&a)[16]) {
-#pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    const uint32_t x = a[i], y = a[i + 8];
-    a[i] = __byte_perm(x, y, 0x6240);
-    a[i + 8] = __byte_perm(x, y, 0x7351);
-  }
-  exchange_stage<16, 4>(a, 0x0F0F0F0Fu);
-  exchange_stage<16, 2>(a, 0x33333333u);
-  exchange_stage<16, 1>(a, 0x55555555u);
-}
-
-// |v| as an integer that orders like it (NaN above +inf above every finite
-// value): the bit pattern without its sign.  float64 masks the high word only:
-// masking the whole pattern is recognised as fabs and emitted on the FP64 pipe.
-__device__ __forceinline__ uint32_t magnitude(float v) { return __float_as_uint(v) & 0x7FFFFFFFu; }
-__device__ __forceinline__ uint64_t magnitude(double v) {
-  return ((uint64_t)((uint32_t)__double2hiint(v) & 0x7FFFFFFFu) << 32) | (uint32_t)__double2loint(v);
-}
-
 // The largest magnitude of a brick: over a lane's 16 values, then its 4 lanes.
-// float32 takes the maximum of |v| with NaN propagated, one instruction per
-// value; a NaN's own bits, which that maximum does not keep, are looked up.
-__device__ __forceinline__ float max_abs_nan(float a, float b) {
-  float r;
-  asm("{\n .reg .f32 t;\n abs.f32 t, %2;\n max.NaN.f32 %0, %1, t;\n}\n" : "=f"(r) : "f"(a), "f"(b));
-  return r;
-}
 template <typename T>
 __device__ __forceinline__ typename Fmt<T>::U brick_max(const T* e) {
   using U = typename Fmt<T>::U;
-  constexpr unsigned FULL = 0xffffffffu;
-  U m;
-  if constexpr (sizeof(T) == 4) {
-    float f = 0.0f;
-#pragma unroll
-    for (int v = 0; v < 16; ++v) f = max_abs_nan(f, e[v]);
-    m = __float_as_uint(f);
-    if (m > Fmt<T>::INF) {
-      m = 0;
-#pragma unroll
-      for (int v = 0; v < 16; ++v) m = max(m, magnitude(e[v]));
-    }
-  } else {
-    m = magnitude(e[0]);
-#pragma unroll
-    for (int v = 1; v < 16; ++v) {
-      const U a = magnitude(e[v]);
-      m = a > m ? a : m;
-    }
-  }
+  U m = lane_max<T, 16>(e);
 #pragma unroll
   for (int o = 1; o <= 2; o <<= 1) {
-    const U a = __shfl_xor_sync(FULL, m, o);
+    const U a = __shfl_xor_sync(0xffffffffu, m, o);
     m = a > m ? a : m;
   }
   return m;
@@ -305,30 +201,6 @@ __device__ __forceinline__ void lift_inv_bricks(S* v, uint4* zw, uint4* yw, int 
   for (int x = 0; x < 4; ++x) lift_inv(v[x], v[x + 4], v[x + 8], v[x + 12]);
 #pragma unroll
   for (int y = 0; y < 4; ++y) lift_inv(v[4 * y], v[4 * y + 1], v[4 * y + 2], v[4 * y + 3]);
-}
-
-// R6 and R13 for blocks whose scale is outside the common range, out of line.
-template <typename T>
-__device__ __noinline__ typename Fmt<T>::S quantize_any(typename Fmt<T>::U b, int s) {
-  return quantize<T>(b, s);
-}
-template <typename T>
-__device__ __noinline__ typename Fmt<T>::U dequantize_any(typename Fmt<T>::S q, int s) {
-  return dequantize_bits<T>(q, s);
-}
-
-// R6 for float64 in a block whose scale s lies in [-960, 1000] (c = 1078 - s):
-// q = sign(e) * ((the 53-bit significand << 3) >> r) with r = c - biased
-// exponent, which is at least 0 because |q| < 2^56.  A subnormal e, taken with
-// a hidden bit it does not have, is shifted out entirely (r >= 78).  c = 4096
-// gives 0 for every e.
-__device__ __forceinline__ int64_t quantize_f64_normal(double e, int c) {
-  const uint32_t hi = (uint32_t)__double2hiint(e), lo = (uint32_t)__double2loint(e);
-  const uint64_t m = ((uint64_t)((hi & 0xFFFFFu) | 0x100000u) << 32) | lo;
-  const int r = min(c - (int)((hi >> 20) & 0x7FFu), 63);
-  const int64_t a = (int64_t)((m << 3) >> r);
-  const int64_t sg = (int64_t)((int32_t)hi >> 31);
-  return (a ^ sg) - sg;
 }
 
 // Staging of a chunk's field values in shared memory with TMA (the
@@ -488,7 +360,7 @@ __device__ __forceinline__ void compress3_chunk(const CompressParams& P, int64_t
   const bool have = b < P.nbricks;
 
   for (int w = tid; w < BUFW / 4; w += kCompressThreads3) reinterpret_cast<uint4*>(cbuf)[w] = make_uint4(0, 0, 0, 0);
-  reinterpret_cast<uint32_t*>(s_spread)[tid] = reinterpret_cast<const uint32_t*>(kSpread3.code)[tid];
+  reinterpret_cast<uint32_t*>(s_spread)[tid] = reinterpret_cast<const uint32_t*>(kSpread.code)[tid];
   static_assert(kSpreadBytes == 4 * kCompressThreads3, "one word per thread");
 
   int64_t bx = 0, by = 0, bz = 0;
@@ -610,9 +482,9 @@ __device__ __forceinline__ void compress3_chunk(const CompressParams& P, int64_t
         }
       } else {
         if (common) {
-          const int c = coded ? 1078 - s : 4096;
+          const int c = coded ? 1022 + Q - s : 4096;
 #pragma unroll
-          for (int k = 0; k < 16; ++k) v[k] = quantize_f64_normal(e[k], c);
+          for (int k = 0; k < 16; ++k) v[k] = quantize_f64_normal<Q - 53>(e[k], c);
         } else {
 #pragma unroll
           for (int k = 0; k < 16; ++k) v[k] = coded ? quantize_any<T>(F::bits(e[k]), s) : S(0);

@@ -528,49 +528,246 @@ __device__ __forceinline__ void load_line(const T* src, int nv, T* v) {
   for (int m = 0; m < 4; ++m) v[m] = src[min(m, nv - 1)];
 }
 
-// Sequential bit reader over a word stream with the two current words in
-// registers: one load per 64 bits consumed.  Positions must not decrease.
-struct BitReader {
-  const uint64_t* __restrict__ w;
-  uint64_t nw, wi, a, b;
-  __device__ __forceinline__ uint64_t ld(uint64_t i) const { return i < nw ? __ldg(w + i) : 0ull; }
-  __device__ __forceinline__ void init(const uint64_t* words, uint64_t nwords, uint64_t pos) {
-    w = words;
-    nw = nwords;
-    wi = pos >> 6;
-    a = ld(wi);
-    b = ld(wi + 1);
+// Bit transposes within a lane.  transpose8: word i holds 8 bits (planes) each
+// of the coefficients i, i + 8, i + 4 and i + 12 (from its low byte up);
+// afterwards word j holds planes j and j + 4 of the 16 coefficients.  transpose16: word i holds 16 bits (planes) of
+// coefficient i in its low half and of coefficient i + 8 in its high half;
+// afterwards word j holds plane j of the 16 coefficients in its low half and
+// plane j + 8 in its high half.  transpose32: word i holds 32 bits of
+// coefficient i; afterwards word j holds planes j and j + 16.  Stages of 4, 2
+// and 1 exchange bit groups between two words with a shift and a logic op per
+// result; the stage of 8 is one byte permute per result.
+template <int N, int K>
+__device__ __forceinline__ void exchange_stage(uint32_t (&a)[N], uint32_t m) {
+#pragma unroll
+  for (int i = 0; i < N; ++i)
+    if (!(i & K)) {
+      const uint32_t x = a[i], y = a[i + K];
+      a[i] = (x & m) | ((y << K) & ~m);
+      a[i + K] = ((x >> K) & m) | (y & ~m);
+    }
+}
+__device__ __forceinline__ void transpose8(uint32_t (&a)[4]) {
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const uint32_t t = (a[i] ^ (a[i] >> 12)) & 0x0000F0F0u;
+    a[i] ^= t ^ (t << 12);
   }
-  __device__ __forceinline__ uint64_t peek(uint64_t pos) {
-    const uint64_t i = pos >> 6;
+  exchange_stage<4, 2>(a, 0x33333333u);
+  exchange_stage<4, 1>(a, 0x55555555u);
+}
+// transpose8 backwards: word j holds planes j and j + 4; afterwards word i holds
+// the bytes of coefficients i, i + 8, i + 4 and i + 12.
+__device__ __forceinline__ void untranspose8(uint32_t (&a)[4]) {
+  exchange_stage<4, 1>(a, 0x55555555u);
+  exchange_stage<4, 2>(a, 0x33333333u);
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const uint32_t t = (a[i] ^ (a[i] >> 12)) & 0x0000F0F0u;
+    a[i] ^= t ^ (t << 12);
+  }
+}
+__device__ __forceinline__ void transpose16(uint32_t (&a)[8]) {
+#pragma unroll
+  for (int i = 0; i < 8; ++i) a[i] = __byte_perm(a[i], 0u, 0x3120);
+  exchange_stage<8, 4>(a, 0x0F0F0F0Fu);
+  exchange_stage<8, 2>(a, 0x33333333u);
+  exchange_stage<8, 1>(a, 0x55555555u);
+}
+__device__ __forceinline__ void transpose32_lane(uint32_t (&a)[16]) {
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const uint32_t x = a[i], y = a[i + 8];
+    a[i] = __byte_perm(x, y, 0x6240);
+    a[i + 8] = __byte_perm(x, y, 0x7351);
+  }
+  exchange_stage<16, 4>(a, 0x0F0F0F0Fu);
+  exchange_stage<16, 2>(a, 0x33333333u);
+  exchange_stage<16, 1>(a, 0x55555555u);
+}
+
+// |v| as an integer that orders like it (NaN above +inf above every finite
+// value): the bit pattern without its sign.  float64 masks the high word only:
+// masking the whole pattern is recognised as fabs and emitted on the FP64 pipe.
+__device__ __forceinline__ uint32_t magnitude(float v) { return __float_as_uint(v) & 0x7FFFFFFFu; }
+__device__ __forceinline__ uint64_t magnitude(double v) {
+  return ((uint64_t)((uint32_t)__double2hiint(v) & 0x7FFFFFFFu) << 32) | (uint32_t)__double2loint(v);
+}
+
+// The largest magnitude of a lane's N values.  float32 takes the maximum of |v|
+// with NaN propagated, one instruction per value; a NaN's own bits, which that
+// maximum does not keep, are looked up.
+__device__ __forceinline__ float max_abs_nan(float a, float b) {
+  float r;
+  asm("{\n .reg .f32 t;\n abs.f32 t, %2;\n max.NaN.f32 %0, %1, t;\n}\n" : "=f"(r) : "f"(a), "f"(b));
+  return r;
+}
+template <typename T, int N>
+__device__ __forceinline__ typename Fmt<T>::U lane_max(const T* e) {
+  using U = typename Fmt<T>::U;
+  U m;
+  if constexpr (sizeof(T) == 4) {
+    float f = 0.0f;
+#pragma unroll
+    for (int v = 0; v < N; ++v) f = max_abs_nan(f, e[v]);
+    m = __float_as_uint(f);
+    if (m > Fmt<T>::INF) {
+      m = 0;
+#pragma unroll
+      for (int v = 0; v < N; ++v) m = max(m, magnitude(e[v]));
+    }
+  } else {
+    m = magnitude(e[0]);
+#pragma unroll
+    for (int v = 1; v < N; ++v) {
+      const U a = magnitude(e[v]);
+      m = a > m ? a : m;
+    }
+  }
+  return m;
+}
+
+// R6 and R13 for blocks whose scale is outside the common range, out of line.
+template <typename T>
+__device__ __noinline__ typename Fmt<T>::S quantize_any(typename Fmt<T>::U b, int s) {
+  return quantize<T>(b, s);
+}
+template <typename T>
+__device__ __noinline__ typename Fmt<T>::U dequantize_any(typename Fmt<T>::S q, int s) {
+  return dequantize_bits<T>(q, s);
+}
+
+// R6 for float64 in a block whose scale s lies in [-960, 1000], with Q = 53 + G
+// quantisation bits (c = 1075 + G - s): q = sign(e) * ((the 53-bit significand
+// << G) >> r) with r = c - biased exponent, which is at least 0 because
+// |q| < 2^Q.  A subnormal e, taken with a hidden bit it does not have, is
+// shifted out entirely (r >= 75 + G).  c = 4096 gives 0 for every e.
+template <int G>
+__device__ __forceinline__ int64_t quantize_f64_normal(double e, int c) {
+  const uint32_t hi = (uint32_t)__double2hiint(e), lo = (uint32_t)__double2loint(e);
+  const uint64_t m = ((uint64_t)((hi & 0xFFFFFu) | 0x100000u) << 32) | lo;
+  const int r = min(c - (int)((hi >> 20) & 0x7FFu), 63);
+  const int64_t a = (int64_t)((m << G) >> r);
+  const int64_t sg = (int64_t)((int32_t)hi >> 31);
+  return (a ^ sg) - sg;
+}
+
+// Group-test code of 8 coefficient bits (R11): each bit in turn, and after
+// each 1 the 1 of the next token's test bit.  Its length is 8 + popc(bits).
+struct alignas(4) SpreadTable {
+  uint16_t code[256];
+};
+constexpr SpreadTable make_spread() {
+  SpreadTable t{};
+  for (int v = 0; v < 256; ++v) {
+    unsigned code = 0, len = 0;
+    for (int j = 0; j < 8; ++j)
+      if ((v >> j) & 1) {
+        code |= 3u << len;
+        len += 2;
+      } else {
+        ++len;
+      }
+    t.code[v] = (uint16_t)code;
+  }
+  return t;
+}
+static __device__ const SpreadTable kSpread = make_spread();
+constexpr int kSpreadBytes = (int)sizeof(SpreadTable);
+
+// Sequential reader of one block's bits with 32-bit positions relative to
+// the start of the word that holds the block's first bit: the two current
+// words in 32-bit halves, one load per 64 bits consumed, and a 64-bit window
+// at any position made of two funnel shifts.  Words at or beyond the
+// payload's end read as zero.  Positions must not decrease.
+struct BlockBits {
+  const uint64_t* __restrict__ w;  // the payload from the block's first word
+  uint32_t nw;                     // words readable from w
+  uint32_t wi;                     // index of the word in a0:a1
+  uint32_t a0, a1, b0, b1;         // words wi and wi + 1
+  __device__ __forceinline__ uint64_t ld(uint32_t i) const { return i < nw ? __ldg(w + i) : 0ull; }
+  __device__ __forceinline__ void set(uint64_t lo, uint64_t hi) {
+    a0 = (uint32_t)lo;
+    a1 = (uint32_t)(lo >> 32);
+    b0 = (uint32_t)hi;
+    b1 = (uint32_t)(hi >> 32);
+  }
+  // bit position of the block's first bit within the reader's frame: off & 63
+  __device__ __forceinline__ void init(const uint64_t* words, uint64_t nwords, uint64_t off) {
+    const uint64_t w0 = off >> 6;
+    w = words + w0;
+    nw = w0 < nwords ? (uint32_t)min(nwords - w0, (uint64_t)0xffffffffu) : 0u;
+    wi = 0;
+    set(ld(0), ld(1));
+  }
+  __device__ __forceinline__ uint64_t peek(uint32_t pos) {
+    const uint32_t i = pos >> 6;
     if (i != wi) {
       if (i == wi + 1) {
-        a = b;
-        b = ld(i + 1);
+        a0 = b0;
+        a1 = b1;
+        const uint64_t nb = ld(i + 1);
+        b0 = (uint32_t)nb;
+        b1 = (uint32_t)(nb >> 32);
       } else {
-        a = ld(i);
-        b = ld(i + 1);
+        set(ld(i), ld(i + 1));
       }
       wi = i;
     }
-    const uint32_t sh = (uint32_t)(pos & 63);
-    return sh ? (a >> sh) | (b << (64 - sh)) : a;
+    const bool up = pos & 32u;  // window starts in the word's upper half
+    const uint32_t x0 = up ? a1 : a0, x1 = up ? b0 : a1, x2 = up ? b1 : b0;
+    return ((uint64_t)__funnelshift_r(x1, x2, pos) << 32) | __funnelshift_r(x0, x1, pos);
   }
 };
 
-// Bits emitted for one plane (R11) given its plane word W (bit r = bit of the
-// r-th coded coefficient) and n coefficients already significant:
-// n verbatim bits, then (if n < N) one test bit per newly significant
-// coefficient, the run of coefficient bits up to and including it, and a
-// closing 0 test bit unless the last coefficient became significant.
-template <int N>
-__device__ __forceinline__ int plane_len(uint64_t W, int n) {
-  if (n >= N) return n;
-  uint64_t rest = n >= 64 ? 0ull : (W >> n);
-  if (!rest) return n + 1;
-  int hi = 64 - __clzll((long long)W);  // one past the highest set position
-  int m = __popcll((long long)rest);
-  return n + m + (hi - n) + (hi < N ? 1 : 0);
+// Byte table of the group-test part as a two-state machine: in state "test"
+// a 0 ends the part and a 1 starts a run; in state "run" every bit is the
+// next coefficient's bit and a 1 ends the run.  Entry [state][byte] (16 bits):
+// bits 0-7 the 1s among the byte's coefficient bits (coefficient-relative),
+// bits 8-11 their count, bit 12 set when the part ends in the byte; then
+// bits 13-15 hold the bits used up to and including the closing test bit,
+// minus 1; otherwise bit 13 is the state after the byte.
+constexpr uint32_t kTokEnded = 1u << 12;
+constexpr int kTokLut = 512;  // entries (2 states x 256 bytes)
+
+struct alignas(4) TokenTable {
+  uint16_t entry[kTokLut];
+};
+constexpr TokenTable make_tokens() {
+  TokenTable t{};
+  for (int idx = 0; idx < kTokLut; ++idx) {
+    int st = idx >> 8;
+    const int byte = idx & 255;
+    unsigned out = 0, cnt = 0, e = 0;
+    bool ended = false;
+    for (int j = 0; j < 8 && !ended; ++j) {
+      const int bit = (byte >> j) & 1;
+      if (st == 0) {
+        if (bit) {
+          st = 1;
+        } else {
+          ended = true;
+          e = kTokEnded | ((unsigned)j << 13);
+        }
+      } else {
+        out |= (unsigned)bit << cnt;
+        ++cnt;
+        if (bit) st = 0;
+      }
+    }
+    if (!ended) e = (unsigned)st << 13;
+    t.entry[idx] = (uint16_t)(out | (cnt << 8) | e);
+  }
+  return t;
+}
+static __device__ const TokenTable kTokens = make_tokens();
+
+// A CTA's copy of the table in shared memory (4-byte aligned); read after the
+// next barrier.
+template <int THREADS>
+__device__ __forceinline__ void load_tokens(uint16_t* at) {
+  uint32_t* w = reinterpret_cast<uint32_t*>(at);
+  for (int i = threadIdx.x; i < kTokLut / 2; i += THREADS) w[i] = reinterpret_cast<const uint32_t*>(kTokens.entry)[i];
 }
 
 }  // namespace pcz

@@ -48,7 +48,6 @@ constexpr int kRWarps = 8;
 constexpr int kRThreads = 32 * kRWarps;
 constexpr int kRound = 8;    // components per round
 constexpr int kTasks = 512;  // parse tasks (block of one brick and component) per round
-constexpr int kTokLut = 512;  // entries of the group-test byte table (2 states x 256 bytes)
 constexpr int kLenBuckets = 64;  // parse tasks are handed out longest block first, by len / 16
 // plane words per block kept in shared memory: as many as let 3 CTAs share an SM
 template <typename T>
@@ -91,83 +90,6 @@ __host__ __device__ constexpr int spill_per_block() {  // planes below a block's
 template <typename T>
 __host__ __device__ constexpr size_t spill_words_per_cta() {
   return (size_t)kTasks * spill_per_block<T>();
-}
-
-// Sequential reader of one block's bits with 32-bit positions relative to
-// the start of the word that holds the block's first bit: the two current
-// words in 32-bit halves, one load per 64 bits consumed, and a 64-bit window
-// at any position made of two funnel shifts.  Words at or beyond the
-// payload's end read as zero.  Positions must not decrease.
-struct BlockBits {
-  const uint64_t* __restrict__ w;  // the payload from the block's first word
-  uint32_t nw;                     // words readable from w
-  uint32_t wi;                     // index of the word in a0:a1
-  uint32_t a0, a1, b0, b1;         // words wi and wi + 1
-  __device__ __forceinline__ uint64_t ld(uint32_t i) const { return i < nw ? __ldg(w + i) : 0ull; }
-  __device__ __forceinline__ void set(uint64_t lo, uint64_t hi) {
-    a0 = (uint32_t)lo;
-    a1 = (uint32_t)(lo >> 32);
-    b0 = (uint32_t)hi;
-    b1 = (uint32_t)(hi >> 32);
-  }
-  // bit position of the block's first bit within the reader's frame: off & 63
-  __device__ __forceinline__ void init(const uint64_t* words, uint64_t nwords, uint64_t off) {
-    const uint64_t w0 = off >> 6;
-    w = words + w0;
-    nw = w0 < nwords ? (uint32_t)min(nwords - w0, (uint64_t)0xffffffffu) : 0u;
-    wi = 0;
-    set(ld(0), ld(1));
-  }
-  __device__ __forceinline__ uint64_t peek(uint32_t pos) {
-    const uint32_t i = pos >> 6;
-    if (i != wi) {
-      if (i == wi + 1) {
-        a0 = b0;
-        a1 = b1;
-        const uint64_t nb = ld(i + 1);
-        b0 = (uint32_t)nb;
-        b1 = (uint32_t)(nb >> 32);
-      } else {
-        set(ld(i), ld(i + 1));
-      }
-      wi = i;
-    }
-    const bool up = pos & 32u;  // window starts in the word's upper half
-    const uint32_t x0 = up ? a1 : a0, x1 = up ? b0 : a1, x2 = up ? b1 : b0;
-    return ((uint64_t)__funnelshift_r(x1, x2, pos) << 32) | __funnelshift_r(x0, x1, pos);
-  }
-};
-
-// Byte table of the group-test part as a two-state machine: in state "test"
-// a 0 ends the part and a 1 starts a run; in state "run" every bit is the
-// next coefficient's bit and a 1 ends the run.  Entry [state][byte] (16 bits):
-// bits 0-7 the 1s among the byte's coefficient bits (coefficient-relative),
-// bits 8-11 their count, bit 12 set when the part ends in the byte; then
-// bits 13-15 hold the bits used up to and including the closing test bit,
-// minus 1; otherwise bit 13 is the state after the byte.
-constexpr uint32_t kTokEnded = 1u << 12;
-
-__device__ __forceinline__ uint16_t token_lut_entry(int idx) {
-  int st = idx >> 8;
-  const int byte = idx & 255;
-  uint32_t out = 0, cnt = 0, e = 0;
-  bool ended = false;
-  for (int j = 0; j < 8 && !ended; ++j) {
-    const int bit = (byte >> j) & 1;
-    if (st == 0) {
-      if (bit) st = 1;
-      else {
-        ended = true;
-        e = kTokEnded | ((uint32_t)j << 13);
-      }
-    } else {
-      out |= (uint32_t)bit << cnt;
-      ++cnt;
-      if (bit) st = 0;
-    }
-  }
-  if (!ended) e = (uint32_t)st << 13;
-  return (uint16_t)(out | (cnt << 8) | e);
 }
 
 // The group-test part of a plane (R11), a byte at a time through the table:
@@ -652,7 +574,7 @@ __global__ void __launch_bounds__(kRThreads, 3) k_retrieve3(const RetrieveParams
   uint16_t* order = lut + kTokLut;                                         // [kTasks]
   int* hist = reinterpret_cast<int*>(order + kTasks);                      // [kLenBuckets]
   if (threadIdx.x < kLenBuckets) hist[threadIdx.x] = 0;
-  for (int i = threadIdx.x; i < kTokLut; i += kRThreads) lut[i] = token_lut_entry(i);  // read after the loop's first barrier
+  load_tokens<kRThreads>(lut);  // read after the loop's first barrier
   __shared__ int s_next;  // next parse task of the round
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, h = lane >> 4, t = lane & 15;
   S* buf = bufs + warp * 128;

@@ -5,29 +5,44 @@
 // in registers (residual, alignment, lifting along x then y, sequency order,
 // negabinary, bit planes from the top down, decode-back and verification),
 // and one warp covers one index chunk of 32 bricks, so the bricks' bit
-// offsets in the chunk come from a warp scan.  The bits are assembled in a
-// per-warp shared buffer and appended to the scratch pool like the 3D
-// kernel's chunks; retrieval mirrors this with one thread per brick and
-// component parsing and rebuilding a brick.
+// offsets in the chunk come from a warp scan.  Each lane's code is formed in its
+// own column of shared memory, shifted into the warp's chunk buffer and appended
+// to the scratch pool like the 3D kernel's chunks; retrieval mirrors this with
+// one thread per brick and component parsing and rebuilding a brick.
 #include "pcz_chunk_small.cuh"
 
 namespace pcz {
 
+// CTAs of 4 warps that share an SM, measured on 2D fields (4096^2 float32, 4096 x
+// 3000 float64, 6 components).  Construction: float32 5 (349 us; 4: 376, 6: 387),
+// float64 3 (613; 2: 709, 4: 640).  Retrieval: float32 8 (278 us; 6: 292, 5:
+// 318), float64 5 (327; 4: 348).
+template <typename T>
+constexpr int kCompressCtas = sizeof(T) == 4 ? 5 : 3;
+template <typename T>
+constexpr int kRetrieveCtas = sizeof(T) == 4 ? 8 : 5;
+
 template <typename T, int D>
-__global__ void __launch_bounds__(kSmallThreads) k_compress_small(const CompressParams P) {
+__global__ void __launch_bounds__(kSmallThreads, kCompressCtas<T>) k_compress_small(const CompressParams P) {
   extern __shared__ __align__(16) unsigned char smem[];
   const int warp = threadIdx.x >> 5;
-  uint32_t* cbuf = reinterpret_cast<uint32_t*>(smem) + (size_t)warp * chunk_words_small<T, D>();
-  compress_small_chunk<T, D>(P, (int64_t)blockIdx.x * kSmallWarps + warp, cbuf);
+  uint32_t* area = reinterpret_cast<uint32_t*>(smem) + (size_t)warp * SmallArea<T, D>::kWords;
+  const uint16_t* spread = load_spread<kSmallThreads>(smem + small_smem<T, D>(kSmallWarps) - kSpreadBytes);
+  __syncthreads();
+  const int64_t chunk = (int64_t)blockIdx.x * kSmallWarps + warp;
+  if (chunk < P.nchunks) compress_small_chunk<T, D>(P, chunk, area, spread);
 }
 
 // One thread per brick: of the single job, or of a job list whose units are
 // bricks (unit_begin = the job's first brick among all jobs' bricks).
 template <typename T, int D>
-__global__ void __launch_bounds__(kSmallThreads) k_retrieve_small(const RetrieveParams R) {
+__global__ void __launch_bounds__(kSmallThreads, kRetrieveCtas<T>) k_retrieve_small(const RetrieveParams R) {
+  __shared__ __align__(4) uint16_t tokens[kTokLut];
+  load_tokens<kSmallThreads>(tokens);
+  __syncthreads();
   const int64_t g = (int64_t)blockIdx.x * kSmallThreads + threadIdx.x;
   if (!R.jobs) {
-    if (g < R.job0.nbox) retrieve_small_brick<T, D>(R.job0, R.write, R.err, g);
+    if (g < R.job0.nbox) retrieve_small_brick<T, D>(R.job0, R.write, R.err, g, tokens);
     return;
   }
   if (g >= R.nunits) return;
@@ -40,12 +55,12 @@ __global__ void __launch_bounds__(kSmallThreads) k_retrieve_small(const Retrieve
       hi = mid - 1;
   }
   const BoxJob& J = R.jobs[lo];
-  retrieve_small_brick<T, D>(J, R.write, R.err, g - J.unit_begin);
+  retrieve_small_brick<T, D>(J, R.write, R.err, g - J.unit_begin, tokens);
 }
 
 template <typename T, int D>
 static cudaError_t launch_compress_small_t(const CompressParams& p, cudaStream_t s) {
-  const size_t smem = small_smem<T, D>();
+  const size_t smem = small_smem<T, D>(kSmallWarps);
   cudaError_t e = cudaFuncSetAttribute(k_compress_small<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   if (p.nchunks == 0) return cudaSuccess;

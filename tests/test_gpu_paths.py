@@ -103,10 +103,11 @@ def test_derivatives_outside_the_normal_range(P, h):
 @pytest.mark.parametrize("dtype", [np.float32, np.float64])
 @pytest.mark.parametrize("exp", ["low", "low+", "mid", "high-", "high"])
 @pytest.mark.parametrize("rel", [[0.25, 2.0 ** -4], [2.0 ** -9, 2.0 ** -14], [2.0 ** -20], [2.0 ** -45]])
-def test_construction_by_span_and_scale(P, dtype, exp, rel):
+@pytest.mark.parametrize("shape", [(9, 10, 37), (21, 37), (203,)])
+def test_construction_by_span_and_scale(P, dtype, exp, rel, shape):
     e = {np.float32: {"low": -103, "low+": -99, "mid": 3, "high-": 117, "high": 121},
          np.float64: {"low": -946, "low+": -940, "mid": 3, "high-": 1012, "high": 1017}}[dtype][exp]
-    x = np.ldexp(S.powerlaw((9, 10, 37), seed=61, dtype=np.float64) / 4.0, e).astype(dtype)
+    x = np.ldexp(S.powerlaw(shape, seed=61, dtype=np.float64) / 4.0, e).astype(dtype)
     tau = [float(np.ldexp(r, e)) for r in rel]
     st, ref = P.compress(torch.from_numpy(x).cuda(), tau), O.Streams(x, tau, nthreads=4)
     d = parse_serialized(st.serialize())
