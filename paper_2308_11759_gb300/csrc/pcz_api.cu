@@ -434,8 +434,8 @@ BoxJob make_job(const pc_streams* s, int k0, int k, const int64_t lo[3], const i
   return J;
 }
 
-// Cuts the jobs of one launch into units (retrieve_unit_mult on the launch's
-// brick total) and places them one after the other; returns the units.  Units
+// Cuts the jobs of one launch into units (retrieve_split on the launch's brick
+// total) and places them one after the other; returns the units.  Units
 // of 1D/2D jobs are bricks.
 int64_t place_job_list(BoxJob* jobs, int nj, int dtype, int ndims) {
   int64_t bricks = 0, units = 0;
@@ -443,9 +443,8 @@ int64_t place_job_list(BoxJob* jobs, int nj, int dtype, int ndims) {
   for (int j = 0; j < nj; ++j) {
     BoxJob& J = jobs[j];
     J.unit_begin = units;
-    J.umult = retrieve_unit_mult(dtype, J.k - J.k0, J.nbox, bricks);
-    const int64_t ub = 16 * (int64_t)J.umult;
-    J.dv_ub = div_magic((uint64_t)ub);
+    retrieve_split(dtype, J.k - J.k0, bricks, &J.round, &J.unit_bricks);
+    const int64_t ub = J.unit_bricks;
     units += ndims == 3 ? (J.nbox + ub - 1) / ub : J.nbox;
   }
   return units;

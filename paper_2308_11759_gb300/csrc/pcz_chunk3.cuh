@@ -15,13 +15,6 @@
 
 namespace pcz {
 
-// Rank of each brick position in coded order (R8).
-constexpr PermTable make_rank() {
-  const PermTable perm = make_perm(64);
-  PermTable t{};
-  for (int r = 0; r < 64; ++r) t.pos[perm.pos[r]] = (int8_t)r;
-  return t;
-}
 static __constant__ PermTable kRank3 = make_rank();
 
 // Largest bit string of one brick and component: the header, at most one
@@ -42,18 +35,14 @@ constexpr int kWarps3 = kCompressThreads3 / 32;
 
 // A warp's work area in shared memory, in u32 words.  Three uses follow one
 // another within a component:
-//  (a) exchanges between the z-planes and the y-planes of the lifting passes:
-//      16-byte vectors of 4 values along x (float64: two such sets, 2 values
-//      each), vector (y, z) of brick b at (b >> 1) * 38 + (b & 1) + 10 z + 2 y.
-//      Both directions are free of bank conflicts.
+//  (a) the exchanges of the lifting passes (LineSet; float64: two sets);
 //  (b) the digits in coded order, brick b from word 72 b (36 b as halves, 20 b
 //      as bytes);
 //  (c) the plane words, brick b from word b * kPlaneStride: word j of the
 //      lane's 16 coefficients q at 4 j + q; a RAW brick's residual in their place.
 template <typename T>
 struct Area3 {
-  static constexpr int kSet = 38 * 4;                                     // vectors of one set of (a)
-  static constexpr int kWords = kSet * 4 * (int)(sizeof(T) / 4);
+  static constexpr int kWords = LineSet::kVectors * 4 * (int)(sizeof(T) / 4);
   static constexpr int kPlaneStride = 16 * (int)sizeof(T) + 4;
   static constexpr int kInfoStride = Fmt<T>::P + 4;                       // plane table, words per brick
 };
@@ -141,68 +130,6 @@ __device__ __forceinline__ void plane_at(const uint32_t* planes, int j, int H, u
   *hi = j >= 0 ? __byte_perm(r.z, r.w, sel) : 0u;
 }
 
-// 4 values along x to and from the work area, in 16-byte vectors (`set`
-// vectors between a 64-bit line's two halves).
-__device__ __forceinline__ void put_line(uint4* a, int, const int32_t* v) {
-  *a = make_uint4((uint32_t)v[0], (uint32_t)v[1], (uint32_t)v[2], (uint32_t)v[3]);
-}
-__device__ __forceinline__ void get_line(const uint4* a, int, int32_t* v) {
-  const uint4 r = *a;
-  v[0] = (int32_t)r.x;
-  v[1] = (int32_t)r.y;
-  v[2] = (int32_t)r.z;
-  v[3] = (int32_t)r.w;
-}
-__device__ __forceinline__ void put_line(uint4* a, int set, const int64_t* v) {
-  longlong2* d = reinterpret_cast<longlong2*>(a);
-  d[0] = make_longlong2(v[0], v[1]);
-  d[set] = make_longlong2(v[2], v[3]);
-}
-__device__ __forceinline__ void get_line(const uint4* a, int set, int64_t* v) {
-  const longlong2* d = reinterpret_cast<const longlong2*>(a);
-  const longlong2 p = d[0], r = d[set];
-  v[0] = p.x;
-  v[1] = p.y;
-  v[2] = r.x;
-  v[3] = r.y;
-}
-
-// R7 on a warp's 8 bricks.  v: the lane's z-plane q (value x + 4 y) on entry;
-// on return its y-plane q of coefficients (coefficient x + 4 z).  One exchange
-// through the work area: a lane lifts along x and y in registers, then along z.
-template <typename S>
-__device__ __forceinline__ void lift_fwd_bricks(S* v, uint4* zw, uint4* yw, int set) {
-#pragma unroll
-  for (int y = 0; y < 4; ++y) lift_fwd(v[4 * y], v[4 * y + 1], v[4 * y + 2], v[4 * y + 3]);
-#pragma unroll
-  for (int x = 0; x < 4; ++x) lift_fwd(v[x], v[x + 4], v[x + 8], v[x + 12]);
-#pragma unroll
-  for (int y = 0; y < 4; ++y) put_line(zw + 2 * y, set, v + 4 * y);
-  __syncwarp();
-#pragma unroll
-  for (int z = 0; z < 4; ++z) get_line(yw + 10 * z, set, v + 4 * z);
-  __syncwarp();
-#pragma unroll
-  for (int x = 0; x < 4; ++x) lift_fwd(v[x], v[x + 4], v[x + 8], v[x + 12]);
-}
-
-// The inverse: coefficients of the lane's y-plane in, values of its z-plane out.
-template <typename S>
-__device__ __forceinline__ void lift_inv_bricks(S* v, uint4* zw, uint4* yw, int set) {
-#pragma unroll
-  for (int x = 0; x < 4; ++x) lift_inv(v[x], v[x + 4], v[x + 8], v[x + 12]);
-#pragma unroll
-  for (int z = 0; z < 4; ++z) put_line(yw + 10 * z, set, v + 4 * z);
-  __syncwarp();
-#pragma unroll
-  for (int y = 0; y < 4; ++y) get_line(zw + 2 * y, set, v + 4 * y);
-  __syncwarp();
-#pragma unroll
-  for (int x = 0; x < 4; ++x) lift_inv(v[x], v[x + 4], v[x + 8], v[x + 12]);
-#pragma unroll
-  for (int y = 0; y < 4; ++y) lift_inv(v[4 * y], v[4 * y + 1], v[4 * y + 2], v[4 * y + 3]);
-}
-
 // Staging of a chunk's field values in shared memory with TMA (the
 // persistent construction kernel, pcz_compress.cu): when the field's rows of
 // bricks are whole chunks (bricks per row a multiple of 32), a chunk is one
@@ -212,10 +139,6 @@ __device__ __forceinline__ void lift_inv_bricks(S* v, uint4* zw, uint4* yw, int 
 // fastest).  The copies signal an mbarrier by their bytes.  Values past the
 // field's end arrive as zeros and are never used: readers clamp to the last
 // in-field line and value (rule R4).
-__device__ __forceinline__ uint32_t smem_addr(const void* p) {
-  return (uint32_t)__cvta_generic_to_shared(p);
-}
-
 // Waits for the barrier's phase with parity `parity` to complete, at most
 // `limit` polls (each poll may itself suspend the thread for a while); false
 // when it gave up.
@@ -338,7 +261,7 @@ __device__ __forceinline__ void compress3_chunk(const CompressParams& P, int64_t
   constexpr int BUFW = chunk_buf_words3<T>();
   constexpr uint32_t CAP = (uint32_t)BUFW * 32;  // bits of the chunk buffer
   constexpr unsigned FULL = 0xffffffffu;
-  constexpr int SET = A3::kSet;
+  constexpr int SET = LineSet::kVectors;
 
   uint32_t* cbuf = reinterpret_cast<uint32_t*>(smem + staging_bytes3<T>(map != nullptr));
   uint32_t* areas = cbuf + BUFW;
@@ -434,23 +357,13 @@ __device__ __forceinline__ void compress3_chunk(const CompressParams& P, int64_t
   if (__any_sync(FULL, m >= F::INF) && lane == 0) atomicOr(P.flags, kFlagNonFinite);
 
   uint32_t* area = areas + warp * A3::kWords;
-  uint4* zw = reinterpret_cast<uint4*>(area) + (bq >> 1) * 38 + (bq & 1) + 10 * q;  // + 2 y: line (y, z = q)
-  uint4* yw = reinterpret_cast<uint4*>(area) + (bq >> 1) * 38 + (bq & 1) + 2 * q;   // + 10 z: line (y = q, z)
+  uint4* zw = reinterpret_cast<uint4*>(area) + LineSet::at(bq, 0, q);  // + 2 y: line (y, z = q)
+  uint4* yw = reinterpret_cast<uint4*>(area) + LineSet::at(bq, q, 0);  // + 10 z: line (y = q, z)
   uint32_t* planes = area + bq * A3::kPlaneStride;
   uint32_t* info = infos + slot * A3::kInfoStride;
-  // places of this lane's coefficients in coded order, a byte each: rank r at
-  // 16 (r / 16) + 4 (r & 3) + 2 ((r >> 2) & 1) + ((r >> 3) & 1), in elements of
-  // 1, 2 or 4 bytes
-  uint32_t place[4];
+  uint32_t place[4];  // coded places of the lane's coefficients x + 4 z (y = q)
 #pragma unroll
-  for (int z = 0; z < 4; ++z) {
-    place[z] = 0u;
-#pragma unroll
-    for (int xx = 0; xx < 4; ++xx) {
-      const int r = kRank3.pos[xx + 4 * q + 16 * z];
-      place[z] |= (uint32_t)((r & 48) + 4 * (r & 3) + 2 * ((r >> 2) & 1) + ((r >> 3) & 1)) << (8 * xx);
-    }
-  }
+  for (int z = 0; z < 4; ++z) place[z] = coded_places(kRank3.pos, q, z);
 
   for (int i = 0; i < P.n; ++i) {  // one component per tau_i
     const U tb = (U)P.tau_bits[i];

@@ -478,7 +478,7 @@ __device__ __forceinline__ void compress_small_chunk(const CompressParams& P, in
 // now 1244; 4096^2 float32, k = 6: 659 -> 278 us.
 template <typename T, int D>
 __device__ __forceinline__ void retrieve_small_brick(const BoxJob& J, int write, unsigned int* err, int64_t g,
-                                                     const uint16_t* tokens) {
+                                                     const uint32_t* tokens) {
   using F = Fmt<T>;
   using U = typename F::U;
   using S = typename F::S;
@@ -559,34 +559,35 @@ __device__ __forceinline__ void retrieve_small_brick(const BoxJob& J, int write,
               W = (uint32_t)w64 & ((1u << n) - 1u);
               uint32_t used = (uint32_t)n;
               if (n < N) {
-                uint64_t gb = w64 >> n;
-                uint32_t st = 0;
-                int c = n;
-                ok = false;
-                for (int t = 0; t < (N == 16 ? 5 : 2); ++t) {  // a valid part is at most 2 (N - n) + 1 bits
-                  const uint32_t e = tokens[st | ((uint32_t)gb & 0xffu)];
-                  const uint32_t o = e & 0xffu;
-                  const int cn = c + (int)((e >> 8) & 15u);
-                  if (cn >= N || (e & kTokEnded)) {  // the part ends in this byte
-                    W |= o << c;
-                    if (cn >= N) {  // the last coefficient's 1 ends it, with no closing test bit
-                      const int l = N - 1 - c;
-                      ok = (o >> l) & 1u;
-                      W &= (1u << N) - 1u;
-                      used += (uint32_t)(l + 1) + (st ? 0u : 1u) + (uint32_t)__popc(o & ((1u << l) - 1u));
-                      n = N;
-                    } else {
-                      ok = true;
-                      used += ((e >> 13) & 7u) + 1u;
-                      n = cn;
-                    }
-                    break;
-                  }
-                  W |= o << c;
-                  c = cn;
-                  st = (e >> 5) & 0x100u;
-                  gb >>= 8;
+                const uint64_t gb = w64 >> n;
+                uint32_t gl = (uint32_t)gb, gh = (uint32_t)(gb >> 32), e = 0, idx = 0, o = 0;
+                int cnt = 0;
+                // a valid part is at most 2 (N - n) + 1 bits; left at one place for
+                // all lanes (see pcz_retrieve.cu)
+#pragma unroll 1
+                for (int t = N == 16 ? 5 : 2; t > 0; --t) {
+                  idx = token_index(e, gl, 0);
+                  e = tokens[idx];
+                  cnt = token_count(e);
+                  o = e & 0xffu;
+                  W |= o << n;
+                  if (n + cnt >= N || (int32_t)e < 0) break;
+                  n += cnt;
+                  cnt = 0;
                   used += 8;
+                  gl = __funnelshift_r(gl, gh, 8);
+                  gh >>= 8;
+                }
+                if (n + cnt >= N) {  // the last coefficient's 1 ends it, with no closing test bit
+                  const int l = N - 1 - n;
+                  ok = (o >> l) & 1u;
+                  W &= (1u << N) - 1u;
+                  used += (uint32_t)(l + 1) + (idx < 256u ? 1u : 0u) + (uint32_t)__popc(o & ((1u << l) - 1u));
+                  n = N;
+                } else {
+                  ok = (int32_t)e < 0;
+                  used += ((e >> 24) & 7u) + 1u;
+                  n += cnt;
                 }
               }
               pos += used;

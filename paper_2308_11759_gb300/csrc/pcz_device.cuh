@@ -126,6 +126,21 @@ __device__ __forceinline__ void lift_inv(S& a, S& b, S& c, S& d) {
   d = wadd(c, d2);
 }
 
+// lift_inv in float, the same values wherever every shift of lift_inv divides an
+// even number and no value needs more than 24 bits: 8 operations instead of 11,
+// on the pipe that integer work leaves idle.
+__device__ __forceinline__ void lift_inv(float& a, float& b, float& c, float& d) {
+  const float s0 = a, d0 = b, e1 = c, e2 = d;
+  const float d1 = __fmaf_rn(0.5f, d0, e1);
+  const float d2 = __fadd_rn(e2, d1);
+  const float s1 = __fmaf_rn(-0.5f, d0, s0);
+  const float s2 = __fadd_rn(s1, d0);
+  a = __fmaf_rn(-0.5f, d1, s1);
+  b = __fadd_rn(a, d1);
+  c = __fmaf_rn(-0.5f, d2, s2);
+  d = __fadd_rn(c, d2);
+}
+
 // R9: negabinary map and its inverse, modulo 2^P.
 template <typename T>
 __device__ __forceinline__ typename Fmt<T>::U nb_fwd(typename Fmt<T>::S q) {
@@ -308,6 +323,14 @@ __device__ __forceinline__ double scaled_i32_to_f64(int32_t r, uint32_t eb) {
   return __hiloint2double(a ? (int)hw : 0, (int)(n << 21));
 }
 
+// r * 2^e for a float r, exactly, where the result is a normal double (or r is
+// 0): adj = (896 + e) << 20, the change of exponent bias in the high word.
+__device__ __forceinline__ double scaled_f32_to_f64(float r, uint32_t adj) {
+  const int b = __float_as_int(r);
+  const uint32_t hi = ((uint32_t)(b >> 3) & 0x8FFFFFFFu) + adj;
+  return __hiloint2double(r == 0.0f ? 0 : (int)hi, b << 29);
+}
+
 // The bit pattern of |v| shifted left by one place (the sign shifted out),
 // in an integer instruction the compiler cannot see through.  Masking the
 // sign bit of a float64 pattern instead is recognised as fabs and emitted as
@@ -434,55 +457,6 @@ __device__ __forceinline__ unsigned long long warp_max_u64(unsigned mask, unsign
 
 __device__ __forceinline__ uint64_t low_mask64(int n) { return n >= 64 ? ~0ull : ((1ull << n) - 1); }
 
-// ---------------------------------------------------------------------------
-// 32x32 bit-matrix transpose across a warp: lane l holds row l; afterwards
-// lane l holds column l (bit r = bit l of row r).  Five exchange stages with
-// the lane l ^ k, k = 16, 8, 4, 2, 1: a lane keeps the k-bit groups of its
-// word on its own side (low groups when bit k of l is 0) and takes the
-// partner's groups of the other side, shifted across by k.  Stages 16 and 8
-// move whole bytes, so one byte permute does the shift and the merge; stages
-// 4, 2 and 1 use a rotation (the bits it wraps around land in the kept
-// groups and are masked off) and one logic op.  keep[] holds this lane's byte
-// selectors for stages 16 and 8 and its kept-bit masks for stages 4, 2, 1,
-// from transpose_masks().
-// ---------------------------------------------------------------------------
-__device__ __forceinline__ void transpose_masks(int lane, uint32_t keep[5]) {
-  keep[0] = (lane & 16) ? 0x3276u : 0x5410u;  // partner's high half down / own low half kept
-  keep[1] = (lane & 8) ? 0x3715u : 0x6240u;   // likewise for the bytes of each half
-  const uint32_t lo[3] = {0x0F0F0F0Fu, 0x33333333u, 0x55555555u};
-#pragma unroll
-  for (int st = 0; st < 3; ++st) {
-    const int k = 4 >> st;
-    keep[2 + st] = (lane & k) ? ~lo[st] : lo[st];
-  }
-}
-
-__device__ __forceinline__ uint32_t transpose32(uint32_t a, int lane, const uint32_t keep[5]) {
-  a = __byte_perm(a, __shfl_xor_sync(0xffffffffu, a, 16), keep[0]);
-  a = __byte_perm(a, __shfl_xor_sync(0xffffffffu, a, 8), keep[1]);
-#pragma unroll
-  for (int st = 0; st < 3; ++st) {
-    const int k = 4 >> st;
-    const uint32_t b = __shfl_xor_sync(0xffffffffu, a, k);
-    // rotate right by k (partner's high groups down) or by 32 - k (low groups up)
-    const uint32_t moved = __funnelshift_r(b, b, (uint32_t)(2 * (lane & k) - k));
-    a = (a & keep[2 + st]) | (moved & ~keep[2 + st]);
-  }
-  return a;
-}
-
-// Index of brick element (x, y, z) of the warp's half h in the shared brick
-// buffer (two bricks, 128 elements).  The rotations make every lifting pass
-// (16 lanes of a brick reading one line position each) and the x-line
-// accesses free of bank conflicts for 4- and 8-byte elements.
-template <typename T>
-__device__ __forceinline__ int sidx(int x, int y, int z, int h) {
-  if constexpr (sizeof(T) == 8)
-    return 64 * h + 16 * z + 4 * ((y + z) & 3) + ((x + z) & 3);
-  else
-    return 32 * z + 16 * h + 4 * ((y + z) & 3) + ((x + z) & 3);
-}
-
 // One x-line of a brick (4 consecutive values) between registers and memory:
 // a single 16-byte access per 16 bytes when the line is whole and aligned
 // (fewer transactions, which matters most when the memory is on the host side
@@ -566,6 +540,13 @@ __device__ __forceinline__ void untranspose8(uint32_t (&a)[4]) {
     const uint32_t t = (a[i] ^ (a[i] >> 12)) & 0x0000F0F0u;
     a[i] ^= t ^ (t << 12);
   }
+}
+__device__ __forceinline__ void untranspose16(uint32_t (&a)[8]) {  // transpose16 backwards
+  exchange_stage<8, 1>(a, 0x55555555u);
+  exchange_stage<8, 2>(a, 0x33333333u);
+  exchange_stage<8, 4>(a, 0x0F0F0F0Fu);
+#pragma unroll
+  for (int i = 0; i < 8; ++i) a[i] = __byte_perm(a[i], 0u, 0x3120);
 }
 __device__ __forceinline__ void transpose16(uint32_t (&a)[8]) {
 #pragma unroll
@@ -700,20 +681,27 @@ struct BlockBits {
     wi = 0;
     set(ld(0), ld(1));
   }
+  __device__ __forceinline__ void advance() {  // by one word
+    a0 = b0;
+    a1 = b1;
+    const uint64_t nb = ld(++wi + 1);
+    b0 = (uint32_t)nb;
+    b1 = (uint32_t)(nb >> 32);
+  }
   __device__ __forceinline__ uint64_t peek(uint32_t pos) {
     const uint32_t i = pos >> 6;
     if (i != wi) {
       if (i == wi + 1) {
-        a0 = b0;
-        a1 = b1;
-        const uint64_t nb = ld(i + 1);
-        b0 = (uint32_t)nb;
-        b1 = (uint32_t)(nb >> 32);
+        advance();
       } else {
         set(ld(i), ld(i + 1));
+        wi = i;
       }
-      wi = i;
     }
+    return window(pos);
+  }
+  // 64 bits from pos, which lies in word wi
+  __device__ __forceinline__ uint64_t window(uint32_t pos) const {
     const bool up = pos & 32u;  // window starts in the word's upper half
     const uint32_t x0 = up ? a1 : a0, x1 = up ? b0 : a1, x2 = up ? b1 : b0;
     return ((uint64_t)__funnelshift_r(x1, x2, pos) << 32) | __funnelshift_r(x0, x1, pos);
@@ -722,52 +710,155 @@ struct BlockBits {
 
 // Byte table of the group-test part as a two-state machine: in state "test"
 // a 0 ends the part and a 1 starts a run; in state "run" every bit is the
-// next coefficient's bit and a 1 ends the run.  Entry [state][byte] (16 bits):
-// bits 0-7 the 1s among the byte's coefficient bits (coefficient-relative),
-// bits 8-11 their count, bit 12 set when the part ends in the byte; then
-// bits 13-15 hold the bits used up to and including the closing test bit,
-// minus 1; otherwise bit 13 is the state after the byte.
-constexpr uint32_t kTokEnded = 1u << 12;
+// next coefficient's bit and a 1 ends the run.  Entry 256 * state + byte: byte 0
+// the byte's coefficient bits, byte 1 the state after it, byte 2 how many
+// coefficients, byte 3 128 when the part ends in the byte, plus the bits used up
+// to and including the closing test bit, minus 1.
 constexpr int kTokLut = 512;  // entries (2 states x 256 bytes)
 
-struct alignas(4) TokenTable {
-  uint16_t entry[kTokLut];
+struct TokenTable {
+  uint32_t entry[kTokLut];
 };
 constexpr TokenTable make_tokens() {
   TokenTable t{};
   for (int idx = 0; idx < kTokLut; ++idx) {
-    int st = idx >> 8;
-    const int byte = idx & 255;
-    unsigned out = 0, cnt = 0, e = 0;
-    bool ended = false;
-    for (int j = 0; j < 8 && !ended; ++j) {
-      const int bit = (byte >> j) & 1;
+    unsigned st = (unsigned)idx >> 8, out = 0, cnt = 0, end = 0;
+    for (int j = 0; j < 8 && !end; ++j) {
+      const unsigned bit = ((unsigned)idx >> j) & 1u;
       if (st == 0) {
-        if (bit) {
+        if (bit)
           st = 1;
-        } else {
-          ended = true;
-          e = kTokEnded | ((unsigned)j << 13);
-        }
+        else
+          end = 128u + (unsigned)j;
       } else {
-        out |= (unsigned)bit << cnt;
+        out |= bit << cnt;
         ++cnt;
         if (bit) st = 0;
       }
     }
-    if (!ended) e = (unsigned)st << 13;
-    t.entry[idx] = (uint16_t)(out | (cnt << 8) | e);
+    t.entry[idx] = out | (st << 8) | (cnt << 16) | (end << 24);
   }
   return t;
 }
 static __device__ const TokenTable kTokens = make_tokens();
 
-// A CTA's copy of the table in shared memory (4-byte aligned); read after the
-// next barrier.
+// A CTA's copy of the table in shared memory; read after the next barrier.
 template <int THREADS>
-__device__ __forceinline__ void load_tokens(uint16_t* at) {
-  uint32_t* w = reinterpret_cast<uint32_t*>(at);
-  for (int i = threadIdx.x; i < kTokLut / 2; i += THREADS) w[i] = reinterpret_cast<const uint32_t*>(kTokens.entry)[i];
+__device__ __forceinline__ void load_tokens(uint32_t* at) {
+  for (int i = threadIdx.x; i < kTokLut; i += THREADS) at[i] = kTokens.entry[i];
+}
+
+// The entry for byte `j` (0..3) of g after entry e (0 at the start of a part):
+// one byte permute forms the index from e's state byte, whose clear sign bit
+// fills the upper bytes.
+__device__ __forceinline__ uint32_t token_index(uint32_t e, uint32_t g, int j) {
+  uint32_t r;
+  asm("prmt.b32 %0, %1, %2, %3;" : "=r"(r) : "r"(e), "r"(g), "r"(0x9914 + j));
+  return r;
+}
+__device__ __forceinline__ int token_count(uint32_t e) { return (int)__byte_perm(e, 0u, 0x4442); }
+
+// Rank of each brick position in coded order (R8).
+constexpr PermTable make_rank() {
+  const PermTable perm = make_perm(64);
+  PermTable t{};
+  for (int r = 0; r < 64; ++r) t.pos[perm.pos[r]] = (int8_t)r;
+  return t;
+}
+// Places of a lane's coefficients x + 4 z (x = 0..3, y = q) in coded order, a
+// byte each: rank r at 16 (r / 16) + 4 (r & 3) + 2 ((r >> 2) & 1) + ((r >> 3) & 1),
+// the order in which the bit transposes take 16 coefficients.
+__device__ __forceinline__ uint32_t coded_places(const int8_t* rank, int q, int z) {
+  uint32_t v = 0;
+#pragma unroll
+  for (int x = 0; x < 4; ++x) {
+    const int r = rank[x + 4 * q + 16 * z];
+    v |= (uint32_t)((r & 48) + 4 * (r & 3) + 2 * ((r >> 2) & 1) + ((r >> 3) & 1)) << (8 * x);
+  }
+  return v;
+}
+
+__device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
+
+// Exchange between the z-planes and the y-planes of a warp's 8 bricks in shared
+// memory: 16-byte vectors of 4 values along x (64-bit values: two sets of 2
+// each), vector (y, z) of brick b at `at`.  Both directions are free of bank
+// conflicts.
+struct LineSet {
+  static constexpr int kVectors = 38 * 4;
+  static __device__ __forceinline__ int at(int b, int y, int z) { return (b >> 1) * 38 + (b & 1) + 10 * z + 2 * y; }
+};
+
+// 4 values along x to and from the work area, in 16-byte vectors (`set`
+// vectors between a 64-bit line's two halves).
+__device__ __forceinline__ void put_line(uint4* a, int, const int32_t* v) {
+  *a = make_uint4((uint32_t)v[0], (uint32_t)v[1], (uint32_t)v[2], (uint32_t)v[3]);
+}
+__device__ __forceinline__ void get_line(const uint4* a, int, int32_t* v) {
+  const uint4 r = *a;
+  v[0] = (int32_t)r.x;
+  v[1] = (int32_t)r.y;
+  v[2] = (int32_t)r.z;
+  v[3] = (int32_t)r.w;
+}
+__device__ __forceinline__ void put_line(uint4* a, int, const float* v) {
+  *reinterpret_cast<float4*>(a) = make_float4(v[0], v[1], v[2], v[3]);
+}
+__device__ __forceinline__ void get_line(const uint4* a, int, float* v) {
+  const float4 r = *reinterpret_cast<const float4*>(a);
+  v[0] = r.x;
+  v[1] = r.y;
+  v[2] = r.z;
+  v[3] = r.w;
+}
+__device__ __forceinline__ void put_line(uint4* a, int set, const int64_t* v) {
+  longlong2* d = reinterpret_cast<longlong2*>(a);
+  d[0] = make_longlong2(v[0], v[1]);
+  d[set] = make_longlong2(v[2], v[3]);
+}
+__device__ __forceinline__ void get_line(const uint4* a, int set, int64_t* v) {
+  const longlong2* d = reinterpret_cast<const longlong2*>(a);
+  const longlong2 p = d[0], r = d[set];
+  v[0] = p.x;
+  v[1] = p.y;
+  v[2] = r.x;
+  v[3] = r.y;
+}
+
+// R7 on a warp's 8 bricks.  v: the lane's z-plane q (value x + 4 y) on entry;
+// on return its y-plane q of coefficients (coefficient x + 4 z).  One exchange
+// through the work area: a lane lifts along x and y in registers, then along z.
+template <typename S>
+__device__ __forceinline__ void lift_fwd_bricks(S* v, uint4* zw, uint4* yw, int set) {
+#pragma unroll
+  for (int y = 0; y < 4; ++y) lift_fwd(v[4 * y], v[4 * y + 1], v[4 * y + 2], v[4 * y + 3]);
+#pragma unroll
+  for (int x = 0; x < 4; ++x) lift_fwd(v[x], v[x + 4], v[x + 8], v[x + 12]);
+#pragma unroll
+  for (int y = 0; y < 4; ++y) put_line(zw + 2 * y, set, v + 4 * y);
+  __syncwarp();
+#pragma unroll
+  for (int z = 0; z < 4; ++z) get_line(yw + 10 * z, set, v + 4 * z);
+  __syncwarp();
+#pragma unroll
+  for (int x = 0; x < 4; ++x) lift_fwd(v[x], v[x + 4], v[x + 8], v[x + 12]);
+}
+
+// The inverse: coefficients of the lane's y-plane in, values of its z-plane out.
+template <typename S>
+__device__ __forceinline__ void lift_inv_bricks(S* v, uint4* zw, uint4* yw, int set) {
+#pragma unroll
+  for (int x = 0; x < 4; ++x) lift_inv(v[x], v[x + 4], v[x + 8], v[x + 12]);
+#pragma unroll
+  for (int z = 0; z < 4; ++z) put_line(yw + 10 * z, set, v + 4 * z);
+  __syncwarp();
+#pragma unroll
+  for (int y = 0; y < 4; ++y) get_line(zw + 2 * y, set, v + 4 * y);
+  __syncwarp();
+#pragma unroll
+  for (int x = 0; x < 4; ++x) lift_inv(v[x], v[x + 4], v[x + 8], v[x + 12]);
+#pragma unroll
+  for (int y = 0; y < 4; ++y) lift_inv(v[4 * y], v[4 * y + 1], v[4 * y + 2], v[4 * y + 3]);
 }
 
 }  // namespace pcz

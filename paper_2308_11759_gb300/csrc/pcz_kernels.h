@@ -65,11 +65,8 @@ struct BoxJob {
   int64_t nbox;                  // bricks meeting the box
   int64_t unit_begin;            // first unit of this job within the launch
   int k0, k;
-  int umult;                     // a unit is 16 * umult bricks
-  int pad_;
+  int round, unit_bricks;        // components decoded at a time; bricks of a unit
   DivMagic dv_bn0, dv_bn1;       // division by bn[0] and bn[1] (used when nbox < 2^32)
-  DivMagic dv_ub;                // division by the bricks of a unit, 16 * umult
-  int32_t pad2_[2];
   void* out;                     // box values of T (read too when k0 > 0)
   const void* cache;             // full-field cached partial sums of T, or null
   const uint8_t* level;          // per brick: k of the cached partial sum (0: none)
@@ -168,11 +165,11 @@ uint32_t check_word_batch(int reset);
 // Sets the message pc_last_error() returns on this thread.
 void set_last_error(const char* msg);
 
-// CTAs of a persistent retrieval launch over nunits units, brick pairs per
-// warp of a unit for a job of nbox bricks and ncomp components in a launch of
-// `bricks` bricks, and the spill words a launch of grid CTAs needs.
+// CTAs of a persistent retrieval launch over nunits units, how a job of ncomp
+// components is split in a launch of `bricks` bricks, and the spill words a
+// launch of grid CTAs needs.
 int retrieve_grid(int dtype, int ndims, int64_t nunits);
-int retrieve_unit_mult(int dtype, int ncomp, int64_t nbox, int64_t bricks);
+void retrieve_split(int dtype, int ncomp, int64_t bricks, int* round, int* unit_bricks);
 size_t retrieve_spill_words(int dtype, int ndims, int grid);
 
 // Finite-difference derivatives (pcz_fd.cu): omega_z = v_x - u_y and the

@@ -14,26 +14,26 @@
 // job's k starts from the cached x~ and decodes only the components above it
 // (Algorithm 2's partial sums are the same whichever way they are reached).
 //
-// Layout: persistent CTAs of 8 warps, each taking units of 16 * umult
-// consecutive bricks of a job's box.  Components are handled in rounds of up
-// to 8.  Parse phase (parse_round): an index pass loads every task's block
-// position and length (a task is one block: one brick and component), a
-// counting sort orders the tasks longest first, and the warps steal them 32
-// at a time, one block per lane (plane parsing is sequential per block, so
-// this is where the lanes' parallelism comes from); a block's plane words go
-// to a shared-memory slot, counted from its top plane down, and the few
-// planes that do not fit to a per-CTA spill area in global memory.  After a
-// barrier, each warp rebuilds its brick pairs (16 lanes per brick, lane t
-// holding the x-line y = t & 3, z = t >> 2): lane p fetches plane p (and
-// p + 32) of both bricks, a 32x32 bit transpose across the warp turns planes
-// back into each lane's coefficients t + 16j, and the inverse reorder,
-// lifting and scaling run through a bank-conflict-free brick buffer; x_j is
-// then added into x~, component by component in ascending order.  Float64
-// pairs whose coded planes span fewer than 16 (most of them at tolerances a
-// few decades apart) are decoded in 32-bit integers scaled to their lowest
-// plane and converted to double without the FP64 pipe, which the partial-sum
-// adds keep busy; this form is a second instantiation of the kernel, used
-// when a brick decodes at least 3 components.
+// Layout: persistent CTAs of 4 warps, each taking units of 32 or more consecutive
+// bricks of a job's box, up to 6 components at a time.  Parse: the warps take
+// tasks of 32 blocks of one component, a block per lane, plane by plane (the
+// blocks of a task are neighbours, so they are of alike length and their index
+// entries are adjacent); the plane words of all blocks lie one after another in
+// shared memory, those that do not fit in global memory.  Rebuild: each warp takes
+// 8 bricks at a time, 4 lanes each.  Lane q of a brick reads the planes' bits of
+// the 16 coefficients q, transposes them back in registers, 8 or 16 planes at
+// once, and hands the digits over through shared memory, each lane taking its
+// y-plane of coefficients; two inverse lifting passes run in registers after one
+// exchange (in float where 8 planes hold a brick's digits: fewer operations, on
+// the otherwise idle pipe), and x_j is added into the lane's z-plane of x~.
+//
+// Bound by instruction issue.  With 16 lanes per brick in the rebuild, CTAs of
+// 512 blocks sorted by length for the parse and an index pass of its own it took
+// 190 (float32, k = 6) and 229 (float64, k = 8) warp instructions per brick and
+// component, now 107 and 127; 512^3 float32: k = 6 2.87 -> 1.71 ms, k = 1 0.86 ->
+// 0.44 ms; 256 x 384 x 384 float64: k = 8 1.29 -> 0.89 ms; refinement from k = 1 to
+// 8 in place 7.06 -> 3.39 and 3.13 -> 1.75 ms (nearly half of it had gone to the
+// index pass and the sort).
 #include <algorithm>
 #include <type_traits>
 
@@ -42,27 +42,24 @@
 
 namespace pcz {
 
-__constant__ PermTable kPerm3r = make_perm(64);
+static __constant__ PermTable kRank3r = make_rank();
 
-constexpr int kRWarps = 8;
+constexpr int kRWarps = 4;
 constexpr int kRThreads = 32 * kRWarps;
-constexpr int kRound = 8;    // components per round
-constexpr int kTasks = 512;  // parse tasks (block of one brick and component) per round
-constexpr int kLenBuckets = 64;  // parse tasks are handed out longest block first, by len / 16
-// plane words per block kept in shared memory: as many as let 3 CTAs share an SM
-template <typename T>
-struct Slots {
-  static constexpr int n = sizeof(T) == 4 ? 15 : 14;
-};
+constexpr int kRoundTasks = 6;                 // warp tasks (32 blocks of one component) parsed at a time, at most
+constexpr int kBlocks = 32 * kRoundTasks;      // their blocks
+constexpr int kPool = 1792;                    // plane words kept in shared memory (a round of the 512^3
+                                               // workload's blocks has 900 to 1730)
+constexpr int kPoolPad = 16;                   // words before and after them that may be read (and are masked)
 
 struct BlockMeta {
   uint64_t off;   // first bit of the brick in the component's payload
   int16_t s;      // scale exponent (R6), within [-1100, 1100]
-  uint16_t len;   // bits of the block from the index; 0: nothing to parse (header final)
-  int8_t p;       // lowest coded plane, 0..64 (64 when the block is not CODED)
-  int8_t top;     // highest non-empty plane, -1 if none
-  int8_t mode;
-  uint8_t comp;   // component within the round
+  int8_t p;       // lowest coded plane, 0..64
+  int8_t top;     // highest non-empty plane, p - 1 if none
+  uint8_t mode;
+  uint8_t pad_;
+  uint16_t at;    // first plane word, from the top plane down: below kPool in shared memory, else spilled
 };
 static_assert(sizeof(BlockMeta) == 16, "block header size");
 
@@ -72,161 +69,133 @@ __device__ __forceinline__ uint32_t div_by(uint32_t n, const DivMagic& D) {
   return (t + ((n - t) >> D.s1)) >> D.s2;
 }
 
+// A warp's work area, in 16-byte vectors: the exchange of the inverse lifting
+// (LineSet), or the digits in coded order (brick b from byte 80 b, 144 b, 272 b
+// or 528 b for 1, 2, 4 or 8 bytes each).
+template <typename T>
+struct AreaR {
+  static constexpr int kVectors = LineSet::kVectors * (int)(sizeof(T) / 4);
+  static_assert(kVectors * 16 >= 8 * (64 * (int)sizeof(T) + 16), "digits fit");
+};
+
 template <typename T>
 __host__ __device__ constexpr size_t retrieve_smem3() {
-  return (size_t)kTasks * Slots<T>::n * sizeof(uint64_t)  // plane slots
-         + (size_t)kTasks * sizeof(BlockMeta)       // block headers
-         + (size_t)kRWarps * 128 * sizeof(typename Fmt<T>::S)  // brick buffers
-         + (size_t)kTokLut * sizeof(uint16_t)                   // group-test byte table
-         + (size_t)kTasks * sizeof(uint16_t)                    // parse order of the round's tasks
-         + (size_t)kLenBuckets * sizeof(int);                   // task counts per length bucket
+  return (size_t)(kPool + 2 * kPoolPad) * sizeof(uint64_t)        // plane words
+         + (size_t)kBlocks * sizeof(BlockMeta)                    // block headers
+         + (size_t)kRWarps * AreaR<T>::kVectors * 16              // work areas
+         + (size_t)kTokLut * sizeof(uint32_t)                     // group-test byte table
+         + (size_t)kBlocks / 8;                                   // decoding of every 8 blocks
 }
 
-template <typename T>
-__host__ __device__ constexpr int spill_per_block() {  // planes below a block's slot
-  return Fmt<T>::P - Slots<T>::n;
-}
-
+// Plane words of a round that may not fit: all of the blocks' planes but the
+// pool's, and one block's that straddles the pool's end.
 template <typename T>
 __host__ __device__ constexpr size_t spill_words_per_cta() {
-  return (size_t)kTasks * spill_per_block<T>();
+  return (size_t)kBlocks * Fmt<T>::P - kPool + Fmt<T>::P;
 }
 
-// The group-test part of a plane (R11), a byte at a time through the table:
-// n coefficients are significant and the part starts at bit pos.  When a
-// byte would carry the count to N, the last coefficient turns significant in
-// it (after which no closing test bit follows) or the block is malformed; the
-// part's end then follows from the byte's entry in closed form.  A valid part
-// is at most 2 (N - n) + 1 <= 129 bits, so 17 bytes bound the loop.
-__device__ __forceinline__ bool parse_group(BlockBits& br, uint32_t& pos, int& n, uint64_t& W, const uint16_t* lut) {
-  constexpr int N = 64;
-  int c = n;
-  uint32_t st = 0;  // state, pre-shifted to index the table's upper half
-  uint32_t used = 0;
-  for (int w = 0; w < 3; ++w) {
-    const uint64_t g = br.peek(pos + used);
-    const uint32_t glo = (uint32_t)g, ghi = (uint32_t)(g >> 32);
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      if (w == 2 && j == 1) return false;  // more than 17 bytes: malformed
-      const uint32_t byte = ((j < 4 ? glo : ghi) >> (8 * (j & 3))) & 0xffu;
-      const uint32_t e = lut[st | byte];
-      const uint32_t out = e & 0xffu;
-      const int cn = c + (int)((e >> 8) & 15u);
-      if (cn >= N || (e & kTokEnded)) {  // the part ends in this byte
-        if (cn >= N) {
-          // coefficient N - 1 is the byte's coefficient bit k; its 1 ends the
-          // part, with no closing test bit.  Bits used through it: k + 1
-          // coefficient bits and the test bits before them (the byte's first
-          // bit in the test state, and one after each earlier 1).
-          const int k = N - 1 - c;
-          if (!((out >> k) & 1u)) return false;  // a run past the last coefficient
-          W |= (uint64_t)(out & ((2u << k) - 1u)) << c;
-          pos += used + (uint32_t)(k + 1) + (st ? 0u : 1u) + (uint32_t)__popc(out & ((1u << k) - 1u));
-          n = N;
-        } else {
-          W |= (uint64_t)out << c;
-          pos += used + ((e >> 13) & 7u) + 1;
-          n = cn;
-        }
-        return true;
-      }
-      W |= (uint64_t)out << c;
-      c = cn;
-      st = (e >> 5) & 0x100u;
-      used += 8;
-    }
-  }
-  return false;
-}
-
-// R11 decoding of planes P-1 .. p of one block, starting at bit pos and ending
-// exactly at end.  Plane pl (for pl in [p, top], top = the highest non-empty
-// plane, -1 if none) goes to slot[top - pl], or to spill[top - pl - Slots<T>::n]
-// below the slot.  Planes above the first significant coefficient are one 0
-// test bit each and are skipped together.  Returns false on a malformed
-// block; every loop is bounded.
+// The place of the block whose plane words start at index `at` of the round.
 template <typename T>
-__device__ bool parse_planes(BlockBits& br, uint32_t pos, uint32_t end, int p, uint64_t* slot, uint64_t* spill,
-                             int& top, const uint16_t* lut) {
-  constexpr int N = 64;
-  int n = 0;
-  top = -1;
-  int pl = Fmt<T>::P - 1;
-  while (pl >= p) {
-    const uint64_t v = br.peek(pos);
-    if (v & 1ull) break;
-    const int z = v ? __ffsll((long long)v) - 1 : 64;
-    const int skip = min(z, pl - p + 1);
-    pos += (uint32_t)skip;
-    pl -= skip;
-    if (skip == z && z < 64) break;  // the bit after the zeros is the first significant plane's test 1
+__device__ __forceinline__ uint64_t* words_at(uint64_t* pool, uint64_t* spill, int at, int nw) {
+  return at + nw <= kPool ? pool + at : spill + (at - (kPool - Fmt<T>::P));
+}
+
+// A plane in which coefficients may turn significant (R11): n < 64 verbatim bits
+// at pos, then the group-test part, a byte at a time through the table.  The
+// plane word is gathered at the top of 64 bits, each byte's coefficient bits
+// funnelled in from above, and moved down at the end.  When a byte would carry the
+// count to 64, the last coefficient turns significant in it (after which no
+// closing test bit follows) or the block is malformed; the part's end then
+// follows from the byte's entry in closed form.  A valid part is at most
+// 2 (64 - n) + 1 <= 129 bits.
+__device__ __forceinline__ bool parse_group_plane(BlockBits& br, uint32_t& pos, int& n, uint64_t& W,
+                                                  const uint32_t* lut) {
+  const uint64_t v = (br.peek(pos) << 1) << (63 - n);
+  uint32_t wlo = (uint32_t)v, whi = (uint32_t)(v >> 32), e = 0, idx = 0;
+  pos += (uint32_t)n;
+  int c = n, cnt = 0;
+  bool end = false;
+  // 4 bytes at a time without branches (a lane whose part has ended shifts by 0):
+  // code at the exits of a loop over bytes would run once for every byte at which
+  // some lane ends.  A byte that does not end the part holds at least 4
+  // coefficients, which bounds the loop.
+#pragma unroll 1
+  for (;;) {
+    const uint64_t g64 = br.peek(pos);
+    auto word = [&](uint32_t g) {
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const uint32_t i1 = token_index(e, g, j), e1 = lut[i1];
+        const int c1 = token_count(e1);
+        if (!end) {
+          idx = i1;
+          e = e1;
+          cnt = c1;
+        }
+        end = end || c + cnt >= 64 || (int32_t)e < 0;  // the part ends in this byte
+        const int add = end ? 0 : cnt;
+        wlo = __funnelshift_r(wlo, whi, add);
+        whi = __funnelshift_r(whi, e, add);
+        c += add;
+        pos += end ? 0u : 8u;
+      }
+    };
+    word((uint32_t)g64);
+    if (!end) word((uint32_t)(g64 >> 32));
+    if (end) break;
   }
-  for (; pl >= p; --pl) {
-    uint64_t W = 0;
-    if (n > 0) {
-      W = br.peek(pos) & low_mask64(n);
-      pos += (uint32_t)n;
+  const int k = min(64 - c, cnt);  // of its coefficients
+  wlo = __funnelshift_r(wlo, whi, k);
+  whi = __funnelshift_r(whi, e, k);
+  c += k;
+  W = (((uint64_t)whi << 32) | wlo) >> (64 - c);
+  n = c;
+  if (c == 64) {
+    // bits used through the last coefficient's 1: its byte's first k coefficient
+    // bits and the test bits before them (the byte's first bit in the test state,
+    // and one after each earlier 1)
+    pos += (uint32_t)k + (idx < 256u ? 1u : 0u) + (uint32_t)__popc(e & ((1u << (k - 1)) - 1u));
+    return whi >> 31;  // (0: a run past the last coefficient)
+  }
+  pos += ((e >> 24) & 7u) + 1u;
+  return true;
+}
+
+// R11 decoding of planes top .. p of one block (top: the highest non-empty one,
+// whose test bit 1 is at bit pos), ending exactly at end, into out[0 .. top - p].
+// Returns false on a malformed block; every loop is bounded.
+__device__ __forceinline__ bool parse_planes(BlockBits& br, uint32_t pos, uint32_t end, int nw, uint64_t* out,
+                                             const uint32_t* lut) {
+  int n = 0;
+  for (int k = 0; k < nw; ++k) {
+    uint64_t W;
+    if (n == 64) {
+      W = br.peek(pos);
+      pos += 64;
+    } else if (!parse_group_plane(br, pos, n, W, lut)) {
+      return false;
     }
-    if (n < N && !parse_group(br, pos, n, W, lut)) return false;
     if (pos > end) return false;
-    if (W && top < 0) top = pl;
-    if (top >= 0) {
-      const int rel = top - pl;
-      if (rel < Slots<T>::n)
-        slot[rel] = W;
-      else if (PCZ_CHECK(rel - Slots<T>::n < spill_per_block<T>(), 3))
-        spill[rel - Slots<T>::n] = W;
-    }
+    out[k] = W;
   }
   return pos == end;
 }
 
-// One brick of the unit as seen by this lane: where it is and which of its
-// values this lane's x-line writes.
-struct BrickLane {
-  bool have, line_ok;
-  bool vm[4];
-  int64_t bx, b, orow, frow;
-};
-
-// FAST_DIV: split g by invariant-integer division (measured faster for
-// float64 fields and slower for float32 ones, where the kernel's register
-// allocation changes with it).
-template <bool FAST_DIV>
-__device__ __forceinline__ BrickLane brick_lane(const BoxJob& J, int64_t g, int t) {
-  BrickLane L;
-  L.have = g < J.nbox;
-  int64_t bx = 0, by = 0, bz = 0;
-  if (L.have) {
-    if (FAST_DIV && J.nbox < (1ll << 32)) {  // 32-bit division by the box's invariant extents
-      const uint32_t g32 = (uint32_t)g;
-      const uint32_t r = div_by(g32, J.dv_bn0);
-      const uint32_t z = div_by(r, J.dv_bn1);
-      bx = J.bl[0] + (int64_t)(g32 - r * (uint32_t)J.bn[0]);
-      by = J.bl[1] + (int64_t)(r - z * (uint32_t)J.bn[1]);
-      bz = J.bl[2] + (int64_t)z;
-    } else {
-      bx = J.bl[0] + g % J.bn[0];
-      const int64_t r = g / J.bn[0];
-      by = J.bl[1] + r % J.bn[1];
-      bz = J.bl[2] + r / J.bn[1];
-    }
+// Brick g of the job's box (x fastest): its coordinates.
+__device__ __forceinline__ void brick_of(const BoxJob& J, int64_t g, int64_t* bx, int64_t* by, int64_t* bz) {
+  if (J.nbox < (1ll << 32)) {  // 32-bit division by the box's invariant extents
+    const uint32_t g32 = (uint32_t)g;
+    const uint32_t r = div_by(g32, J.dv_bn0);
+    const uint32_t z = div_by(r, J.dv_bn1);
+    *bx = J.bl[0] + (int64_t)(g32 - r * (uint32_t)J.bn[0]);
+    *by = J.bl[1] + (int64_t)(r - z * (uint32_t)J.bn[1]);
+    *bz = J.bl[2] + (int64_t)z;
+  } else {
+    *bx = J.bl[0] + g % J.bn[0];
+    const int64_t r = g / J.bn[0];
+    *by = J.bl[1] + r % J.bn[1];
+    *bz = J.bl[2] + r / J.bn[1];
   }
-  L.bx = bx;
-  L.b = bx + J.nb[0] * (by + J.nb[1] * bz);
-  const int64_t gy = 4 * by + (t & 3), gz = 4 * bz + (t >> 2);
-  L.line_ok = L.have && gy < J.dims[1] && gz < J.dims[2] && gy >= J.lo[1] && gy < J.hi[1] && gz >= J.lo[2] &&
-              gz < J.hi[2];
-  const int64_t ext0 = J.hi[0] - J.lo[0], ext1 = J.hi[1] - J.lo[1];
-  L.orow = ((gz - J.lo[2]) * ext1 + (gy - J.lo[1])) * ext0 + 4 * bx - J.lo[0];
-  L.frow = (gz * J.dims[1] + gy) * J.dims[0] + 4 * bx;
-#pragma unroll
-  for (int m = 0; m < 4; ++m) {
-    const int64_t gx = 4 * bx + m;
-    L.vm[m] = L.line_ok && gx < J.dims[0] && gx >= J.lo[0] && gx < J.hi[0];
-  }
-  return L;
 }
 
 // Level of brick b's cached partial sum that a job at k may start from (0:
@@ -237,447 +206,509 @@ __device__ __forceinline__ int cached_level(const BoxJob& J, int64_t b) {
   return lv <= J.k ? lv : 0;
 }
 
-// x~ of this lane's 4 values at the start of a job: 0, the caller's partial
-// sum x~_k0 (refinement), or the cache.
-template <typename T>
-__device__ __forceinline__ void start_sum(const BoxJob& J, int write, const BrickLane& BL, T* xt) {
-  const int lv = BL.have ? cached_level(J, BL.b) : 0;
-  const T* cache = reinterpret_cast<const T*>(J.cache);
-  const T* out = reinterpret_cast<const T*>(J.out);
-#pragma unroll
-  for (int m = 0; m < 4; ++m) {
-    xt[m] = T(0);
-    if (lv > 0 && BL.vm[m])
-      xt[m] = cache[BL.frow + m];
-    else if (write && J.k0 > 0 && BL.vm[m])
-      xt[m] = out[BL.orow + m];
-  }
-}
+// How 8 blocks (one component of a rebuild's bricks) are decoded: the largest of
+// theirs, and whether one is RAW.
+enum : int { kDecodeNone = 0, kDecodeFloat8 = 1, kDecodeInt16 = 2, kDecodeAny = 3, kHasRaw = 4 };
 
-// Rebuilds one component of the warp's brick pair (lanes 0-15: brick A,
-// 16-31: brick B) from the parsed blocks mA/mB (slots sA/sB, spill pA/pB):
-// returns this lane's 4 values of x_j.  SC (float64): pairs whose coded
-// planes span fewer than 16 take the 32-bit integer decoding.
-template <typename T, bool SC>
-__device__ __forceinline__ void rebuild_pair(const BlockMeta& mA, const BlockMeta& mB, const uint64_t* sA,
-                                             const uint64_t* sB, const uint64_t* pA, const uint64_t* pB,
-                                             const CompDesc* cd, typename Fmt<T>::S* buf, const int* ix,
-                                             const int* iy, const int* iz, const int* ir, const uint32_t* tkeep,
-                                             int lane, int h, int t, T* xi) {
-  using F = Fmt<T>;
-  using U = typename F::U;
-  using S = typename F::S;
-  constexpr bool WIDE = F::P == 64;
-  const BlockMeta& my = h ? mB : mA;
-#pragma unroll
-  for (int m = 0; m < 4; ++m) xi[m] = T(0);
-  const bool cA = mA.mode == kModeCoded, cB = mB.mode == kModeCoded;
-  if (cA || cB) {
-    // lane l fetches plane l (and l + 32) of both bricks; planes outside
-    // [p, top] are zero
-    auto fetch = [&](const BlockMeta& mX, const uint64_t* sX, const uint64_t* pX, int pl) {
-      if (pl < mX.p || pl > mX.top) return (uint64_t)0;  // a block not CODED has p = 64, top = -1
-      const int rel = mX.top - pl;
-      if (rel < Slots<T>::n) return sX[rel];
-      return PCZ_CHECK(rel - Slots<T>::n < spill_per_block<T>(), 3) ? pX[rel - Slots<T>::n] : (uint64_t)0;
-    };
-    const int lo = min((int)mA.p, (int)mB.p);
-    const int hi = max((int)mA.top, (int)mB.top);
-    S r[4];            // the coefficients after the inverse transform
-    bool conv = true;  // r still to be dequantised into xi
-    bool scaled = false;
-    if constexpr (WIDE && SC) scaled = hi - lo < 16 && lo >= 6 && hi <= 58;
-    if (scaled) {
-      // 64-bit coefficients whose coded planes lie in [lo, lo + 16), lo >= 6,
-      // below plane 59, decoded in 32-bit integers in units of 2^(lo - 6).  A
-      // coefficient with negabinary digits v from plane lo is
-      // ((v ^ M) - M) * 2^lo with M = NBM >> lo (M's bits above v's do not
-      // matter).  In these units each pass of the inverse lifting turns
-      // multiples of 2^a into multiples of 2^(a - 2), so from 2^6 every shift
-      // divides an even number exactly; and |value| < 2^(hi - lo + 6.42) *
-      // 2.75^3 < 2^26 (2.75: the largest row sum of the inverse lifting's
-      // coefficients), while the unscaled value stays below 2^(hi + 4.8) <= 2^63.
-      // Neither form wraps, so the result is the 64-bit decoding's exactly.
-      const int pl = lo + (lane & 15);
-      const uint64_t WA = fetch(mA, sA, pA, pl), WB = fetch(mB, sB, pB, pl);
-      const uint32_t sel = h ? 0x7632u : 0x5410u;
-      const uint32_t M = (uint32_t)(F::NBM >> min(lo, 63));  // lo = 64: no digit at all
-      int32_t* b32 = reinterpret_cast<int32_t*>(buf);
-#pragma unroll
-      for (int t2 = 0; t2 < 2; ++t2) {
-        const uint32_t row = __byte_perm((uint32_t)(WA >> (32 * t2)), (uint32_t)(WB >> (32 * t2)), sel);
-        const uint32_t w = transpose32(row, lane, tkeep);
-        b32[ir[2 * t2]] = (int32_t)((((w & 0xffffu) ^ M) - M) << 6);
-        b32[ir[2 * t2 + 1]] = (int32_t)((((w >> 16) ^ M) - M) << 6);
-      }
-      __syncwarp();
-      {
-        int32_t a = b32[iz[0]], bq = b32[iz[1]], c = b32[iz[2]], d = b32[iz[3]];
-        lift_inv(a, bq, c, d);
-        b32[iz[0]] = a; b32[iz[1]] = bq; b32[iz[2]] = c; b32[iz[3]] = d;
-      }
-      __syncwarp();
-      {
-        int32_t a = b32[iy[0]], bq = b32[iy[1]], c = b32[iy[2]], d = b32[iy[3]];
-        lift_inv(a, bq, c, d);
-        b32[iy[0]] = a; b32[iy[1]] = bq; b32[iy[2]] = c; b32[iy[3]] = d;
-      }
-      __syncwarp();
-      int32_t q[4];
-#pragma unroll
-      for (int m = 0; m < 4; ++m) q[m] = b32[ix[m]];
-      __syncwarp();
-      lift_inv(q[0], q[1], q[2], q[3]);
-      if (my.s >= -960 && my.s <= 1022) {  // R13 without rounding (scaled_i32_to_f64)
-        if constexpr (WIDE) {
-          if (my.mode == kModeCoded) {
-            const uint32_t eb = (uint32_t)(1053 + (lo - 6) - my.s) << 20;
-#pragma unroll
-            for (int m = 0; m < 4; ++m) xi[m] = scaled_i32_to_f64(q[m], eb);
-          }
-        }
-        conv = false;
-      } else {  // the general path below, on the unscaled coefficients
-#pragma unroll
-        for (int m = 0; m < 4; ++m) r[m] = (S)((U)(int64_t)q[m] << (lo - 6));
-      }
-    } else {
-      U u[4];
-      if ((!WIDE || !SC) && hi - lo < 16) {
-        // every coded plane of the pair lies in [lo, lo + 16): one transpose
-        // carries two coefficient groups, rows 0-15 the planes of group 2t and
-        // rows 16-31 those of group 2t + 1 (lane l fetches plane lo + (l & 15))
-        const int pl = lo + (lane & 15);
-        const uint64_t WA = fetch(mA, sA, pA, pl), WB = fetch(mB, sB, pB, pl);
-        const uint32_t sel = h ? 0x7632u : 0x5410u;  // 16-bit group 2 t2 + h of both words
-#pragma unroll
-        for (int t2 = 0; t2 < 2; ++t2) {
-          const uint32_t row = __byte_perm((uint32_t)(WA >> (32 * t2)), (uint32_t)(WB >> (32 * t2)), sel);
-          const uint32_t w = transpose32(row, lane, tkeep);
-          u[2 * t2] = (U)((U)(w & 0xffffu) << lo);
-          u[2 * t2 + 1] = (U)((U)(w >> 16) << lo);
-        }
-      } else {
-        // lane l fetches plane base + l (and base + 32 + l for 64-bit
-        // coefficients when the coded planes of the pair span more than 32)
-        int base = 0;
-        bool two = WIDE;
-        if constexpr (WIDE) {
-          if (hi - lo < 32) {  // one 32-plane window holds every coded plane
-            base = lo;
-            two = false;
-          }
-        }
-        const uint64_t WA0 = fetch(mA, sA, pA, base + lane), WB0 = fetch(mB, sB, pB, base + lane);
-        {
-          uint32_t tl[4];
-          tl[0] = __byte_perm((uint32_t)WA0, (uint32_t)WB0, 0x5410);
-          tl[1] = __byte_perm((uint32_t)WA0, (uint32_t)WB0, 0x7632);
-          tl[2] = __byte_perm((uint32_t)(WA0 >> 32), (uint32_t)(WB0 >> 32), 0x5410);
-          tl[3] = __byte_perm((uint32_t)(WA0 >> 32), (uint32_t)(WB0 >> 32), 0x7632);
-#pragma unroll
-          for (int j = 0; j < 4; ++j) u[j] = (U)transpose32(tl[j], lane, tkeep) << base;
-        }
-        if constexpr (WIDE) {
-          if (two) {
-            const uint64_t WA1 = fetch(mA, sA, pA, lane + 32), WB1 = fetch(mB, sB, pB, lane + 32);
-            uint32_t th[4];
-            th[0] = __byte_perm((uint32_t)WA1, (uint32_t)WB1, 0x5410);
-            th[1] = __byte_perm((uint32_t)WA1, (uint32_t)WB1, 0x7632);
-            th[2] = __byte_perm((uint32_t)(WA1 >> 32), (uint32_t)(WB1 >> 32), 0x5410);
-            th[3] = __byte_perm((uint32_t)(WA1 >> 32), (uint32_t)(WB1 >> 32), 0x7632);
-#pragma unroll
-            for (int j = 0; j < 4; ++j) u[j] |= (U)((uint64_t)transpose32(th[j], lane, tkeep) << 32);
-          }
-        }
-      }
-#pragma unroll
-      for (int j = 0; j < 4; ++j) buf[ir[j]] = nb_inv<T>(u[j]);
-      __syncwarp();
-      {
-        S a = buf[iz[0]], bq = buf[iz[1]], c = buf[iz[2]], d = buf[iz[3]];
-        lift_inv(a, bq, c, d);
-        buf[iz[0]] = a; buf[iz[1]] = bq; buf[iz[2]] = c; buf[iz[3]] = d;
-      }
-      __syncwarp();
-      {
-        S a = buf[iy[0]], bq = buf[iy[1]], c = buf[iy[2]], d = buf[iy[3]];
-        lift_inv(a, bq, c, d);
-        buf[iy[0]] = a; buf[iy[1]] = bq; buf[iy[2]] = c; buf[iy[3]] = d;
-      }
-      __syncwarp();
-#pragma unroll
-      for (int m = 0; m < 4; ++m) r[m] = buf[ix[m]];
-      __syncwarp();
-      lift_inv(r[0], r[1], r[2], r[3]);
-    }
-    if (conv && my.mode == kModeCoded) dequantize_line<T, true>(r, my.s, xi);
-  }
-  if (my.mode == kModeRaw) {
-#pragma unroll
-    for (int m = 0; m < 4; ++m)
-      xi[m] = F::val((U)peek64(cd->payload, cd->nwords, my.off + 2 + (uint64_t)F::P * (4 * t + m)));
-  }
-}
-
-// Parse task L decodes the block that the round's index pass placed in
-// meta[L] (component base + comp, its first bit and length) into slot L and
-// replaces meta[L] by the block's header.  An entry of length 0 (a brick past
-// the box, or a component the brick takes from the cache) is final already.
+// One warp task: each lane parses component comp's block of box brick g into
+// the round's plane words and its header.  A brick past the box, or a component
+// the brick takes from the cache, has nothing to parse.  Every lane of the warp
+// calls it.
 template <typename T>
-__device__ __forceinline__ void parse_task(const BoxJob& J, unsigned int* err, int base, int L, uint64_t* slots,
-                                           BlockMeta* meta, uint64_t* spill, const uint16_t* lut) {
+__device__ __forceinline__ void parse_task(const BoxJob& J, unsigned int* err, int64_t g, int comp, BlockMeta* meta,
+                                           uint8_t* how, uint64_t* pool, uint64_t* spill, int* used,
+                                           const uint32_t* lut) {
   using F = Fmt<T>;
   constexpr int N = 64;
   constexpr int Q = F::P - 2 - Geo<3>::G;
   constexpr int C = Geo<3>::C;
   constexpr int HDR = 2 + 3 + F::EBITS;
   constexpr int EMAXT = (1 << (F::EXPW - 1));  // frexp exponent of the largest finite T
-  constexpr int SP = spill_per_block<T>();
-  const BlockMeta in = meta[L];
-  if (in.len == 0) return;
-  const CompDesc& cd = J.comp[base + in.comp];
+  const int lane = threadIdx.x & 31;
+  int mode = kModeZero, s = 0, p = 0, top = -1;
+  uint64_t off = 0;
+  uint32_t pos = 0, end = 0;
+  bool ok = true;
   BlockBits br;  // positions from the start of the block's first word
-  br.init(cd.payload, cd.nwords, in.off);
-  const uint32_t start = (uint32_t)(in.off & 63u), end = start + in.len;
-  const uint64_t v = br.peek(start);
-  int mode = (int)(v & 3ull), s = 0, p = 0, top = -1;
-  bool ok;
-  if (mode == kModeZero) {
-    ok = in.len == 2;
-  } else if (mode == kModeRaw) {
-    ok = in.len == 2 + N * F::P;
-  } else if (mode == kModeCoded) {
-    const int esc = (int)((v >> 2) & 7ull);
-    const int emax = (int)((v >> 5) & ((1ull << F::EBITS) - 1)) - F::EBIAS;
-    ok = emax >= F::EMIN && emax <= EMAXT;
-    if (ok) {
-      s = Q - emax;
-      p = min(max(cd.L + s - C - esc, 0), F::P);
-      ok = parse_planes<T>(br, start + HDR, end, p, slots + L * Slots<T>::n, spill + L * SP, top, lut);
+  br.init(nullptr, 0, 0);
+  int64_t bx, by, bz;
+  if (g < J.nbox) {
+    brick_of(J, g, &bx, &by, &bz);
+    const int64_t b = bx + J.nb[0] * (by + J.nb[1] * bz);
+    if (comp >= cached_level(J, b)) {
+      const CompDesc& cd = J.comp[comp];
+      off = cd.chunk_word[b / kChunk] * 64ull + cd.brick_off[b];
+      const uint32_t len = cd.brick_len[b];
+      br.init(cd.payload, cd.nwords, off);
+      pos = (uint32_t)(off & 63u);
+      end = pos + len;
+      const uint64_t v = br.peek(pos);
+      mode = (int)(v & 3ull);
+      if (mode == kModeCoded) {
+        const int esc = (int)((v >> 2) & 7ull);
+        const int emax = (int)((v >> 5) & ((1ull << F::EBITS) - 1)) - F::EBIAS;
+        ok = emax >= F::EMIN && emax <= EMAXT;
+        if (ok) {
+          s = Q - emax;
+          p = min(max(cd.L + s - C - esc, 0), F::P);
+          pos += HDR;
+          // planes above the first significant coefficient are single 0 test bits
+          top = F::P - 1;
+          while (top >= p) {
+            const uint64_t t = br.peek(pos);
+            const int z = t ? __ffsll((long long)t) - 1 : 64;
+            const int skip = min(z, top - p + 1);
+            pos += (uint32_t)skip;
+            top -= skip;
+            if (z < 64) break;  // the bit after the zeros is the first significant plane's test 1
+          }
+          ok = pos <= end;
+        }
+      } else if (mode == kModeZero) {
+        ok = len == 2;
+      } else {
+        ok = mode == kModeRaw && len == 2 + N * F::P;
+      }
     }
-  } else {
-    ok = false;
   }
+  // places of the lanes' plane words: a warp scan, and one atomic per task
+  const bool coded = ok && mode == kModeCoded;
+  const int nw = coded ? top - p + 1 : 0;
+  int incl = nw;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int y = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += y;
+  }
+  int at = 0;
+  if (lane == 31) at = atomicAdd(used, incl);
+  at = __shfl_sync(0xffffffffu, at, 31) + incl - nw;
+  if (coded) ok = parse_planes(br, pos, end, nw, words_at<T>(pool, spill, at, nw), lut);
   if (!ok) {
     atomicOr(err, 1u);
     mode = kModeZero;
   }
-  BlockMeta bm = in;
-  bm.mode = (int8_t)mode;
+  BlockMeta bm;
+  bm.off = off;
   bm.s = (int16_t)s;
-  bm.p = (int8_t)(mode == kModeCoded ? p : 64);  // no plane of a ZERO or RAW block is coded
+  bm.p = (int8_t)p;
   bm.top = (int8_t)top;
-  meta[L] = bm;
+  bm.mode = (uint8_t)mode;
+  bm.pad_ = 0;
+  bm.at = (uint16_t)at;
+  *meta = bm;
+  // Exactness of the two short decodings (see add_component): no value of the
+  // inverse lifting is odd where it is halved (p >= 6), and none reaches 2^31
+  // (planes up to 26) or 2^63 (up to 58) -- 2^(top + 1) * 2/3 * 2.75^3, with
+  // 2.75 the largest row sum of the inverse lifting's coefficients.  Float64
+  // blocks with higher planes (the first component's, mostly) take the decoding
+  // of 16 planes after a look at their coefficients.
+  int h = kDecodeNone;
+  if (mode == kModeCoded && nw > 0) {
+    const bool common = sizeof(T) == 8 ? s >= -960 && s <= 1022 : s >= -96 && s <= 126;
+    const bool scaled = p >= 6 && common, low = top <= (sizeof(T) == 8 ? 58 : 26);
+    h = at + nw > kPool || nw > 16 || (sizeof(T) == 8 && !scaled) ? kDecodeAny
+        : nw <= 8 && scaled && low                                ? kDecodeFloat8
+                                                                  : kDecodeInt16;
+  }
+#pragma unroll
+  for (int o = 1; o <= 4; o <<= 1) h = max(h, __shfl_xor_sync(0xffffffffu, h, o));
+  const unsigned raw = __ballot_sync(0xffffffffu, mode == kModeRaw);
+  if ((lane & 7) == 0) *how = (uint8_t)(h | ((raw >> lane) & 0xffu ? kHasRaw : 0));
 }
 
-// Parse phase of a round: task L is component base + L / ub of unit brick
-// L % ub (ub = bricks per unit).
-//  1. Index pass: every thread looks up the index of its tasks (first bit and
-//     length of the block; the loads of the whole round are in flight
-//     together) into meta[L], and counts them per length bucket.
-//  2. A counting sort of the tasks by block length, longest first (each warp
-//     scans the bucket counts itself), into order[].
-//  3. Warp-granular work stealing over order[]: each warp takes the next 32
-//     tasks until none is left.  The 32 blocks a warp parses side by side are
-//     then of alike length, so lanes wait little for one another, and the
-//     short blocks at the end fill the gaps before the barrier.
-// Every thread of the CTA calls it; hist[] is zero on entry and on return.
+// A lane's share of a brick: z-plane q, values x + 4 y.  Which of them lie in
+// the box, and where they are in the output and in the field.
+struct BrickLane {
+  bool have;
+  int x0, x1, y0, y1;  // values [x0, x1) of rows [y0, y1); y1 = 0 where the plane is outside
+  int64_t b, out, field;
+};
+
+__device__ __forceinline__ BrickLane brick_lane(const BoxJob& J, int64_t g, int q) {
+  BrickLane L;
+  L.have = g < J.nbox;
+  int64_t bx = 0, by = 0, bz = 0;
+  if (L.have) brick_of(J, g, &bx, &by, &bz);
+  L.b = bx + J.nb[0] * (by + J.nb[1] * bz);
+  const int64_t gy = 4 * by, gz = 4 * bz + q;
+  L.x0 = (int)max(J.lo[0] - 4 * bx, (int64_t)0);
+  L.x1 = (int)min(J.hi[0] - 4 * bx, (int64_t)4);
+  L.y0 = (int)max(J.lo[1] - gy, (int64_t)0);
+  L.y1 = L.have && gz >= J.lo[2] && gz < J.hi[2] ? (int)min(J.hi[1] - gy, (int64_t)4) : 0;
+  const int64_t ext0 = J.hi[0] - J.lo[0], ext1 = J.hi[1] - J.lo[1];
+  L.out = ((gz - J.lo[2]) * ext1 + (gy - J.lo[1])) * ext0 + 4 * bx - J.lo[0];
+  L.field = (gz * J.dims[1] + gy) * J.dims[0] + 4 * bx;
+  return L;
+}
+
+// x~ of the lane's values at the start of a job: 0, the caller's partial sum
+// x~_k0 (refinement), or the cache.  -0 is read as +0, which is what adding a
+// component makes of it even where the component is zero.  Returns whether the
+// sum starts from 0.
 template <typename T>
-__device__ __forceinline__ void parse_round(const BoxJob& J, unsigned int* err, int64_t unit0, int ub, int base,
-                                            int nc, int* next, uint64_t* slots, BlockMeta* meta, uint64_t* spill,
-                                            const uint16_t* lut, uint16_t* order, int* hist) {
-  constexpr unsigned FULL = 0xffffffffu;
-  const int lane = threadIdx.x & 31;
-  const int ntask = nc * ub;
-  constexpr int PER = kTasks / kRThreads;  // tasks per thread in the index pass
-  int key[PER], rank[PER];
+__device__ __forceinline__ bool start_sum(const BoxJob& J, int write, const BrickLane& L, T* xt) {
+  using F = Fmt<T>;
 #pragma unroll
-  for (int q = 0; q < PER; ++q) {
-    const int L = threadIdx.x + q * kRThreads;
-    key[q] = -1;
-    if (L >= ntask) continue;
-    const int jj = (int)div_by((uint32_t)L, J.dv_ub);  // ub = 16 * umult
-    const int64_t g = unit0 + (L - jj * ub);
-    BlockMeta bm;
-    bm.off = 0;
-    bm.s = 0;
-    bm.len = 0;
-    bm.p = 64;
-    bm.top = -1;
-    bm.mode = kModeZero;
-    bm.comp = (uint8_t)jj;
-    if (g < J.nbox) {
-      int64_t bx, by, bz;
-      if (J.nbox < (1ll << 32)) {  // 32-bit division by the box's invariant extents
-        const uint32_t g32 = (uint32_t)g;
-        const uint32_t r = div_by(g32, J.dv_bn0);
-        const uint32_t z = div_by(r, J.dv_bn1);
-        bx = J.bl[0] + (int64_t)(g32 - r * (uint32_t)J.bn[0]);
-        by = J.bl[1] + (int64_t)(r - z * (uint32_t)J.bn[1]);
-        bz = J.bl[2] + (int64_t)z;
-      } else {
-        bx = J.bl[0] + g % J.bn[0];
-        const int64_t r = g / J.bn[0];
-        by = J.bl[1] + r % J.bn[1];
-        bz = J.bl[2] + r / J.bn[1];
+  for (int v = 0; v < 16; ++v) xt[v] = T(0);
+  const int lv = L.have ? cached_level(J, L.b) : 0;
+  if (lv == 0 && !(write && J.k0 > 0)) return true;
+  const T* src = lv > 0 ? reinterpret_cast<const T*>(J.cache) + L.field : reinterpret_cast<const T*>(J.out) + L.out;
+  const int64_t row = lv > 0 ? J.dims[0] : J.hi[0] - J.lo[0];
+#pragma unroll
+  for (int y = 0; y < 4; ++y) {
+    if (y < L.y0 || y >= L.y1) continue;
+    const T* line = src + y * row;
+    if (L.x0 == 0 && L.x1 == 4) {
+      load_line<T>(line, 4, xt + 4 * y);
+    } else {
+#pragma unroll
+      for (int x = 0; x < 4; ++x)
+        if (x >= L.x0 && x < L.x1) xt[x + 4 * y] = line[x];
+    }
+  }
+#pragma unroll
+  for (int v = 0; v < 16; ++v)
+    if (F::bits(xt[v]) == F::SIGN) xt[v] = T(0);
+  return false;
+}
+
+// The lane's values into the output: whole aligned lines with 16-byte stores.
+template <typename T>
+__device__ __forceinline__ void store_lines(const BoxJob& J, const BrickLane& L, const T* xt) {
+  T* out = reinterpret_cast<T*>(J.out) + L.out;
+  const int64_t row = J.hi[0] - J.lo[0];
+  const bool whole = L.x0 == 0 && L.x1 == 4 && (((uintptr_t)out | ((uintptr_t)row * sizeof(T))) & 15) == 0;
+#pragma unroll
+  for (int y = 0; y < 4; ++y) {
+    if (y < L.y0 || y >= L.y1) continue;
+    T* line = out + y * row;
+    if (whole) {
+      constexpr bool all[4] = {true, true, true, true};
+      store_line<T>(line, xt + 4 * y, all);
+    } else {
+#pragma unroll
+      for (int x = 0; x < 4; ++x)
+        if (x >= L.x0 && x < L.x1) line[x] = xt[4 * y + x];
+    }
+  }
+}
+
+// Float64 partial sums in fixed point.  As long as every partial sum of a brick
+// is a multiple of some 2^e below 2^(e + 51), no addition rounds, and the sums can
+// be kept as 64-bit integers in units of 2^e: the FP64 pipe (2 lanes per SM and
+// clock, 64 cycles for a warp's addition) then sees one operation per value
+// instead of one per component.  `lead` is the first coded component's highest
+// plane, as an exponent (each component is below 2^(lead + 5)), depth = 46 -
+// ceil(log2 k) the bits below it, e = lead - depth.  A component that does not
+// fit (deeper, larger, RAW) ends it: the sums so far become doubles.  256 x 384 x
+// 384, k = 8: 1070 -> 888 us.
+struct FixedSum {
+  bool on;    // (the same in the whole warp)
+  int lead;   // kNoLead before the brick's first coded component
+  int depth;
+};
+constexpr int kNoLead = -(1 << 20);
+
+// units of 2^ue (|v| below 2^51, the result normal or 0) as a double
+__device__ __forceinline__ double fixed_to_f64(double v, int ue) {
+  const double m = __dsub_rn(__longlong_as_double(__double_as_longlong(v) + 0x4338000000000000ll), 6755399441055744.0);
+  const int hi = __double2hiint(m);
+  return __hiloint2double(hi ? hi + ue * (1 << 20) : 0, __double2loint(m));
+}
+
+__device__ __forceinline__ void end_fixed(FixedSum& fx, double* xt) {
+  const int ue = fx.lead == kNoLead ? 0 : fx.lead - fx.depth;
+#pragma unroll
+  for (int k = 0; k < 16; ++k) xt[k] = fixed_to_f64(xt[k], ue);
+  fx.on = false;
+}
+
+// i * 2^sh into a fixed-point sum: sh is at most 33, |i| below 2^27 (in the
+// decoding of 16 planes) and |i| * 2^3 below 2^31.
+__device__ __forceinline__ double fixed_add(double sum, int32_t i, int sh) {
+  const int32_t hi = i * (1 << max(sh - 30, 0));
+  return __longlong_as_double(__double_as_longlong(sum) + (int64_t)hi * (int64_t)(1 << min(sh, 30)));
+}
+
+// Adds one component into the z-planes of a warp's 8 bricks.  how: kDecode* and
+// kHasRaw of the 8; m: header of the lane's brick; pool, spill: the round's plane
+// words; zw, yw: the lane's lines of the exchange; place: the coded places of its
+// coefficients.
+template <typename T>
+__device__ __forceinline__ void add_component(int how, const BlockMeta& m, const CompDesc* cd, uint64_t* pool,
+                                              uint64_t* spill, uint4* area, uint4* zw, uint4* yw,
+                                              const uint32_t* place, int lane, T* xt, FixedSum& fx) {
+  using F = Fmt<T>;
+  using U = typename F::U;
+  using S = typename F::S;
+  constexpr bool WIDE = F::P == 64;
+  constexpr unsigned FULL = 0xffffffffu;
+  const int bq = lane >> 2, q = lane & 3;
+  const bool coded = m.mode == kModeCoded;
+  const int p = m.p, top = m.top, s = coded ? (int)m.s : 0;
+  const int nw = coded ? top - p + 1 : 0;  // planes with digits
+  const uint32_t areas = smem_addr(area);
+  bool any = (how & 3) == kDecodeAny;
+  if constexpr (WIDE) {
+    if (fx.on) {
+      bool fits = !any && !(how & kHasRaw);
+      if (nw > 0) {
+        if (fx.lead == kNoLead) {
+          fx.lead = top - s;
+          fits = fits && fx.lead >= -900 && fx.lead <= 900;
+        }
+        const int H = (how & 3) == kDecodeFloat8 ? 8 : 16;  // the decoding's units: 2^(base - 6 - s)
+        fits = fits && top - s <= fx.lead && max(top, H - 1) - (H - 1) - 6 - s >= fx.lead - fx.depth;
       }
-      const int64_t b = bx + J.nb[0] * (by + J.nb[1] * bz);
-      if (base + jj >= cached_level(J, b)) {
-        const CompDesc& cd = J.comp[base + jj];
-        bm.off = cd.chunk_word[b / kChunk] * 64ull + cd.brick_off[b];
-        bm.len = cd.brick_len[b];
+      if (!__all_sync(FULL, fits)) end_fixed(fx, xt);
+    }
+  }
+  // The short decodings take the planes top .. top - H + 1 of the lane's 16
+  // coefficients, transposed to digits: bit i of a digit is plane base + i.  What
+  // lies outside [p, top] (other blocks' words) is masked off.
+  if ((how & 3) == kDecodeFloat8) {
+    const int base = max(top, 7) - 7;
+    const uint32_t keep = nw > 0 ? ((1u << nw) - 1u) << (p - base) : 0u;
+    const uint16_t* pc = reinterpret_cast<const uint16_t*>(pool + (nw > 0 ? m.at + top - base : 7)) + q;  // plane base
+    uint32_t a[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) a[j] = (uint32_t)pc[-4 * j] | ((uint32_t)pc[-4 * (j + 4)] << 16);
+    untranspose8(a);
+    area[5 * bq + q] = make_uint4(a[0], a[1], a[2], a[3]);
+    __syncwarp();
+    // R9: with M = NBM >> base (8 bits), digits d stand for (d ^ M) - M in units of
+    // 2^base.  With 2^23's bit pattern in M, the difference of two floats.
+    const uint32_t M = (uint32_t)(F::NBM >> base) & 0xffu | 0x4B000000u;
+    const uint32_t get = areas + 80u * bq;
+    float r[16];
+#pragma unroll
+    for (int k = 0; k < 16; ++k) {
+      uint32_t d;  // the address: get + byte k & 3 of place
+      asm volatile("ld.shared.u8 %0, [%1];" : "=r"(d) : "r"(__dp4a(place[k >> 2], 1u << (8 * (k & 3)), get)) : "memory");
+      r[k] = __fsub_rn(__uint_as_float((d & keep) ^ M), __uint_as_float(M));
+    }
+    __syncwarp();
+    // values below 2^12.8 units and multiples of 2^-6: 19 bits
+    lift_inv_bricks<float>(r, zw, yw, LineSet::kVectors);
+    if constexpr (WIDE) {
+      if (fx.on) {  // r in units of 2^-6: the float sum with 1.5 * 2^17 holds it in its low bits
+        const int sh = nw > 0 ? (base - 6 - s) - (fx.lead - fx.depth) : 0;
+#pragma unroll
+        for (int k = 0; k < 16; ++k)
+          xt[k] = fixed_add(xt[k], __float_as_int(__fadd_rn(r[k], 196608.0f)) - 0x48400000, sh);
+      } else {
+        const uint32_t adj = (uint32_t)(896 + base - s) << 20;
+#pragma unroll
+        for (int k = 0; k < 16; ++k) xt[k] = F::add(xt[k], scaled_f32_to_f64(r[k], adj));
+      }
+    } else {
+      const float sc = __uint_as_float((uint32_t)(127 + base - s) << 23);  // x_j = r * sc exactly
+#pragma unroll
+      for (int k = 0; k < 16; ++k) xt[k] = __fmaf_rn(r[k], sc, xt[k]);
+    }
+  } else if ((how & 3) == kDecodeInt16) {
+    const int base = max(top, 15) - 15;
+    const uint32_t keep = nw > 0 ? ((1u << nw) - 1u) << (p - base) : 0u;
+    const uint16_t* pc = reinterpret_cast<const uint16_t*>(pool + (nw > 0 ? m.at + top - base : 15)) + q;
+    uint32_t a[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) a[j] = (uint32_t)pc[-4 * j] | ((uint32_t)pc[-4 * (j + 8)] << 16);
+    untranspose16(a);
+    area[9 * bq + 2 * q] = make_uint4(a[0], a[4], a[1], a[5]);
+    area[9 * bq + 2 * q + 1] = make_uint4(a[2], a[6], a[3], a[7]);
+    __syncwarp();
+    const uint32_t M = (uint32_t)(F::NBM >> base);
+    const uint32_t unit = WIDE ? 64u : 1u << base;  // float64: units of 2^(base - 6), values below 2^27
+    const uint32_t get = areas + 144u * bq;
+    int32_t r[16];
+#pragma unroll
+    for (int k = 0; k < 16; ++k) {
+      uint16_t d;
+      asm volatile("ld.shared.u16 %0, [%1];" : "=h"(d) : "r"(__dp4a(place[k >> 2], 2u << (8 * (k & 3)), get)) : "memory");
+      r[k] = (int32_t)((((uint32_t)d & keep) ^ M) * unit - M * unit);
+    }
+    if constexpr (WIDE) {
+      // planes above 58: no value of the inverse lifting is larger than the sum of
+      // the brick's 64 coefficients' magnitudes (its matrix has no entry above 1)
+      if (__any_sync(FULL, nw > 0 && top > 58)) {
+        uint32_t sum = 0;
+#pragma unroll
+        for (int k = 0; k < 16; ++k) sum += (uint32_t)abs(r[k]);  // each below 2^22
+        sum += __shfl_xor_sync(FULL, sum, 1);
+        sum += __shfl_xor_sync(FULL, sum, 2);
+        any = __any_sync(FULL, nw > 0 && top > 58 && sum >= 1u << (69 - base));
       }
     }
-    meta[L] = bm;
-    key[q] = kLenBuckets - 1 - min((int)(bm.len >> 4), kLenBuckets - 1);  // longest first
-    rank[q] = atomicAdd(hist + key[q], 1);
-  }
-  __syncthreads();
-  // bucket bases: an exclusive scan of the 64 counts, two per lane, in every warp
-  const int h0 = hist[2 * lane], h1 = hist[2 * lane + 1];
-  int incl = h0 + h1;
+    __syncwarp();
+    if (!any) lift_inv_bricks<int32_t>(r, zw, yw, LineSet::kVectors);
+    if constexpr (WIDE) {
+      if (any) {
+        if (fx.on) end_fixed(fx, xt);
+      } else if (fx.on) {
+        const int sh = nw > 0 ? (base - 6 - s) - (fx.lead - fx.depth) : 0;
 #pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const int y = __shfl_up_sync(FULL, incl, o);
-    if (lane >= o) incl += y;
-  }
-  const int b0 = incl - h0 - h1, b1 = incl - h1;
+        for (int k = 0; k < 16; ++k) xt[k] = fixed_add(xt[k], r[k], sh);
+      } else {
+        const uint32_t eb = (uint32_t)(1053 + (base - 6) - s) << 20;
 #pragma unroll
-  for (int q = 0; q < PER; ++q) {
-    const int k = key[q] < 0 ? 0 : key[q];
-    const int e0 = __shfl_sync(FULL, b0, k >> 1), e1 = __shfl_sync(FULL, b1, k >> 1);
-    if (key[q] >= 0) order[((k & 1) ? e1 : e0) + rank[q]] = (uint16_t)(threadIdx.x + q * kRThreads);
+        for (int k = 0; k < 16; ++k) xt[k] = F::add(xt[k], scaled_i32_to_f64(r[k], eb));
+      }
+    } else if (__all_sync(FULL, s >= -96 && s <= 126)) {
+      // one rounding to float; the product by 2^-s is exact (normal, and below
+      // 2^127 for s >= -96), so one fused add is x~ + x_j
+      const float sc = __uint_as_float((uint32_t)(127 - s) << 23);
+#pragma unroll
+      for (int k = 0; k < 16; ++k) xt[k] = __fmaf_rn(__int2float_rn(r[k]), sc, xt[k]);
+    } else {
+#pragma unroll
+      for (int k = 0; k < 16; ++k) xt[k] = F::add(xt[k], F::val(dequantize_any<T>(r[k], s)));
+    }
   }
-  __syncthreads();
-  if (threadIdx.x < kLenBuckets) hist[threadIdx.x] = 0;  // read by every warp before the barrier
-  for (;;) {
-    int t0 = 0;
-    if (lane == 0) t0 = atomicAdd(next, 32);
-    t0 = __shfl_sync(FULL, t0, 0);
-    if (t0 >= ntask) break;
-    if (t0 + lane < ntask) parse_task<T>(J, err, base, order[t0 + lane], slots, meta, spill, lut);
+  if (any) {
+    // any planes, 16 at a time from plane 0, each 16 digits a half-word of the
+    // coefficients in coded order
+    const uint32_t stride = 64u * sizeof(T) + 16u;
+    unsigned char* dig = reinterpret_cast<unsigned char*>(area) + stride * bq;
+    const uint64_t* words = words_at<T>(pool, spill, m.at, nw);
+#pragma unroll 1
+    for (int h = 0; h < F::P / 16; ++h) {
+      auto plane = [&](int pl) {
+        if (nw <= 0 || pl < p || pl > top) return 0u;
+        return (uint32_t)reinterpret_cast<const uint16_t*>(words + (top - pl))[q];
+      };
+      uint32_t a[8];
+#pragma unroll
+      for (int j = 0; j < 8; ++j) a[j] = plane(16 * h + j) | (plane(16 * h + j + 8) << 16);
+      untranspose16(a);
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {  // ranks i and i + 8 of the lane's 16, at their places
+        uint16_t* e = reinterpret_cast<uint16_t*>(dig + (16 * q + 4 * (i & 3) + 2 * (i >> 2)) * sizeof(T)) + h;
+        e[0] = (uint16_t)a[i];
+        e[sizeof(T) / 2] = (uint16_t)(a[i] >> 16);
+      }
+    }
+    __syncwarp();
+    S r[16];
+#pragma unroll
+    for (int k = 0; k < 16; ++k)
+      r[k] = nb_inv<T>(*reinterpret_cast<const U*>(dig + ((place[k >> 2] >> (8 * (k & 3))) & 0xffu) * sizeof(T)));
+    __syncwarp();
+    lift_inv_bricks<S>(r, zw, yw, LineSet::kVectors);
+    const bool common = __all_sync(FULL, WIDE ? s >= -960 && s <= 1022 : s >= -127 && s <= 126);
+#pragma unroll
+    for (int y = 0; y < 4; ++y) {
+      T xi[4];
+      if (common) {
+        dequantize_line<T, true>(r + 4 * y, s, xi);
+      } else {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) xi[k] = F::val(dequantize_any<T>(r[4 * y + k], s));
+      }
+#pragma unroll
+      for (int k = 0; k < 4; ++k) xt[4 * y + k] = F::add(xt[4 * y + k], xi[k]);
+    }
+  }
+  if ((how & kHasRaw) && m.mode == kModeRaw) {
+#pragma unroll
+    for (int k = 0; k < 16; ++k)
+      xt[k] = F::add(xt[k], F::val((U)peek64(cd->payload, cd->nwords, m.off + 2 + (uint64_t)F::P * (16 * q + k))));
   }
 }
 
-template <typename T, bool SC>
-__global__ void __launch_bounds__(kRThreads, 3) k_retrieve3(const RetrieveParams R) {
-  using F = Fmt<T>;
-  using S = typename F::S;
-  constexpr int SP = spill_per_block<T>();
+// CTAs that share an SM, as their shared memory allows: 31 KB for float32, 40 KB
+// for float64 (6 and 4 measured 2 and 7 % slower).
+template <typename T>
+constexpr int kRetrieveCtas3 = sizeof(T) == 4 ? 7 : 5;
 
+template <typename T>
+__global__ void __launch_bounds__(kRThreads, kRetrieveCtas3<T>) k_retrieve3(const RetrieveParams R) {
   extern __shared__ __align__(16) unsigned char smem[];
-  uint64_t* slots = reinterpret_cast<uint64_t*>(smem);                // [kTasks][Slots<T>::n]
-  BlockMeta* meta = reinterpret_cast<BlockMeta*>(slots + kTasks * Slots<T>::n);  // [kTasks]
-  S* bufs = reinterpret_cast<S*>(meta + kTasks);                           // [kRWarps][128]
-  uint16_t* lut = reinterpret_cast<uint16_t*>(bufs + kRWarps * 128);       // [kTokLut]
-  uint16_t* order = lut + kTokLut;                                         // [kTasks]
-  int* hist = reinterpret_cast<int*>(order + kTasks);                      // [kLenBuckets]
-  if (threadIdx.x < kLenBuckets) hist[threadIdx.x] = 0;
+  uint64_t* pool = reinterpret_cast<uint64_t*>(smem) + kPoolPad;                // [kPool]
+  BlockMeta* meta = reinterpret_cast<BlockMeta*>(pool + kPool + kPoolPad);     // [kBlocks]
+  uint4* areas = reinterpret_cast<uint4*>(meta + kBlocks);                     // [kRWarps]
+  uint32_t* lut = reinterpret_cast<uint32_t*>(areas + kRWarps * AreaR<T>::kVectors);
+  uint8_t* how = reinterpret_cast<uint8_t*>(lut + kTokLut);                    // [kBlocks / 8]
   load_tokens<kRThreads>(lut);  // read after the loop's first barrier
-  __shared__ int s_next;  // next parse task of the round
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, h = lane >> 4, t = lane & 15;
-  S* buf = bufs + warp * 128;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, bq = lane >> 2, q = lane & 3;
+  uint4* area = areas + warp * AreaR<T>::kVectors;
+  uint4* zw = area + LineSet::at(bq, 0, q);  // + 2 y: line (y, z = q)
+  uint4* yw = area + LineSet::at(bq, q, 0);  // + 10 z: line (y = q, z)
   uint64_t* spill = R.spill + (size_t)blockIdx.x * spill_words_per_cta<T>();
-
-  const int xx = t & 3, yq = t >> 2, ly = t & 3, lz = t >> 2;
-  int ix[4], iy[4], iz[4], ir[4];
+  uint32_t place[4];  // coded places of the lane's coefficients x + 4 z (y = q)
 #pragma unroll
-  for (int m = 0; m < 4; ++m) {
-    ix[m] = sidx<T>(m, ly, lz, h);
-    iy[m] = sidx<T>(xx, m, yq, h);
-    iz[m] = sidx<T>(xx, yq, m, h);
-    const int pos = kPerm3r.pos[t + 16 * m];
-    ir[m] = sidx<T>(pos & 3, (pos >> 2) & 3, pos >> 4, h);
-  }
-  uint32_t tkeep[5];
-  transpose_masks(lane, tkeep);
+  for (int z = 0; z < 4; ++z) place[z] = coded_places(kRank3r.pos, q, z);
+
   __shared__ BoxJob sJ;
+  __shared__ int s_task, s_used;  // the round's next warp task, and its plane words so far
   const BoxJob& J = sJ;
   constexpr int JW = (int)(sizeof(BoxJob) / 8);
   static_assert(sizeof(BoxJob) % 8 == 0 && JW <= kRThreads, "job copy");
-
+  if (tid == 0) s_task = s_used = 0;
+  int64_t job_end = 0;  // the units of the job in sJ end here
   for (int64_t unit = blockIdx.x; unit < R.nunits; unit += gridDim.x) {
-    __syncthreads();  // the previous unit is done with sJ
-    if (!R.jobs) {
-      if (threadIdx.x == 0) sJ = R.job0;
-    } else if (threadIdx.x < JW) {  // the job whose units contain this one
-      int lo = 0, hi = R.njobs - 1;
-      while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (R.jobs[mid].unit_begin <= unit)
-          lo = mid;
-        else
-          hi = mid - 1;
+    if (unit >= job_end) {  // the job whose units contain this one
+      __syncthreads();      // the previous unit is done with sJ
+      if (!R.jobs) {
+        if (tid == 0) sJ = R.job0;
+        job_end = R.nunits;
+      } else {
+        int lo = 0, hi = R.njobs - 1;
+        while (lo < hi) {
+          const int mid = (lo + hi + 1) >> 1;
+          if (R.jobs[mid].unit_begin <= unit)
+            lo = mid;
+          else
+            hi = mid - 1;
+        }
+        if (tid < JW) reinterpret_cast<uint64_t*>(&sJ)[tid] = reinterpret_cast<const uint64_t*>(R.jobs + lo)[tid];
+        job_end = lo + 1 < R.njobs ? R.jobs[lo + 1].unit_begin : R.nunits;
       }
-      reinterpret_cast<uint64_t*>(&sJ)[threadIdx.x] = reinterpret_cast<const uint64_t*>(R.jobs + lo)[threadIdx.x];
-    }
-    if (threadIdx.x == kRThreads - 1) s_next = 0;
-    __syncthreads();
-    T* out = reinterpret_cast<T*>(J.out);
-    const int umult = J.umult;
-    const int ub = 16 * umult;  // bricks per unit: umult brick pairs per warp
-    const int64_t unit0 = (unit - J.unit_begin) * ub;
-    if (J.k - J.k0 <= kRound) {
-      // one round: every warp parses, then each warp rebuilds its umult
-      // brick pairs and writes them out
-      const int nc = J.k - J.k0;
-      parse_round<T>(J, R.err, unit0, ub, J.k0, nc, &s_next, slots, meta, spill, lut, order, hist);
       __syncthreads();
-      for (int q = 0; q < umult; ++q) {
-        const int uA = 2 * (kRWarps * q + warp);  // unit-local index of the pair's first brick
-        const BrickLane BL = brick_lane<sizeof(T) == 8>(J, unit0 + uA + h, t);
-        T xt[4];
-        start_sum<T>(J, R.write, BL, xt);
-        for (int jj = 0; jj < nc; ++jj) {  // Algorithm 2, components in ascending order
-          const int L = jj * ub + uA;
-          const BlockMeta mA = meta[L], mB = meta[L + 1];
-          T xi[4];
-          rebuild_pair<T, SC>(mA, mB, slots + L * Slots<T>::n, slots + (L + 1) * Slots<T>::n, spill + L * SP, spill + (L + 1) * SP,
-                          &J.comp[J.k0 + jj], buf, ix, iy, iz, ir, tkeep, lane, h, t, xi);
-#pragma unroll
-          for (int m = 0; m < 4; ++m) xt[m] = F::add(xt[m], xi[m]);  // x~ += x_j
-        }
-        if (R.write) {
-          store_line<T>(out + BL.orow, xt, BL.vm);
-        }
+    }
+    const int ub = J.unit_bricks, sets = ub / 32;  // bricks of a unit; sets of 32
+    const int64_t unit0 = (unit - J.unit_begin) * ub;
+    T xt[16];
+    BrickLane BL;
+    FixedSum fx;
+    for (int c0 = J.k0; c0 < J.k; c0 += J.round) {
+      const int nc = min(J.round, J.k - c0), ntask = nc * sets;
+      for (;;) {  // the warps take tasks, the first component's (mostly the longest) first
+        int t = 0;
+        if (lane == 0) t = atomicAdd(&s_task, 1);
+        t = __shfl_sync(0xffffffffu, t, 0);
+        if (t >= ntask) break;
+        const int c = t / sets, u = 32 * (t - c * sets) + lane;
+        const int blk = c * ub + u;
+        parse_task<T>(J, R.err, unit0 + u, c0 + c, meta + blk, how + blk / 8, pool, spill, &s_used, lut);
       }
-    } else {
-      // several rounds (umult = 2, units of 32 bricks): x~ of the warp's 4
-      // bricks stays in registers across rounds
-      BrickLane BL[2];
-      T xt[2][4];
-#pragma unroll
-      for (int q = 0; q < 2; ++q) {
-        BL[q] = brick_lane<sizeof(T) == 8>(J, unit0 + 4 * warp + 2 * q + h, t);
-        start_sum<T>(J, R.write, BL[q], xt[q]);
-      }
-      for (int base = J.k0; base < J.k; base += kRound) {
-        const int nc = min(kRound, J.k - base);
-        parse_round<T>(J, R.err, unit0, 32, base, nc, &s_next, slots, meta, spill, lut, order, hist);
-        __syncthreads();
-        for (int jj = 0; jj < nc; ++jj) {
-#pragma unroll
-          for (int q = 0; q < 2; ++q) {
-            const int uA = 4 * warp + 2 * q;
-            const int L = jj * 32 + uA;
-            const BlockMeta mA = meta[L], mB = meta[L + 1];
-            T xi[4];
-            rebuild_pair<T, SC>(mA, mB, slots + L * Slots<T>::n, slots + (L + 1) * Slots<T>::n, spill + L * SP,
-                            spill + (L + 1) * SP, &J.comp[base + jj], buf, ix, iy, iz, ir, tkeep, lane, h, t, xi);
-#pragma unroll
-            for (int m = 0; m < 4; ++m) xt[q][m] = F::add(xt[q][m], xi[m]);
+      __syncthreads();
+      if (tid == 0) s_task = s_used = 0;
+      if (R.write) {
+        // (more than one set: the unit's components are all in this round)
+        for (int g = 0; g < sets; ++g) {
+          const int u = 8 * (kRWarps * g + warp) + bq;
+          if (c0 == J.k0) {
+            BL = brick_lane(J, unit0 + u, q);
+            const bool zero = start_sum<T>(J, R.write, BL, xt);
+            fx.on = sizeof(T) == 8 && __all_sync(0xffffffffu, zero) && J.k > 1;
+            fx.lead = kNoLead;
+            fx.depth = 46 - (32 - __clz(J.k - 1));
+          }
+          for (int c = 0; c < nc; ++c) {  // Algorithm 2, components in ascending order
+            const int blk = c * ub + u, h = how[blk / 8];
+            if (h == kDecodeNone) continue;
+            const BlockMeta m = meta[blk];
+            add_component<T>(h, m, &J.comp[c0 + c], pool, spill, area, zw, yw, place, lane, xt, fx);
+          }
+          if (c0 + nc >= J.k) {
+            if constexpr (sizeof(T) == 8)
+              if (fx.on) end_fixed(fx, xt);
+            store_lines<T>(J, BL, xt);
           }
         }
-        __syncthreads();  // the next round's parse reuses the slots and the task counter
-        if (threadIdx.x == 0) s_next = 0;
-        __syncthreads();
       }
-      if (R.write) {
-#pragma unroll
-        for (int q = 0; q < 2; ++q)
-          store_line<T>(out + BL[q].orow, xt[q], BL[q].vm);
-      }
+      __syncthreads();  // the next blocks take the places
     }
   }
 }
@@ -690,8 +721,8 @@ static int retrieve_grid_t(int64_t nunits) {
     int dev = 0, sms = 0, ps = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaFuncSetAttribute(k_retrieve3<T, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)retrieve_smem3<T>());
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ps, k_retrieve3<T, false>, kRThreads, retrieve_smem3<T>()) !=
+    cudaFuncSetAttribute(k_retrieve3<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)retrieve_smem3<T>());
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ps, k_retrieve3<T>, kRThreads, retrieve_smem3<T>()) !=
         cudaSuccess) {
       cudaGetLastError();
       ps = 1;
@@ -701,20 +732,18 @@ static int retrieve_grid_t(int64_t nunits) {
   return (int)(nunits < g ? (nunits > 0 ? nunits : 1) : g);
 }
 
-// Brick pairs per warp in a unit (a unit is 16 * umult bricks): as many as
-// keep one round's parse tasks (bricks x components) within kTasks, two per
-// thread, so that warps can steal work -- but no more than leave every CTA
-// that fits on the GPU two units of the launch's bricks, and no more than the
-// job fills.  A 64^3 box at k = 4 (4096 bricks) in units of 128 ran on 32 of
-// 456 CTAs: 43.6 us, in units of 16 26 us; four reconstructions of a 64^3
-// field took 240 us, now 90 us.  (One, two and four units per CTA measured
-// alike.)  Several rounds use 2 pairs per warp.
-int retrieve_unit_mult(int dtype, int ncomp, int64_t nbox, int64_t bricks) {
-  if (ncomp <= 0 || ncomp > kRound) return 2;
+// How a job of ncomp components is decoded in a launch of `bricks` bricks: in
+// rounds of equal size of at most kRoundTasks components, units of so many
+// bricks that a round has up to kRoundTasks warp tasks (4 where there is one
+// component: its first planes are many) -- unless the units would then not fill
+// the GPU.
+void retrieve_split(int dtype, int ncomp, int64_t bricks, int* round, int* unit_bricks) {
+  const int rounds = std::max((ncomp + kRoundTasks - 1) / kRoundTasks, 1);
+  *round = std::max((ncomp + rounds - 1) / rounds, 1);
+  int sets = *round == 1 ? 4 : std::max(kRoundTasks / *round, 1);
   const int64_t fit = dtype == 1 ? retrieve_grid_t<float>(INT64_MAX) : retrieve_grid_t<double>(INT64_MAX);
-  const int64_t most = std::max((kTasks / 16) / ncomp, 1);
-  const int64_t share = bricks / (16 * fit * 2);
-  return (int)std::max<int64_t>(1, std::min(std::min(most, share), (nbox + 15) / 16));
+  while (sets > 1 && bricks < fit * 32 * sets) --sets;
+  *unit_bricks = 32 * (rounds > 1 ? 1 : sets);
 }
 
 int retrieve_grid(int dtype, int ndims, int64_t nunits) {
@@ -727,31 +756,13 @@ size_t retrieve_spill_words(int dtype, int ndims, int grid) {
   return (dtype == 1 ? spill_words_per_cta<float>() : spill_words_per_cta<double>()) * (size_t)grid;
 }
 
-// Float64 retrieval decoding at least this many components per brick takes
-// the kernel with the 32-bit decoding of narrow pairs (SC): measured 7.5 %
-// faster over k = 1..8 of a 512^3 field with 8 components (11 % at k = 8), but
-// 8 % slower at k = 1 and 1 % slower at k = 2, where the parse, whose
-// registers the extra path crowds, dominates.  Lists of jobs (batches, served
-// queries) take it too.
-constexpr int kScaledMinComponents = 3;
-
 template <typename T>
 static cudaError_t launch_retrieve_t(const RetrieveParams& p, cudaStream_t s) {
   const size_t smem = retrieve_smem3<T>();
-  cudaError_t e = cudaFuncSetAttribute(k_retrieve3<T, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if constexpr (sizeof(T) == 8)
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(k_retrieve3<T, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = cudaFuncSetAttribute(k_retrieve3<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   if (p.nunits == 0) return cudaSuccess;
-  bool sc = false;
-  if constexpr (sizeof(T) == 8) sc = p.jobs != nullptr || p.job0.k - p.job0.k0 >= kScaledMinComponents;
-  if constexpr (sizeof(T) == 8)
-    if (sc) {
-      k_retrieve3<T, true><<<(unsigned)p.grid, kRThreads, smem, s>>>(p);
-      return cudaGetLastError();
-    }
-  k_retrieve3<T, false><<<(unsigned)p.grid, kRThreads, smem, s>>>(p);
+  k_retrieve3<T><<<(unsigned)p.grid, kRThreads, smem, s>>>(p);
   return cudaGetLastError();
 }
 

@@ -37,7 +37,7 @@ __global__ void __launch_bounds__(kSmallThreads, kCompressCtas<T>) k_compress_sm
 // bricks (unit_begin = the job's first brick among all jobs' bricks).
 template <typename T, int D>
 __global__ void __launch_bounds__(kSmallThreads, kRetrieveCtas<T>) k_retrieve_small(const RetrieveParams R) {
-  __shared__ __align__(4) uint16_t tokens[kTokLut];
+  __shared__ uint32_t tokens[kTokLut];
   load_tokens<kSmallThreads>(tokens);
   __syncthreads();
   const int64_t g = (int64_t)blockIdx.x * kSmallThreads + threadIdx.x;
