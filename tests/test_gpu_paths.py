@@ -119,3 +119,47 @@ def test_construction_by_span_and_scale(P, dtype, exp, rel, shape):
         assert c["measured"] == ref.measured(i)
     got = st.retrieve(k=len(tau)).cpu().numpy()
     assert np.array_equal(_bits(got), _bits(ref.retrieve(len(tau))))
+
+
+# results of a server batch written into the callers' buffers: buffers that
+# start at any byte of an allocation, 140 of them (more than one list of
+# copies holds), some without a buffer; buffers shared by two queries
+# (the later one's result stays: the boxes all hold the field's centre, so
+# batches wait for one another)
+@pytest.mark.parametrize("where", ["apart", "shared"])
+def test_server_results(P, where):
+    x = torch.from_numpy(S.powerlaw((40, 44, 52), seed=67, dtype=np.float32)).cuda()
+    st = P.compress(x, [0.1, 0.01, 0.001])
+    rng = np.random.default_rng(68)
+    qs, off, at = [], [], 0
+    for i in range(140):
+        lo = [int(rng.integers(0, s // 2)) for s in x.shape]
+        hi = [int(rng.integers(s // 2 + 1, s + 1)) for s in x.shape]
+        qs.append((0, (lo, hi), 0.0, int(rng.integers(1, 4))))
+        at += int(rng.integers(0, 9)) * 4 if i % 3 else int(rng.integers(0, 300))
+        off.append(at)
+        at += 4 * int(np.prod([h - l for l, h in zip(lo, hi)]))
+    memory = torch.full((at + 64,), 7, dtype=torch.uint8, device="cuda")
+    if where == "shared":
+        off = [off[i - 1] if i and i % 4 == 0 else o for i, o in enumerate(off)]
+
+    class Out:  # a buffer at any byte address (a tensor's must be a multiple of its type)
+        def __init__(self, p):
+            self.p = p
+
+        def data_ptr(self):
+            return self.p
+
+    outs = [None if i % 11 == 10 else Out(memory.data_ptr() + o) for i, o in enumerate(off)]
+    want = memory.cpu().numpy().copy()
+    for q, o, out in zip(qs, off, outs):
+        if out is not None:
+            b = st.retrieve(k=q[3], box=q[1]).cpu().numpy().view(np.uint8).reshape(-1)
+            want[o:o + b.size] = b
+    srv = P.Server(1 << 30)
+    srv.add_field(st)
+    srv.replay(qs[:1], [0.0], None)  # (starts the dispatcher)
+    srv.replay(qs, [0.0] * len(qs), outs)
+    torch.cuda.synchronize()
+    srv.close()
+    assert np.array_equal(memory.cpu().numpy(), want)
