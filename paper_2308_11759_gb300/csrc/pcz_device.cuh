@@ -861,4 +861,27 @@ __device__ __forceinline__ void lift_inv_bricks(S* v, uint4* zw, uint4* yw, int 
   for (int y = 0; y < 4; ++y) lift_inv(v[4 * y], v[4 * y + 1], v[4 * y + 2], v[4 * y + 3]);
 }
 
+// n / d for an invariant d, by one high multiply (DivMagic).
+__device__ __forceinline__ uint32_t div_by(uint32_t n, const DivMagic& D) {
+  const uint32_t t = __umulhi(D.m, n);
+  return (t + ((n - t) >> D.s1)) >> D.s2;
+}
+
+// Brick g of the job's box (x fastest): its coordinates.
+__device__ __forceinline__ void brick_of(const BoxJob& J, int64_t g, int64_t* bx, int64_t* by, int64_t* bz) {
+  if (J.nbox < (1ll << 32)) {  // 32-bit division by the box's invariant extents
+    const uint32_t g32 = (uint32_t)g;
+    const uint32_t r = div_by(g32, J.dv_bn0);
+    const uint32_t z = div_by(r, J.dv_bn1);
+    *bx = J.bl[0] + (int64_t)(g32 - r * (uint32_t)J.bn[0]);
+    *by = J.bl[1] + (int64_t)(r - z * (uint32_t)J.bn[1]);
+    *bz = J.bl[2] + (int64_t)z;
+  } else {
+    *bx = J.bl[0] + g % J.bn[0];
+    const int64_t r = g / J.bn[0];
+    *by = J.bl[1] + r % J.bn[1];
+    *bz = J.bl[2] + r / J.bn[1];
+  }
+}
+
 }  // namespace pcz
