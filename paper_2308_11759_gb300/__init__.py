@@ -34,6 +34,10 @@ class PczError(RuntimeError):
         self.name = STATUS.get(status, str(status))
 
 
+# A bytes object of a given length whose contents are written before it is handed on.
+_new_bytes = C.PYFUNCTYPE(C.py_object, C.c_void_p, C.c_ssize_t)(("PyBytes_FromStringAndSize", C.pythonapi))
+
+
 class Box(C.Structure):
     _fields_ = [("lo", C.c_int64 * 3), ("hi", C.c_int64 * 3)]
 
@@ -154,18 +158,23 @@ def _stream_ptr(stream):
     return C.c_void_p(stream.cuda_stream)
 
 
-def _box(box, shape):
-    if box is None:
-        return None, tuple(shape)
-    lo, hi = [int(v) for v in box[0]], [int(v) for v in box[1]]
+def _span(box, shape):
+    """A Box's six numbers (lo, then hi, x first) and the box's extents in array axis order."""
+    lo, hi = list(map(int, box[0])), list(map(int, box[1]))
     nd = len(shape)
     if len(lo) != nd or len(hi) != nd:
         raise ValueError("box rank differs from the field's")
-    b = Box()
-    for a in range(3):
-        b.lo[a] = lo[nd - 1 - a] if a < nd else 0
-        b.hi[a] = hi[nd - 1 - a] if a < nd else 1
-    return b, tuple(h - l for l, h in zip(lo, hi))
+    ext = tuple(map(int.__sub__, hi, lo))
+    lo.reverse()
+    hi.reverse()
+    return (lo + [0, 0, 0])[:3] + (hi + [1, 1, 1])[:3], ext
+
+
+def _box(box, shape):
+    if box is None:
+        return None, tuple(shape)
+    v, ext = _span(box, shape)
+    return Box.from_buffer((C.c_int64 * 6)(*v)), ext
 
 
 def _ptr(x):
@@ -211,9 +220,11 @@ class Streams:
     @classmethod
     def deserialize(cls, data: bytes, stream=None):
         torch = _torch()
-        buf = C.create_string_buffer(bytes(data), len(data))
+        raw = bytes(data)  # (bytes themselves are not copied)
+        if len(raw) > len(data):  # the length of `data` counts items wider than a byte
+            raise ValueError("byte string too long")
         h = C.c_void_p()
-        _check(lib().pc_streams_deserialize(buf, len(data), _stream_ptr(stream), C.byref(h)))
+        _check(lib().pc_streams_deserialize(raw, len(raw), _stream_ptr(stream), C.byref(h)))
         nd = C.c_int()
         dims = (C.c_int64 * 3)()
         dt = C.c_int()
@@ -322,9 +333,11 @@ class Streams:
     def serialize(self, stream=None) -> bytes:
         n = C.c_size_t()
         _check(lib().pc_streams_serialize(self._h, None, C.byref(n), _stream_ptr(stream)))
-        buf = C.create_string_buffer(n.value)
-        _check(lib().pc_streams_serialize(self._h, buf, C.byref(n), _stream_ptr(stream)))
-        return buf.raw[: n.value]
+        # the streams are copied straight into the bytes object returned, not
+        # through a zero-filled buffer and a copy of that
+        data = _new_bytes(None, n.value)
+        _check(lib().pc_streams_serialize(self._h, data, C.byref(n), _stream_ptr(stream)))
+        return data
 
 
 class Batch:
@@ -392,16 +405,15 @@ def retrieve_batch(streams, ks, boxes=None, outs=None, stream=None):
     and dimensionality (pc_retrieve_batch).  Returns the output tensors."""
     torch = _torch()
     nq = len(streams)
-    bx = (Box * max(nq, 1))()
+    bx = []  # (a Box written field by field takes twice as long)
     res = []
     for q in range(nq):
         st = streams[q]
         box = boxes[q] if boxes is not None else None
-        b, ext = _box(box, st.shape)
-        if b is None:
-            b, ext = _box(([0] * len(st.shape), list(st.shape)), st.shape)
-        bx[q] = b
+        v, ext = _span(([0] * len(st.shape), st.shape) if box is None else box, st.shape)
+        bx += v
         res.append(outs[q] if outs is not None else torch.empty(ext, dtype=st.dtype, device="cuda"))
+    bx = (Box * max(nq, 1)).from_buffer((C.c_int64 * max(6 * nq, 6))(*bx))
     sp = (C.c_void_p * max(nq, 1))(*[st._h.value for st in streams])
     kk = (C.c_int * max(nq, 1))(*[int(k) for k in ks])
     op = (C.c_void_p * max(nq, 1))(*[o.data_ptr() for o in res])
@@ -435,14 +447,15 @@ class Server:
         results.  Returns (latencies in seconds as a numpy array, stats dict)."""
         nq = len(queries)
         qa = (Query * max(nq, 1))()
-        for j, (field, box, tau, k) in enumerate(queries):
+        for q, (field, box, tau, k) in zip(qa, queries):
             known = 0 <= field < len(self._fields)  # the library rejects other indices
             shape = self._fields[field].shape if known else tuple(box[1])
-            b, _ = _box(box, shape)
-            qa[j].field = int(field)
-            qa[j].k = int(k)
-            qa[j].tau = float(tau)
-            qa[j].box = b if b is not None else _box(([0] * len(shape), list(shape)), shape)[0]
+            v, _ = _span(([0] * len(shape), shape) if box is None else box, shape)
+            q.field = int(field)
+            q.k = int(k)
+            q.tau = float(tau)
+            q.box.lo[:] = v[:3]
+            q.box.hi[:] = v[3:]
         arr = (C.c_double * max(nq, 1))(*[float(t) for t in arrival_s])
         lat = (C.c_double * max(nq, 1))()
         outp = None

@@ -1028,8 +1028,13 @@ pc_status pc_streams_deserialize(const void* h_buf, size_t len, void* cuda_strea
       const uint16_t* bl = (const uint16_t*)(p + q + 8 * nch);
       uint64_t w = 0;
       for (int64_t c = 0; c < nch; ++c) {
-        uint64_t bits = 0;
-        for (int64_t b = c * kChunk; b < nbr && b < (c + 1) * kChunk; ++b) bits += bl[b];
+        const uint16_t* b = bl + c * kChunk;
+        uint32_t bits = 0;
+        if (nbr - c * kChunk >= kChunk) {  // (a fixed count: the compiler adds whole vectors)
+          for (int j = 0; j < kChunk; ++j) bits += b[j];
+        } else {
+          for (int j = 0; j < (int)(nbr - c * kChunk); ++j) bits += b[j];
+        }
         if (cw[c] != w) {
           delete s;
           return fail(PC_ERR_CORRUPT_STREAM, "chunk offsets inconsistent with brick lengths");

@@ -1023,8 +1023,12 @@ pc_status pc_retrieve_batch(int nq, const pc_streams* const* s, const int* k, co
       cudaFreeAsync(mem, st);
       if (e != cudaSuccess) return api_cuda_fail(e, "batched retrieval");
     }
+  std::vector<const pc_streams*> used;  // each once: an event record per query took 1.5 us
   for (int q = 0; q < nq; ++q)
-    if (k[q] > 0) note_use(s[q], st);
+    if (k[q] > 0) used.push_back(s[q]);
+  std::sort(used.begin(), used.end());
+  used.erase(std::unique(used.begin(), used.end()), used.end());
+  for (const pc_streams* u : used) note_use(u, st);
   return PC_OK;
 }
 
