@@ -242,7 +242,7 @@ __device__ __forceinline__ void append_chunk(const CompressParams& P, uint32_t* 
 // values.  With 16 lanes per brick and 4 values per lane it took 582 (float32)
 // and 997 (float64) warp instructions per brick and component, now 187 and 284;
 // 512^3 float32, 8 components: 10.16 -> 3.52 ms, 256 x 384 x 384 float64, 12
-// components: 8.77 -> 3.35 ms.  It runs at 0.71 (float32; ALU pipe 0.67) and
+// components: 8.77 -> 3.22 ms.  It runs at 0.71 (float32; ALU pipe 0.67) and
 // 0.47 (float64) of the issue peak.
 template <typename T>
 __device__ __forceinline__ void compress3_chunk(const CompressParams& P, int64_t chunk, unsigned char* smem,
@@ -578,14 +578,32 @@ __device__ __forceinline__ void compress3_chunk(const CompressParams& P, int64_t
           uint32_t w[16];
 #pragma unroll
           for (int k = 0; k < 16; ++k) w[k] = digits(k);
-          int32_t r[16];
-          const uint32_t M = (uint32_t)(F::NBM >> min(p, 63)), M64 = M << 6;
+          // Within 13 planes the same in float, in units of 2^p: d and M's 13 bits
+          // with 2^23's bit pattern in front are floats whose difference is the
+          // coefficient, and values below 2^(13 + 4.4) that are multiples of
+          // 2^-6 need 24 bits.  8 operations a line instead of 11, off the ALU
+          // pipe, and a shorter conversion: 256 x 384 x 384, 12 components, 3.35
+          // -> 3.22 ms.  (Float32, whose conversion is one instruction, became 3 %
+          // slower with both forms in the kernel and keeps the integers.)
+          if (span <= 13) {
+            float r[16];
+            const uint32_t M = ((uint32_t)(F::NBM >> min(p, 63)) & 0x1fffu) | 0x4B000000u;
 #pragma unroll
-          for (int k = 0; k < 16; ++k) r[k] = (int32_t)(((w[k] ^ M) << 6) - M64);
-          lift_inv_bricks<int32_t>(r, zw, yw, SET);
-          const uint32_t eb = (uint32_t)(1053 + (p - 6) - s) << 20;
+            for (int k = 0; k < 16; ++k) r[k] = __fsub_rn(__uint_as_float(w[k] ^ M), __uint_as_float(M));
+            lift_inv_bricks<float>(r, zw, yw, SET);
+            const uint32_t adj = (uint32_t)(896 + p - s) << 20;
 #pragma unroll
-          for (int k = 0; k < 16; ++k) add(k, scaled_i32_to_f64(r[k], eb));
+            for (int k = 0; k < 16; ++k) add(k, scaled_f32_to_f64(r[k], adj));
+          } else {
+            int32_t r[16];
+            const uint32_t M = (uint32_t)(F::NBM >> min(p, 63)), M64 = M << 6;
+#pragma unroll
+            for (int k = 0; k < 16; ++k) r[k] = (int32_t)(((w[k] ^ M) << 6) - M64);
+            lift_inv_bricks<int32_t>(r, zw, yw, SET);
+            const uint32_t eb = (uint32_t)(1053 + (p - 6) - s) << 20;
+#pragma unroll
+            for (int k = 0; k < 16; ++k) add(k, scaled_i32_to_f64(r[k], eb));
+          }
           residual_of(xtn, en);
           H = planes_of(w);
         } else {
