@@ -33,7 +33,11 @@
 // component, now 107 and 127; 512^3 float32: k = 6 2.87 -> 1.71 ms, k = 1 0.86 ->
 // 0.44 ms; 256 x 384 x 384 float64: k = 8 1.29 -> 0.89 ms; refinement from k = 1 to
 // 8 in place 7.06 -> 3.39 and 3.13 -> 1.75 ms (nearly half of it had gone to the
-// index pass and the sort).
+// index pass and the sort).  With what few bricks need (any planes, RAW) out of
+// line, nothing spills and the common path is shorter to fetch: 512^3 float32 k =
+// 6 1.72 -> 1.68 ms, 252 x 380 x 384 float64 k = 1 204 -> 185 us, refinement by one
+// component 198 -> 183 us.  (Code that does not even run costs here: a prefetch
+// behind a condition that is never true made k = 6 7 % slower.)
 #include <algorithm>
 #include <type_traits>
 
@@ -408,12 +412,83 @@ __device__ __forceinline__ double fixed_add(double sum, int32_t i, int sh) {
   return __longlong_as_double(__double_as_longlong(sum) + (int64_t)hi * (int64_t)(1 << min(sh, 30)));
 }
 
+// The decoding of any planes, and RAW blocks: rare, and out of line, so that the
+// common path stays short.  xt: the lane's partial sums.
+template <typename T>
+__device__ __noinline__ void add_any(const BlockMeta* bm, uint64_t* pool, uint64_t* spill, uint4* area, int lane, T* xt) {
+  using F = Fmt<T>;
+  using U = typename F::U;
+  using S = typename F::S;
+  constexpr bool WIDE = F::P == 64;
+  constexpr unsigned FULL = 0xffffffffu;
+  const BlockMeta m = *bm;
+  const int bq = lane >> 2, q = lane & 3;
+  const bool coded = m.mode == kModeCoded;
+  const int p = m.p, top = m.top, s = coded ? (int)m.s : 0;
+  const int nw = coded ? top - p + 1 : 0;
+  uint4* zw = area + LineSet::at(bq, 0, q);
+  uint4* yw = area + LineSet::at(bq, q, 0);
+  uint32_t place[4];
+#pragma unroll
+  for (int z = 0; z < 4; ++z) place[z] = coded_places(kRank3r.pos, q, z);
+      // any planes, 16 at a time from plane 0, each 16 digits a half-word of the
+      // coefficients in coded order
+      const uint32_t stride = 64u * sizeof(T) + 16u;
+      unsigned char* dig = reinterpret_cast<unsigned char*>(area) + stride * bq;
+      const uint64_t* words = words_at<T>(pool, spill, m.at, nw);
+#pragma unroll 1
+      for (int h = 0; h < F::P / 16; ++h) {
+        auto plane = [&](int pl) {
+          if (nw <= 0 || pl < p || pl > top) return 0u;
+          return (uint32_t)reinterpret_cast<const uint16_t*>(words + (top - pl))[q];
+        };
+        uint32_t a[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) a[j] = plane(16 * h + j) | (plane(16 * h + j + 8) << 16);
+        untranspose16(a);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {  // ranks i and i + 8 of the lane's 16, at their places
+          uint16_t* e = reinterpret_cast<uint16_t*>(dig + (16 * q + 4 * (i & 3) + 2 * (i >> 2)) * sizeof(T)) + h;
+          e[0] = (uint16_t)a[i];
+          e[sizeof(T) / 2] = (uint16_t)(a[i] >> 16);
+        }
+      }
+      __syncwarp();
+      S r[16];
+#pragma unroll
+      for (int k = 0; k < 16; ++k)
+        r[k] = nb_inv<T>(*reinterpret_cast<const U*>(dig + ((place[k >> 2] >> (8 * (k & 3))) & 0xffu) * sizeof(T)));
+      __syncwarp();
+      lift_inv_bricks<S>(r, zw, yw, LineSet::kVectors);
+      const bool common = __all_sync(FULL, WIDE ? s >= -960 && s <= 1022 : s >= -127 && s <= 126);
+#pragma unroll
+      for (int y = 0; y < 4; ++y) {
+        T xi[4];
+        if (common) {
+          dequantize_line<T, true>(r + 4 * y, s, xi);
+        } else {
+#pragma unroll
+          for (int k = 0; k < 4; ++k) xi[k] = F::val(dequantize_any<T>(r[4 * y + k], s));
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) xt[4 * y + k] = F::add(xt[4 * y + k], xi[k]);
+      }
+}
+
+template <typename T>
+__device__ __noinline__ void add_raw(const BlockMeta* bm, const CompDesc* cd, int q, T* xt) {
+  using F = Fmt<T>;
+  using U = typename F::U;
+  const uint64_t off = bm->off + 2 + (uint64_t)F::P * 16 * q;
+  for (int k = 0; k < 16; ++k) xt[k] = F::add(xt[k], F::val((U)peek64(cd->payload, cd->nwords, off + (uint64_t)F::P * k)));
+}
+
 // Adds one component into the z-planes of a warp's 8 bricks.  how: kDecode* and
 // kHasRaw of the 8; m: header of the lane's brick; pool, spill: the round's plane
 // words; zw, yw: the lane's lines of the exchange; place: the coded places of its
 // coefficients.
 template <typename T>
-__device__ __forceinline__ void add_component(int how, const BlockMeta& m, const CompDesc* cd, uint64_t* pool,
+__device__ __forceinline__ void add_component(int how, const BlockMeta* bm, const CompDesc* cd, uint64_t* pool,
                                               uint64_t* spill, uint4* area, uint4* zw, uint4* yw,
                                               const uint32_t* place, int lane, T* xt, FixedSum& fx) {
   using F = Fmt<T>;
@@ -421,6 +496,7 @@ __device__ __forceinline__ void add_component(int how, const BlockMeta& m, const
   using S = typename F::S;
   constexpr bool WIDE = F::P == 64;
   constexpr unsigned FULL = 0xffffffffu;
+  const BlockMeta m = *bm;
   const int bq = lane >> 2, q = lane & 3;
   const bool coded = m.mode == kModeCoded;
   const int p = m.p, top = m.top, s = coded ? (int)m.s : 0;
@@ -543,53 +619,20 @@ __device__ __forceinline__ void add_component(int how, const BlockMeta& m, const
     }
   }
   if (any) {
-    // any planes, 16 at a time from plane 0, each 16 digits a half-word of the
-    // coefficients in coded order
-    const uint32_t stride = 64u * sizeof(T) + 16u;
-    unsigned char* dig = reinterpret_cast<unsigned char*>(area) + stride * bq;
-    const uint64_t* words = words_at<T>(pool, spill, m.at, nw);
-#pragma unroll 1
-    for (int h = 0; h < F::P / 16; ++h) {
-      auto plane = [&](int pl) {
-        if (nw <= 0 || pl < p || pl > top) return 0u;
-        return (uint32_t)reinterpret_cast<const uint16_t*>(words + (top - pl))[q];
-      };
-      uint32_t a[8];
+    T t[16];
 #pragma unroll
-      for (int j = 0; j < 8; ++j) a[j] = plane(16 * h + j) | (plane(16 * h + j + 8) << 16);
-      untranspose16(a);
+    for (int k = 0; k < 16; ++k) t[k] = xt[k];
+    add_any<T>(bm, pool, spill, area, lane, t);
 #pragma unroll
-      for (int i = 0; i < 8; ++i) {  // ranks i and i + 8 of the lane's 16, at their places
-        uint16_t* e = reinterpret_cast<uint16_t*>(dig + (16 * q + 4 * (i & 3) + 2 * (i >> 2)) * sizeof(T)) + h;
-        e[0] = (uint16_t)a[i];
-        e[sizeof(T) / 2] = (uint16_t)(a[i] >> 16);
-      }
-    }
-    __syncwarp();
-    S r[16];
-#pragma unroll
-    for (int k = 0; k < 16; ++k)
-      r[k] = nb_inv<T>(*reinterpret_cast<const U*>(dig + ((place[k >> 2] >> (8 * (k & 3))) & 0xffu) * sizeof(T)));
-    __syncwarp();
-    lift_inv_bricks<S>(r, zw, yw, LineSet::kVectors);
-    const bool common = __all_sync(FULL, WIDE ? s >= -960 && s <= 1022 : s >= -127 && s <= 126);
-#pragma unroll
-    for (int y = 0; y < 4; ++y) {
-      T xi[4];
-      if (common) {
-        dequantize_line<T, true>(r + 4 * y, s, xi);
-      } else {
-#pragma unroll
-        for (int k = 0; k < 4; ++k) xi[k] = F::val(dequantize_any<T>(r[4 * y + k], s));
-      }
-#pragma unroll
-      for (int k = 0; k < 4; ++k) xt[4 * y + k] = F::add(xt[4 * y + k], xi[k]);
-    }
+    for (int k = 0; k < 16; ++k) xt[k] = t[k];
   }
   if ((how & kHasRaw) && m.mode == kModeRaw) {
+    T t[16];
 #pragma unroll
-    for (int k = 0; k < 16; ++k)
-      xt[k] = F::add(xt[k], F::val((U)peek64(cd->payload, cd->nwords, m.off + 2 + (uint64_t)F::P * (16 * q + k))));
+    for (int k = 0; k < 16; ++k) t[k] = xt[k];
+    add_raw<T>(bm, cd, q, t);
+#pragma unroll
+    for (int k = 0; k < 16; ++k) xt[k] = t[k];
   }
 }
 
@@ -675,8 +718,7 @@ __global__ void __launch_bounds__(kRThreads, kRetrieveCtas3<T>) k_retrieve3(cons
           for (int c = 0; c < nc; ++c) {  // Algorithm 2, components in ascending order
             const int blk = c * ub + u, h = how[blk / 8];
             if (h == kDecodeNone) continue;
-            const BlockMeta m = meta[blk];
-            add_component<T>(h, m, &J.comp[c0 + c], pool, spill, area, zw, yw, place, lane, xt, fx);
+            add_component<T>(h, meta + blk, &J.comp[c0 + c], pool, spill, area, zw, yw, place, lane, xt, fx);
           }
           if (c0 + nc >= J.k) {
             if constexpr (sizeof(T) == 8)
