@@ -223,6 +223,47 @@ __device__ __forceinline__ void append_chunk(const CompressParams& P, uint32_t* 
   }
 }
 
+// r = x - a, padded: x in shared memory, part h of the lane's at s_x[h * threads].
+template <typename T>
+__device__ __forceinline__ void residual_from(const uint4* s_x, bool any_partial, int nvx, int nvy, int nvz, int lane,
+                                              const T* a, T* r) {
+  constexpr int XV = 16 / (int)sizeof(T);  // values of a 16-byte part
+  union Part {
+    uint4 w;
+    T v[XV];
+    __device__ Part() {}
+  };
+#pragma unroll
+  for (int h = 0; h < 16 / XV; ++h) {
+    Part t;
+    t.w = s_x[h * kCompressThreads3];
+#pragma unroll
+    for (int o = 0; o < XV; ++o) r[XV * h + o] = Fmt<T>::sub(t.v[o], a[XV * h + o]);
+  }
+  if (any_partial) pad_brick<T>(r, nvx, nvy, nvz, lane);
+}
+
+// A RAW block's outcome (R14), out of line: a holds x~ and receives the residual
+// that is stored, xr x~ and er the residual after it; returns the brick's largest
+// |er|.  (In line it made float64 spill 520 bytes a thread, now 12: 256 x 384 x
+// 384, 12 components, 3.21 -> 3.10 ms.)
+template <typename T>
+static __device__ __noinline__ typename Fmt<T>::U raw_form(const uint4* s_x, bool any_partial, int nvx, int nvy, int nvz,
+                                                           int lane, T* a, T* xr, T* er) {
+  T e[16], x[16], r[16];
+  residual_from<T>(s_x, any_partial, nvx, nvy, nvz, lane, a, e);
+#pragma unroll
+  for (int k = 0; k < 16; ++k) x[k] = Fmt<T>::add(a[k], e[k]);
+  residual_from<T>(s_x, any_partial, nvx, nvy, nvz, lane, x, r);
+#pragma unroll
+  for (int k = 0; k < 16; ++k) {
+    a[k] = e[k];
+    xr[k] = x[k];
+    er[k] = r[k];
+  }
+  return brick_max<T>(r);
+}
+
 // Algorithm 1 on every brick of index chunk `chunk` of a 3D field, all
 // components, by 4 warps (barrier `bar_id`); smem holds compress_smem3<T>(map
 // != nullptr) bytes, 128-byte aligned.  With a tensor map, xs (= smem) holds
@@ -242,7 +283,7 @@ __device__ __forceinline__ void append_chunk(const CompressParams& P, uint32_t* 
 // values.  With 16 lanes per brick and 4 values per lane it took 582 (float32)
 // and 997 (float64) warp instructions per brick and component, now 187 and 284;
 // 512^3 float32, 8 components: 10.16 -> 3.52 ms, 256 x 384 x 384 float64, 12
-// components: 8.77 -> 3.22 ms.  It runs at 0.71 (float32; ALU pipe 0.67) and
+// components: 8.77 -> 3.10 ms.  It runs at 0.71 (float32; ALU pipe 0.67) and
 // 0.47 (float64) of the issue peak.
 template <typename T>
 __device__ __forceinline__ void compress3_chunk(const CompressParams& P, int64_t chunk, unsigned char* smem,
@@ -343,16 +384,7 @@ __device__ __forceinline__ void compress3_chunk(const CompressParams& P, int64_t
     s_x[h * kCompressThreads3 + tid] = t.w;
   }
   // r = x - a, padded
-  auto residual_of = [&](const T* a, T* r) {
-#pragma unroll
-    for (int h = 0; h < 16 / XV; ++h) {
-      Part t;
-      t.w = s_x[h * kCompressThreads3 + tid];
-#pragma unroll
-      for (int o = 0; o < XV; ++o) r[XV * h + o] = F::sub(t.v[o], a[XV * h + o]);
-    }
-    if (any_partial) pad_brick<T>(r, nvx, nvy, nvz, lane);
-  };
+  auto residual_of = [&](const T* a, T* r) { residual_from<T>(s_x + tid, any_partial, nvx, nvy, nvz, lane, a, r); };
   U m = brick_max<T>(e);  // the largest magnitude of the residual, by brick
   if (__any_sync(FULL, m >= F::INF) && lane == 0) atomicOr(P.flags, kFlagNonFinite);
 
@@ -684,20 +716,17 @@ __device__ __forceinline__ void compress3_chunk(const CompressParams& P, int64_t
       int viol = 0;  // Eq. 1 failures left (only a RAW brick can have them)
       U mnew = mn;
       if (__any_sync(FULL, mode == kModeRaw || (pass && lenC > LEN_RAW))) {
-        // the residual the brick started from, and x~ and the residual after it
-        T eo[16], xr[16], er[16];
-        residual_of(xt, eo);
+        T a[16], xr[16], er[16];
 #pragma unroll
-        for (int k = 0; k < 16; ++k) xr[k] = F::add(xt[k], eo[k]);
-        residual_of(xr, er);
-        const U mr = brick_max<T>(er);
+        for (int k = 0; k < 16; ++k) a[k] = xt[k];
+        const U mr = raw_form<T>(s_x + tid, any_partial, nvx, nvy, nvz, lane, a, xr, er);
         if (pass && lenC > LEN_RAW && mr <= tb) mode = kModeRaw;
         if (mode == kModeRaw) {
           S* raw = reinterpret_cast<S*>(planes);  // the residual, for the bit writes
           mnew = mr;
 #pragma unroll
           for (int k = 0; k < 16; ++k) {
-            raw[16 * q + k] = (S)F::bits(eo[k]);
+            raw[16 * q + k] = (S)F::bits(a[k]);
             xtn[k] = xr[k];
             en[k] = er[k];
             if ((k & 3) < nvx && (k >> 2) < nvy && q < nvz && magnitude(er[k]) > tb) ++viol;
