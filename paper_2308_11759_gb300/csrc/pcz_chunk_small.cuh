@@ -475,7 +475,7 @@ __device__ __forceinline__ void compress_small_chunk(const CompressParams& P, in
 // transposed back into digits in registers, aligned to the brick's highest
 // plane.  With planes scattered bit by bit into the coefficients and a loop over
 // tokens it took 2877 warp instructions per 32 float32 2D bricks and component,
-// now 1244; 4096^2 float32, k = 6: 659 -> 278 us.
+// now 1244; 4096^2 float32, k = 6: 659 -> 284 us.
 template <typename T, int D>
 __device__ __forceinline__ void retrieve_small_brick(const BoxJob& J, int write, unsigned int* err, int64_t g,
                                                      const uint32_t* tokens) {

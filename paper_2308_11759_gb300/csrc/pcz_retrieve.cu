@@ -431,50 +431,51 @@ __device__ __noinline__ void add_any(const BlockMeta* bm, uint64_t* pool, uint64
   uint32_t place[4];
 #pragma unroll
   for (int z = 0; z < 4; ++z) place[z] = coded_places(kRank3r.pos, q, z);
-      // any planes, 16 at a time from plane 0, each 16 digits a half-word of the
-      // coefficients in coded order
-      const uint32_t stride = 64u * sizeof(T) + 16u;
-      unsigned char* dig = reinterpret_cast<unsigned char*>(area) + stride * bq;
-      const uint64_t* words = words_at<T>(pool, spill, m.at, nw);
+  // any planes, 16 at a time from plane 0, each 16 digits a half-word of the
+  // coefficients in coded order
+  const uint32_t stride = 64u * sizeof(T) + 16u;
+  unsigned char* dig = reinterpret_cast<unsigned char*>(area) + stride * bq;
+  const uint64_t* words = words_at<T>(pool, spill, m.at, nw);
 #pragma unroll 1
-      for (int h = 0; h < F::P / 16; ++h) {
-        auto plane = [&](int pl) {
-          if (nw <= 0 || pl < p || pl > top) return 0u;
-          return (uint32_t)reinterpret_cast<const uint16_t*>(words + (top - pl))[q];
-        };
-        uint32_t a[8];
+  for (int h = 0; h < F::P / 16; ++h) {
+    auto plane = [&](int pl) {
+      if (nw <= 0 || pl < p || pl > top) return 0u;
+      return (uint32_t)reinterpret_cast<const uint16_t*>(words + (top - pl))[q];
+    };
+    uint32_t a[8];
 #pragma unroll
-        for (int j = 0; j < 8; ++j) a[j] = plane(16 * h + j) | (plane(16 * h + j + 8) << 16);
-        untranspose16(a);
+    for (int j = 0; j < 8; ++j) a[j] = plane(16 * h + j) | (plane(16 * h + j + 8) << 16);
+    untranspose16(a);
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {  // ranks i and i + 8 of the lane's 16, at their places
-          uint16_t* e = reinterpret_cast<uint16_t*>(dig + (16 * q + 4 * (i & 3) + 2 * (i >> 2)) * sizeof(T)) + h;
-          e[0] = (uint16_t)a[i];
-          e[sizeof(T) / 2] = (uint16_t)(a[i] >> 16);
-        }
-      }
-      __syncwarp();
-      S r[16];
+    for (int i = 0; i < 8; ++i) {  // ranks i and i + 8 of the lane's 16, at their places
+      uint16_t* e = reinterpret_cast<uint16_t*>(dig + (16 * q + 4 * (i & 3) + 2 * (i >> 2)) * sizeof(T)) + h;
+      e[0] = (uint16_t)a[i];
+      e[sizeof(T) / 2] = (uint16_t)(a[i] >> 16);
+    }
+  }
+  __syncwarp();
+  S r[16];
 #pragma unroll
-      for (int k = 0; k < 16; ++k)
-        r[k] = nb_inv<T>(*reinterpret_cast<const U*>(dig + ((place[k >> 2] >> (8 * (k & 3))) & 0xffu) * sizeof(T)));
-      __syncwarp();
-      lift_inv_bricks<S>(r, zw, yw, LineSet::kVectors);
-      const bool common = __all_sync(FULL, WIDE ? s >= -960 && s <= 1022 : s >= -127 && s <= 126);
+  for (int k = 0; k < 16; ++k)
+    r[k] = nb_inv<T>(*reinterpret_cast<const U*>(dig + ((place[k >> 2] >> (8 * (k & 3))) & 0xffu) * sizeof(T)));
+  __syncwarp();
+  lift_inv_bricks<S>(r, zw, yw, LineSet::kVectors);
+  const bool common = __all_sync(FULL, WIDE ? s >= -960 && s <= 1022 : s >= -127 && s <= 126);
 #pragma unroll
-      for (int y = 0; y < 4; ++y) {
-        T xi[4];
-        if (common) {
-          dequantize_line<T, true>(r + 4 * y, s, xi);
-        } else {
+  for (int y = 0; y < 4; ++y) {
+    T xi[4];
+    if (common) {
+      dequantize_line<T, true>(r + 4 * y, s, xi);
+    } else {
 #pragma unroll
-          for (int k = 0; k < 4; ++k) xi[k] = F::val(dequantize_any<T>(r[4 * y + k], s));
-        }
+      for (int k = 0; k < 4; ++k) xi[k] = F::val(dequantize_any<T>(r[4 * y + k], s));
+    }
 #pragma unroll
-        for (int k = 0; k < 4; ++k) xt[4 * y + k] = F::add(xt[4 * y + k], xi[k]);
-      }
+    for (int k = 0; k < 4; ++k) xt[4 * y + k] = F::add(xt[4 * y + k], xi[k]);
+  }
 }
 
+// A RAW block of the lane's brick into its sums.
 template <typename T>
 __device__ __noinline__ void add_raw(const BlockMeta* bm, const CompDesc* cd, int q, T* xt) {
   using F = Fmt<T>;

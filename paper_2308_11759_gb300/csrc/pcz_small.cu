@@ -15,8 +15,8 @@ namespace pcz {
 
 // CTAs of 4 warps that share an SM, measured on 2D fields (4096^2 float32, 4096 x
 // 3000 float64, 6 components).  Construction: float32 5 (349 us; 4: 376, 6: 387),
-// float64 3 (613; 2: 709, 4: 640).  Retrieval: float32 8 (278 us; 6: 292, 5:
-// 318), float64 5 (327; 4: 348).
+// float64 3 (613; 2: 709, 4: 640).  Retrieval: float32 8 (284 us; 6 and 5
+// 5 and 14 % slower), float64 5 (330; 4 6 % slower).
 template <typename T>
 constexpr int kCompressCtas = sizeof(T) == 4 ? 5 : 3;
 template <typename T>
