@@ -55,27 +55,20 @@ METRIC = "compress/retrieve GB/s vs HBM roofline; progressive-query p50/p99 late
 # workload, means over the 16 retrieval launches of a step (k = 1..8, float32 and float64), from
 # ncu captures of the current kernels at 512^3 (gpu__time_duration, dram__bytes_read/write,
 # smsp__inst_executed: one pass), one per type.
-TRAFFIC = {"retrieve": 1298626048}
+TRAFFIC = {"retrieve": 1280814160}
 TRAFFIC_SOURCE = ("ncu dram__bytes_read.sum + dram__bytes_write.sum per launch, mean over the 16 retrieval launches "
                   "(k = 1..8, float32 and float64) of this workload at 512^3")
-INSTRUCTIONS = {"retrieve": 2046510995}
-# Pipe utilisation (ncu --set full on the 320^3 case of this workload): the retrieval (k = 8)
-# and compression kernels are bound by instruction issue, not by HBM.  The float32 retrieval
-# figures are of the current kernel; the float64 ones of the kernel before the 32-bit decoding
-# of narrow brick pairs (11 % less time at k = 8 since, with the int -> double conversions off
-# the FP64 pipe); compression has since dropped a warp vote and some FP64 operations (2-4 %
-# less time; float64 9 %, its magnitude tests no longer compiling to FP64 adds), its figures
-# are of the kernel before that.
+INSTRUCTIONS = {"retrieve": 1143428190}
+# Pipe utilisation (ncu on the 320^3 case of this workload): the retrieval (k = 8) and
+# compression kernels are bound by instruction issue, not by HBM.
 PIPES = {"launch": "320^3, retrieval at k = 8, compression of 8 components",
-         "retrieve": {"alu": {"f32": 0.569, "f64": 0.574}, "fp64": {"f32": 0.0, "f64": 0.662},
-                      "issue_active": {"f32": 0.677, "f64": 0.604}},
-         "compress": {"alu": {"f32": 0.708, "f64": 0.598}, "fp64": {"f32": 0.0, "f64": 0.464},
-                      "issue_active": {"f32": 0.762, "f64": 0.584}},
-         "source": "ncu sm__inst_executed_pipe_{alu,fp64}.avg.pct_of_peak_sustained_active, "
-                   "smsp__issue_active.avg.pct_of_peak_sustained_active; compression figures from the "
-                   "kernel before its last changes (2-4 % less time since for float32, 9 % for float64, whose "
-                   "magnitude tests no longer compile to FP64 adds); float64 retrieval figures from the "
-                   "kernel before its 32-bit decoding of narrow brick pairs (11 % less time at k = 8 since)"}
+         "retrieve": {"alu": {"f32": 0.487, "f64": 0.463}, "fp64": {"f32": 0.0, "f64": 0.142},
+                      "issue_active": {"f32": 0.646, "f64": 0.556}},
+         "compress": {"alu": {"f32": 0.662, "f64": 0.507}, "fp64": {"f32": 0.0, "f64": 0.449},
+                      "issue_active": {"f32": 0.705, "f64": 0.475}},
+         "source": "ncu sm__inst_executed_pipe_alu.avg.pct_of_peak_sustained_active, "
+                   "sm__pipe_fp64_cycles_active.avg.pct_of_peak_sustained_active, "
+                   "smsp__issue_active.avg.pct_of_peak_sustained_active"}
 BATCH_WORKLOAD = ("64 float32 fields, half 2D with extents in [256, 4096], half 3D between 32^3 and "
                   "384x384x256 (not multiples of 4), half sums of Gaussians and half k^-5/3 spectra, 6 components "
                   "(tau_i = 1e-(i+1) * range)")
@@ -670,8 +663,8 @@ def run_batched(args, device):
                           "chunks_per_item": info["chunks_per_item"], "items_per_claim": info["items_per_claim"],
                           "ctas_per_sm_3d": info["ctas_per_sm"], "warps_per_cta_1d2d": info["warps_small"],
                           "one_kernel_for_both": bool(info["mixed"]),
-                          "candidates": "3D CTAs of 16 warps per SM {2, 1} x 1D/2D warps per CTA {4, 8, 16}, and "
-                                        "for 2 CTAs: 1D/2D warps {2, 4, 8, 16} x chunks per warp per item {1, 2} "
+                          "candidates": "3D CTAs of 4 warps per SM {6, 5} x 1D/2D warps per CTA {4, 8, 16}, and "
+                                        "for 6 CTAs: 1D/2D warps {2, 4, 8, 16} x chunks per warp per item {1, 2} "
                                         "(two kernels); one kernel for both with 1 or 2 chunks per warp; two items "
                                         "per claim or the fields in the given order for 3 shapes",
                           "candidate_ms": [round(v, 3) for v in info["candidate_ms"]],
