@@ -84,7 +84,7 @@ __device__ __forceinline__ void scan_segment(const uint32_t* __restrict__ in, ui
   // by warps first: 1024 threads' atomics on one word each took most of the 185
   // us of a batch's 384 segments (51 us now)
 #pragma unroll
-  for (int k = 0; k < 5; ++k) {  // (32 bits: 32 bricks a chunk, below 2^27 chunks)
+  for (int k = 0; k < 5; ++k) {  // (32 bits: at most 2048 a chunk, a warp has a 32nd of below 2^26 chunks)
     const unsigned x = __reduce_add_sync(0xffffffffu, my_cnt[k]);
     if (lane == 0 && x) atomicAdd(&cnt_s[k], (unsigned long long)x);
   }
