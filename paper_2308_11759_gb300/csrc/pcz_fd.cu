@@ -170,7 +170,7 @@ __device__ __noinline__ void vorticity_value(const T* __restrict__ u, const T* _
 
 // omega_z = v_x - u_y.  float64 is bound by the FP64 pipe (3 subtractions per
 // value at 2 lanes per SM and clock) next to HBM: 384 x 384 x 256 527 us ->
-// 267 us.
+// 236 us.
 template <typename T, bool POW2>
 __global__ void __launch_bounds__(kTileX * kTileY) k_vorticity_z(const T* __restrict__ u, const T* __restrict__ v,
                                                                  T* __restrict__ out, int nx, int ny, int nz,
@@ -277,13 +277,24 @@ __device__ __noinline__ void second_value(const T* __restrict__ w, T* __restrict
   out[i] = second_at<T>(w + i, c, n, s, hh);
 }
 
+// (float32: in line, since its multiplications cost nothing and a call's registers
+// and stack do: y and z 15 to 25 % slower)
+template <typename T>
+__device__ __forceinline__ void second_one(const T* __restrict__ w, T* __restrict__ out, int64_t i, int c, int n,
+                                           int64_t s, const Den<T>& hh) {
+  if constexpr (sizeof(T) == 4)
+    out[i] = second_at<T>(w + i, c, n, s, hh);
+  else
+    second_value<T>(w, out, i, c, n, s, hh);
+}
+
 // d2w/da2 along x (axis 0) or y (axis 1).
 template <typename T, bool POW2>
 __global__ void __launch_bounds__(kTileX * kTileY) k_second_xy(const T* __restrict__ w, T* __restrict__ out, int nx,
                                                                int ny, int nz, int zchunk, int axis, Den<T> hh) {
   if (axis == 0 && blockIdx.x == gridDim.x - 1) {
     x_ends(nx, ny, nz, zchunk, [&](int x, int y, int z) {
-      second_value<T>(w, out, ((int64_t)z * ny + y) * nx + x, x, nx, 1, hh);
+      second_one<T>(w, out, ((int64_t)z * ny + y) * nx + x, x, nx, 1, hh);
     });
     return;
   }
@@ -308,16 +319,16 @@ __global__ void __launch_bounds__(kTileX * kTileY) k_second_xy(const T* __restri
 #pragma unroll
       for (int j = 0; j < 4; ++j) out[i + j * plane] = second_fast<T, POW2>(fp[j], f0[j], fm[j], hh, rare);
       if (rare)
-        for (int j = 0; j < 4; ++j) second_value<T>(w, out, i + j * plane, cc, n, s, hh);
+        for (int j = 0; j < 4; ++j) second_one<T>(w, out, i + j * plane, cc, n, s, hh);
     }
   }
-  for (; z < c.z1; ++z) second_value<T>(w, out, i0 + (int64_t)(z - c.z0) * plane, cc, n, s, hh);
+  for (; z < c.z1; ++z) second_one<T>(w, out, i0 + (int64_t)(z - c.z0) * plane, cc, n, s, hh);
 }
 
 // d2w/dz2: the column's window w[z-1], w[z], w[z+1] stays in registers.
-// float64 384 x 384 x 256: 288 us -> 160 us.
+// float64 384 x 384 x 256: 288 us -> 158 us.
 template <typename T, bool POW2>
-__global__ void __launch_bounds__(kTileX * kTileY) k_second_z(const T* __restrict__ w, T* __restrict__ out, int nx,
+__global__ void __launch_bounds__(kTileX * kTileY, sizeof(T) == 4 && !POW2 ? 8 : 0) k_second_z(const T* __restrict__ w, T* __restrict__ out, int nx,
                                                               int ny, int nz, int zchunk, Den<T> hh) {
   const Column c = column(nx, ny, nz, zchunk);
   if (!c.ok) return;
@@ -325,11 +336,11 @@ __global__ void __launch_bounds__(kTileX * kTileY) k_second_z(const T* __restric
   const int64_t col = (int64_t)c.y * nx + c.x;
   int za = c.z0, zb = c.z1;  // the slice's interior planes [za, zb)
   if (za == 0) {             // the four-point ends
-    second_value<T>(w, out, col, 0, nz, plane, hh);
+    second_one<T>(w, out, col, 0, nz, plane, hh);
     za = 1;
   }
   if (zb == nz) {
-    second_value<T>(w, out, col + (int64_t)(nz - 1) * plane, nz - 1, nz, plane, hh);
+    second_one<T>(w, out, col + (int64_t)(nz - 1) * plane, nz - 1, nz, plane, hh);
     zb = nz - 1;
   }
   if (za >= zb) return;
@@ -345,14 +356,26 @@ __global__ void __launch_bounds__(kTileX * kTileY) k_second_z(const T* __restric
     bool rare = false;
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-      q[o + j * plane] = second_fast<T, POW2>(wp[j], w0, wm, hh, rare);
+      if constexpr (sizeof(T) == 4 && !POW2)
+        q[o + j * plane] = second_inner<T>(wp[j], w0, wm, hh);
+      else
+        q[o + j * plane] = second_fast<T, POW2>(wp[j], w0, wm, hh, rare);
       wm = w0;
       w0 = wp[j];
     }
     if (rare)
-      for (int j = 0; j < 4; ++j) second_value<T>(w, out, col + (int64_t)(z + j) * plane, z + j, nz, plane, hh);
+      for (int j = 0; j < 4; ++j) second_one<T>(w, out, col + (int64_t)(z + j) * plane, z + j, nz, plane, hh);
   }
-  for (; z < zb; ++z) second_value<T>(w, out, col + (int64_t)z * plane, z, nz, plane, hh);
+  for (; z < zb; ++z) {
+    if constexpr (sizeof(T) == 4) {
+      const T wp = __ldg(w + col + (int64_t)(z + 1) * plane);
+      out[col + (int64_t)z * plane] = second_inner<T>(wp, w0, wm, hh);
+      wm = w0;
+      w0 = wp;
+    } else {
+      second_one<T>(w, out, col + (int64_t)z * plane, z, nz, plane, hh);
+    }
+  }
 }
 
 template <typename T>
@@ -369,9 +392,20 @@ Den<T> make_den(double h, int twice) {
   return D;
 }
 
-// Grid of tiles, with z split so that about 16 CTAs per SM are launched.
-// ends: one more CTA along x, for the columns at the ends of x.
-dim3 fd_grid(int nx, int ny, int nz, bool ends, int* zchunk) {
+// CTAs launched per SM.  A kernel's last CTAs no longer fill the SMs (float64: the
+// FP64 pipe), so short slices of z keep that tail short; k_second_z reads 2 planes
+// more per slice, and the slices of k_vorticity_z4 are short already (a value
+// takes less than one load).  16 -> 64 and 128 CTAs per SM: float64 vorticity, 256
+// x 384 x 384, 268 -> 236 us (251 x 379 x 381: 269 -> 229), along y 175 -> 155;
+// float32 along y, 512^3, 250 -> 207 us; vorticity of 251 x 379 x 381 116 -> 88.
+constexpr int kPerSm32 = 64, kPerSm64 = 128, kPerSmVec4 = 24;
+
+// Grid of tiles, with z split so that about per_sm CTAs per SM are launched, in
+// chunks of a multiple of the 4 planes that a thread handles at once (the rest go
+// one by one).  Where that would take fewer planes, 16 CTAs per SM of at most 4:
+// a small field's time is one thread's chain of operations.  ends: one more CTA
+// along x, for the columns at the ends of x.
+dim3 fd_grid(int nx, int ny, int nz, bool ends, int per_sm, int* zchunk) {
   static const int sms = [] {  // once, thread-safe
     int dev = 0, n = 0;
     cudaGetDevice(&dev);
@@ -379,9 +413,12 @@ dim3 fd_grid(int nx, int ny, int nz, bool ends, int* zchunk) {
     return n > 0 ? n : 1;
   }();
   const int64_t tiles = (int64_t)((nx + kTileX - 1) / kTileX) * ((ny + kTileY - 1) / kTileY);
-  int64_t split = (16 * (int64_t)sms + tiles - 1) / tiles;
-  split = std::max<int64_t>(1, std::min<int64_t>(split, nz));
-  *zchunk = (int)((nz + split - 1) / split);
+  auto chunk = [&](int per) {
+    const int64_t split = std::max<int64_t>(1, std::min<int64_t>((per * (int64_t)sms + tiles - 1) / tiles, nz));
+    return (int)((nz + split - 1) / split);
+  };
+  const int zc = chunk(per_sm);
+  *zchunk = zc >= 4 ? (zc + 3) & ~3 : std::min(chunk(16), 4);
   const int gz = (nz + *zchunk - 1) / *zchunk;
   return dim3((unsigned)((nx + kTileX - 1) / kTileX + (ends ? 1 : 0)), (unsigned)((ny + kTileY - 1) / kTileY), (unsigned)gz);
 }
@@ -394,12 +431,12 @@ cudaError_t launch_fd_vorticity_z(int dtype, const void* u, const void* v, void*
   const dim3 block(kTileX, kTileY);
   const bool vec4 = dtype == 1 && nx % 4 == 0 && ((uintptr_t)u | (uintptr_t)v | (uintptr_t)out) % 16 == 0;
   if (vec4) {  // the tiles are 128 values wide
-    dim3 grid = fd_grid((int)(nx / 4), (int)ny, (int)nz, false, &zc);
+    dim3 grid = fd_grid((int)(nx / 4), (int)ny, (int)nz, false, kPerSmVec4, &zc);
     k_vorticity_z4<<<grid, block, 0, st>>>((const float*)u, (const float*)v, (float*)out, (int)nx, (int)ny, (int)nz,
                                            zc, make_den<float>(h, 1));
     return cudaGetLastError();
   }
-  const dim3 grid = fd_grid((int)nx, (int)ny, (int)nz, true, &zc);
+  const dim3 grid = fd_grid((int)nx, (int)ny, (int)nz, true, dtype == 1 ? kPerSm32 : kPerSm64, &zc);
   auto run = [&](auto one) {
     using T = decltype(one);
     const Den<T> D = make_den<T>(h, 1);
@@ -416,7 +453,7 @@ cudaError_t launch_fd_vorticity_z(int dtype, const void* u, const void* v, void*
 cudaError_t launch_fd_second(int dtype, const void* w, void* out, int64_t nx, int64_t ny, int64_t nz, int axis,
                              double h, cudaStream_t st) {
   int zc = 1;
-  const dim3 grid = fd_grid((int)nx, (int)ny, (int)nz, axis == 0, &zc);
+  const dim3 grid = fd_grid((int)nx, (int)ny, (int)nz, axis == 0, dtype == 1 ? kPerSm32 : kPerSm64, &zc);
   const dim3 block(kTileX, kTileY);
   auto run = [&](auto one) {
     using T = decltype(one);
