@@ -168,6 +168,17 @@ __device__ __noinline__ void vorticity_value(const T* __restrict__ u, const T* _
   out[i] = Ar<T>::sub(first_at<T>(v + i, x, nx, 1, h2), first_at<T>(u + i, y, ny, nx, h2));
 }
 
+template <typename T, bool POW2>
+__device__ __forceinline__ void vorticity_one(const T* __restrict__ u, const T* __restrict__ v, T* __restrict__ out,
+                                              int x, int y, int z, int nx, int ny, const Den<T>& h2) {
+  if constexpr (sizeof(T) == 8 && !POW2) {
+    const int64_t i = ((int64_t)z * ny + y) * nx + x;
+    out[i] = Ar<T>::sub(first_at<T>(v + i, x, nx, 1, h2), first_at<T>(u + i, y, ny, nx, h2));
+  } else {
+    vorticity_value<T>(u, v, out, x, y, z, nx, ny, h2);
+  }
+}
+
 // omega_z = v_x - u_y.  float64 is bound by the FP64 pipe (3 subtractions per
 // value at 2 lanes per SM and clock) next to HBM: 384 x 384 x 256 527 us ->
 // 236 us.
@@ -176,7 +187,7 @@ __global__ void __launch_bounds__(kTileX * kTileY) k_vorticity_z(const T* __rest
                                                                  T* __restrict__ out, int nx, int ny, int nz,
                                                                  int zchunk, Den<T> h2) {
   if (blockIdx.x == gridDim.x - 1) {
-    x_ends(nx, ny, nz, zchunk, [&](int x, int y, int z) { vorticity_value<T>(u, v, out, x, y, z, nx, ny, h2); });
+    x_ends(nx, ny, nz, zchunk, [&](int x, int y, int z) { vorticity_one<T, POW2>(u, v, out, x, y, z, nx, ny, h2); });
     return;
   }
   const Column c = column(nx, ny, nz, zchunk);
@@ -206,7 +217,7 @@ __global__ void __launch_bounds__(kTileX * kTileY) k_vorticity_z(const T* __rest
         for (int j = 0; j < 4; ++j) vorticity_value<T>(u, v, out, c.x, c.y, z + j, nx, ny, h2);
     }
   }
-  for (; z < c.z1; ++z) vorticity_value<T>(u, v, out, c.x, c.y, z, nx, ny, h2);
+  for (; z < c.z1; ++z) vorticity_one<T, POW2>(u, v, out, c.x, c.y, z, nx, ny, h2);
 }
 
 // omega_z = v_x - u_y for float32 rows whose length is a multiple of 4 (and
@@ -277,12 +288,13 @@ __device__ __noinline__ void second_value(const T* __restrict__ w, T* __restrict
   out[i] = second_at<T>(w + i, c, n, s, hh);
 }
 
-// (float32: in line, since its multiplications cost nothing and a call's registers
-// and stack do: y and z 15 to 25 % slower)
-template <typename T>
+// (In line for float32, whose multiplications cost nothing while a call's registers
+// and stack do: y and z 15 to 25 % slower.  Also in kernels built for the
+// division: small fields, where every value comes here, 10 % slower as calls.)
+template <typename T, bool POW2>
 __device__ __forceinline__ void second_one(const T* __restrict__ w, T* __restrict__ out, int64_t i, int c, int n,
                                            int64_t s, const Den<T>& hh) {
-  if constexpr (sizeof(T) == 4)
+  if constexpr (sizeof(T) == 4 || !POW2)
     out[i] = second_at<T>(w + i, c, n, s, hh);
   else
     second_value<T>(w, out, i, c, n, s, hh);
@@ -294,7 +306,7 @@ __global__ void __launch_bounds__(kTileX * kTileY) k_second_xy(const T* __restri
                                                                int ny, int nz, int zchunk, int axis, Den<T> hh) {
   if (axis == 0 && blockIdx.x == gridDim.x - 1) {
     x_ends(nx, ny, nz, zchunk, [&](int x, int y, int z) {
-      second_one<T>(w, out, ((int64_t)z * ny + y) * nx + x, x, nx, 1, hh);
+      second_one<T, POW2>(w, out, ((int64_t)z * ny + y) * nx + x, x, nx, 1, hh);
     });
     return;
   }
@@ -319,10 +331,10 @@ __global__ void __launch_bounds__(kTileX * kTileY) k_second_xy(const T* __restri
 #pragma unroll
       for (int j = 0; j < 4; ++j) out[i + j * plane] = second_fast<T, POW2>(fp[j], f0[j], fm[j], hh, rare);
       if (rare)
-        for (int j = 0; j < 4; ++j) second_one<T>(w, out, i + j * plane, cc, n, s, hh);
+        for (int j = 0; j < 4; ++j) second_one<T, POW2>(w, out, i + j * plane, cc, n, s, hh);
     }
   }
-  for (; z < c.z1; ++z) second_one<T>(w, out, i0 + (int64_t)(z - c.z0) * plane, cc, n, s, hh);
+  for (; z < c.z1; ++z) second_one<T, POW2>(w, out, i0 + (int64_t)(z - c.z0) * plane, cc, n, s, hh);
 }
 
 // d2w/dz2: the column's window w[z-1], w[z], w[z+1] stays in registers.
@@ -336,11 +348,11 @@ __global__ void __launch_bounds__(kTileX * kTileY, sizeof(T) == 4 && !POW2 ? 8 :
   const int64_t col = (int64_t)c.y * nx + c.x;
   int za = c.z0, zb = c.z1;  // the slice's interior planes [za, zb)
   if (za == 0) {             // the four-point ends
-    second_one<T>(w, out, col, 0, nz, plane, hh);
+    second_one<T, POW2>(w, out, col, 0, nz, plane, hh);
     za = 1;
   }
   if (zb == nz) {
-    second_one<T>(w, out, col + (int64_t)(nz - 1) * plane, nz - 1, nz, plane, hh);
+    second_one<T, POW2>(w, out, col + (int64_t)(nz - 1) * plane, nz - 1, nz, plane, hh);
     zb = nz - 1;
   }
   if (za >= zb) return;
@@ -364,7 +376,7 @@ __global__ void __launch_bounds__(kTileX * kTileY, sizeof(T) == 4 && !POW2 ? 8 :
       w0 = wp[j];
     }
     if (rare)
-      for (int j = 0; j < 4; ++j) second_one<T>(w, out, col + (int64_t)(z + j) * plane, z + j, nz, plane, hh);
+      for (int j = 0; j < 4; ++j) second_one<T, POW2>(w, out, col + (int64_t)(z + j) * plane, z + j, nz, plane, hh);
   }
   for (; z < zb; ++z) {
     if constexpr (sizeof(T) == 4) {
@@ -373,7 +385,7 @@ __global__ void __launch_bounds__(kTileX * kTileY, sizeof(T) == 4 && !POW2 ? 8 :
       wm = w0;
       w0 = wp;
     } else {
-      second_one<T>(w, out, col + (int64_t)z * plane, z, nz, plane, hh);
+      second_one<T, POW2>(w, out, col + (int64_t)z * plane, z, nz, plane, hh);
     }
   }
 }
