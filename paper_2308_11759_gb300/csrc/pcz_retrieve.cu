@@ -499,9 +499,9 @@ __device__ __forceinline__ void add_component(int how, const BlockMeta* bm, cons
   constexpr unsigned FULL = 0xffffffffu;
   const BlockMeta m = *bm;
   const int bq = lane >> 2, q = lane & 3;
-  const bool coded = m.mode == kModeCoded;
-  const int p = m.p, top = m.top, s = coded ? (int)m.s : 0;
-  const int nw = coded ? top - p + 1 : 0;  // planes with digits
+  const int p = m.p, top = m.top;
+  const int nw = m.mode == kModeCoded ? top - p + 1 : 0;  // planes with digits
+  const int s = nw > 0 ? (int)m.s : 0;  // (a CODED block without any may have a scale outside the others' range)
   const uint32_t areas = smem_addr(area);
   bool any = (how & 3) == kDecodeAny;
   if constexpr (WIDE) {
