@@ -97,6 +97,12 @@ template <typename T>
 __device__ __forceinline__ uint64_t* words_at(uint64_t* pool, uint64_t* spill, int at, int nw) {
   return at + nw <= kPool ? pool + at : spill + (at - (kPool - Fmt<T>::P));
 }
+// Whether its nw words lie in one of the two (debug builds check it).
+template <typename T>
+__device__ __forceinline__ bool words_in(int at, int nw) {
+  const int64_t end = (int64_t)at - (kPool - Fmt<T>::P) + nw;
+  return at >= 0 && nw >= 0 && nw <= Fmt<T>::P && (at + nw <= kPool || end <= (int64_t)spill_words_per_cta<T>());
+}
 
 // A plane in which coefficients may turn significant (R11): n < 64 verbatim bits
 // at pos, then the group-test part, a byte at a time through the table.  The
@@ -187,6 +193,12 @@ __device__ __forceinline__ int cached_level(const BoxJob& J, int64_t b) {
   return lv <= J.k ? lv : 0;
 }
 
+// Whether a block has planes, of which a short decoding reads the word at
+// `last` and the `more` before it: within the pool and its pads (debug builds check it).
+__device__ __forceinline__ bool from_pool(int nw, int last, int more) {
+  return nw > 0 && PCZ_CHECK(last - more >= -kPoolPad && last < kPool + kPoolPad, 3);
+}
+
 // How 8 blocks (one component of a rebuild's bricks) are decoded: the largest of
 // theirs, and whether one is RAW.
 enum : int { kDecodeNone = 0, kDecodeFloat8 = 1, kDecodeInt16 = 2, kDecodeAny = 3, kHasRaw = 4 };
@@ -264,7 +276,7 @@ __device__ __forceinline__ void parse_task(const BoxJob& J, unsigned int* err, i
   int at = 0;
   if (lane == 31) at = atomicAdd(used, incl);
   at = __shfl_sync(0xffffffffu, at, 31) + incl - nw;
-  if (coded) ok = parse_planes(br, pos, end, nw, words_at<T>(pool, spill, at, nw), lut);
+  if (coded) ok = PCZ_CHECK(words_in<T>(at, nw), 3) && parse_planes(br, pos, end, nw, words_at<T>(pool, spill, at, nw), lut);
   if (!ok) {
     atomicOr(err, 1u);
     mode = kModeZero;
@@ -425,7 +437,7 @@ __device__ __noinline__ void add_any(const BlockMeta* bm, uint64_t* pool, uint64
   const int bq = lane >> 2, q = lane & 3;
   const bool coded = m.mode == kModeCoded;
   const int p = m.p, top = m.top, s = coded ? (int)m.s : 0;
-  const int nw = coded ? top - p + 1 : 0;
+  const int nw = coded && PCZ_CHECK(words_in<T>(m.at, top - p + 1), 3) ? top - p + 1 : 0;
   uint4* zw = area + LineSet::at(bq, 0, q);
   uint4* yw = area + LineSet::at(bq, q, 0);
   uint32_t place[4];
@@ -524,7 +536,7 @@ __device__ __forceinline__ void add_component(int how, const BlockMeta* bm, cons
   if ((how & 3) == kDecodeFloat8) {
     const int base = max(top, 7) - 7;
     const uint32_t keep = nw > 0 ? ((1u << nw) - 1u) << (p - base) : 0u;
-    const uint16_t* pc = reinterpret_cast<const uint16_t*>(pool + (nw > 0 ? m.at + top - base : 7)) + q;  // plane base
+    const uint16_t* pc = reinterpret_cast<const uint16_t*>(pool + (from_pool(nw, m.at + top - base, 7) ? m.at + top - base : 7)) + q;  // plane base
     uint32_t a[4];
 #pragma unroll
     for (int j = 0; j < 4; ++j) a[j] = (uint32_t)pc[-4 * j] | ((uint32_t)pc[-4 * (j + 4)] << 16);
@@ -564,7 +576,7 @@ __device__ __forceinline__ void add_component(int how, const BlockMeta* bm, cons
   } else if ((how & 3) == kDecodeInt16) {
     const int base = max(top, 15) - 15;
     const uint32_t keep = nw > 0 ? ((1u << nw) - 1u) << (p - base) : 0u;
-    const uint16_t* pc = reinterpret_cast<const uint16_t*>(pool + (nw > 0 ? m.at + top - base : 15)) + q;
+    const uint16_t* pc = reinterpret_cast<const uint16_t*>(pool + (from_pool(nw, m.at + top - base, 15) ? m.at + top - base : 15)) + q;
     uint32_t a[8];
 #pragma unroll
     for (int j = 0; j < 8; ++j) a[j] = (uint32_t)pc[-4 * j] | ((uint32_t)pc[-4 * (j + 8)] << 16);
