@@ -427,6 +427,7 @@ BoxJob make_job(const pc_streams* s, int k0, int k, const int64_t lo[3], const i
   J.nbox = J.bn[0] * J.bn[1] * J.bn[2];
   J.k0 = k0;
   J.k = k;
+  if (s->ndims == 3) retrieve_split(s->words + k0, k - k0, s->nbricks, &J.round, &J.unit_bricks);
   if (J.nbox < (1ll << 32)) {
     J.dv_bn0 = div_magic((uint64_t)J.bn[0]);
     J.dv_bn1 = div_magic((uint64_t)J.bn[1]);
@@ -435,18 +436,17 @@ BoxJob make_job(const pc_streams* s, int k0, int k, const int64_t lo[3], const i
   return J;
 }
 
-// Cuts the jobs of one launch into units (retrieve_split on the launch's brick
-// total) and places them one after the other; returns the units.  Units
-// of 1D/2D jobs are bricks.
+// Cuts the jobs of one launch into units (retrieve_split's, or smaller ones where
+// the launch's bricks are few) and places them one after the other; returns the
+// units.  Units of 1D/2D jobs are bricks.
 int64_t place_job_list(BoxJob* jobs, int nj, int dtype, int ndims) {
   int64_t bricks = 0, units = 0;
   for (int j = 0; j < nj; ++j) bricks += jobs[j].nbox;
   for (int j = 0; j < nj; ++j) {
     BoxJob& J = jobs[j];
     J.unit_begin = units;
-    retrieve_split(dtype, J.k - J.k0, bricks, &J.round, &J.unit_bricks);
-    const int64_t ub = J.unit_bricks;
-    units += ndims == 3 ? (J.nbox + ub - 1) / ub : J.nbox;
+    if (ndims == 3) J.unit_bricks = retrieve_unit(dtype, J.unit_bricks, bricks);
+    units += ndims == 3 ? (J.nbox + J.unit_bricks - 1) / J.unit_bricks : J.nbox;
   }
   return units;
 }

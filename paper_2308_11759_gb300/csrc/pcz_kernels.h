@@ -165,11 +165,13 @@ uint32_t check_word_batch(int reset);
 // Sets the message pc_last_error() returns on this thread.
 void set_last_error(const char* msg);
 
-// CTAs of a persistent retrieval launch over nunits units, how a job of ncomp
-// components is split in a launch of `bricks` bricks, and the spill words a
-// launch of grid CTAs needs.
+// CTAs of a persistent retrieval launch over nunits units; how a 3D job is split
+// whose ncomp components have `words` payload words over a field of nbricks
+// bricks, and the unit it gets in a launch of `bricks` bricks; and the spill words
+// a launch of grid CTAs needs.
 int retrieve_grid(int dtype, int ndims, int64_t nunits);
-void retrieve_split(int dtype, int ncomp, int64_t bricks, int* round, int* unit_bricks);
+void retrieve_split(const uint64_t* words, int ncomp, int64_t nbricks, int* round, int* unit_bricks);
+int retrieve_unit(int dtype, int unit_bricks, int64_t bricks);
 size_t retrieve_spill_words(int dtype, int ndims, int grid);
 
 // Finite-difference derivatives (pcz_fd.cu): omega_z = v_x - u_y and the

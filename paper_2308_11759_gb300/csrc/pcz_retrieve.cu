@@ -424,8 +424,11 @@ __device__ __forceinline__ double fixed_add(double sum, int32_t i, int sh) {
   return __longlong_as_double(__double_as_longlong(sum) + (int64_t)hi * (int64_t)(1 << min(sh, 30)));
 }
 
-// The decoding of any planes, and RAW blocks: rare, and out of line, so that the
-// common path stays short.  xt: the lane's partial sums.
+// The decoding of any planes, out of line, so that the common path stays short.  xt:
+// the lane's partial sums.  Components of more than 16 planes (steps of 12 bits and
+// more) come here with every brick.  Two aligned windows instead of four, and 32-bit
+// integers up to 20 planes: 256^3 float64, 2 components of 20 and 17 words a brick
+// 347 -> 312 us, of 17 and 13 290 -> 235.
 template <typename T>
 __device__ __noinline__ void add_any(const BlockMeta* bm, uint64_t* pool, uint64_t* spill, uint4* area, int lane, T* xt) {
   using F = Fmt<T>;
@@ -443,36 +446,64 @@ __device__ __noinline__ void add_any(const BlockMeta* bm, uint64_t* pool, uint64
   uint32_t place[4];
 #pragma unroll
   for (int z = 0; z < 4; ++z) place[z] = coded_places(kRank3r.pos, q, z);
-  // any planes, 16 at a time from plane 0, each 16 digits a half-word of the
-  // coefficients in coded order
-  const uint32_t stride = 64u * sizeof(T) + 16u;
-  unsigned char* dig = reinterpret_cast<unsigned char*>(area) + stride * bq;
+  // 16 planes at a time from plane `base`, 16 digits a half-word of the coefficients
+  // in coded order.  Float64 blocks of at most 32 planes, aligned to the highest, take
+  // two such windows and 32-bit digits: d stands for ((d ^ M) - M) * 2^base with M =
+  // NBM >> base (as in add_component; 32 bits of M suffice).
+  const bool two = WIDE && __all_sync(FULL, nw <= 32);
+  const int base = two ? max(top, 31) - 31 : 0;
+  const int bytes = two ? 4 : (int)sizeof(T);
+  unsigned char* dig = reinterpret_cast<unsigned char*>(area) + (64 * bytes + 16) * bq;
   const uint64_t* words = words_at<T>(pool, spill, m.at, nw);
 #pragma unroll 1
-  for (int h = 0; h < F::P / 16; ++h) {
+  for (int h = 0; h < 8 * bytes / 16; ++h) {
     auto plane = [&](int pl) {
       if (nw <= 0 || pl < p || pl > top) return 0u;
       return (uint32_t)reinterpret_cast<const uint16_t*>(words + (top - pl))[q];
     };
     uint32_t a[8];
 #pragma unroll
-    for (int j = 0; j < 8; ++j) a[j] = plane(16 * h + j) | (plane(16 * h + j + 8) << 16);
+    for (int j = 0; j < 8; ++j) a[j] = plane(base + 16 * h + j) | (plane(base + 16 * h + j + 8) << 16);
     untranspose16(a);
 #pragma unroll
     for (int i = 0; i < 8; ++i) {  // ranks i and i + 8 of the lane's 16, at their places
-      uint16_t* e = reinterpret_cast<uint16_t*>(dig + (16 * q + 4 * (i & 3) + 2 * (i >> 2)) * sizeof(T)) + h;
+      uint16_t* e = reinterpret_cast<uint16_t*>(dig + (16 * q + 4 * (i & 3) + 2 * (i >> 2)) * bytes) + h;
       e[0] = (uint16_t)a[i];
-      e[sizeof(T) / 2] = (uint16_t)(a[i] >> 16);
+      e[bytes / 2] = (uint16_t)(a[i] >> 16);
     }
   }
   __syncwarp();
-  S r[16];
+  auto digits = [&](int k) { return dig + ((place[k >> 2] >> (8 * (k & 3))) & 0xffu) * bytes; };
+  const bool common = __all_sync(FULL, WIDE ? s >= -960 && s <= 1022 : s >= -127 && s <= 126);
+  if constexpr (WIDE) {
+    // at most 20 planes: in 32-bit integers, as add_component's 16
+    if (common && __all_sync(FULL, nw <= 0 || (nw <= 20 && p >= 6 && top <= 58))) {
+      const int low = max(top, 19) - 19;
+      const uint32_t M = (uint32_t)(F::NBM >> low);
+      int32_t r[16];
 #pragma unroll
-  for (int k = 0; k < 16; ++k)
-    r[k] = nb_inv<T>(*reinterpret_cast<const U*>(dig + ((place[k >> 2] >> (8 * (k & 3))) & 0xffu) * sizeof(T)));
+      for (int k = 0; k < 16; ++k)
+        r[k] = (int32_t)((((*reinterpret_cast<const uint32_t*>(digits(k)) >> (low - base)) ^ M) - M) << 6);
+      __syncwarp();
+      lift_inv_bricks<int32_t>(r, zw, yw, LineSet::kVectors);
+      const uint32_t eb = (uint32_t)(1053 + (low - 6) - s) << 20;
+#pragma unroll
+      for (int k = 0; k < 16; ++k) xt[k] = F::add(xt[k], scaled_i32_to_f64(r[k], eb));
+      return;
+    }
+  }
+  S r[16];
+  if (two) {
+    const uint32_t M = (uint32_t)(F::NBM >> base);
+#pragma unroll
+    for (int k = 0; k < 16; ++k)
+      r[k] = (S)(((int64_t)(*reinterpret_cast<const uint32_t*>(digits(k)) ^ M) - (int64_t)M) << base);
+  } else {
+#pragma unroll
+    for (int k = 0; k < 16; ++k) r[k] = nb_inv<T>(*reinterpret_cast<const U*>(digits(k)));
+  }
   __syncwarp();
   lift_inv_bricks<S>(r, zw, yw, LineSet::kVectors);
-  const bool common = __all_sync(FULL, WIDE ? s >= -960 && s <= 1022 : s >= -127 && s <= 126);
 #pragma unroll
   for (int y = 0; y < 4; ++y) {
     T xi[4];
@@ -764,18 +795,34 @@ static int retrieve_grid_t(int64_t nunits) {
   return (int)(nunits < g ? (nunits > 0 ? nunits : 1) : g);
 }
 
-// How a job of ncomp components is decoded in a launch of `bricks` bricks: in
-// rounds of equal size of at most kRoundTasks components, units of so many
-// bricks that a round has up to kRoundTasks warp tasks (4 where there is one
-// component: its first planes are many) -- unless the units would then not fill
-// the GPU.
-void retrieve_split(int dtype, int ncomp, int64_t bricks, int* round, int* unit_bricks) {
+// How a job of ncomp components is decoded: in rounds of equal size of at most
+// kRoundTasks components, units of so many bricks that a round has up to
+// kRoundTasks warp tasks (4 where there is one component: its first planes are
+// many).  Two or three components take fewer bricks, but no fewer than 3 tasks,
+// where their blocks' plane words -- nearly the payload's words a brick -- would
+// otherwise not fit in the pool: blocks past it take the decoding of any planes
+// (192^3 float64, 2 components of 17 and 13 words 169 -> 139 us, 3 of 17, 13 and 13
+// 211 -> 161; float32, 2 of 21 and 10 113 -> 87).  One component gains or loses
+// little (0 to 10 %).
+void retrieve_split(const uint64_t* words, int ncomp, int64_t nbricks, int* round, int* unit_bricks) {
   const int rounds = std::max((ncomp + kRoundTasks - 1) / kRoundTasks, 1);
   *round = std::max((ncomp + rounds - 1) / rounds, 1);
   int sets = *round == 1 ? 4 : std::max(kRoundTasks / *round, 1);
+  if (rounds > 1) sets = 1;
+  if (*round > 1) {
+    double per = 0;  // a brick's words
+    for (int i = 0; i < *round; ++i) per += (double)words[i] / (double)nbricks;
+    while ((sets - 1) * *round >= 3 && 32 * sets * per > kPool) --sets;
+  }
+  *unit_bricks = 32 * sets;
+}
+
+// The unit of a job in a launch of `bricks` bricks: smaller ones where the units
+// would otherwise not fill the GPU.
+int retrieve_unit(int dtype, int unit_bricks, int64_t bricks) {
   const int64_t fit = dtype == 1 ? retrieve_grid_t<float>(INT64_MAX) : retrieve_grid_t<double>(INT64_MAX);
-  while (sets > 1 && bricks < fit * 32 * sets) --sets;
-  *unit_bricks = 32 * (rounds > 1 ? 1 : sets);
+  while (unit_bricks > 32 && bricks < fit * unit_bricks) unit_bricks -= 32;
+  return unit_bricks;
 }
 
 int retrieve_grid(int dtype, int ndims, int64_t nunits) {

@@ -96,3 +96,45 @@ def test_coded_blocks_without_planes(dtype, log_tau):
         got = st.retrieve(k=k).cpu().numpy()
         assert np.array_equal(got.view(np.uint8), want[k].view(np.uint8))
     st.close()
+
+
+# Every decoding of the 3D retrieval -- 8, 16, 20 and 32 planes aligned to the
+# highest, and any -- with digits up to the largest, whose values wrap as the
+# oracle's do, at scales on both sides of the common range: 8 blocks of one kind
+# together, then the same blocks in any order
+@pytest.mark.parametrize("dtype,log_tau", [(np.float32, 0), (np.float32, -112), (np.float32, 100), (np.float64, 0),
+                                           (np.float64, -1000), (np.float64, 968)])
+def test_blocks_of_any_planes(dtype, log_tau):
+    import paper_2308_11759_gb300 as P
+
+    rng = np.random.default_rng(37)
+    width = PLANES[dtype]
+    blocks = []
+    for p in range(width):
+        emax = width - 8 - (p + 4 - log_tau)
+        if not EXP_MIN[dtype] <= emax <= EXP_MAX[dtype]:
+            continue
+        assert _lowest(dtype, log_tau, emax, 0)[1] == p
+        for planes in (1, 7, 8, 9, 15, 16, 17, 19, 20, 21, 31, 32, 33, 47, 64):
+            if p + planes > width:
+                continue
+            for i in range(8):
+                few = 64 if i % 2 else 3  # (a few coefficients only: blocks that do not wrap)
+                u = [(int(rng.integers(0, 1 << 63)) * 2 + int(rng.integers(0, 2))) % (1 << planes) << p
+                     if r < few else 0 for r in range(64)]
+                u[int(rng.integers(0, few))] |= 1 << (p + planes - 1)
+                blocks.append(_block(dtype, log_tau, emax, 0, u))
+    assert len(blocks) > 300
+    blocks += [blocks[i] for i in rng.permutation(len(blocks))]
+    shape, tau = (4, 4, 4 * len(blocks)), [2.0 ** log_tau]
+    x = torch.zeros(shape, dtype=torch.float32 if dtype == np.float32 else torch.float64, device="cuda")
+    st = P.Streams.deserialize(_serialized(P.compress(x, tau).serialize()[:64], tau, [blocks]))
+    want = np.empty(shape, dtype)
+    for b, bits in enumerate(blocks):
+        words = np.zeros((1, 160), dtype=np.uint64)
+        w = O.str_to_bits(bits)[0]
+        words[0, :len(w)] = w
+        want[:, :, 4 * b:4 * b + 4] = O.decode_brick(dtype, 3, tau, 1, words, np.array([len(bits)])).reshape(4, 4, 4)
+    got = st.retrieve(k=1).cpu().numpy()
+    assert np.array_equal(got.view(np.uint8), want.view(np.uint8))
+    st.close()
