@@ -133,6 +133,12 @@ __device__ __forceinline__ T second_at(const T* __restrict__ p, int c, int n, in
 
 constexpr int kTileX = 32, kTileY = 8;
 
+// CTAs per SM that k_vorticity_z and k_second_z are built for.  float32 is bound by
+// the loads in flight and takes all 64 warps of an SM at 32 registers a thread:
+// vorticity of 4095 x 4093 (one plane), 2h a power of two, 115 -> 90 us.
+template <typename T>
+constexpr int kFdCtas = sizeof(T) == 4 ? 8 : 0;
+
 // Thread (x, y) of a tile: its column and slice [z0, z1) of z.
 struct Column {
   int x, y, z0, z1;
@@ -168,10 +174,12 @@ __device__ __noinline__ void vorticity_value(const T* __restrict__ u, const T* _
   out[i] = Ar<T>::sub(first_at<T>(v + i, x, nx, 1, h2), first_at<T>(u + i, y, ny, nx, h2));
 }
 
+// (In line except for float64 powers of two, as second_one: a call took 4095 x 4093
+// float32, where every value comes here, from 122 to 187 us; now 103.)
 template <typename T, bool POW2>
 __device__ __forceinline__ void vorticity_one(const T* __restrict__ u, const T* __restrict__ v, T* __restrict__ out,
                                               int x, int y, int z, int nx, int ny, const Den<T>& h2) {
-  if constexpr (sizeof(T) == 8 && !POW2) {
+  if constexpr (sizeof(T) == 4 || !POW2) {
     const int64_t i = ((int64_t)z * ny + y) * nx + x;
     out[i] = Ar<T>::sub(first_at<T>(v + i, x, nx, 1, h2), first_at<T>(u + i, y, ny, nx, h2));
   } else {
@@ -183,9 +191,10 @@ __device__ __forceinline__ void vorticity_one(const T* __restrict__ u, const T* 
 // value at 2 lanes per SM and clock) next to HBM: 384 x 384 x 256 527 us ->
 // 236 us.
 template <typename T, bool POW2>
-__global__ void __launch_bounds__(kTileX * kTileY) k_vorticity_z(const T* __restrict__ u, const T* __restrict__ v,
-                                                                 T* __restrict__ out, int nx, int ny, int nz,
-                                                                 int zchunk, Den<T> h2) {
+__global__ void __launch_bounds__(kTileX * kTileY, kFdCtas<T>) k_vorticity_z(const T* __restrict__ u,
+                                                                              const T* __restrict__ v,
+                                                                              T* __restrict__ out, int nx, int ny,
+                                                                              int nz, int zchunk, Den<T> h2) {
   if (blockIdx.x == gridDim.x - 1) {
     x_ends(nx, ny, nz, zchunk, [&](int x, int y, int z) { vorticity_one<T, POW2>(u, v, out, x, y, z, nx, ny, h2); });
     return;
@@ -196,13 +205,15 @@ __global__ void __launch_bounds__(kTileX * kTileY) k_vorticity_z(const T* __rest
   const int64_t i0 = ((int64_t)c.z0 * ny + c.y) * nx + c.x;
   int z = c.z0;
   if (c.y > 0 && c.y < ny - 1) {
-    // interior column: the loads of 4 planes are issued before any is used
+    // interior column: the loads of 4 planes are issued before any is used (of 2
+    // for float32 divisions, which need the registers: 512 x 512 x 511 361 -> 324 us)
     using A = Ar<T>;
-    for (; z + 4 <= c.z1; z += 4) {
+    constexpr int N = sizeof(T) == 4 && !POW2 ? 2 : 4;
+    for (; z + N <= c.z1; z += N) {
       const int64_t i = i0 + (int64_t)(z - c.z0) * plane;
-      T vp[4], vm[4], up[4], um[4];
+      T vp[N], vm[N], up[N], um[N];
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
+      for (int j = 0; j < N; ++j) {
         vp[j] = __ldg(v + i + j * plane + 1);
         vm[j] = __ldg(v + i + j * plane - 1);
         up[j] = __ldg(u + i + j * plane + nx);
@@ -210,11 +221,11 @@ __global__ void __launch_bounds__(kTileX * kTileY) k_vorticity_z(const T* __rest
       }
       bool rare = false;
 #pragma unroll
-      for (int j = 0; j < 4; ++j)
+      for (int j = 0; j < N; ++j)
         out[i + j * plane] = A::sub(h2.template fast<POW2>(A::sub(vp[j], vm[j]), rare),
                                     h2.template fast<POW2>(A::sub(up[j], um[j]), rare));
       if (rare)
-        for (int j = 0; j < 4; ++j) vorticity_value<T>(u, v, out, c.x, c.y, z + j, nx, ny, h2);
+        for (int j = 0; j < N; ++j) vorticity_value<T>(u, v, out, c.x, c.y, z + j, nx, ny, h2);
     }
   }
   for (; z < c.z1; ++z) vorticity_one<T, POW2>(u, v, out, c.x, c.y, z, nx, ny, h2);
@@ -340,8 +351,9 @@ __global__ void __launch_bounds__(kTileX * kTileY) k_second_xy(const T* __restri
 // d2w/dz2: the column's window w[z-1], w[z], w[z+1] stays in registers.
 // float64 384 x 384 x 256: 288 us -> 158 us.
 template <typename T, bool POW2>
-__global__ void __launch_bounds__(kTileX * kTileY, sizeof(T) == 4 && !POW2 ? 8 : 0) k_second_z(const T* __restrict__ w, T* __restrict__ out, int nx,
-                                                              int ny, int nz, int zchunk, Den<T> hh) {
+__global__ void __launch_bounds__(kTileX * kTileY, kFdCtas<T>) k_second_z(const T* __restrict__ w, T* __restrict__ out,
+                                                                          int nx, int ny, int nz, int zchunk,
+                                                                          Den<T> hh) {
   const Column c = column(nx, ny, nz, zchunk);
   if (!c.ok) return;
   const int64_t plane = (int64_t)nx * ny;
@@ -405,19 +417,21 @@ Den<T> make_den(double h, int twice) {
 }
 
 // CTAs launched per SM.  A kernel's last CTAs no longer fill the SMs (float64: the
-// FP64 pipe), so short slices of z keep that tail short; k_second_z reads 2 planes
-// more per slice, and the slices of k_vorticity_z4 are short already (a value
-// takes less than one load).  16 -> 64 and 128 CTAs per SM: float64 vorticity, 256
-// x 384 x 384, 268 -> 236 us (251 x 379 x 381: 269 -> 229), along y 175 -> 155;
-// float32 along y, 512^3, 250 -> 207 us; vorticity of 251 x 379 x 381 116 -> 88.
+// FP64 pipe), so short slices of z keep that tail short; the slices of
+// k_vorticity_z4 are short already (a value takes less than one load).  16 -> 64 and
+// 128 CTAs per SM: float64 vorticity, 256 x 384 x 384, 268 -> 236 us (251 x 379 x
+// 381: 269 -> 229), along y 175 -> 155; float32 along y, 512^3, 250 -> 207 us;
+// vorticity of 251 x 379 x 381 116 -> 88.
 constexpr int kPerSm32 = 64, kPerSm64 = 128, kPerSmVec4 = 24;
 
 // Grid of tiles, with z split so that about per_sm CTAs per SM are launched, in
 // chunks of a multiple of the 4 planes that a thread handles at once (the rest go
 // one by one).  Where that would take fewer planes, 16 CTAs per SM of at most 4:
-// a small field's time is one thread's chain of operations.  ends: one more CTA
-// along x, for the columns at the ends of x.
-dim3 fd_grid(int nx, int ny, int nz, bool ends, int per_sm, int* zchunk) {
+// a small field's time is one thread's chain of operations.  But no slice takes
+// fewer planes than `least` where 16 CTAs per SM are reached with more: k_second_z
+// reads 2 planes more per slice (8 x 1501 x 1503 float32 41.7 -> 35 us with one
+// slice).  ends: one more CTA along x, for the columns at the ends of x.
+dim3 fd_grid(int nx, int ny, int nz, bool ends, int per_sm, int* zchunk, int least = 4) {
   static const int sms = [] {  // once, thread-safe
     int dev = 0, n = 0;
     cudaGetDevice(&dev);
@@ -430,7 +444,8 @@ dim3 fd_grid(int nx, int ny, int nz, bool ends, int per_sm, int* zchunk) {
     return (int)((nz + split - 1) / split);
   };
   const int zc = chunk(per_sm);
-  *zchunk = zc >= 4 ? (zc + 3) & ~3 : std::min(chunk(16), 4);
+  const int most = chunk(16);
+  *zchunk = std::max(zc >= 4 ? (zc + 3) & ~3 : std::min(most, 4), std::min(most, least));
   const int gz = (nz + *zchunk - 1) / *zchunk;
   return dim3((unsigned)((nx + kTileX - 1) / kTileX + (ends ? 1 : 0)), (unsigned)((ny + kTileY - 1) / kTileY), (unsigned)gz);
 }
@@ -465,7 +480,8 @@ cudaError_t launch_fd_vorticity_z(int dtype, const void* u, const void* v, void*
 cudaError_t launch_fd_second(int dtype, const void* w, void* out, int64_t nx, int64_t ny, int64_t nz, int axis,
                              double h, cudaStream_t st) {
   int zc = 1;
-  const dim3 grid = fd_grid((int)nx, (int)ny, (int)nz, axis == 0, dtype == 1 ? kPerSm32 : kPerSm64, &zc);
+  const dim3 grid = fd_grid((int)nx, (int)ny, (int)nz, axis == 0, dtype == 1 ? kPerSm32 : kPerSm64, &zc,
+                            dtype == 1 && axis == 2 ? 16 : 4);
   const dim3 block(kTileX, kTileY);
   auto run = [&](auto one) {
     using T = decltype(one);
