@@ -466,9 +466,10 @@ __device__ __forceinline__ void compress_small_chunk(const CompressParams& P, in
 }
 
 // Retrieval of brick g (box order) of job J by one thread: components
-// k0+1..k parsed and rebuilt in ascending order and summed into x~
-// (Algorithm 2).  No warp-collective operations.  tokens: the CTA's byte table
-// of the group-test part (kTokens).
+// k0+1..k (at least one) parsed and rebuilt in ascending order and summed into x~
+// (Algorithm 2).  No warp-collective operations.  tokens: the CTA's byte table of the
+// group-test part (kTokens), there once ready() returns (false: this thread has no
+// brick of its own); 1D requests the first block's bits before.
 //
 // A plane takes one look at the stream (at most 33 bits) and, while
 // coefficients turn significant, a table step per byte; 8 planes at a time are
@@ -476,9 +477,9 @@ __device__ __forceinline__ void compress_small_chunk(const CompressParams& P, in
 // plane.  With planes scattered bit by bit into the coefficients and a loop over
 // tokens it took 2877 warp instructions per 32 float32 2D bricks and component,
 // now 1244; 4096^2 float32, k = 6: 659 -> 284 us.
-template <typename T, int D>
+template <typename T, int D, typename Ready>
 __device__ __forceinline__ void retrieve_small_brick(const BoxJob& J, int write, unsigned int* err, int64_t g,
-                                                     const uint32_t* tokens) {
+                                                     const uint32_t* tokens, Ready ready) {
   using F = Fmt<T>;
   using U = typename F::U;
   using S = typename F::S;
@@ -505,13 +506,18 @@ __device__ __forceinline__ void retrieve_small_brick(const BoxJob& J, int write,
       xt[k] = out[(k >> 2) * ext0 + (k & 3)];  // the partial sum so far
   }
   const int64_t chunk = b / kChunk;
-  for (int j = J.k0; j < J.k; ++j) {  // Algorithm 2: x~ += D(y_j)
-    const CompDesc& cd = J.comp[j];
+  uint32_t blen, pos;
+  BlockBits br;  // positions from the start of the block's first word
+  auto block = [&](const CompDesc& cd) {
     const uint64_t off = cd.chunk_word[chunk] * 64ull + cd.brick_off[b];
-    const uint32_t blen = cd.brick_len[b];
-    BlockBits br;  // positions from the start of the block's first word
+    blen = cd.brick_len[b];
     br.init(cd.payload, cd.nwords, off);
-    uint32_t pos = (uint32_t)(off & 63u);
+    pos = (uint32_t)(off & 63u);
+  };
+  if constexpr (D == 1) block(J.comp[J.k0]);  // (2D has no registers for it: k = 6 2 % slower)
+  if (!ready()) return;
+  for (int j = J.k0; j < J.k; ++j) {  // Algorithm 2: x~ += D(y_j)
+    if (D == 2 || j > J.k0) block(J.comp[j]);
     const uint32_t end = pos + blen;
     const uint64_t v = br.peek(pos);
     const int mode = (int)(v & 3ull);
@@ -533,7 +539,7 @@ __device__ __forceinline__ void retrieve_small_brick(const BoxJob& J, int write,
       ok = emax >= F::EMIN && emax <= EMAXT;
       if (ok) {
         const int s = Q - emax;
-        const int p = min(max(cd.L + s - C - esc, 0), F::P);
+        const int p = min(max(J.comp[j].L + s - C - esc, 0), F::P);
         pos += HDR;
         int top = F::P - 1;  // highest plane with a significant coefficient; planes above it are a 0 test bit each
         while (top >= p) {

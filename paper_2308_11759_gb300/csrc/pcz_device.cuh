@@ -716,7 +716,7 @@ struct BlockBits {
 // to and including the closing test bit, minus 1.
 constexpr int kTokLut = 512;  // entries (2 states x 256 bytes)
 
-struct TokenTable {
+struct alignas(16) TokenTable {
   uint32_t entry[kTokLut];
 };
 constexpr TokenTable make_tokens() {
