@@ -23,7 +23,8 @@
  *    computation), except that a retrieval output of 32 MiB or more in
  *    pinned memory is decoded into device staging slabs of whole brick
  *    layers that the copy engines move to the host while the next slab
- *    decodes.  Results in pinned host memory are complete in stream order,
+ *    decodes, and a smaller one of 2 MiB or more may be decoded into device
+ *    memory and copied.  Results in pinned host memory are complete in stream order,
  *    as after a cudaMemcpyAsync: synchronise cuda_stream before reading them.
  *    Pageable host memory is copied through the same stream, and such calls
  *    return with the data in place.

@@ -818,6 +818,21 @@ static pc_status retrieve_pinned_slabs(const pc_streams* s, int k0, int k, const
   return PC_OK;
 }
 
+// Whether a 3D box in pinned host memory (below the slabs' size) is decoded into
+// device memory and copied, rather than written (and read, when refining) in place.
+// In place, a store that fills only part of a 32-byte sector crosses the link on its
+// own: rows that are not whole 16-byte words, and float64, whose lanes store a line
+// in halves.  float64, in place / copied: 128 x 127 x 129, k = 4 343 / 142 us,
+// refining from 2 to 4 329 / 224; 128^3 165 / 139 and 212 / 220; 64^3 38 / 41 and 36 /
+// 52.  float32 128 x 127 x 129 114 / 84 and 162 / 124, 128^3 69 / 83.
+static bool copied_box(const pc_streams* s, const int64_t lo[3], const int64_t hi[3], const void* at, size_t bytes,
+                       int read_in) {
+  const size_t row = (size_t)(hi[0] - lo[0]) * dsize(s->dtype);
+  const bool words = (((uintptr_t)at | row) & 15) == 0;
+  if (words && s->dtype == PC_F32) return false;
+  return bytes >= size_t(2) << (20 + (read_in ? 1 : 0) + (words ? 1 : 0));
+}
+
 static pc_status retrieve_common(const pc_streams* s, int k0, int k, const pc_box* box, void* buf, int read_in,
                                  void* cuda_stream) {
   cudaStream_t st = (cudaStream_t)cuda_stream;
@@ -832,6 +847,18 @@ static pc_status retrieve_common(const pc_streams* s, int k0, int k, const pc_bo
       // a large box in pinned host memory: decoded into device slabs and copied by the copy engines
       cudaStream_t cs = copy_stream();
       if (cs) return retrieve_pinned_slabs(s, k0, k, lo, hi, static_cast<char*>(buf), read_in, st, cs);
+    }
+    if (host && s->ndims == 3 && k > k0 && copied_box(s, lo, hi, kp, bytes, read_in)) {
+      Scratch scr(st);
+      void* d = nullptr;
+      if (scr.get(&d, bytes) == cudaSuccess) {
+        if (read_in) CK(cudaMemcpyAsync(d, buf, bytes, cudaMemcpyHostToDevice, st));
+        r = run_retrieve(s, k0, k, lo, hi, d, 1, st);
+        if (r != PC_OK) return r;
+        CK(cudaMemcpyAsync(buf, d, bytes, cudaMemcpyDeviceToHost, st));
+        return PC_OK;
+      }
+      cudaGetLastError();  // no memory for it: in place
     }
     // device memory, or pinned host memory written in place by the kernel
     return run_retrieve(s, k0, k, lo, hi, const_cast<void*>(kp), 1, st);
