@@ -551,9 +551,9 @@ void set_schedule(pc_batch* B, const Schedule& sc) {
 }
 
 // Captures H2D of the parameter blocks, the counters' reset, the batched
-// construction (kernel variant v: the 3D kernel for v / 3 + 1 CTAs per SM and,
-// on a parallel branch, the 1D/2D kernel with kSmallShapes[v % 3] warps per
-// CTA), the segmented scan and the D2H of the results.
+// construction (kernel variant v: variant v / 4 + 1 of the 3D kernel, see
+// batch3_ctas, and, on a parallel branch, the 1D/2D kernel with kSmallShapes[v % 4]
+// warps per CTA; the last variant is the kernel for both), the segmented scan and the D2H of the results.
 pc_status capture_graph(pc_batch* B, int v) {
   cudaStream_t st = B->st;
   cudaGraph_t g = nullptr;

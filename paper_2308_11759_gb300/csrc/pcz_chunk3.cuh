@@ -281,7 +281,7 @@ static __device__ __noinline__ typename Fmt<T>::U raw_form(const uint4* s_x, boo
 // transposed in registers, reductions over a brick take two shuffles, and what
 // a component costs per warp (votes, scans, the barrier) is shared by 512
 // values.  With 16 lanes per brick and 4 values per lane it took 582 (float32)
-// and 997 (float64) warp instructions per brick and component, now 187 and 284;
+// and 997 (float64) warp instructions per brick and component, now 187 and 270;
 // 512^3 float32, 8 components: 10.16 -> 3.52 ms, 256 x 384 x 384 float64, 12
 // components: 8.77 -> 3.10 ms.  It runs at 0.71 (float32; ALU pipe 0.67) and
 // 0.47 (float64) of the issue peak.

@@ -7,9 +7,13 @@
 // coefficients and group-tested bit planes (Sec. 2).  The paper does not fix
 // the coder's internals; the project rules R4..R15 do, and each is restated
 // where it is implemented.  All floating-point work here is IEEE
-// round-to-nearest with no contraction: the only arithmetic on T values is
-// one add or one subtract (explicit _rn intrinsics); scaling and conversions
-// are done on the bit patterns with integer operations.
+// round-to-nearest with no contraction by the compiler, and the only arithmetic
+// on T values that rounds is one add or one subtract (explicit _rn intrinsics) and
+// the conversion of an integer coefficient.  What else runs in floating point is
+// exact: products by powers of two that stay normal, their fused adds (which round
+// once, as the add does), and the lifting, in float, of values that need at most
+// 24 bits.  Scales outside those ranges work on the bit patterns with integer
+// operations.
 #pragma once
 
 #include <cstdint>
@@ -226,19 +230,6 @@ __device__ __forceinline__ typename Fmt<T>::U dequantize_bits(typename Fmt<T>::S
   return q < 0 ? (out | F::SIGN) : out;
 }
 
-// R13 for float fields, the common case in a few instructions: when 2^-s is a
-// normal float and the result is normal or overflows, int->float rounding
-// followed by an exact power-of-two scaling is the single correct rounding.
-// Other cases take the general path.
-__device__ __forceinline__ float dequantize_f32(int32_t q, int s) {
-  if (q == 0) return 0.0f;
-  const uint32_t a = q < 0 ? 0u - (uint32_t)q : (uint32_t)q;
-  const int nb = 32 - __clz(a);
-  if (s >= -127 && s <= 126 && nb - s >= -125)
-    return __fmul_rn(__int2float_rn(q), __uint_as_float((uint32_t)(127 - s) << 23));
-  return __uint_as_float(dequantize_bits<float>(q, s));
-}
-
 // R13 for float64 when the result is known to be normal and finite (s in
 // [-960, 1022], see dequantize_line): the 53 leading bits of |q| rounded to
 // nearest, ties to even, by adding half an ulp less one plus the kept lsb
@@ -255,14 +246,6 @@ __device__ __forceinline__ uint64_t dequantize_f64_normal(int64_t q, int s) {
     r = a << (-sh);
   const uint64_t bits = ((uint64_t)(nb - s + 1021) << 52) + r;  // r's bit 52 completes the exponent
   return q < 0 ? (bits | Fmt<double>::SIGN) : bits;
-}
-
-template <typename T>
-__device__ __forceinline__ T dequantize_val(typename Fmt<T>::S q, int s) {
-  if constexpr (sizeof(T) == 4)
-    return dequantize_f32(q, s);
-  else
-    return Fmt<T>::val(dequantize_bits<T>(q, s));
 }
 
 // R13 for the 4 values of a line that share the block's scale s.
@@ -331,39 +314,11 @@ __device__ __forceinline__ double scaled_f32_to_f64(float r, uint32_t adj) {
   return __hiloint2double(r == 0.0f ? 0 : (int)hi, b << 29);
 }
 
-// The bit pattern of |v| shifted left by one place (the sign shifted out),
-// in an integer instruction the compiler cannot see through.  Masking the
-// sign bit of a float64 pattern instead is recognised as fabs and emitted as
-// an add on the FP64 pipe, which on this part costs as much as a real add.
-// Shifted patterns order like the magnitudes (NaN above +inf above every
-// finite value).
-__device__ __forceinline__ uint64_t mag2_bits(double v) {
-  uint64_t r;
-  asm("shl.b64 %0, %1, 1;" : "=l"(r) : "l"((uint64_t)__double_as_longlong(v)));
-  return r;
-}
-
-// |e| <= tau on bit patterns: tb is the pattern of the largest T value not
-// above tau, so the comparison is exact; NaN and +-inf fail it.
-template <typename T>
-__device__ __forceinline__ bool within(T e, typename Fmt<T>::U tb) {
-  using F = Fmt<T>;
-  if constexpr (sizeof(T) == 8)
-    return mag2_bits(e) <= (tb << 1);
-  else
-    return (F::bits(e) & F::ABS) <= tb;
-}
-
-template <typename T>
-__device__ __forceinline__ bool not_finite(T v) {
-  using F = Fmt<T>;
-  return (F::bits(v) & F::INF) == F::INF;
-}
-
 // ---------------------------------------------------------------------------
-// R8: sequency order of the 4^3 coefficients, ties by brick position.
-// kPerm3.pos[r] = brick position of the r-th coded coefficient.  Built at
-// compile time by ranking every position.
+// R8: sequency order of the coefficients, ties by brick position.  make_perm(n).pos[r]
+// = brick position of the r-th coded coefficient of n; make_rank below is the
+// inverse for 4^3 (kRank3 in the 3D kernels).  Built at compile time by ranking
+// every position.
 // ---------------------------------------------------------------------------
 struct PermTable {
   int8_t pos[64];
@@ -454,8 +409,6 @@ __device__ __forceinline__ unsigned long long warp_max_u64(unsigned mask, unsign
   const unsigned lo = __reduce_max_sync(mask, (unsigned)(v >> 32) == hi ? (unsigned)v : 0u);
   return ((unsigned long long)hi << 32) | lo;
 }
-
-__device__ __forceinline__ uint64_t low_mask64(int n) { return n >= 64 ? ~0ull : ((1ull << n) - 1); }
 
 // One x-line of a brick (4 consecutive values) between registers and memory:
 // a single 16-byte access per 16 bytes when the line is whole and aligned
@@ -569,7 +522,8 @@ __device__ __forceinline__ void transpose32_lane(uint32_t (&a)[16]) {
 
 // |v| as an integer that orders like it (NaN above +inf above every finite
 // value): the bit pattern without its sign.  float64 masks the high word only:
-// masking the whole pattern is recognised as fabs and emitted on the FP64 pipe.
+// masking the whole pattern is recognised as fabs and emitted as an add on the
+// FP64 pipe, which costs as much as a real one.
 __device__ __forceinline__ uint32_t magnitude(float v) { return __float_as_uint(v) & 0x7FFFFFFFu; }
 __device__ __forceinline__ uint64_t magnitude(double v) {
   return ((uint64_t)((uint32_t)__double2hiint(v) & 0x7FFFFFFFu) << 32) | (uint32_t)__double2loint(v);

@@ -33,8 +33,8 @@
 // component, now 107 and 127; 512^3 float32: k = 6 2.87 -> 1.71 ms, k = 1 0.86 ->
 // 0.44 ms; 256 x 384 x 384 float64: k = 8 1.29 -> 0.89 ms; refinement from k = 1 to
 // 8 in place 7.06 -> 3.39 and 3.13 -> 1.75 ms (nearly half of it had gone to the
-// index pass and the sort).  With what few bricks need (any planes, RAW) out of
-// line, nothing spills and the common path is shorter to fetch: 512^3 float32 k =
+// index pass and the sort).  With what most streams' bricks do not need (more than
+// 16 planes of a component, RAW) out of line, nothing spills and the common path is shorter to fetch: 512^3 float32 k =
 // 6 1.72 -> 1.68 ms, 252 x 380 x 384 float64 k = 1 204 -> 185 us, refinement by one
 // component 198 -> 183 us.  (Code that does not even run costs here: a prefetch
 // behind a condition that is never true made k = 6 7 % slower.)
@@ -390,7 +390,7 @@ __device__ __forceinline__ void store_lines(const BoxJob& J, const BrickLane& L,
 // Float64 partial sums in fixed point.  As long as every partial sum of a brick
 // is a multiple of some 2^e below 2^(e + 51), no addition rounds, and the sums can
 // be kept as 64-bit integers in units of 2^e: the FP64 pipe (2 lanes per SM and
-// clock, 64 cycles for a warp's addition) then sees one operation per value
+// clock, 16 clocks for a warp's addition) then sees one operation per value
 // instead of one per component.  `lead` is the first coded component's highest
 // plane, as an exponent (each component is below 2^(lead + 5)), depth = 46 -
 // ceil(log2 k) the bits below it, e = lead - depth.  A component that does not
