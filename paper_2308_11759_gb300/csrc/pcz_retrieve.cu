@@ -276,7 +276,9 @@ __device__ __forceinline__ void parse_task(const BoxJob& J, unsigned int* err, i
   int at = 0;
   if (lane == 31) at = atomicAdd(used, incl);
   at = __shfl_sync(0xffffffffu, at, 31) + incl - nw;
-  if (coded) ok = PCZ_CHECK(words_in<T>(at, nw), 3) && parse_planes(br, pos, end, nw, words_at<T>(pool, spill, at, nw), lut);
+  if (coded)
+    ok = PCZ_CHECK(words_in<T>(at, nw), 3) &&
+         parse_planes(br, pos, end, nw, words_at<T>(pool, spill, at, nw), lut);
   if (!ok) {
     atomicOr(err, 1u);
     mode = kModeZero;
@@ -582,7 +584,8 @@ __device__ __forceinline__ void add_component(int how, const BlockMeta* bm, cons
   if ((how & 3) == kDecodeFloat8) {
     const int base = max(top, 7) - 7;
     const uint32_t keep = nw > 0 ? ((1u << nw) - 1u) << (p - base) : 0u;
-    const uint16_t* pc = reinterpret_cast<const uint16_t*>(pool + (from_pool(nw, m.at + top - base, 7) ? m.at + top - base : 7)) + q;  // plane base
+    const int last = m.at + top - base;  // word of plane base
+    const uint16_t* pc = reinterpret_cast<const uint16_t*>(pool + (from_pool(nw, last, 7) ? last : 7)) + q;
     uint32_t a[4];
 #pragma unroll
     for (int j = 0; j < 4; ++j) a[j] = (uint32_t)pc[-4 * j] | ((uint32_t)pc[-4 * (j + 4)] << 16);
@@ -622,7 +625,8 @@ __device__ __forceinline__ void add_component(int how, const BlockMeta* bm, cons
   } else if ((how & 3) == kDecodeInt16) {
     const int base = max(top, 15) - 15;
     const uint32_t keep = nw > 0 ? ((1u << nw) - 1u) << (p - base) : 0u;
-    const uint16_t* pc = reinterpret_cast<const uint16_t*>(pool + (from_pool(nw, m.at + top - base, 15) ? m.at + top - base : 15)) + q;
+    const int last = m.at + top - base;
+    const uint16_t* pc = reinterpret_cast<const uint16_t*>(pool + (from_pool(nw, last, 15) ? last : 15)) + q;
     uint32_t a[8];
 #pragma unroll
     for (int j = 0; j < 8; ++j) a[j] = (uint32_t)pc[-4 * j] | ((uint32_t)pc[-4 * (j + 8)] << 16);
